@@ -161,12 +161,12 @@ extern "C" tdcfie_status tdcfie_assemble(tdcfie_t h) {
     CK(zalloc(&h->G, ne * ne));
     CK(cudaStreamSynchronize(s));
     t0 = now_s();
-    launch_retarded_efie(h->dm, h->dt, h->K, h->T0, M.D, h->S, h->Phi, h->opts.time_order, s);
+    launch_retarded_efie(h->dm, h->dt, h->K, h->T0, h->S, h->Phi, h->opts.time_order, s);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s));
     h->asm_s[1] = now_s() - t0;
     t0 = now_s();
-    launch_retarded_mfie(h->dm, h->dt, h->K, M.D, h->MM, h->opts.time_order, s);
+    launch_retarded_mfie(h->dm, h->dt, h->K, h->MM, h->opts.time_order, s);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s));
     h->asm_s[2] = now_s() - t0;

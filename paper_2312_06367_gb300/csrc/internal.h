@@ -43,7 +43,7 @@ void gauss_legendre(int n, double* x, double* w);
 constexpr int NANG = 6;       // Gauss points per angular piece
 constexpr int NRAD = 5;       // Gauss points per radial piece
 constexpr double PIECE = 1.0; // largest psi / u width of a piece
-constexpr int LAGW = 16;      // lag window held per thread in the retarded kernels
+constexpr int LAGW = 16;      // lags formed per pass of a thread in the retarded kernels
 
 struct RuleTables {
     double ax[NANG], aw[NANG], rx[NRAD], rw[NRAD];
@@ -60,9 +60,9 @@ struct DevMesh {
 void set_rule_tables(const RuleTables& r, cudaStream_t s);
 // symmetric degree-5 rule on a triangle: per point barycentric (a, b, c) and weight (sum 1)
 void triangle_rule7(double r7[7][4]);
-void launch_retarded_efie(const DevMesh& m, double dt, int K, double T0, double D, double* S, double* Phi,
-                          int order, cudaStream_t s);
-void launch_retarded_mfie(const DevMesh& m, double dt, int K, double D, double* MM, int order, cudaStream_t s);
+void launch_retarded_efie(const DevMesh& m, double dt, int K, double T0, double* S, double* Phi, int order,
+                          cudaStream_t s);
+void launch_retarded_mfie(const DevMesh& m, double dt, int K, double* MM, int order, cudaStream_t s);
 void launch_static(const DevMesh& m, double kappa, double* Zs, double* Psi, double* M, double* G, cudaStream_t s);
 
 // ---------------------------------------------------------------- dense FP64 helpers (linalg.cu)
