@@ -112,15 +112,18 @@ static tdcfie_status upload_mesh(tdcfie_t h) {
     const Mesh& M = h->mesh;
     DevMesh& d = h->dm;
     double *V, *tsign, *fV, *bc_phi;
-    int *F, *tedge, *cp, *cm, *fF, *fparent, *fvert, *val, *bc_ptr, *bc_fn;
+    int *F, *tedge, *cp, *cm, *fF, *fparent, *fvert, *val, *bc_ptr, *bc_fn, *touch;
     if ((e = put(h, &V, M.V)) || (e = put(h, &F, M.F)) || (e = put(h, &tedge, M.tedge)) || (e = put(h, &tsign, M.tsign)) ||
         (e = put(h, &cp, M.cplus)) || (e = put(h, &cm, M.cminus)) || (e = put(h, &fV, M.fV)) || (e = put(h, &fF, M.fF)) ||
         (e = put(h, &fparent, M.fparent)) || (e = put(h, &fvert, M.fvert)) || (e = put(h, &val, M.valence)) ||
-        (e = put(h, &bc_ptr, M.bc_ptr)) || (e = put(h, &bc_fn, M.bc_fn)) || (e = put(h, &bc_phi, M.bc_phi)))
+        (e = put(h, &bc_ptr, M.bc_ptr)) || (e = put(h, &bc_fn, M.bc_fn)) || (e = put(h, &bc_phi, M.bc_phi)) ||
+        (e = put(h, &touch, M.touch)))
         return cuda_fail(h, e, "upload mesh");
     d.V = V; d.F = F; d.tedge = tedge; d.tsign = tsign; d.cplus_ = cp; d.cminus_ = cm;
     d.fV = fV; d.fF = fF; d.fparent = fparent; d.fvert = fvert; d.valence = val;
     d.bc_ptr = bc_ptr; d.bc_fn = bc_fn; d.bc_phi = bc_phi;
+    d.touch = touch;
+    d.ntouch = (int)(M.touch.size() / 2);
     d.nv = M.nv; d.nc = M.nc; d.ne = M.ne; d.nf = M.nf;
     e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "upload mesh");
@@ -161,12 +164,12 @@ extern "C" tdcfie_status tdcfie_assemble(tdcfie_t h) {
     CK(zalloc(&h->G, ne * ne));
     CK(cudaStreamSynchronize(s));
     t0 = now_s();
-    launch_retarded_efie(h->dm, h->dt, h->K, h->T0, h->S, h->Phi, h->opts.time_order, s);
+    launch_retarded_efie(h->dm, h->dt, h->K, h->T0, M.lmax, h->S, h->Phi, h->opts.time_order, s);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s));
     h->asm_s[1] = now_s() - t0;
     t0 = now_s();
-    launch_retarded_mfie(h->dm, h->dt, h->K, h->MM, h->opts.time_order, s);
+    launch_retarded_mfie(h->dm, h->dt, h->K, M.lmax, h->MM, h->opts.time_order, s);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s));
     h->asm_s[2] = now_s() - t0;
@@ -480,7 +483,7 @@ extern "C" tdcfie_status tdcfie_destroy(tdcfie_t h) {
     if (!h) return TDCFIE_OK;
     free_plan(h);
     const void* ptrs[] = {h->dm.V, h->dm.F, h->dm.tedge, h->dm.tsign, h->dm.cplus_, h->dm.cminus_, h->dm.fV, h->dm.fF,
-                          h->dm.fparent, h->dm.fvert, h->dm.valence, h->dm.bc_ptr, h->dm.bc_fn, h->dm.bc_phi,
+                          h->dm.fparent, h->dm.fvert, h->dm.valence, h->dm.bc_ptr, h->dm.bc_fn, h->dm.bc_phi, h->dm.touch,
                           h->S, h->Phi, h->MM, h->Zs, h->Psi, h->Mst, h->G, h->PS, h->L1, h->L2, h->A, h->T, h->T0inv,
                           h->H, h->Zh, h->PinvS, h->dexc};
     for (const void* p : ptrs) if (p) cudaFree(const_cast<void*>(p));

@@ -22,6 +22,8 @@ struct Mesh {
     std::vector<double> tsign;    // nc x 3: +1 if the triangle is c+ of that edge
     std::vector<int> valence;     // nv: triangles at each vertex
     double D = 0.0;               // largest vertex-to-vertex distance
+    double lmax = 0.0;            // longest edge
+    std::vector<int> touch;       // pairs of triangles that share a vertex (ordered, each with itself too)
     // barycentric refinement
     int nf = 0;
     std::vector<double> fV;       // (nv + ne + nc) x 3
@@ -43,7 +45,7 @@ void gauss_legendre(int n, double* x, double* w);
 constexpr int NANG = 6;       // Gauss points per angular piece
 constexpr int NRAD = 5;       // Gauss points per radial piece
 constexpr double PIECE = 1.0; // largest psi / u width of a piece
-constexpr int LAGW = 16;      // lags formed per pass of a thread in the retarded kernels
+constexpr int LAGW = 8;       // most lags formed per window of the retarded kernels
 
 struct RuleTables {
     double ax[NANG], aw[NANG], rx[NRAD], rw[NRAD];
@@ -54,15 +56,16 @@ struct DevMesh {
     const double* V; const int* F; const int* tedge; const double* tsign; const int* cplus_; const int* cminus_;
     const double* fV; const int* fF; const int* fparent; const int* fvert; const int* valence;
     const int* bc_ptr; const int* bc_fn; const double* bc_phi;
-    int nv, nc, ne, nf;
+    const int* touch;             // ntouch x 2: ordered pairs of triangles that share a vertex
+    int nv, nc, ne, nf, ntouch;
 };
 
 void set_rule_tables(const RuleTables& r, cudaStream_t s);
 // symmetric degree-5 rule on a triangle: per point barycentric (a, b, c) and weight (sum 1)
 void triangle_rule7(double r7[7][4]);
-void launch_retarded_efie(const DevMesh& m, double dt, int K, double T0, double* S, double* Phi, int order,
+void launch_retarded_efie(const DevMesh& m, double dt, int K, double T0, double lmax, double* S, double* Phi, int order,
                           cudaStream_t s);
-void launch_retarded_mfie(const DevMesh& m, double dt, int K, double* MM, int order, cudaStream_t s);
+void launch_retarded_mfie(const DevMesh& m, double dt, int K, double lmax, double* MM, int order, cudaStream_t s);
 void launch_static(const DevMesh& m, double kappa, double* Zs, double* Psi, double* M, double* G, cudaStream_t s);
 
 // ---------------------------------------------------------------- dense FP64 helpers (linalg.cu)

@@ -97,6 +97,28 @@ std::string build_mesh(const double* V, int64_t nv64, const int32_t* F, int64_t 
     m.D = std::sqrt(D);
 
     // ---------------- barycentric refinement
+    // longest edge; ordered pairs of triangles that share a vertex
+    for (int e = 0; e < ne; ++e) {
+        double l2 = 0.0;
+        for (int k = 0; k < 3; ++k) {
+            const double x = m.V[3 * m.E[2 * e] + k] - m.V[3 * m.E[2 * e + 1] + k];
+            l2 += x * x;
+        }
+        m.lmax = std::max(m.lmax, std::sqrt(l2));
+    }
+    {
+        std::vector<std::vector<int>> at(nv);
+        for (int c = 0; c < nc; ++c)
+            for (int j = 0; j < 3; ++j) at[m.F[3 * c + j]].push_back(c);
+        std::vector<int> nb;
+        for (int c = 0; c < nc; ++c) {
+            nb.clear();
+            for (int j = 0; j < 3; ++j) nb.insert(nb.end(), at[m.F[3 * c + j]].begin(), at[m.F[3 * c + j]].end());
+            std::sort(nb.begin(), nb.end());
+            nb.erase(std::unique(nb.begin(), nb.end()), nb.end());
+            for (int o : nb) { m.touch.push_back(c); m.touch.push_back(o); }
+        }
+    }
     const int nfv = nv + ne + nc;
     m.fV.resize(3 * (size_t)nfv);
     for (int i = 0; i < 3 * nv; ++i) m.fV[i] = m.V[i];
