@@ -205,7 +205,7 @@ extern "C" tdcfie_status tdcfie_set_excitation(tdcfie_t h, const tdcfie_plane_wa
         if (!(exc->width[r] > 0.0)) return fail(h, TDCFIE_E_ARG, "width must be positive");
         for (int i = 0; i < 9; ++i) if (!std::isfinite(buf[11 * r + i])) return fail(h, TDCFIE_E_ARG, "non-finite excitation");
     }
-    if (!h->dexc) CK(cudaMalloc(&h->dexc, sizeof(double) * buf.size()));
+    if (!h->dexc) CK(cudaMalloc(&h->dexc, sizeof(double) * buf.size()));     // (build_plan allocates it)
     CK(cudaMemcpyAsync(h->dexc, buf.data(), sizeof(double) * buf.size(), cudaMemcpyHostToDevice, h->stream));
     h->excited = true;
     return plan_reset(h);

@@ -1,15 +1,14 @@
 // Several scatterers marched together (the uneven batch).  Two forms, chosen at creation:
 //
 //  * Persistent (every member FP32, one incident wave, direct solve: the uneven-batch workload):
-//    ONE cooperative kernel per step walks a work list of all members' items -- plane-wave tests
-//    (32 edges), history partial sums (BCH rows of BQ blocks, into the member's per-block partial
-//    buffer), their reduction over the blocks in block order (32 edges), T_0^-1 rows, projector
-//    gathers (32 triangles), pseudo-inverse rows, post-processing (32 edges) -- with grid-wide
-//    barriers between the seven phases.  Warps take items from a per-phase counter; the items are listed
-//    longest first, so big scatterers start early and small ones fill the tail.  The row dot
-//    products use the same arithmetic as the per-handle step (simt.h), so every member's
-//    currents equal those of tdcfie_step bit for bit.  Rows per warp, warps per block and blocks
-//    per SM come from a measuring autotuner (tdcfie_batch_tune).
+//    ONE cooperative kernel per step runs the phases of the step of every member -- where a chunk
+//    starts, the envelopes, tests and pre-sums of its steps; the history rows inside the chunk, T_0^-1
+//    rows, projector gathers, pseudo-inverse rows, post-processing -- with grid-wide barriers in
+//    between.  The units of a phase (rows, edges, triangles of all members) are dealt to the warps in
+//    turn, so that every member spreads over the whole grid; no unit waits for a counter.  The
+//    arithmetic is that of the per-handle step (simt.h), so every member's currents equal those of
+//    tdcfie_step bit for bit.  Units per turn, warps per block and blocks per SM come from a
+//    measuring autotuner (tdcfie_batch_tune).
 //  * Graph branches (any other mix of precisions, waves or solvers): one CUDA graph holds one step
 //    of every handle, each on its own forked stream.
 // Either way a single graph launch advances all members; the handles keep their own blocks,
@@ -27,63 +26,48 @@ using namespace tdc;
 
 namespace tdc {
 
-struct BMember {            // device view of one member handle (FP32, one wave)
-    int ne, nc, nblk, ring;
-    const float* blocks;    // nblk x ne x ne: -A, alpha L2, -T_1 .. -T_{K-1}
-    const float* t0inv;     // ne x ne
-    const float* pinv;      // nc x nc
-    float *E, *H, *ringbuf, *b, *z, *u;
-    double* partial;        // nblk x ne per-block history sums
-    const int* pptr;
-    const int* pnE;
-    const float* px;
-    const float* pc;
-    const double* exc;
-    DevMesh m;
-    double dt, dtt;
-    Ctl* ctl;
-};
-
-struct BItem {
-    int member, first, count, block;   // block: first block of a history item (else 0)
-};
-
-enum { PH_RHS = 0, PH_HIST, PH_RED, PH_SOLVE, PH_PIN, PH_PINV, PH_POUT, NPH };
-constexpr int BCH = 8;                 // rows per work item of the row phases
-constexpr int BQ = 4;                  // blocks per history work item
+enum { PH_ENV = 0, PH_GATHER, PH_PRE, PH_HIST, PH_SOLVE, PH_PIN, PH_PINV, PH_POUT, NPH };
 constexpr uint64_t BWAIT_NS = 2000000000ull;
 
 struct BArgs {
-    const BMember* mem;
+    const SimtDev<float>* mem;
     int nmem;
-    const BItem* items[NPH];
-    int nitems[NPH];
-    unsigned* sync;     // [NPH] take counters, arrival count, generation, timeout flag
+    const int* first[NPH];   // first unit of every member in a phase, [nmem + 1]
+    unsigned* sync;          // arrival count, generation, timeout flag
 };
 
-__device__ __forceinline__ uint64_t bclock() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
+// units of a phase for one member (one warp works on a unit)
+static int phase_units(const StepPlan* p, int ph) {
+    const auto up = [](int64_t a, int b) { return (int)((a + b - 1) / b); };
+    switch (ph) {
+        case PH_ENV: return up((int64_t)p->npts * p->C, 32);
+        case PH_GATHER: return p->ne;
+        case PH_PRE: return up(p->ne, PRE_ROWS) * p->ngroups * up(p->C, PRE_COLS);
+        case PH_PIN: return up(p->nc, 32);
+        case PH_PINV: return up(p->nc, PRE_ROWS);
+        case PH_POUT: return up(p->ne, 32);
+        // rows of the history, of every lag that may be pushed, and of the solve
+        case PH_HIST: return up(p->ne, step_rows<1>()) * (1 + std::max(0, std::min(p->C - 1, p->K - 1) - 1));
+        default: return up(p->ne, step_rows<1>());
+    }
 }
 
 // grid-wide barrier of the co-resident blocks (cooperative launch); bounded spin
 __device__ __forceinline__ void grid_barrier(unsigned* sync) {
-    unsigned* count = sync + NPH;
-    volatile unsigned* gen = sync + NPH + 1;
+    volatile unsigned* gen = sync + 1;
     __syncthreads();
     if (threadIdx.x == 0) {
         const unsigned g = *gen;
         __threadfence();
-        if (atomicAdd(count, 1u) == gridDim.x - 1) {
-            *count = 0;
+        if (atomicAdd(sync, 1u) == gridDim.x - 1) {
+            *sync = 0;
             __threadfence();
-            atomicAdd(sync + NPH + 1, 1u);
+            atomicAdd(sync + 1, 1u);
         } else {
-            const uint64_t t0 = bclock();
+            const uint64_t t0 = device_ns();
             while (*gen == g) {
-                if (bclock() - t0 > BWAIT_NS) {
-                    atomicExch(sync + NPH + 2, 1u);
+                if (device_ns() - t0 > BWAIT_NS) {
+                    atomicExch(sync + 2, 1u);
                     break;
                 }
             }
@@ -93,142 +77,72 @@ __device__ __forceinline__ void grid_barrier(unsigned* sync) {
     __syncthreads();
 }
 
-// acc[i] = B_i . x for the nrows (<= ROWS) rows B_i = B0 + i ld of one warp, R = 1; the per-row
-// arithmetic is that of RowDot<float, 1> (four compensated lanes accumulators, FP64 combination),
-// but each float4 of x is loaded once for all rows
-template <int ROWS>
-__device__ __forceinline__ void rows_dot(const float* __restrict__ B0, int64_t ld, int nrows, int ncols,
-                                         const float* __restrict__ x, double* acc) {
-    const bool vec = ((ncols | (int)ld) & 3) == 0 &&
-                     ((reinterpret_cast<uintptr_t>(B0) | reinterpret_cast<uintptr_t>(x)) & 15) == 0;
-    if (!vec) {
-        for (int i = 0; i < nrows; ++i) RowDot<float, 1>::run(B0 + i * ld, ncols, x, 1, ncols, acc + i);
-        return;
-    }
-    const int lane = threadIdx.x & 31;
-    float hi[ROWS][4], lo[ROWS][4];
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) hi[i][c] = lo[i][c] = 0.f;
-    const float4* x4 = reinterpret_cast<const float4*>(x);
-    for (int j = lane; j < (ncols >> 2); j += 32) {
-        const float4 v = x4[j];
-#pragma unroll
-        for (int i = 0; i < ROWS; ++i)
-            if (i < nrows) {
-                const float4 a = reinterpret_cast<const float4*>(B0 + i * ld)[j];
-                ff_add(hi[i][0], lo[i][0], a.x, v.x);
-                ff_add(hi[i][1], lo[i][1], a.y, v.y);
-                ff_add(hi[i][2], lo[i][2], a.z, v.z);
-                ff_add(hi[i][3], lo[i][3], a.w, v.w);
-            }
-    }
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i) {
-        double v = 0.0;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) v += (double)hi[i][c] + (double)lo[i][c];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (i < nrows) acc[i] = v;
+__device__ __forceinline__ void batch_unit(int ph, const SimtDev<float>& d, int u, int lane) {
+    const int64_t n = d.ctl->n;
+    if (ph == PH_ENV) {
+        const int idx = 32 * u + lane;
+        if (idx < d.npts * d.C) {
+            const int i = idx % d.C, pt = idx / d.C;
+            d.env[idx] = env_point<float>(d.exc, n + i, d.dt, d.pts[3 * pt], d.pts[3 * pt + 1], d.pts[3 * pt + 2]);
+        }
+    } else if (ph == PH_GATHER) {
+        gather_edge<float>(d, u, 0, lane);
+    } else if (ph == PH_PRE) {
+        const int ctiles = (d.C + PRE_COLS - 1) / PRE_COLS, t = u % ctiles, g = u / ctiles % d.ngroups;
+        pre_item<float>(d, n, u / ctiles / d.ngroups * PRE_ROWS, g, t * PRE_COLS, lane);
+    } else if (ph == PH_HIST) {
+        hist_unit<float, 1>(d, n, u, lane);
+    } else if (ph == PH_SOLVE) {
+        solve_unit<float, 1>(d, n, u, lane);
+    } else if (ph == PH_PIN) {
+        if (32 * u + lane < d.nc) pin_value<float>(d, n, 0, 0, 32 * u + lane);
+    } else if (ph == PH_PINV) {
+        pinv_item<float>(d, 1, u * PRE_ROWS, 0, lane);
+    } else {
+        if (32 * u + lane < d.ne) pout_value<float>(d, n, 0, 0, 32 * u + lane);
     }
 }
 
-template <int ROWS>
-__device__ __forceinline__ void batch_item(int phase, const BMember& M, const BItem& it) {
+// one MOT step of every member; rows: consecutive units per turn of a warp
+__global__ void __launch_bounds__(256) k_batch_step(const __grid_constant__ BArgs a, int rows) {
     const int lane = threadIdx.x & 31;
-    const int64_t n = M.ctl->n;
-    const int ne = M.ne;
-    float* yn = M.ringbuf + (n % M.ring) * (int64_t)ne;
-    if (phase == PH_RHS) {
-        const int e = it.first + lane;
-        if (lane < it.count) {
-            float ev, hv;
-            rhs_edge<float>(M.exc, n, M.dt, e, M.pptr, M.px, M.pc, M.pnE, ev, hv);
-            M.E[e] = ev;
-            M.H[e] = hv;
-        }
-    } else if (phase == PH_HIST) {
-        // per-block partial sums (the arithmetic of k_history_rows), reduced in block order by PH_RED
-        const int q1 = min(M.nblk, it.block + BQ);
-        for (int q = it.block; q < q1; ++q) {
-            const float* x;
-            if (q == 0) x = M.E;
-            else if (q == 1) x = M.H;
-            else {
-                int64_t slot = (n - (q - 1)) % M.ring;
-                if (slot < 0) slot += M.ring;
-                x = M.ringbuf + slot * (int64_t)ne;
+    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    bool start = false;      // some member starts a chunk (uniform: no counter moves before the end)
+    for (int s = 0; s < a.nmem; ++s) start |= (a.mem[s].ctl->n - 1) % a.mem[s].C == 0;
+    for (int ph = start ? PH_ENV : PH_HIST; ph < NPH; ++ph) {
+        const int* first = a.first[ph];
+        const int total = first[a.nmem];
+        int s = 0;
+        for (int64_t u0 = warp * rows; u0 < total; u0 += nwarps * rows)
+            for (int64_t u = u0; u < min(u0 + rows, (int64_t)total); ++u) {
+                while (u >= first[s + 1]) ++s;
+                const SimtDev<float>& d = a.mem[s];
+                if (ph <= PH_PRE && (d.ctl->n - 1) % d.C != 0) continue;
+                batch_unit(ph, d, (int)(u - first[s]), lane);
             }
-            for (int r0 = it.first; r0 < it.first + it.count; r0 += ROWS) {
-                const int nr = min(ROWS, it.first + it.count - r0);
-                double acc[ROWS];
-                rows_dot<ROWS>(M.blocks + ((int64_t)q * ne + r0) * ne, ne, nr, ne, x, acc);
-                if (lane == 0)
-                    for (int i = 0; i < nr; ++i) M.partial[(int64_t)q * ne + r0 + i] = acc[i];
-            }
-        }
-    } else if (phase == PH_RED) {
-        const int e = it.first + lane;
-        if (lane < it.count) {
-            double v = 0.0;
-            for (int q = 0; q < M.nblk; ++q) v += M.partial[(int64_t)q * ne + e];
-            M.b[e] = (float)v;
-        }
-    } else if (phase == PH_SOLVE || phase == PH_PINV) {
-        const bool solve = phase == PH_SOLVE;
-        const int cols = solve ? ne : M.nc;
-        const float* Mx = solve ? M.t0inv : M.pinv;
-        const float* x = solve ? M.b : M.z;
-        float* dst = solve ? yn : M.u;
-        for (int r0 = it.first; r0 < it.first + it.count; r0 += ROWS) {
-            const int nr = min(ROWS, it.first + it.count - r0);
-            double acc[ROWS];
-            rows_dot<ROWS>(Mx + (int64_t)r0 * cols, cols, nr, cols, x, acc);
-            if (lane == 0)
-                for (int i = 0; i < nr; ++i) dst[r0 + i] = (float)acc[i];
-        }
-    } else if (phase == PH_PIN) {
-        const int c = it.first + lane;
-        if (lane < it.count) {
-            const float* yp = M.ringbuf + ((n - 1) % M.ring) * (int64_t)ne;
-            M.z[c] = (float)project_in_value<float>(M.m, c, yn, yp, n == 1, M.dtt);
-        }
-    } else {   // PH_POUT
-        const int e = it.first + lane;
-        if (lane < it.count) {
-            const float val = yn[e] + M.u[M.m.cplus_[e]] - M.u[M.m.cminus_[e]];
-            Ctl* ctl = M.ctl;
-            if (!isfinite((double)val) && atomicCAS(&ctl->status, 0, (int)TDCFIE_E_NONFINITE) == 0) ctl->bad_step = n;
-            if (ctl->out) reinterpret_cast<float*>(ctl->out)[(n - ctl->n0) * (int64_t)ne + e] = val;
-            if (ctl->yout) reinterpret_cast<float*>(ctl->yout)[(n - ctl->n0) * (int64_t)ne + e] = yn[e];
-        }
-    }
-}
-
-// one MOT step of every member: seven phases over the work lists, grid barriers in between
-template <int ROWS>
-__global__ void k_batch_step(BArgs a) {
-    const int lane = threadIdx.x & 31;
-    for (int ph = 0; ph < NPH; ++ph) {
-        const BItem* items = a.items[ph];
-        const int nitems = a.nitems[ph];
-        for (;;) {
-            int i = 0;
-            if (lane == 0) i = (int)atomicAdd(a.sync + ph, 1u);
-            i = __shfl_sync(0xffffffffu, i, 0);
-            if (i >= nitems) break;
-            const BItem it = items[i];
-            batch_item<ROWS>(ph, a.mem[it.member], it);
-        }
         grid_barrier(a.sync);
     }
-    // every block has passed the last barrier: advance the members and rearm the counters
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        for (int s = 0; s < a.nmem; ++s) a.mem[s].ctl->n += 1;
-        for (int ph = 0; ph < NPH; ++ph) a.sync[ph] = 0;
-        __threadfence();
+    // every block has passed the last barrier: advance the members
+    if (blockIdx.x == 0)
+        for (int s = threadIdx.x; s < a.nmem; s += blockDim.x) {
+            Ctl* c = a.mem[s].ctl;
+            c->n += 1;
+            c->p0 = c->n;
+        }
+}
+
+// output base of the next steps of every member
+__global__ void k_batch_outputs(const __grid_constant__ BArgs a, void* const* outs) {
+    for (int s = threadIdx.x; s < a.nmem; s += blockDim.x) {
+        Ctl* c = a.mem[s].ctl;
+        c->n0 = c->n;
+        c->out = outs ? outs[s] : nullptr;
+        c->yout = nullptr;
     }
+}
+__global__ void k_batch_status(const __grid_constant__ BArgs a, Ctl* out) {
+    for (int s = threadIdx.x; s < a.nmem; s += blockDim.x) out[s] = *a.mem[s].ctl;
 }
 
 }  // namespace tdc
@@ -245,11 +159,13 @@ struct tdcfie_batch_s {
     int64_t launches_per_step = 0;
     // persistent form
     bool persistent = false;
-    BMember* dmem = nullptr;
-    BItem* ditems = nullptr;
+    SimtDev<float>* dmem = nullptr;
+    int* dfirst = nullptr;
     unsigned* dsync = nullptr;
+    void** douts = nullptr;       // the members' output pointers of a call
+    Ctl* dstat = nullptr;         // the members' step states after a call
     BArgs args{};
-    int rows = 2, threads = 256, blocks_per_sm = 1, grid = 0, sms = 0;
+    int rows = 1, threads = 256, blocks_per_sm = 1, grid = 0, sms = 0;
     double hist_bytes = 0.0;
 };
 
@@ -262,7 +178,7 @@ static void destroy_batch(tdcfie_batch_t b) {
     for (cudaEvent_t e : {b->fork, b->t0, b->t1})
         if (e) cudaEventDestroy(e);
     if (b->main) cudaStreamDestroy(b->main);
-    for (void* p : {(void*)b->dmem, (void*)b->ditems, (void*)b->dsync})
+    for (void* p : {(void*)b->dmem, (void*)b->dfirst, (void*)b->dsync, (void*)b->douts, (void*)b->dstat})
         if (p) cudaFree(p);
     delete b;
 }
@@ -273,8 +189,7 @@ static bool persistent_member(tdcfie_t h) {
     return h->plan && h->plan->prec == TDCFIE_FP32 && h->plan->R == 1 && !h->plan->gmres_on && h->plan->blocks;
 }
 
-template <int ROWS>
-static cudaError_t launch_persistent_t(tdcfie_batch_t b, cudaStream_t s) {
+static cudaError_t launch_persistent(tdcfie_batch_t b, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(b->grid);
     cfg.blockDim = dim3(b->threads);
@@ -285,86 +200,46 @@ static cudaError_t launch_persistent_t(tdcfie_batch_t b, cudaStream_t s) {
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_batch_step<ROWS>, b->args);
+    return cudaLaunchKernelEx(&cfg, k_batch_step, b->args, b->rows);
 }
 
-static cudaError_t launch_persistent(tdcfie_batch_t b, cudaStream_t s) {
-    switch (b->rows) {
-        case 1: return launch_persistent_t<1>(b, s);
-        case 4: return launch_persistent_t<4>(b, s);
-        default: return launch_persistent_t<2>(b, s);
-    }
-}
-
-static int max_blocks_per_sm(int rows, int threads) {
+static int max_blocks_per_sm(int threads) {
     int nb = 0;
-    cudaError_t e;
-    if (rows == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_step<1>, threads, 0);
-    else if (rows == 4) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_step<4>, threads, 0);
-    else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_step<2>, threads, 0);
-    return e == cudaSuccess ? nb : 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_step, threads, 0) == cudaSuccess ? nb : 0;
 }
 
-// work lists of the seven phases, longest items first (by the bytes they stream)
+// members' views and the units of every phase
 static cudaError_t build_persistent(tdcfie_batch_t b) {
     const int n = (int)b->hs.size();
-    std::vector<BMember> mem(n);
-    std::vector<std::vector<std::pair<double, BItem>>> lists(NPH);
+    std::vector<SimtDev<float>> mem(n);
+    std::vector<int> first((size_t)NPH * (n + 1), 0);
     b->hist_bytes = 0.0;
     for (int s = 0; s < n; ++s) {
-        tdcfie_t h = b->hs[s];
-        StepPlan* p = h->plan;
-        BMember& M = mem[s];
-        M.ne = p->ne; M.nc = p->nc; M.nblk = p->nblk; M.ring = p->ring;
-        M.blocks = (const float*)p->blocks; M.t0inv = (const float*)p->t0inv; M.pinv = (const float*)p->pinv;
-        M.E = (float*)p->E; M.H = (float*)p->Hv; M.ringbuf = (float*)p->ringbuf;
-        M.b = (float*)p->b; M.z = (float*)p->z; M.u = (float*)p->u; M.partial = (double*)p->partial;
-        M.pptr = p->pptr; M.pnE = p->pnE; M.px = (const float*)p->px; M.pc = (const float*)p->pc;
-        M.exc = h->dexc; M.m = h->dm; M.dt = h->dt; M.dtt = h->dtt; M.ctl = p->ctl;
+        const StepPlan* p = b->hs[s]->plan;
+        mem[s] = simt_view<float>(b->hs[s], *p);
         b->hist_bytes += (double)p->nblk * p->ne * p->ne * 4.0;
-        for (int e = 0; e < p->ne; e += 32) {
-            const BItem it{s, e, std::min(32, p->ne - e), 0};
-            lists[PH_RHS].push_back({(double)p->ne, it});
-            lists[PH_RED].push_back({(double)p->nblk, it});
-            lists[PH_POUT].push_back({(double)p->ne, it});
-        }
-        for (int c = 0; c < p->nc; c += 32) lists[PH_PIN].push_back({(double)p->nc, BItem{s, c, std::min(32, p->nc - c), 0}});
-        for (int r = 0; r < p->ne; r += BCH) {
-            const int cnt = std::min(BCH, p->ne - r);
-            for (int q = 0; q < p->nblk; q += BQ)
-                lists[PH_HIST].push_back({(double)std::min(BQ, p->nblk - q) * p->ne * cnt, BItem{s, r, cnt, q}});
-            lists[PH_SOLVE].push_back({(double)p->ne * cnt, BItem{s, r, cnt, 0}});
-        }
-        for (int r = 0; r < p->nc; r += BCH)
-            lists[PH_PINV].push_back({(double)p->nc * std::min(BCH, p->nc - r), BItem{s, r, std::min(BCH, p->nc - r), 0}});
-    }
-    std::vector<BItem> all;
-    std::vector<size_t> off(NPH);
-    for (int ph = 0; ph < NPH; ++ph) {
-        std::stable_sort(lists[ph].begin(), lists[ph].end(),
-                         [](const std::pair<double, BItem>& x, const std::pair<double, BItem>& y) { return x.first > y.first; });
-        off[ph] = all.size();
-        for (auto& pr : lists[ph]) all.push_back(pr.second);
-        b->args.nitems[ph] = (int)lists[ph].size();
+        for (int ph = 0; ph < NPH; ++ph) first[ph * (n + 1) + s + 1] = first[ph * (n + 1) + s] + phase_units(p, ph);
     }
     cudaError_t e;
-    if ((e = cudaMalloc(&b->dmem, sizeof(BMember) * n)) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&b->ditems, sizeof(BItem) * all.size())) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&b->dsync, sizeof(unsigned) * (NPH + 3))) != cudaSuccess) return e;
-    if ((e = cudaMemcpy(b->dmem, mem.data(), sizeof(BMember) * n, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
-    if ((e = cudaMemcpy(b->ditems, all.data(), sizeof(BItem) * all.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
-    if ((e = cudaMemset(b->dsync, 0, sizeof(unsigned) * (NPH + 3))) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&b->dmem, sizeof(SimtDev<float>) * n)) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&b->dfirst, sizeof(int) * first.size())) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&b->dsync, sizeof(unsigned) * 3)) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&b->douts, sizeof(void*) * n)) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&b->dstat, sizeof(Ctl) * n)) != cudaSuccess) return e;
+    if ((e = cudaMemcpy(b->dmem, mem.data(), sizeof(SimtDev<float>) * n, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    if ((e = cudaMemcpy(b->dfirst, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    if ((e = cudaMemset(b->dsync, 0, sizeof(unsigned) * 3)) != cudaSuccess) return e;
     b->args.mem = b->dmem;
     b->args.nmem = n;
-    for (int ph = 0; ph < NPH; ++ph) b->args.items[ph] = b->ditems + off[ph];
+    for (int ph = 0; ph < NPH; ++ph) b->args.first[ph] = b->dfirst + ph * (n + 1);
     b->args.sync = b->dsync;
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    b->rows = 2;
+    b->rows = 1;
     b->threads = 256;
-    b->blocks_per_sm = std::max(1, std::min(2, max_blocks_per_sm(b->rows, b->threads)));
-    b->grid = b->sms * b->blocks_per_sm;
+    b->blocks_per_sm = 1;
+    b->grid = b->sms;
     return cudaSuccess;
 }
 }  // namespace tdc
@@ -415,9 +290,19 @@ extern "C" tdcfie_status tdcfie_batch_step(tdcfie_batch_t b, int64_t nsteps, voi
     if (nsteps == 0) return TDCFIE_OK;
     cudaError_t e = cudaSetDevice(b->hs[0]->opts.device);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaSetDevice");
-    for (int64_t i = 0; i < n; ++i) {
-        const tdcfie_status st = plan_set_outputs(b->hs[i], currents_out ? currents_out[i] : nullptr, nullptr);
-        if (st != TDCFIE_OK) return fail(nullptr, st, "batch handle " + std::to_string(i) + ": " + b->hs[i]->err);
+    if (b->persistent) {
+        // one kernel sets every member's output base
+        if (currents_out) e = cudaMemcpyAsync(b->douts, currents_out, sizeof(void*) * n, cudaMemcpyHostToDevice, b->main);
+        if (e == cudaSuccess) {
+            k_batch_outputs<<<1, 256, 0, b->main>>>(b->args, currents_out ? b->douts : nullptr);
+            e = cudaGetLastError();
+        }
+        if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch outputs");
+    } else {
+        for (int64_t i = 0; i < n; ++i) {
+            const tdcfie_status st = plan_set_outputs(b->hs[i], currents_out ? currents_out[i] : nullptr, nullptr);
+            if (st != TDCFIE_OK) return fail(nullptr, st, "batch handle " + std::to_string(i) + ": " + b->hs[i]->err);
+        }
     }
     if (!b->exec) {
         e = cudaStreamBeginCapture(b->main, cudaStreamCaptureModeThreadLocal);
@@ -447,22 +332,24 @@ extern "C" tdcfie_status tdcfie_batch_step(tdcfie_batch_t b, int64_t nsteps, voi
         e = cudaGraphInstantiate(&b->exec, b->graph, 0);
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaGraphInstantiate (batch)");
     }
+    std::vector<Ctl> ctl(n);
+    unsigned timeout = 0;
     e = cudaEventRecord(b->t0, b->main);
     for (int64_t i = 0; i < nsteps && e == cudaSuccess; ++i) e = cudaGraphLaunch(b->exec, b->main);
     if (e == cudaSuccess) e = cudaEventRecord(b->t1, b->main);
+    if (e == cudaSuccess && b->persistent) {
+        k_batch_status<<<1, 256, 0, b->main>>>(b->args, b->dstat);
+        e = cudaMemcpyAsync(ctl.data(), b->dstat, sizeof(Ctl) * n, cudaMemcpyDeviceToHost, b->main);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&timeout, b->dsync + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, b->main);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->main);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch step");
     float ms = 0.f;
     cudaEventElapsedTime(&ms, b->t0, b->t1);
     b->last_step_ms = ms / (double)nsteps;
-    if (b->persistent) {
-        unsigned timeout = 0;
-        e = cudaMemcpy(&timeout, b->dsync + NPH + 2, sizeof(unsigned), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch status");
-        if (timeout) return fail(nullptr, TDCFIE_E_TIMEOUT, "a bounded grid-wide wait of the batch kernel ran out");
-    }
+    if (timeout) return fail(nullptr, TDCFIE_E_TIMEOUT, "a bounded grid-wide wait of the batch kernel ran out");
     for (int64_t i = 0; i < n; ++i) {
-        const tdcfie_status st = plan_check(b->hs[i]);
+        const tdcfie_status st = b->persistent ? plan_status(b->hs[i], ctl[i]) : plan_check(b->hs[i]);
         if (st != TDCFIE_OK) return fail(nullptr, st, "batch handle " + std::to_string(i) + ": " + b->hs[i]->err);
     }
     return TDCFIE_OK;
@@ -481,11 +368,13 @@ extern "C" tdcfie_status tdcfie_batch_tune(tdcfie_batch_t b, int64_t steps_per_c
             const tdcfie_status st = plan_set_outputs(h, nullptr, nullptr);
             if (st != TDCFIE_OK) return st;
         }
+        // whole chunks of every member, so that each candidate sees as many chunk starts
+        steps_per_candidate = (steps_per_candidate + 15) / 16 * 16;
         double best = 1e300;
         int br = b->rows, bt = b->threads, bb = b->blocks_per_sm;
         for (int rows : {1, 2, 4})
-            for (int threads : {128, 256, 512}) {
-                const int maxb = max_blocks_per_sm(rows, threads);
+            for (int threads : {64, 128, 256}) {
+                const int maxb = max_blocks_per_sm(threads);
                 for (int bps : {1, 2, 4}) {
                     if (bps > maxb) continue;
                     b->rows = rows; b->threads = threads; b->blocks_per_sm = bps; b->grid = b->sms * bps;
@@ -504,7 +393,7 @@ extern "C" tdcfie_status tdcfie_batch_tune(tdcfie_batch_t b, int64_t steps_per_c
         if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
         if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
         unsigned timeout = 0;
-        e = cudaMemcpy(&timeout, b->dsync + NPH + 2, sizeof(unsigned), cudaMemcpyDeviceToHost);
+        e = cudaMemcpy(&timeout, b->dsync + 2, sizeof(unsigned), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch status");
         if (timeout) return fail(nullptr, TDCFIE_E_TIMEOUT, "a bounded grid-wide wait of the batch kernel ran out");
         // the candidates marched the members: back to the start of the march

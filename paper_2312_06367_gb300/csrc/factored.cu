@@ -9,8 +9,7 @@
 // an entry is nonzero only for the few lags k whose time-basis support meets the distances of the
 // two basis functions, so that sum_k nnz is a few N^2 for every K, against K N^2 for the T_k.
 //
-// Per step n (one CUDA graph):
-//   rhs       e_n, h_n (the plane-wave tests of the dense path)
+// Per chunk of steps: e_n, h_n (the plane-wave tests of the dense path, simt.h).  Per step n:
 //   shells    z = [e_n + es ; h_n - mm ; eh]   (one warp per row of [S ; -MM' ; Phi], all lags)
 //   solve     y_n = W z,  W = T_0^-1 [-A | alpha L2 | -L1 Sigma]   (formed once in FP64)
 //   charges   q_n = Sigma^T y_n
@@ -164,9 +163,21 @@ struct ShellDot<double> {
     }
 };
 
+// hi + lo += a b, error-free (FMA product error, TwoSum); rounded operations only: a contracted
+// multiply-add here would break the error-free sums
+__device__ __forceinline__ void ff_add(float& hi, float& lo, float a, float b) {
+    const float p = __fmul_rn(a, b);
+    const float pe = fmaf(a, b, -p);        // a b = p + pe exactly
+    const float t = __fadd_rn(hi, p);        // TwoSum(hi, p) = t + te
+    const float bp = __fsub_rn(t, hi);
+    const float te = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bp)), __fsub_rn(p, bp));
+    hi = t;
+    lo = __fadd_rn(lo, __fadd_rn(te, pe));
+}
+
 template <>
 struct ShellDot<float> {
-    // error-free products and sums as in the dense FP32 row sums (RowDot<float>)
+    // error-free products and sums as in the dense FP32 row sums (simt.h)
     template <int RMAX>
     __device__ static void run(const uint32_t* __restrict__ idx, const float* __restrict__ val, int64_t b, int64_t e,
                                const float* __restrict__ ring, int64_t slot_stride, int ld, int nb, int K, int R,
@@ -207,11 +218,12 @@ __global__ void __launch_bounds__(256) k_shells(int ne, int nc, int K, int R, in
                                                 const int64_t* __restrict__ rowptr, const uint32_t* __restrict__ idx,
                                                 const T* __restrict__ val, const T* __restrict__ xring,
                                                 const T* __restrict__ qring, const T* __restrict__ E,
-                                                const T* __restrict__ Hv, T* __restrict__ z) {
+                                                const T* __restrict__ Hv, int C, int ld, T* __restrict__ z) {
     __shared__ double part[256 / 32][RMAX];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = blockIdx.x * (256 / 32 / WPR) + warp / WPR;
     const int w = warp % WPR;
+    if (blockIdx.x == 0 && threadIdx.x == 0) const_cast<Ctl*>(ctl)->t_mark = device_ns();
     const bool live = row < 2 * ne + nc;
     double acc[RMAX];
     if (live) {
@@ -231,16 +243,17 @@ __global__ void __launch_bounds__(256) k_shells(int ne, int nc, int K, int R, in
         double v = 0.0;
         for (int q = 0; q < WPR; ++q) v += part[warp + q][lane];
         double base = 0.0;
-        if (row < ne) base = (double)E[(int64_t)lane * ne + row];
-        else if (row < 2 * ne) base = (double)Hv[(int64_t)lane * ne + row - ne];
+        const int col = (int)((ctl->n - 1) % C) * R + lane;      // the step's column of the chunk's tests
+        if (row < ne) base = (double)E[(int64_t)col * ld + row];
+        else if (row < 2 * ne) base = (double)Hv[(int64_t)col * ld + row - ne];
         z[(int64_t)lane * ldz + row] = (T)(base + v);
     }
 }
 
 // q_n = Sigma^T y_n into the charge ring and qcur
 template <typename T>
-__global__ void k_fact_charges(DevMesh m, int R, int K, const Ctl* ctl, const T* __restrict__ y2, T* __restrict__ qring,
-                               T* __restrict__ qcur) {
+__global__ void k_fact_charges(DevMesh m, int R, int K, int ldc, const Ctl* ctl, const T* __restrict__ y2,
+                               T* __restrict__ qring, T* __restrict__ qcur) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= m.nc * R) return;
     const int r = t / m.nc, c = t % m.nc;
@@ -250,7 +263,7 @@ __global__ void k_fact_charges(DevMesh m, int R, int K, const Ctl* ctl, const T*
     for (int j = 0; j < 3; ++j) s = fma(m.tsign[3 * c + j], (double)y[m.tedge[3 * c + j]], s);
     const T q = (T)s;
     qring[((n % K) * R + r) * (int64_t)m.nc + c] = q;
-    qcur[(int64_t)r * m.nc + c] = q;
+    qcur[(int64_t)r * ldc + c] = q;
 }
 
 // j_n = y_n + Sigma((1/dtt - 1) v_n - v_{n-1}/dtt) -> x ring slot n, outputs; c_{n+1} -> slot n+1
@@ -276,20 +289,26 @@ __global__ void k_fact_post(DevMesh m, int R, int K, Ctl* ctl, const T* __restri
     if (ctl->yout) reinterpret_cast<T*>(ctl->yout)[((n - ctl->n0) * R + r) * (int64_t)m.ne + e] = y[e];
 }
 
-// y = M x for one matrix, one warp per row, result into slot n mod 2 of a two-slot buffer
-template <typename T, int RMAX>
-__global__ void k_fact_apply(const T* __restrict__ Mtx, int nrow, int ncol, int R, const T* __restrict__ x,
-                             T* __restrict__ y2, const Ctl* ctl) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (warp >= nrow) return;
-    double acc[RMAX];
-    warp_rows<T, RMAX>(Mtx + (int64_t)warp * ncol, ncol, x, R, ncol, acc);
-    T* dst = y2 + (ctl->n & 1) * (int64_t)R * nrow;
-    if ((threadIdx.x & 31) == 0) {
+// y = M x for one matrix (rows and vectors of ncol entries, a multiple of 16 bytes), one warp per row,
+// result into slot n mod 2 of a two-slot buffer; mark: close the device time of the shells' kernel
+template <typename T, int RM>
+__global__ void __launch_bounds__(256) k_fact_apply(const T* __restrict__ Mtx, int nrow, int ncol, int R, const T* __restrict__ x,
+                                                    T* __restrict__ y2, Ctl* ctl, bool mark) {
+    if (mark && blockIdx.x == 0 && threadIdx.x == 0) ctl->hist_ns += device_ns() - ctl->t_mark;
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (row >= nrow) return;
+    Acc<T> acc[1][RM];
+    int off[RM];
 #pragma unroll
-        for (int r = 0; r < RMAX; ++r)
-            if (r < R) dst[(int64_t)r * nrow + warp] = (T)acc[r];
-    }
+    for (int r = 0; r < RM; ++r) off[r] = min(r, R - 1) * ncol;
+    const T* rp[1] = {Mtx + (int64_t)row * ncol};
+    tile_rows<T, 1, RM>(rp, x, off, ncol / VecOf<T>::W, lane, acc);
+    typename SumOf<T>::S v[RM];
+#pragma unroll
+    for (int r = 0; r < RM; ++r) v[r] = acc[0][r].sum();
+    const auto s = multi_reduce<RM>(v, lane);
+    const int r = multi_index<RM>(lane);
+    if (multi_owner<RM>(lane) && r < R) y2[((ctl->n & 1) * R + r) * (int64_t)nrow + row] = (T)sum_value(s);
 }
 
 __global__ void k_fact_advance(Ctl* ctl) { ctl->n += 1; }
@@ -352,16 +371,16 @@ tdcfie_status build_fact(tdcfie_t h, StepPlan* p) {
     FK(cudaMalloc(&f->W, es * nW));
     if (p->prec == TDCFIE_FP64) FK(cudaMemcpyAsync(f->W, W64, 8 * nW, cudaMemcpyDeviceToDevice, s));
     else cast_f64_f32(s, W64, (float*)f->W, nW);
-    FK(cudaMalloc(&p->pinv, es * (int64_t)nc * nc));
-    if (p->prec == TDCFIE_FP64) FK(cudaMemcpyAsync(p->pinv, h->PinvS, 8 * (int64_t)nc * nc, cudaMemcpyDeviceToDevice, s));
-    else cast_f64_f32(s, h->PinvS, (float*)p->pinv, (int64_t)nc * nc);
+    FK(cudaMalloc(&p->pinv, es * (int64_t)nc * p->ldc));
+    to_path(s, p->prec, h->PinvS, p->pinv, nc, nc, p->ldc, 1.0);
     FK(cudaStreamSynchronize(s));
     cudaFree(B);
     cudaFree(W64);
     // march state
     FK(cudaMalloc(&f->xring, es * K * R * ne));
     FK(cudaMalloc(&f->qring, es * K * R * nc));
-    FK(cudaMalloc(&f->qcur, es * R * nc));
+    FK(cudaMalloc(&f->qcur, es * R * p->ldc));
+    FK(cudaMemsetAsync(f->qcur, 0, es * R * p->ldc, s));
     FK(cudaMalloc(&f->y2, es * 2 * R * ne));
     FK(cudaMalloc(&f->v2, es * 2 * R * nc));
     FK(cudaMalloc(&f->z, es * R * f->ldz));
@@ -393,33 +412,29 @@ static void launch_fact_r(tdcfie_t h, StepPlan& p, cudaStream_t s) {
     FactPlan& f = *p.fact;
     const tdc::DevMesh& m = h->dm;
     const int ne = p.ne, nc = p.nc, R = p.R, tb = 256, wpb = 8;
-    launch_rhs<T>(h, p, s);
-    cudaEventRecordWithFlags(p.evA, s, cudaEventRecordExternal);
     k_shells<T, RMAX><<<(f.nrows + wpb / WPR - 1) / (wpb / WPR), 32 * wpb, 0, s>>>(ne, nc, f.K, R, f.ldz, p.ctl, f.rowptr, f.idx,
                                                                       (const T*)f.val, (const T*)f.xring,
                                                                       (const T*)f.qring, (const T*)p.E,
-                                                                      (const T*)p.Hv, (T*)f.z);
-    cudaEventRecordWithFlags(p.evB, s, cudaEventRecordExternal);
+                                                                      (const T*)p.Hv, p.C, p.ld, (T*)f.z);
     k_fact_apply<T, RMAX><<<(ne + wpb - 1) / wpb, 32 * wpb, 0, s>>>((const T*)f.W, ne, f.ldz, R, (const T*)f.z,
-                                                                     (T*)f.y2, p.ctl);
-    k_fact_charges<T><<<(nc * R + tb - 1) / tb, tb, 0, s>>>(m, R, f.K, p.ctl, (const T*)f.y2, (T*)f.qring, (T*)f.qcur);
-    k_fact_apply<T, RMAX><<<(nc + wpb - 1) / wpb, 32 * wpb, 0, s>>>((const T*)p.pinv, nc, nc, R, (const T*)f.qcur,
-                                                                     (T*)f.v2, p.ctl);
+                                                                     (T*)f.y2, p.ctl, true);
+    k_fact_charges<T><<<(nc * R + tb - 1) / tb, tb, 0, s>>>(m, R, f.K, p.ldc, p.ctl, (const T*)f.y2, (T*)f.qring, (T*)f.qcur);
+    k_fact_apply<T, RMAX><<<(nc + wpb - 1) / wpb, 32 * wpb, 0, s>>>((const T*)p.pinv, nc, p.ldc, R, (const T*)f.qcur,
+                                                                     (T*)f.v2, p.ctl, false);
     k_fact_post<T><<<(ne * R + tb - 1) / tb, tb, 0, s>>>(m, R, f.K, p.ctl, (const T*)f.y2, (const T*)f.v2,
                                                          (T*)f.xring, h->dtt);
     k_fact_advance<<<1, 1, 0, s>>>(p.ctl);
-    p.launches_per_step = 7;
 }
 
 template <typename T>
-cudaError_t launch_step_fact(tdcfie_t h, StepPlan& p, cudaStream_t s) {
+int launch_step_fact(tdcfie_t h, StepPlan& p, cudaStream_t s) {
     if (p.R == 1) launch_fact_r<T, 1>(h, p, s);
     else if (p.R <= 4) launch_fact_r<T, 4>(h, p, s);
     else launch_fact_r<T, 8>(h, p, s);
-    return cudaGetLastError();
+    return 6;
 }
 
-template cudaError_t launch_step_fact<double>(tdcfie_t, StepPlan&, cudaStream_t);
-template cudaError_t launch_step_fact<float>(tdcfie_t, StepPlan&, cudaStream_t);
+template int launch_step_fact<double>(tdcfie_t, StepPlan&, cudaStream_t);
+template int launch_step_fact<float>(tdcfie_t, StepPlan&, cudaStream_t);
 
 }  // namespace tdc

@@ -13,6 +13,7 @@
 
 #include "gmres.h"
 #include "plan.h"
+#include "simt.h"
 
 namespace tdc {
 
@@ -26,7 +27,7 @@ enum { NSTATS = 8 };
 constexpr int MV_WPB = 16;   // rows (warps) per block of the Arnoldi matvec
 
 struct GmDev {
-    int R, ne, m, maxit, pass_cap;
+    int R, ne, ld, m, maxit, pass_cap;     // ld: row length of the step's vectors (b, ring, guess)
     double tol, inner_tol;
     double *x, *r, *V, *w, *hdot, *H, *cs, *sn, *g, *yv, *scal;
     int* flags;
@@ -48,7 +49,7 @@ __global__ void k_gm_init(GmDev d, const T* __restrict__ b, int mode, const T* _
     const int r = blockIdx.y;
     const int64_t n = ctl->n;
     const T* guess = nullptr;
-    if (mode == 1 && n > 1) guess = ringbuf + ((n - 1) % ring) * (int64_t)d.R * d.ne;
+    if (mode == 1 && n > 1) guess = ringbuf + ((n - 1) % ring) * (int64_t)d.R * d.ld;
     if ((mode == 2 || mode == 4) && n > 1) guess = learned;
     if (i == 0) {
         d.flags[r * NFLAGS + F_DONE] = DONE_OPEN;
@@ -61,20 +62,21 @@ __global__ void k_gm_init(GmDev d, const T* __restrict__ b, int mode, const T* _
     if (i < (d.m + 1) * d.m) d.H[(int64_t)r * (d.m + 1) * d.m + i] = 0.0;
     if (i < 2 * (d.m + 1)) d.hdot[(int64_t)r * 2 * (d.m + 1) + i] = 0.0;
     if (i >= d.ne) return;
-    const double bi = (double)b[(int64_t)r * d.ne + i];
-    double x0 = guess ? (double)guess[(int64_t)r * d.ne + i] : 0.0;
+    const double bi = (double)b[(int64_t)r * d.ld + i];
+    double x0 = guess ? (double)guess[(int64_t)r * d.ld + i] : 0.0;
     if (mode == 3) {
         const double c[4] = {4.0, -6.0, 4.0, -1.0};
         x0 = 0.0;
         for (int k = 1; k <= 4 && k <= ring; ++k)
-            if (n - k >= 1) x0 += c[k - 1] * (double)ringbuf[((n - k) % ring) * (int64_t)d.R * d.ne + (int64_t)r * d.ne + i];
+            if (n - k >= 1) x0 += c[k - 1] * (double)ringbuf[(((n - k) % ring) * d.R + r) * (int64_t)d.ld + i];
     }
     d.x[(int64_t)r * d.ne + i] = x0;
     atomicAdd(d.scal + r * NSCAL + S_BN2, bi * bi);
 }
 
-__global__ void k_gm_zero_scal(GmDev d) {
+__global__ void k_gm_zero_scal(GmDev d, Ctl* ctl) {
     const int t = threadIdx.x;
+    if (t == 0) ctl->hist_ns += device_ns() - ctl->t_mark;      // the history kernel ran just before
     if (t < d.R * NSCAL) d.scal[t] = 0.0;
 }
 
@@ -91,7 +93,7 @@ __global__ void k_gm_resid(GmDev d, const double* __restrict__ T0, const T* __re
     for (int j = lane; j < d.ne; j += 32) s += a[j] * xr[j];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
-        const double v = (double)b[(int64_t)r * d.ne + row] - s;
+        const double v = (double)b[(int64_t)r * d.ld + row] - s;
         d.r[(int64_t)r * d.ne + row] = v;
         atomicAdd(d.scal + r * NSCAL + S_RN2, v * v);
     }
@@ -298,8 +300,8 @@ __global__ void k_gm_store(GmDev d, T* __restrict__ ringbuf, int ring, Ctl* ctl)
             }
     }
     if (i >= d.ne) return;
-    T* dst = ringbuf + (ctl->n % ring) * (int64_t)d.R * d.ne;
-    dst[(int64_t)r * d.ne + i] = (T)d.x[(int64_t)r * d.ne + i];
+    T* dst = ringbuf + (ctl->n % ring) * (int64_t)d.R * d.ld;
+    dst[(int64_t)r * d.ld + i] = (T)d.x[(int64_t)r * d.ne + i];
 }
 
 // ---------------------------------------------------------------- host side
@@ -321,7 +323,7 @@ cudaError_t build_gmres(tdcfie_t h, StepPlan* p) {
     const int R = p->R, ne = p->ne;
     const int m = std::max(2, std::min(60, h->opts.gmres_restart));
     GmDev& d = g->d;
-    d.R = R; d.ne = ne; d.m = m;
+    d.R = R; d.ne = ne; d.ld = p->ld; d.m = m;
     d.tol = h->opts.gmres_tol;
     d.inner_tol = 1e-4;   // each cycle gains four digits; the restarts refine against the FP64 residual
     d.maxit = std::max(1, h->opts.gmres_maxit);
@@ -368,14 +370,14 @@ int gmres_body_launches() { return 7; }
 // captured on the plan's own stream), then the store into the ring.
 template <typename T>
 cudaError_t launch_gmres(tdcfie_t h, StepPlan* p, const T* b, const T* learned, const T* T0p, T* ringbuf,
-                         cudaStream_t s) {
+                         cudaStream_t s, int& kernels) {
     GmresPlan* g = p->gm;
     const GmDev& d = g->d;
     const int ne = d.ne, R = d.R, tb = 256, wpb = 8;
     const int ninit = std::max(ne, (d.m + 1) * d.m + 1);
     const dim3 gi((ninit + tb - 1) / tb, R), ge((ne + tb - 1) / tb, R), gw((ne + wpb - 1) / wpb, R),
         gm((ne + MV_WPB - 1) / MV_WPB, R);
-    k_gm_zero_scal<<<1, 64, 0, s>>>(d);
+    k_gm_zero_scal<<<1, 64, 0, s>>>(d, p->ctl);
     k_gm_init<T><<<gi, tb, 0, s>>>(d, b, h->opts.guess, ringbuf, p->ring, learned, p->ctl);
 
     cudaStreamCaptureStatus cs;
@@ -417,13 +419,13 @@ cudaError_t launch_gmres(tdcfie_t h, StepPlan* p, const T* b, const T* learned, 
     if (le != cudaSuccess) return le;
 
     k_gm_store<T><<<ge, tb, 0, s>>>(d, ringbuf, p->ring, p->ctl);
-    p->launches_per_step += 3;   // zero_scal, init, store; the loop passes are counted on the device
+    kernels += 3;   // zero_scal, init, store; the loop passes are counted on the device
     return cudaGetLastError();
 }
 
 template cudaError_t launch_gmres<double>(tdcfie_t, StepPlan*, const double*, const double*, const double*, double*,
-                                          cudaStream_t);
+                                          cudaStream_t, int&);
 template cudaError_t launch_gmres<float>(tdcfie_t, StepPlan*, const float*, const float*, const float*, float*,
-                                         cudaStream_t);
+                                         cudaStream_t, int&);
 
 }  // namespace tdc

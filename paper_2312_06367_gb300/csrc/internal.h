@@ -92,11 +92,13 @@ struct Ctl {              // device-resident step state read by every kernel of 
     int64_t n0;           // step of the first output row of this tdcfie_step call
     void* out;            // currents_out of this call (nullptr: discard)
     int status;           // 0 ok, else a tdcfie_status recorded with bad_step
-    int64_t bad_step;
+    int64_t bad_step;     // first step with a non-finite current (INT64_MAX: none)
     int timeout;          // set by a device-side bounded wait that ran out
     void* yout;           // optional y_n output of this call (nullptr: none)
     int noconv;           // set when a GMRES solve stopped above its tolerance (gmres_maxit reached)
     int64_t noconv_step;  // the first such step
+    int64_t p0;           // SIMT paths: first step not yet post-processed
+    unsigned long long t_mark, hist_ns;   // SIMT paths: device time of the history kernels (ns)
 };
 }  // namespace tdc
 
@@ -142,13 +144,16 @@ tdcfie_status fail(tdcfie_t h, tdcfie_status st, const std::string& msg);
 tdcfie_status cuda_fail(tdcfie_t h, cudaError_t e, const char* where);
 tdcfie_status build_plan(tdcfie_t h);
 void free_plan(tdcfie_t h);
+// dst[i][j] = scale src[i][j] in the path precision, rows padded with zeros from cols to ld (march.cu)
+void to_path(cudaStream_t s, int prec, const double* src, void* dst, int64_t rows, int cols, int ld, double scale);
 tdcfie_status plan_reset(tdcfie_t h);
 tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout = nullptr);
 tdcfie_status plan_gmres_stats(tdcfie_t h, long long* out6);
 tdcfie_status plan_set_solver(tdcfie_t h, int solver, int guess, double tol);
-cudaError_t capture_step(tdcfie_t h, cudaStream_t s);
+cudaError_t capture_step(tdcfie_t h, cudaStream_t s);   // one whole step of any path and position in a chunk
 tdcfie_status plan_set_outputs(tdcfie_t h, void* out, void* yout);
 tdcfie_status plan_check(tdcfie_t h);
+tdcfie_status plan_status(tdcfie_t h, const Ctl& c);      // what the step state words say
 int plan_launches_per_step(tdcfie_t h);
 tdcfie_status far_field(tdcfie_t h, const void* currents, int64_t nt, double w, const double* rhat, int64_t ndir,
                         double* out);

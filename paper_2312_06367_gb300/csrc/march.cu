@@ -1,4 +1,4 @@
-// Hot path of the marching-on-in-time solver (Sec. IV-B), one CUDA graph per step.
+// Hot path of the marching-on-in-time solver (Sec. IV-B), CUDA graphs over chunks of steps.
 //
 // Per step n (t_n = n dt), with y_i = 0 for i <= 0:
 //   rhs:      e_m(t_n) = int f_m . e_in(t_n),  h_m(t_n) = int g_m . h_in(t_n)         (Sec. II-C)
@@ -7,13 +7,13 @@
 //   solve:    y_n = T_0^-1 b_n
 //   project:  z = Sigma^T w_n, w_n = (1/dtt - 1) y_n - y_{n-1}/dtt;  u = (Sigma^T Sigma)^+ z
 //   post:     j_n = y_n + Sigma u = P^LH y_n + P^S (y_n - y_{n-1})/dtt                (Eq. post_processing)
-// Layouts (HBM): matrices row-major; vectors right-hand-side-major (R x N per slot); the ring
-// holds y_{n-1} .. y_{n-K+1} in K-1 slots, slot = i mod (K-1); y_n overwrites the slot of
-// y_{n-K+1} after the history sum has consumed it.
-#include <cuda_bf16.h>
-
-#include <cmath>
+// How the steps of a chunk share the passes over the matrices: simt.h.
+// Layouts (HBM): matrices row-major; vectors right-hand-side-major (R x ld per slot).  The ring holds
+// the last K - 1 + C y, slot = i mod (K - 1 + C): the K - 1 that the history reads and those of the
+// chunk, which the post-processing reads at its end.
 #include <algorithm>
+#include <cmath>
+#include <cstdint>
 #include <cstring>
 #include <string>
 
@@ -25,238 +25,197 @@
 
 namespace tdc {
 
-// ---------------------------------------------------------------- plane-wave tests
-// e_m(t_n), h_m(t_n) for every (edge, wave), waves fastest (a warp shares one edge's points)
+// ---------------------------------------------------------------- kernels (arithmetic in simt.h)
+// The tests and pre-sums of a chunk: no work unless the current step starts one
 template <typename T>
-__global__ void k_rhs(int ne, const double* __restrict__ exc, int R, double dt, const Ctl* ctl,
-                      const int* __restrict__ pptr, const T* __restrict__ px, const T* __restrict__ pc,
-                      const int* __restrict__ nE, T* __restrict__ E, T* __restrict__ H) {
+__device__ __forceinline__ bool chunk_start(const SimtDev<T>& d, int64_t n) { return (n - 1) % d.C == 0; }
+
+template <typename T>
+__global__ void __launch_bounds__(128) k_env(const __grid_constant__ SimtDev<T> d) {
+    const int64_t n = d.ctl->n;
+    if (!chunk_start(d, n)) return;
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (int64_t)d.npts * d.R * d.C) return;
+    const int i = (int)(idx % d.C), r = (int)(idx / d.C % d.R), pt = (int)(idx / d.C / d.R);
+    d.env[idx] = env_point<T>(d.exc + 11 * r, n + i, d.dt, d.pts[3 * pt], d.pts[3 * pt + 1], d.pts[3 * pt + 2]);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(128) k_gather(const __grid_constant__ SimtDev<T> d) {
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (w >= d.ne * d.R || !chunk_start(d, d.ctl->n)) return;
+    gather_edge<T>(d, w / d.R, w % d.R, threadIdx.x & 31);
+}
+
+// grid: (column tiles x row blocks, groups), the column tiles fastest so that blocks that share rows
+// run together
+template <typename T>
+__global__ void __launch_bounds__(128) k_pre(const __grid_constant__ SimtDev<T> d, int ctiles) {
+    const int64_t n = d.ctl->n;
+    if (!chunk_start(d, n)) return;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) d.ctl->t_mark = device_ns();
+    const int tile = blockIdx.x % ctiles, rb = blockIdx.x / ctiles;
+    const int row0 = (rb * 4 + (threadIdx.x >> 5)) * PRE_ROWS;
+    if (row0 < d.ne) pre_item<T>(d, n, row0, blockIdx.y, tile * PRE_COLS, threadIdx.x & 31);
+}
+
+// b_n; step = ctl->n + off
+template <typename T, int RM>
+__global__ void __launch_bounds__(128) k_hist(const __grid_constant__ SimtDev<T> d, int off) {
+    const int64_t n = d.ctl->n + off;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const unsigned long long t = device_ns();
+        if (chunk_start(d, n)) d.ctl->hist_ns += t - d.ctl->t_mark;     // the pre-sums ran just before
+        d.ctl->t_mark = t;
+    }
+    hist_unit<T, RM>(d, n, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31);
+}
+
+template <typename T, int RM>
+__global__ void __launch_bounds__(128) k_solve(const __grid_constant__ SimtDev<T> d, int off) {
+    const int64_t n = d.ctl->n + off;
+    if (blockIdx.x == 0 && threadIdx.x == 0) d.ctl->hist_ns += device_ns() - d.ctl->t_mark;
+    const int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (u * step_rows<RM>() < d.ne) solve_unit<T, RM>(d, n, u, threadIdx.x & 31);
+}
+
+// Post-processing of the steps p0 .. ctl->n + adv - 1 (at most C); the last kernel advances the step
+// counter by adv
+template <typename T>
+__global__ void __launch_bounds__(256) k_pin(const __grid_constant__ SimtDev<T> d, int adv) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= ne * R) return;
-    const int r = idx % R, mm = idx / R;
-    T e, h;
-    rhs_edge<T>(exc + 11 * r, ctl->n, dt, mm, pptr, px, pc, nE, e, h);
-    E[(int64_t)r * ne + mm] = e;
-    H[(int64_t)r * ne + mm] = h;
-}
-
-// Per-block partial sums of the history, kept in FP64 for every path precision
-template <typename T, int RMAX>
-__global__ void k_history(const T* __restrict__ blocks, int nblk, int ne, int R, int ring, const Ctl* ctl,
-                          const T* __restrict__ E, const T* __restrict__ H, const T* __restrict__ ringbuf,
-                          double* __restrict__ partial) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int q = blockIdx.y;
-    if (warp >= ne) return;
-    const int64_t n = ctl->n;
-    const T* x;
-    if (q == 0) x = E;
-    else if (q == 1) x = H;
-    else {
-        const int64_t k = q - 1;                 // lag of this history block
-        int64_t slot = (n - k) % ring;
-        if (slot < 0) slot += ring;
-        x = ringbuf + slot * (int64_t)R * ne;
-    }
-    double acc[RMAX];
-    warp_rows<T, RMAX>(blocks + ((int64_t)q * ne + warp) * ne, ne, x, R, ne, acc);
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int r = 0; r < RMAX; ++r)
-            if (r < R) partial[((int64_t)q * R + r) * ne + warp] = acc[r];
-    }
-}
-
-// FP32 history for several right-hand sides: one warp per ROWS rows, so that each lane's loads of
-// the R history vectors serve ROWS rows; error-free accumulation as in RowDot<float>
-template <int RMAX, int ROWS>
-__global__ void __launch_bounds__(256) k_history_rows(const float* __restrict__ blocks, int ne, int R, int ring,
-                                                      const Ctl* ctl, const float* __restrict__ E,
-                                                      const float* __restrict__ H, const float* __restrict__ ringbuf,
-                                                      double* __restrict__ partial) {
-    const int row0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * ROWS;
-    const int q = blockIdx.y;
-    if (row0 >= ne) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t n = ctl->n;
-    const float* x;
-    if (q == 0) x = E;
-    else if (q == 1) x = H;
-    else {
-        int64_t slot = (n - (q - 1)) % ring;
-        if (slot < 0) slot += ring;
-        x = ringbuf + slot * (int64_t)R * ne;
-    }
-    const float* Bq = blocks + (int64_t)q * ne * ne;
-    float hi[ROWS][RMAX], lo[ROWS][RMAX];
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i)
-#pragma unroll
-        for (int r = 0; r < RMAX; ++r) hi[i][r] = lo[i][r] = 0.f;
-    if ((ne & 3) == 0) {     // rows and vectors start on 16-byte boundaries
-        for (int j = lane; j < (ne >> 2); j += 32) {
-            float4 xv[RMAX];
-#pragma unroll
-            for (int r = 0; r < RMAX; ++r)
-                if (r < R) xv[r] = reinterpret_cast<const float4*>(x + (int64_t)r * ne)[j];
-#pragma unroll
-            for (int i = 0; i < ROWS; ++i) {
-                if (row0 + i >= ne) break;
-                const float4 a = reinterpret_cast<const float4*>(Bq + (int64_t)(row0 + i) * ne)[j];
-#pragma unroll
-                for (int r = 0; r < RMAX; ++r)
-                    if (r < R) {
-                        ff_add(hi[i][r], lo[i][r], a.x, xv[r].x);
-                        ff_add(hi[i][r], lo[i][r], a.y, xv[r].y);
-                        ff_add(hi[i][r], lo[i][r], a.z, xv[r].z);
-                        ff_add(hi[i][r], lo[i][r], a.w, xv[r].w);
-                    }
-            }
-        }
-    } else {
-        for (int j = lane; j < ne; j += 32) {
-            float xv[RMAX];
-#pragma unroll
-            for (int r = 0; r < RMAX; ++r)
-                if (r < R) xv[r] = x[(int64_t)r * ne + j];
-#pragma unroll
-            for (int i = 0; i < ROWS; ++i) {
-                if (row0 + i >= ne) break;
-                const float a = Bq[(int64_t)(row0 + i) * ne + j];
-#pragma unroll
-                for (int r = 0; r < RMAX; ++r)
-                    if (r < R) ff_add(hi[i][r], lo[i][r], a, xv[r]);
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i)
-#pragma unroll
-        for (int r = 0; r < RMAX; ++r) {
-            double v = (double)hi[i][r] + (double)lo[i][r];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0 && r < R && row0 + i < ne) partial[((int64_t)q * R + r) * ne + row0 + i] = v;
-        }
+    const int c = idx % d.nc, col = idx / d.nc;
+    const int64_t n = d.ctl->p0 + col / d.R;
+    if (n < d.ctl->n + adv && col < d.C * d.R) pin_value<T>(d, n, col, col % d.R, c);
 }
 
 template <typename T>
-__global__ void k_reduce(const double* __restrict__ partial, int nblk, int ne, int R, T* __restrict__ b) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ne * R) return;
-    double s = 0;
-    for (int q = 0; q < nblk; ++q) s += partial[(int64_t)q * R * ne + i];
-    b[i] = (T)s;
+__global__ void __launch_bounds__(128) k_pinv(const __grid_constant__ SimtDev<T> d, int adv, int ctiles) {
+    const int ncol = min((int)(d.ctl->n + adv - d.ctl->p0), d.C) * d.R;
+    const int col0 = blockIdx.x % ctiles * PRE_COLS, row0 = (blockIdx.x / ctiles * 4 + (threadIdx.x >> 5)) * PRE_ROWS;
+    if (col0 < ncol && row0 < d.nc) pinv_item<T>(d, ncol, row0, col0, threadIdx.x & 31);
 }
 
-// y = M x for one square matrix, one warp per row; result to a ring slot or plain buffer
-template <typename T, int RMAX>
-__global__ void k_apply(const T* __restrict__ Mtx, int nrow, int ncol, int R, const T* __restrict__ x,
-                        T* __restrict__ y, int ring, const Ctl* ctl) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (warp >= nrow) return;
-    double acc[RMAX];
-    warp_rows<T, RMAX>(Mtx + (int64_t)warp * ncol, ncol, x, R, ncol, acc);
-    T* dst = y;
-    if (ring > 0) dst = y + (ctl->n % ring) * (int64_t)R * nrow;
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int r = 0; r < RMAX; ++r)
-            if (r < R) dst[(int64_t)r * nrow + warp] = (T)acc[r];
-    }
-}
-
-// z[r][c] = sum_j tsign[c][j] w[r][tedge[c][j]],  w = (1/dtt - 1) y_n - y_{n-1}/dtt
 template <typename T>
-__global__ void k_project_in(DevMesh m, int R, int ring, const Ctl* ctl, const T* __restrict__ ringbuf, double dtt,
-                             T* __restrict__ z) {
+__global__ void __launch_bounds__(256) k_pout(const __grid_constant__ SimtDev<T> d, int adv) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= m.nc * R) return;
-    const int r = idx / m.nc, c = idx % m.nc;
-    const int64_t n = ctl->n;
-    const T* yn = ringbuf + (n % ring) * (int64_t)R * m.ne + (int64_t)r * m.ne;
-    const T* yp = ringbuf + ((n - 1) % ring) * (int64_t)R * m.ne + (int64_t)r * m.ne;
-    z[(int64_t)r * m.nc + c] = (T)project_in_value<T>(m, c, yn, yp, n == 1, dtt);
-}
-
-// j[r][m] = y_n[r][m] + u[r][c+(m)] - u[r][c-(m)]; write to out, check finiteness
-template <typename T>
-__global__ void k_project_out(DevMesh m, int R, int ring, Ctl* ctl, const T* __restrict__ ringbuf,
-                              const T* __restrict__ u) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= m.ne * R) return;
-    const int r = idx / m.ne, e = idx % m.ne;
-    const int64_t n = ctl->n;
-    const T* yn = ringbuf + (n % ring) * (int64_t)R * m.ne + (int64_t)r * m.ne;
-    const T val = yn[e] + u[(int64_t)r * m.nc + m.cplus_[e]] - u[(int64_t)r * m.nc + m.cminus_[e]];
-    if (!isfinite((double)val) && atomicCAS(&ctl->status, 0, (int)TDCFIE_E_NONFINITE) == 0) ctl->bad_step = n;
-    if (ctl->out) {
-        T* o = reinterpret_cast<T*>(ctl->out);
-        o[((n - ctl->n0) * R + r) * (int64_t)m.ne + e] = val;
-    }
-    if (ctl->yout) {
-        T* o = reinterpret_cast<T*>(ctl->yout);
-        o[((n - ctl->n0) * R + r) * (int64_t)m.ne + e] = yn[e];
+    const int e = idx % d.ne, col = idx / d.ne;
+    const int64_t end = d.ctl->n + adv, n = d.ctl->p0 + col / d.R;
+    if (n < end && col < d.C * d.R) pout_value<T>(d, n, col, col % d.R, e);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(d.done, 1) == (int)gridDim.x - 1) {     // every block has read n and p0
+            *d.done = 0;
+            d.ctl->n = end;
+            d.ctl->p0 = end;
+            __threadfence();
+        }
     }
 }
 
 __global__ void k_advance(Ctl* ctl) { ctl->n += 1; }
 
-// ---------------------------------------------------------------- plan construction
+// ---------------------------------------------------------------- launches
 static size_t esize(int prec) { return prec == TDCFIE_FP64 ? 8 : 4; }
 
 template <typename T>
-void launch_rhs(tdcfie_t h, StepPlan& p, cudaStream_t s) {
-    const int tb = 256;
-    k_rhs<T><<<(p.ne * p.R + tb - 1) / tb, tb, 0, s>>>(p.ne, h->dexc, p.R, h->dt, p.ctl, p.pptr, (const T*)p.px,
-                                                        (const T*)p.pc, p.pnE, (T*)p.E, (T*)p.Hv);
+SimtDev<T> simt_view(tdcfie_t h, const StepPlan& p) {
+    SimtDev<T> d;
+    d.ne = p.ne; d.nc = p.nc; d.R = p.R; d.C = p.C; d.K = p.K; d.ring = p.ring; d.ld = p.ld; d.ldc = p.ldc;
+    d.ngroups = p.ngroups; d.npts = p.npts;
+    d.blocks = (const T*)p.blocks; d.t0inv = (const T*)p.t0inv; d.pinv = (const T*)p.pinv;
+    d.E = (T*)p.E; d.H = (T*)p.Hv; d.rbuf = (T*)p.ringbuf; d.b = (T*)p.b; d.z = (T*)p.z; d.u = (T*)p.u;
+    using S = typename SumOf<T>::S;
+    d.partial = (S*)p.partial; d.inner = (S*)p.inner; d.env = (T*)p.env; d.pts = (const T*)p.pts;
+    d.eptr = p.eptr; d.enE = p.enE; d.eidx = p.eidx; d.ecoef = (const T*)p.ecoef;
+    d.exc = h->dexc; d.m = h->dm; d.dt = h->dt; d.dtt = h->dtt; d.ctl = p.ctl; d.done = p.done;
+    return d;
 }
-template void launch_rhs<double>(tdcfie_t, StepPlan&, cudaStream_t);
-template void launch_rhs<float>(tdcfie_t, StepPlan&, cudaStream_t);
+template SimtDev<float> simt_view<float>(tdcfie_t, const StepPlan&);
+
+static unsigned div_up(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
 template <typename T>
-static cudaError_t launch_step(tdcfie_t h, StepPlan& p, cudaStream_t s) {
-    if (p.fact) return launch_step_fact<T>(h, p, s);
-    const tdc::DevMesh& m = h->dm;
-    const int R = p.R, ne = p.ne;
-    const int tb = 256;
-    launch_rhs<T>(h, p, s);
-    const int wpb = 8;   // warps per block
-    dim3 g((ne + wpb - 1) / wpb, p.nblk);
-#define HIST(RM) k_history<T, RM><<<g, 32 * wpb, 0, s>>>((const T*)p.blocks, p.nblk, ne, R, p.ring, p.ctl, \
-                                                           (const T*)p.E, (const T*)p.Hv, (const T*)p.ringbuf, (double*)p.partial)
-#define APPLY(RM, M, nr, nc_, x, y, rg) k_apply<T, RM><<<((nr) + wpb - 1) / wpb, 32 * wpb, 0, s>>>((const T*)(M), nr, nc_, R, (const T*)(x), (T*)(y), rg, p.ctl)
-    cudaEventRecordWithFlags(p.evA, s, cudaEventRecordExternal);
-    if (R == 1 || sizeof(T) == 8) {
-        if (R == 1) HIST(1); else if (R <= 4) HIST(4); else HIST(8);
-    } else {
-        // FP32 with several waves: 4 rows per warp up to 4 waves, 2 rows (fewer registers) above
-#define HISTR(RM, ROWS) k_history_rows<RM, ROWS><<<dim3((ne + wpb * ROWS - 1) / (wpb * ROWS), p.nblk), 32 * wpb, 0, s>>>( \
-            (const float*)p.blocks, ne, R, p.ring, p.ctl, (const float*)p.E, (const float*)p.Hv,                       \
-            (const float*)p.ringbuf, (double*)p.partial)
-        if (R <= 4) HISTR(4, 4); else HISTR(8, 2);
-#undef HISTR
+int launch_tests(tdcfie_t h, StepPlan& p, cudaStream_t s) {
+    const SimtDev<T> d = simt_view<T>(h, p);
+    k_env<T><<<div_up((int64_t)p.npts * p.R * p.C, 128), 128, 0, s>>>(d);
+    k_gather<T><<<div_up((int64_t)p.ne * p.R, 4), 128, 0, s>>>(d);
+    return 2;
+}
+template int launch_tests<double>(tdcfie_t, StepPlan&, cudaStream_t);
+template int launch_tests<float>(tdcfie_t, StepPlan&, cudaStream_t);
+
+template <typename T>
+static int launch_pre(tdcfie_t h, StepPlan& p, cudaStream_t s) {
+    int n = launch_tests<T>(h, p, s);
+    if (p.fact) return n;
+    const int ctiles = (int)div_up(p.C * p.R, PRE_COLS);
+    k_pre<T><<<dim3(ctiles * div_up(p.ne, 4 * PRE_ROWS), p.ngroups), 128, 0, s>>>(simt_view<T>(h, p), ctiles);
+    return n + 1;
+}
+
+// history and solve of step ctl->n + off (chunk: of a whole chunk that starts at ctl->n)
+template <typename T>
+static cudaError_t launch_inner(tdcfie_t h, StepPlan& p, bool chunk, int off, cudaStream_t s, int& kernels) {
+    if (p.fact) {
+        kernels += launch_step_fact<T>(h, p, s);
+        return cudaGetLastError();
     }
-    k_reduce<T><<<(ne * R + tb - 1) / tb, tb, 0, s>>>((const double*)p.partial, p.nblk, ne, R, (T*)p.b);
-    cudaEventRecordWithFlags(p.evB, s, cudaEventRecordExternal);
-    p.launches_per_step = 0;
-    if (p.mlp_on) launch_mlp_guess<T>(&p, s);
+    const SimtDev<T> d = simt_view<T>(h, p);
+    const int units = (int)div_up(p.ne, p.R <= 2 ? 2 : 1);
+    // units of the history: the step's rows, and the rows of every lag that can be pushed (chunk: the
+    // step's column is known)
+    const int lags = 1 + std::max(0, std::min(chunk ? p.C - off : p.C - 1, p.K - 1) - 1) * (chunk && off == 0 ? 0 : 1);
+    unsigned g = div_up((int64_t)units * lags, 4);
+#define BY_R(K, ...) (p.R == 1 ? K<T, 1><<<g, 128, 0, s>>>(__VA_ARGS__) : p.R == 2 ? K<T, 2><<<g, 128, 0, s>>>(__VA_ARGS__) : \
+                      p.R <= 4 ? K<T, 4><<<g, 128, 0, s>>>(__VA_ARGS__) : K<T, 8><<<g, 128, 0, s>>>(__VA_ARGS__))
+    BY_R(k_hist, d, off);
+    kernels += 1;
+    g = div_up(units, 4);
+    if (p.mlp_on) kernels += launch_mlp_guess<T>(&p, s);
     if (p.gmres_on) {
         const cudaError_t e = launch_gmres<T>(h, &p, (const T*)p.b, (const T*)p.guessbuf, (const T*)p.t0mat,
-                                              (T*)p.ringbuf, s);
+                                              (T*)p.ringbuf, s, kernels);
         if (e != cudaSuccess) return e;
-    } else if (R == 1) APPLY(1, p.t0inv, ne, ne, p.b, p.ringbuf, p.ring);
-    else if (R <= 4) APPLY(4, p.t0inv, ne, ne, p.b, p.ringbuf, p.ring);
-    else APPLY(8, p.t0inv, ne, ne, p.b, p.ringbuf, p.ring);
-    k_project_in<T><<<(p.nc * R + tb - 1) / tb, tb, 0, s>>>(m, R, p.ring, p.ctl, (const T*)p.ringbuf, h->dtt, (T*)p.z);
-    if (R == 1) APPLY(1, p.pinv, p.nc, p.nc, p.z, p.u, 0);
-    else if (R <= 4) APPLY(4, p.pinv, p.nc, p.nc, p.z, p.u, 0);
-    else APPLY(8, p.pinv, p.nc, p.nc, p.z, p.u, 0);
-    k_project_out<T><<<(ne * R + tb - 1) / tb, tb, 0, s>>>(m, R, p.ring, p.ctl, (const T*)p.ringbuf, (const T*)p.u);
-    k_advance<<<1, 1, 0, s>>>(p.ctl);
-#undef HIST
-#undef APPLY
-    p.launches_per_step += 8 - (p.gmres_on ? 1 : 0);
+    } else {
+        BY_R(k_solve, d, off);
+        kernels += 1;
+    }
+#undef BY_R
     return cudaGetLastError();
+}
+
+template <typename T>
+static int launch_post(tdcfie_t h, StepPlan& p, int adv, cudaStream_t s) {
+    if (p.fact) return 0;      // part of the step
+    const SimtDev<T> d = simt_view<T>(h, p);
+    const int CR = p.C * p.R, ctiles = (int)div_up(CR, PRE_COLS);
+    k_pin<T><<<div_up((int64_t)p.nc * CR, 256), 256, 0, s>>>(d, adv);
+    k_pinv<T><<<ctiles * div_up(p.nc, 4 * PRE_ROWS), 128, 0, s>>>(d, adv, ctiles);
+    k_pout<T><<<div_up((int64_t)p.ne * CR, 256), 256, 0, s>>>(d, adv);
+    return 3;
+}
+
+// enqueue the kernels of one of the plan's graphs (s must be capturing)
+template <typename T>
+static cudaError_t launch_graph(tdcfie_t h, StepPlan& p, int which, cudaStream_t s) {
+    int k = 0;
+    cudaError_t e = cudaSuccess;
+    if (which == StepPlan::G_PRE || which == StepPlan::G_CHUNK) k += launch_pre<T>(h, p, s);
+    if (which == StepPlan::G_STEP) {
+        e = launch_inner<T>(h, p, false, 0, s, k);
+        if (!p.fact) {                      // the factored step advances the counter itself
+            k_advance<<<1, 1, 0, s>>>(p.ctl);
+            k += 1;
+        }
+    }
+    if (which == StepPlan::G_CHUNK)
+        for (int i = 0; i < p.C && e == cudaSuccess; ++i) e = launch_inner<T>(h, p, true, p.fact ? 0 : i, s, k);
+    if (which == StepPlan::G_POST) k += launch_post<T>(h, p, 0, s);
+    if (which == StepPlan::G_CHUNK) k += launch_post<T>(h, p, p.C, s);
+    p.nodes[which] = k;
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 tdcfie_status plan_gmres_stats(tdcfie_t h, long long* out6) {
@@ -267,14 +226,21 @@ tdcfie_status plan_gmres_stats(tdcfie_t h, long long* out6) {
     return TDCFIE_OK;
 }
 
+static void drop_graphs(StepPlan* p) {
+    for (int g = 0; g < StepPlan::NGRAPH; ++g) {
+        if (p->exec[g]) { cudaGraphExecDestroy(p->exec[g]); p->exec[g] = nullptr; }
+        if (p->graph[g]) { cudaGraphDestroy(p->graph[g]); p->graph[g] = nullptr; }
+    }
+    p->nodeA = p->nodeB = nullptr;
+}
+
 void free_plan(tdcfie_t h) {
     StepPlan* p = h->plan;
     if (!p) return;
-    void* bufs[] = {p->blocks, p->t0inv, p->pinv, p->E, p->Hv, p->ringbuf, p->b, p->partial, p->w, p->z, p->u,
-                    p->ctl, p->pptr, p->pnE, p->px, p->pc};
+    void* bufs[] = {p->blocks, p->t0inv, p->pinv, p->E, p->Hv, p->ringbuf, p->b, p->partial, p->inner, p->z, p->u, p->done,
+                    p->ctl, p->pptr, p->pnE, p->px, p->pc, p->env, p->pts, p->ecoef, p->eptr, p->enE, p->eidx};
     for (void* b : bufs) if (b) cudaFree(b);
-    if (p->exec) cudaGraphExecDestroy(p->exec);
-    if (p->graph) cudaGraphDestroy(p->graph);
+    drop_graphs(p);
     if (p->ev0) cudaEventDestroy(p->ev0);
     if (p->ev1) cudaEventDestroy(p->ev1);
     if (p->ev2) cudaEventDestroy(p->ev2);
@@ -294,9 +260,19 @@ void free_plan(tdcfie_t h) {
 
 #define CK(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return cuda_fail(h, e_, #x); } while (0)
 
-static void to_path(cudaStream_t s, int prec, const double* src, void* dst, int64_t n) {
-    if (prec == TDCFIE_FP64) cudaMemcpyAsync(dst, src, n * 8, cudaMemcpyDeviceToDevice, s);
-    else cast_f64_f32(s, src, (float*)dst, n);
+// dst[i][j] = scale src[i][j] in the path precision, rows padded with zeros from cols to ld
+template <typename T>
+__global__ void k_to_path(const double* __restrict__ src, T* __restrict__ dst, int64_t rows, int cols, int ld, double scale) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= rows * ld) return;
+    const int64_t i = t / ld;
+    const int j = (int)(t - i * ld);
+    dst[t] = j < cols ? (T)(scale * src[i * cols + j]) : (T)0;
+}
+void to_path(cudaStream_t s, int prec, const double* src, void* dst, int64_t rows, int cols, int ld, double scale) {
+    const unsigned g = div_up(rows * ld, 256);
+    if (prec == TDCFIE_FP64) k_to_path<double><<<g, 256, 0, s>>>(src, (double*)dst, rows, cols, ld, scale);
+    else k_to_path<float><<<g, 256, 0, s>>>(src, (float*)dst, rows, cols, ld, scale);
 }
 
 tdcfie_status build_plan(tdcfie_t h) {
@@ -309,7 +285,6 @@ tdcfie_status build_plan(tdcfie_t h) {
     p->R = (int)h->R;
     p->ne = M.ne; p->nc = M.nc; p->K = h->K;
     p->nblk = h->K + 1;              // -A, alpha L2, -T_1..-T_{K-1}
-    p->ring = h->K - 1;
     p->esz = esize(p->prec);
     const int64_t ne = M.ne, nc = M.nc, R = p->R;
     const bool tensor = p->prec == TDCFIE_BF16X3 || p->prec == TDCFIE_FP16X3;
@@ -317,6 +292,16 @@ tdcfie_status build_plan(tdcfie_t h) {
         return fail(h, TDCFIE_E_UNSUPPORTED, "the comparison formulation runs on the dense FP64 and FP32 paths");
     if (tensor) p->esz = 4;   // the tensor-core paths keep FP32 vectors, 16-bit hi/lo matrices
     const size_t es = p->esz;
+    // Steps per chunk.  Matrix blocks read per step: (K + 1) / C + (C - 1) / 2 + 1 + 1 / C, least near
+    // C = sqrt(2 (K + 2)) = 9 at K = 42; where everything sits in L2 (up to about 1000 edges) the
+    // kernels per chunk count, not the bytes, and 16 steps share them.  The tests' kernel needs a
+    // divisor of 32.
+    p->C = tensor ? 1 : (ne <= 1024 && R <= 2 ? 16 : 8);
+    p->ring = tensor ? h->K - 1 : h->K - 1 + p->C;
+    const int vw = (int)(16 / es);      // elements per 16-byte vector
+    p->ld = (int)(ne + vw - 1) / vw * vw;
+    p->ldc = (int)(nc + vw - 1) / vw * vw;
+    p->ngroups = (h->K + 1 + 3) / 4;
     // rhs quadrature tables (host, FP64), uploaded in the path precision
     {
         const double s15 = std::sqrt(15.0);
@@ -326,8 +311,12 @@ tdcfie_status build_plan(tdcfie_t h) {
                                  {b1, b1, a1, w1}, {a2, b2, b2, w2}, {b2, a2, b2, w2}, {b2, b2, a2, w2}};
         const double r3[3][4] = {{2.0 / 3, 1.0 / 6, 1.0 / 6, 1.0 / 3}, {1.0 / 6, 2.0 / 3, 1.0 / 6, 1.0 / 3},
                                  {1.0 / 6, 1.0 / 6, 2.0 / 3, 1.0 / 3}};
-        std::vector<std::vector<double>> pts(ne), cfs(ne);
+        // entries of every edge, e-points first (the coarse loop precedes the fine loop), over the
+        // distinct points: 7 per triangle, 3 per fine triangle
+        std::vector<std::vector<double>> cfs(ne);
+        std::vector<std::vector<int>> ids(ne);
         std::vector<int> nE(ne, 0);
+        std::vector<double> X(3 * (size_t)(7 * M.nc + 3 * M.nf));
         auto area = [](const double* a, const double* b, const double* c) {
             const double ex = b[0] - a[0], ey = b[1] - a[1], ez = b[2] - a[2];
             const double fx = c[0] - a[0], fy = c[1] - a[1], fz = c[2] - a[2];
@@ -337,16 +326,16 @@ tdcfie_status build_plan(tdcfie_t h) {
         for (int c = 0; c < M.nc; ++c) {
             const double* v[3] = {&M.V[3 * M.F[3 * c]], &M.V[3 * M.F[3 * c + 1]], &M.V[3 * M.F[3 * c + 2]]};
             const double A = area(v[0], v[1], v[2]);
+            for (int q = 0; q < 7; ++q) {
+                const int id = 7 * c + q;
+                for (int k = 0; k < 3; ++k) X[3 * (size_t)id + k] = r7[q][0] * v[0][k] + r7[q][1] * v[1][k] + r7[q][2] * v[2][k];
+            }
             for (int j = 0; j < 3; ++j) {
                 const int m = M.tedge[3 * c + j];
                 const double sgn = M.tsign[3 * c + j] / (2.0 * A);
                 for (int q = 0; q < 7; ++q) {
-                    double x[3];
-                    for (int k = 0; k < 3; ++k) x[k] = r7[q][0] * v[0][k] + r7[q][1] * v[1][k] + r7[q][2] * v[2][k];
-                    for (int k = 0; k < 3; ++k) {
-                        pts[m].push_back(x[k]);
-                        cfs[m].push_back(r7[q][3] * A * sgn * (x[k] - v[j][k]));
-                    }
+                    ids[m].push_back(7 * c + q);
+                    for (int k = 0; k < 3; ++k) cfs[m].push_back(r7[q][3] * A * sgn * (X[3 * (size_t)(7 * c + q) + k] - v[j][k]));
                     nE[m]++;
                 }
             }
@@ -354,54 +343,79 @@ tdcfie_status build_plan(tdcfie_t h) {
         for (int t = 0; t < M.nf; ++t) {
             const double* v[3] = {&M.fV[3 * M.fF[3 * t]], &M.fV[3 * M.fF[3 * t + 1]], &M.fV[3 * M.fF[3 * t + 2]]};
             const double A = area(v[0], v[1], v[2]);
+            for (int q = 0; q < 3; ++q) {
+                const size_t id = 7 * (size_t)M.nc + 3 * t + q;
+                for (int k = 0; k < 3; ++k) X[3 * id + k] = r3[q][0] * v[0][k] + r3[q][1] * v[1][k] + r3[q][2] * v[2][k];
+            }
             for (int e = M.bc_ptr[t]; e < M.bc_ptr[t + 1]; ++e) {
                 const int m = M.bc_fn[e];
                 const double* ph = &M.bc_phi[3 * e];
                 for (int q = 0; q < 3; ++q) {
-                    double x[3];
-                    for (int k = 0; k < 3; ++k) x[k] = r3[q][0] * v[0][k] + r3[q][1] * v[1][k] + r3[q][2] * v[2][k];
+                    const int id = 7 * M.nc + 3 * t + q;
+                    ids[m].push_back(id);
                     for (int k = 0; k < 3; ++k) {
-                        pts[m].push_back(x[k]);
                         double g = 0.0;
-                        for (int j = 0; j < 3; ++j) g += ph[j] * (x[k] - v[j][k]);
+                        for (int j = 0; j < 3; ++j) g += ph[j] * (X[3 * (size_t)id + k] - v[j][k]);
                         cfs[m].push_back(r3[q][3] * A * g / (2.0 * A));
                     }
                 }
             }
         }
-        // e-points were pushed before any h-point of the same edge only if all coarse passes ran
-        // first, which they did (coarse loop precedes fine loop)
         std::vector<int> ptr(ne + 1, 0);
-        for (int64_t m = 0; m < ne; ++m) ptr[m + 1] = ptr[m] + (int)(pts[m].size() / 3);
-        std::vector<double> X(3 * (size_t)ptr[ne]), C(3 * (size_t)ptr[ne]);
+        for (int64_t m = 0; m < ne; ++m) ptr[m + 1] = ptr[m] + (int)ids[m].size();
+        std::vector<double> C(3 * (size_t)ptr[ne]);
+        std::vector<int> I(ptr[ne]);
         for (int64_t m = 0; m < ne; ++m) {
-            std::copy(pts[m].begin(), pts[m].end(), X.begin() + 3 * ptr[m]);
-            std::copy(cfs[m].begin(), cfs[m].end(), C.begin() + 3 * ptr[m]);
+            std::copy(ids[m].begin(), ids[m].end(), I.begin() + ptr[m]);
+            std::copy(cfs[m].begin(), cfs[m].end(), C.begin() + 3 * (size_t)ptr[m]);
         }
-        const size_t pes = (p->prec == TDCFIE_FP64) ? 8 : 4;
-        CK(cudaMalloc(&p->pptr, sizeof(int) * (ne + 1)));
-        CK(cudaMalloc(&p->pnE, sizeof(int) * ne));
-        CK(cudaMalloc(&p->px, pes * X.size()));
-        CK(cudaMalloc(&p->pc, pes * C.size()));
-        CK(cudaMemcpy(p->pptr, ptr.data(), sizeof(int) * (ne + 1), cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(p->pnE, nE.data(), sizeof(int) * ne, cudaMemcpyHostToDevice));
-        if (pes == 8) {
-            CK(cudaMemcpy(p->px, X.data(), 8 * X.size(), cudaMemcpyHostToDevice));
-            CK(cudaMemcpy(p->pc, C.data(), 8 * C.size(), cudaMemcpyHostToDevice));
+        auto put = [&](void** dst, const std::vector<double>& v) -> cudaError_t {      // path precision
+            const bool f64 = p->prec == TDCFIE_FP64;
+            std::vector<float> vf;
+            if (!f64) vf.assign(v.begin(), v.end());
+            const size_t bytes = v.size() * (f64 ? 8 : 4);
+            const cudaError_t e = cudaMalloc(dst, bytes);
+            return e != cudaSuccess ? e : cudaMemcpy(*dst, f64 ? (const void*)v.data() : vf.data(), bytes, cudaMemcpyHostToDevice);
+        };
+        auto puti = [&](int** dst, const std::vector<int>& v) -> cudaError_t {
+            const cudaError_t e = cudaMalloc(dst, sizeof(int) * v.size());
+            return e != cudaSuccess ? e : cudaMemcpy(*dst, v.data(), sizeof(int) * v.size(), cudaMemcpyHostToDevice);
+        };
+        if (tensor) {
+            std::vector<double> XE(3 * I.size());      // the points per entry
+            for (size_t q = 0; q < I.size(); ++q)
+                for (int k = 0; k < 3; ++k) XE[3 * q + k] = X[3 * (size_t)I[q] + k];
+            CK(puti(&p->pptr, ptr));
+            CK(puti(&p->pnE, nE));
+            CK(put(&p->px, XE));
+            CK(put(&p->pc, C));
         } else {
-            std::vector<float> Xf(X.begin(), X.end()), Cf(C.begin(), C.end());
-            CK(cudaMemcpy(p->px, Xf.data(), 4 * Xf.size(), cudaMemcpyHostToDevice));
-            CK(cudaMemcpy(p->pc, Cf.data(), 4 * Cf.size(), cudaMemcpyHostToDevice));
+            p->npts = (int)(X.size() / 3);
+            CK(puti(&p->eptr, ptr));
+            CK(puti(&p->enE, nE));
+            CK(puti(&p->eidx, I));
+            CK(put(&p->pts, X));
+            CK(put(&p->ecoef, C));
+            CK(cudaMalloc(&p->env, es * p->npts * R * p->C));
         }
     }
     CK(cudaMalloc(&p->ctl, sizeof(Ctl)));
-    CK(cudaMalloc(&p->E, es * R * ne));
-    CK(cudaMalloc(&p->Hv, es * R * ne));
-    CK(cudaMalloc(&p->ringbuf, es * p->ring * R * ne));
-    CK(cudaMalloc(&p->b, es * R * ne));
-    CK(cudaMalloc(&p->partial, sizeof(double) * p->nblk * R * ne));
-    CK(cudaMalloc(&p->z, es * R * nc));
-    CK(cudaMalloc(&p->u, es * R * nc));
+    if (!h->dexc) {     // with the plan, so that whoever keeps a view of the plan has its address
+        CK(cudaMalloc(&h->dexc, sizeof(double) * 11 * R));
+        CK(cudaMemsetAsync(h->dexc, 0, sizeof(double) * 11 * R, s));
+    }
+    if (!tensor) {
+        const size_t CR = (size_t)p->C * R;
+        struct { void** p; size_t n; } bufs[] = {{&p->E, es * CR * p->ld}, {&p->Hv, es * CR * p->ld},
+                                                 {&p->ringbuf, es * (p->ring + 1) * R * p->ld}, {&p->b, es * R * p->ld},
+                                                 {&p->partial, 8 * p->ngroups * CR * p->ld},
+                                                 {&p->inner, 8 * p->C * CR * p->ld},
+                                                 {&p->z, es * CR * p->ldc}, {&p->u, es * CR * p->ldc}, {(void**)&p->done, sizeof(int)}};
+        for (auto& b : bufs) {      // the padding stays zero
+            CK(cudaMalloc(b.p, b.n));
+            CK(cudaMemsetAsync(*b.p, 0, b.n, s));
+        }
+    }
     if (tensor) {
         tdcfie_status st = build_tc(h, p);
         if (st != TDCFIE_OK) return st;
@@ -409,25 +423,23 @@ tdcfie_status build_plan(tdcfie_t h) {
         // mixed TD-MFIE (a comparison formulation of Sec. V): sum_k MM'_k j_{n-k} = h_n with
         // MM'_0 = MM_0 + G/2; block 0 (e) zero, block 1 (h) the identity, block 1+k: -MM_k; the
         // unknown is j itself, so the projector product is zero and the post-processing returns y
-        CK(cudaMalloc(&p->blocks, es * p->nblk * ne * ne));
-        CK(cudaMalloc(&p->t0inv, es * ne * ne));
-        CK(cudaMalloc(&p->pinv, es * nc * nc));
-        CK(cudaMemsetAsync(p->blocks, 0, es * ne * ne, s));
-        CK(cudaMemsetAsync(p->pinv, 0, es * nc * nc, s));
+        const int ld = p->ld, ldc = p->ldc;
+        CK(cudaMalloc(&p->blocks, es * p->nblk * ne * ld));
+        CK(cudaMalloc(&p->t0inv, es * ne * ld));
+        CK(cudaMalloc(&p->pinv, es * nc * ldc));
+        CK(cudaMemsetAsync(p->blocks, 0, es * ne * ld, s));
+        CK(cudaMemsetAsync(p->pinv, 0, es * nc * ldc, s));
         double *tmp = nullptr, *work = nullptr;
         CK(cudaMalloc(&tmp, 8 * ne * ne));
         CK(cudaMalloc(&work, 8 * (2 * ne + 2)));
         fill_identity(s, tmp, (int)ne, 1.0);
-        to_path(s, p->prec, tmp, (char*)p->blocks + es * ne * ne, ne * ne);
-        for (int k = 1; k < h->K; ++k) {
-            CK(cudaMemcpyAsync(tmp, h->MM + (int64_t)k * ne * ne, 8 * ne * ne, cudaMemcpyDeviceToDevice, s));
-            axpby(s, ne * ne, 0.0, tmp, -1.0, tmp);
-            to_path(s, p->prec, tmp, (char*)p->blocks + es * (1 + k) * ne * ne, ne * ne);
-        }
+        to_path(s, p->prec, tmp, (char*)p->blocks + es * ne * ld, ne, (int)ne, ld, 1.0);
+        for (int k = 1; k < h->K; ++k)
+            to_path(s, p->prec, h->MM + (int64_t)k * ne * ne, (char*)p->blocks + es * (1 + k) * ne * ld, ne, (int)ne, ld, -1.0);
         CK(cudaMemcpyAsync(tmp, h->MM, 8 * ne * ne, cudaMemcpyDeviceToDevice, s));
         axpby(s, ne * ne, 0.5, h->G, 1.0, tmp);
         const int singular = invert(s, tmp, (int)ne, work);
-        to_path(s, p->prec, tmp, p->t0inv, ne * ne);
+        to_path(s, p->prec, tmp, p->t0inv, ne, (int)ne, ld, 1.0);
         CK(cudaStreamSynchronize(s));
         cudaFree(tmp);
         cudaFree(work);
@@ -437,27 +449,17 @@ tdcfie_status build_plan(tdcfie_t h) {
         if (st != TDCFIE_OK) return st;
         h->step_bytes = fact_step_bytes(p);
     } else {
-        CK(cudaMalloc(&p->blocks, es * p->nblk * ne * ne));
-        CK(cudaMalloc(&p->t0inv, es * ne * ne));
-        CK(cudaMalloc(&p->pinv, es * nc * nc));
         // block 0: -A, block 1: alpha L2, block 1+k: -T_k
-        double* tmp = nullptr;
-        CK(cudaMalloc(&tmp, 8 * ne * ne));
-        CK(cudaMemcpyAsync(tmp, h->A, 8 * ne * ne, cudaMemcpyDeviceToDevice, s));
-        axpby(s, ne * ne, 0.0, tmp, -1.0, tmp);
-        to_path(s, p->prec, tmp, p->blocks, ne * ne);
-        CK(cudaMemcpyAsync(tmp, h->L2, 8 * ne * ne, cudaMemcpyDeviceToDevice, s));
-        axpby(s, ne * ne, 0.0, tmp, h->alpha, tmp);
-        to_path(s, p->prec, tmp, (char*)p->blocks + es * ne * ne, ne * ne);
-        for (int k = 1; k < h->K; ++k) {
-            CK(cudaMemcpyAsync(tmp, h->T + (int64_t)k * ne * ne, 8 * ne * ne, cudaMemcpyDeviceToDevice, s));
-            axpby(s, ne * ne, 0.0, tmp, -1.0, tmp);
-            to_path(s, p->prec, tmp, (char*)p->blocks + es * (1 + k) * ne * ne, ne * ne);
-        }
-        to_path(s, p->prec, h->T0inv, p->t0inv, ne * ne);
-        to_path(s, p->prec, h->PinvS, p->pinv, nc * nc);
+        const int ld = p->ld, ldc = p->ldc;
+        CK(cudaMalloc(&p->blocks, es * p->nblk * ne * ld));
+        CK(cudaMalloc(&p->t0inv, es * ne * ld));
+        CK(cudaMalloc(&p->pinv, es * nc * ldc));
+        to_path(s, p->prec, h->A, p->blocks, ne, (int)ne, ld, -1.0);
+        to_path(s, p->prec, h->L2, (char*)p->blocks + es * ne * ld, ne, (int)ne, ld, h->alpha);
+        to_path(s, p->prec, h->T + ne * ne, (char*)p->blocks + es * 2 * ne * ld, ne * (h->K - 1), (int)ne, ld, -1.0);
+        to_path(s, p->prec, h->T0inv, p->t0inv, ne, (int)ne, ld, 1.0);
+        to_path(s, p->prec, h->PinvS, p->pinv, nc, (int)nc, ldc, 1.0);
         CK(cudaStreamSynchronize(s));
-        cudaFree(tmp);
     }
     CK(cudaEventCreate(&p->ev0));
     CK(cudaEventCreate(&p->ev1));
@@ -490,9 +492,9 @@ tdcfie_status plan_set_solver(tdcfie_t h, int solver, int guess, double tol) {
     if (solver == TDCFIE_SOLVE_GMRES && h->formulation != TDCFIE_FORMULATION_QHP_CFIE)
         return fail(h, TDCFIE_E_UNSUPPORTED, "the comparison formulation uses the direct solve");
     const bool learned = guess == TDCFIE_GUESS_MLP || guess == TDCFIE_GUESS_MLP_EXTRAP;
-    if (solver == TDCFIE_SOLVE_GMRES && guess == TDCFIE_GUESS_EXTRAP && p->ring < 4)
+    if (solver == TDCFIE_SOLVE_GMRES && guess == TDCFIE_GUESS_EXTRAP && p->K - 1 < 4)
         return fail(h, TDCFIE_E_UNSUPPORTED, "the extrapolated guess needs K - 1 >= 4 stored steps");
-    if (solver == TDCFIE_SOLVE_GMRES && learned && p->ring < 8)
+    if (solver == TDCFIE_SOLVE_GMRES && learned && p->K - 1 < 8)
         return fail(h, TDCFIE_E_UNSUPPORTED, "the learned guess needs K - 1 >= 8 stored steps");
     h->opts.solver = solver;
     h->opts.guess = guess;
@@ -500,9 +502,9 @@ tdcfie_status plan_set_solver(tdcfie_t h, int solver, int guess, double tol) {
     if (solver == TDCFIE_SOLVE_GMRES) {
         if (!p->t0mat) {
             CK(cudaMalloc(&p->t0mat, es * ne * ne));
-            to_path(s, p->prec, h->T, p->t0mat, ne * ne);
-            CK(cudaMalloc(&p->guessbuf, es * R * ne));
-            CK(cudaMemsetAsync(p->guessbuf, 0, es * R * ne, s));
+            to_path(s, p->prec, h->T, p->t0mat, ne, (int)ne, (int)ne, 1.0);
+            CK(cudaMalloc(&p->guessbuf, es * R * p->ld));
+            CK(cudaMemsetAsync(p->guessbuf, 0, es * R * p->ld, s));
             CK(cudaStreamSynchronize(s));
         }
         if (!p->gm) CK(build_gmres(h, p));
@@ -512,19 +514,19 @@ tdcfie_status plan_set_solver(tdcfie_t h, int solver, int guess, double tol) {
     p->gmres_on = solver == TDCFIE_SOLVE_GMRES;
     p->mlp_on = p->gmres_on && learned;
     p->guess_extrap = guess == TDCFIE_GUESS_MLP_EXTRAP;
-    if (p->exec) { cudaGraphExecDestroy(p->exec); p->exec = nullptr; }
-    if (p->graph) { cudaGraphDestroy(p->graph); p->graph = nullptr; }
-    p->nodeA = p->nodeB = nullptr;
+    drop_graphs(p);
     return TDCFIE_OK;
 }
 
 tdcfie_status plan_reset(tdcfie_t h) {
     StepPlan* p = h->plan;
     cudaStream_t s = h->stream;
-    Ctl c{1, 1, nullptr, 0, 0, 0, nullptr};
+    Ctl c{};
+    c.n = c.n0 = c.p0 = 1;
+    c.bad_step = INT64_MAX;
     if (p->gm) CK(reset_gmres_stats(p->gm));
     CK(cudaMemcpyAsync(p->ctl, &c, sizeof(Ctl), cudaMemcpyHostToDevice, s));
-    CK(cudaMemsetAsync(p->ringbuf, 0, p->esz * p->ring * p->R * p->ne, s));
+    if (p->ringbuf) CK(cudaMemsetAsync(p->ringbuf, 0, p->esz * p->ring * p->R * p->ld, s));
     if (p->fact) {
         const tdcfie_status st = reset_fact(h, p);
         if (st != TDCFIE_OK) return st;
@@ -534,13 +536,61 @@ tdcfie_status plan_reset(tdcfie_t h) {
     return TDCFIE_OK;
 }
 
-// Enqueue one step of h on s (s must be capturing a graph).
+// Enqueue one whole step of h on s (s must be capturing a graph): on the SIMT paths the tests and
+// pre-sums (which return at once unless a chunk starts), the step, its post-processing.
 cudaError_t capture_step(tdcfie_t h, cudaStream_t s) {
     StepPlan* p = h->plan;
-    if (p->prec == TDCFIE_FP64) return launch_step<double>(h, *p, s);
-    if (p->prec == TDCFIE_FP32) return launch_step<float>(h, *p, s);
+    auto simt = [&](auto t) -> cudaError_t {
+        using T = decltype(t);
+        int k = launch_pre<T>(h, *p, s);
+        const cudaError_t e = launch_inner<T>(h, *p, false, 0, s, k);
+        k += launch_post<T>(h, *p, 1, s);
+        p->launches_per_step = k;
+        return e == cudaSuccess ? cudaGetLastError() : e;
+    };
+    if (p->prec == TDCFIE_FP64) return simt(0.0);
+    if (p->prec == TDCFIE_FP32) return simt(0.f);
     launch_step_tc(h, p, s);
     return cudaGetLastError();
+}
+
+// the executable graph `which` of the plan, captured on first use
+static tdcfie_status plan_graph(tdcfie_t h, int which) {
+    StepPlan* p = h->plan;
+    cudaStream_t s = h->stream;
+    if (p->exec[which]) return TDCFIE_OK;
+    CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+    cudaError_t ce;
+    if (p->gemm) {
+        ce = capture_step(h, s);
+        p->nodes[which] = p->launches_per_step;
+    } else if (p->prec == TDCFIE_FP64) {
+        ce = launch_graph<double>(h, *p, which, s);
+    } else {
+        ce = launch_graph<float>(h, *p, which, s);
+    }
+    const cudaError_t ee = cudaStreamEndCapture(s, &p->graph[which]);
+    if (ce != cudaSuccess) {
+        if (p->graph[which]) { cudaGraphDestroy(p->graph[which]); p->graph[which] = nullptr; }
+        return cuda_fail(h, ce, "capturing the step graph");
+    }
+    CK(ee);
+    CK(cudaGraphInstantiate(&p->exec[which], p->graph[which], 0));
+    if (!p->gemm) return TDCFIE_OK;
+    size_t nn = 0;
+    CK(cudaGraphGetNodes(p->graph[which], nullptr, &nn));
+    std::vector<cudaGraphNode_t> nodes(nn);
+    CK(cudaGraphGetNodes(p->graph[which], nodes.data(), &nn));
+    for (auto nd : nodes) {
+        cudaGraphNodeType ty;
+        CK(cudaGraphNodeGetType(nd, &ty));
+        if (ty != cudaGraphNodeTypeEventRecord) continue;
+        cudaEvent_t ev;
+        CK(cudaGraphEventRecordNodeGetEvent(nd, &ev));
+        if (ev == p->evA) p->nodeA = nd;
+        if (ev == p->evB) p->nodeB = nd;
+    }
+    return TDCFIE_OK;
 }
 
 // Output base of the next steps of h (synchronous on h's stream): step n writes row n - n0.
@@ -560,7 +610,7 @@ tdcfie_status plan_set_outputs(tdcfie_t h, void* out, void* yout) {
 
 // Status of the step state words: device timeout, then a non-finite current, then a GMRES solve that
 // stopped above its tolerance (each with the first step it happened at)
-static tdcfie_status status_of(tdcfie_t h, const Ctl& c) {
+tdcfie_status plan_status(tdcfie_t h, const Ctl& c) {
     if (c.timeout)
         return fail(h, TDCFIE_E_TIMEOUT, "a bounded device-side wait ran out (tensor-core pipeline)");
     if (c.status != 0)
@@ -576,7 +626,7 @@ tdcfie_status plan_check(tdcfie_t h) {
     StepPlan* p = h->plan;
     Ctl c;
     CK(cudaMemcpy(&c, p->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
-    return status_of(h, c);
+    return plan_status(h, c);
 }
 
 int plan_launches_per_step(tdcfie_t h) { return h->plan ? h->plan->launches_per_step : 0; }
@@ -589,40 +639,6 @@ tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout) {
         CK(cudaEventRecord(h->ev_in, 0));
         CK(cudaStreamWaitEvent(s, h->ev_in, 0));
     }
-    if (!p->exec) {
-        // capture one step
-        CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-        const cudaError_t ce = capture_step(h, s);
-        const cudaError_t ee = cudaStreamEndCapture(s, &p->graph);
-        if (ce != cudaSuccess) {
-            if (p->graph) { cudaGraphDestroy(p->graph); p->graph = nullptr; }
-            return cuda_fail(h, ce, "capturing the step graph");
-        }
-        CK(ee);
-        CK(cudaGraphInstantiate(&p->exec, p->graph, 0));
-        size_t nn = 0;
-        CK(cudaGraphGetNodes(p->graph, nullptr, &nn));
-        std::vector<cudaGraphNode_t> nodes(nn);
-        CK(cudaGraphGetNodes(p->graph, nodes.data(), &nn));
-        for (auto nd : nodes) {
-            cudaGraphNodeType ty;
-            CK(cudaGraphNodeGetType(nd, &ty));
-            if (ty != cudaGraphNodeTypeEventRecord) continue;
-            cudaEvent_t ev;
-            CK(cudaGraphEventRecordNodeGetEvent(nd, &ev));
-            if (ev == p->evA) p->nodeA = nd;
-            if (ev == p->evB) p->nodeB = nd;
-        }
-    }
-    // per-step events around the history sum (rotated into the executable graph before each launch)
-    const int64_t nev = std::min<int64_t>(nsteps, 4096);
-    while ((int64_t)p->hA.size() < nev) {
-        cudaEvent_t a, b;
-        CK(cudaEventCreate(&a));
-        CK(cudaEventCreate(&b));
-        p->hA.push_back(a);
-        p->hB.push_back(b);
-    }
     // set the output base of this call: n0 = current n
     Ctl c;
     CK(cudaMemcpyAsync(&c, p->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
@@ -630,17 +646,58 @@ tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout) {
     c.n0 = c.n;
     c.out = out;
     c.yout = yout;
+    c.hist_ns = 0;
     CK(cudaMemcpyAsync(p->ctl, &c, sizeof(Ctl), cudaMemcpyHostToDevice, s));
     long long g0[6] = {0, 0, 0, 0, 0, 0}, g1[6] = {0, 0, 0, 0, 0, 0};
     if (p->gm) CK(gmres_stats(p->gm, g0));
-    CK(cudaEventRecord(p->ev0, s));
-    for (int64_t i = 0; i < nsteps; ++i) {
-        if (i < nev && p->nodeA && p->nodeB) {
-            CK(cudaGraphExecEventRecordNodeSetEvent(p->exec, p->nodeA, p->hA[i]));
-            CK(cudaGraphExecEventRecordNodeSetEvent(p->exec, p->nodeB, p->hB[i]));
+    int64_t kernels = 0;
+    auto run = [&](int which) -> tdcfie_status {
+        const tdcfie_status st = plan_graph(h, which);
+        if (st != TDCFIE_OK) return st;
+        CK(cudaGraphLaunch(p->exec[which], s));
+        kernels += p->nodes[which];
+        return TDCFIE_OK;
+    };
+#define RUN(g) do { const tdcfie_status st_ = run(g); if (st_ != TDCFIE_OK) return st_; } while (0)
+    int64_t nev = 0;
+    if (p->gemm) {
+        // per-step events around the history sum (rotated into the executable graph before each launch)
+        nev = std::min<int64_t>(nsteps, 4096);
+        while ((int64_t)p->hA.size() < nev) {
+            cudaEvent_t a, b;
+            CK(cudaEventCreate(&a));
+            CK(cudaEventCreate(&b));
+            p->hA.push_back(a);
+            p->hB.push_back(b);
         }
-        CK(cudaGraphLaunch(p->exec, s));
+        const tdcfie_status st = plan_graph(h, StepPlan::G_STEP);
+        if (st != TDCFIE_OK) return st;
+        CK(cudaEventRecord(p->ev0, s));
+        for (int64_t i = 0; i < nsteps; ++i) {
+            if (i < nev && p->nodeA && p->nodeB) {
+                CK(cudaGraphExecEventRecordNodeSetEvent(p->exec[0], p->nodeA, p->hA[i]));
+                CK(cudaGraphExecEventRecordNodeSetEvent(p->exec[0], p->nodeB, p->hB[i]));
+            }
+            RUN(StepPlan::G_STEP);
+        }
+    } else {
+        // whole chunks by one graph (the GMRES loop nodes only step by step), the rest step by step;
+        // the post-processing runs when a chunk ends and when the call does
+        const int64_t C = p->C;
+        CK(cudaEventRecord(p->ev0, s));
+        for (int64_t n = c.n, end = c.n + nsteps; n < end;) {
+            const int64_t i = (n - 1) % C, m = std::min(C - i, end - n);
+            if (m == C && !p->gmres_on) {
+                RUN(StepPlan::G_CHUNK);
+            } else {
+                if (i == 0) RUN(StepPlan::G_PRE);
+                for (int64_t q = 0; q < m; ++q) RUN(StepPlan::G_STEP);
+                if (!p->fact) RUN(StepPlan::G_POST);
+            }
+            n += m;
+        }
     }
+#undef RUN
     CK(cudaEventRecord(p->ev1, s));
     CK(cudaMemcpyAsync(&c, p->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -653,13 +710,13 @@ tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout) {
         float e = 0.f;
         if (cudaEventElapsedTime(&e, p->hA[i], p->hB[i]) == cudaSuccess) { hs += e; ++cnt; }
     }
-    h->last_hist_ms = cnt ? hs / cnt : 0.0;
-    h->last_launches = nsteps * p->launches_per_step;
+    h->last_hist_ms = p->gemm ? (cnt ? hs / cnt : 0.0) : 1e-6 * (double)c.hist_ns / (double)nsteps;
+    h->last_launches = kernels;
     if (p->gm) {
         CK(gmres_stats(p->gm, g1));
         h->last_launches += (g1[5] - g0[5]) * gmres_body_launches();
     }
-    return status_of(h, c);
+    return plan_status(h, c);
 }
 
 }  // namespace tdc

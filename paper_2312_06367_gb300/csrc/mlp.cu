@@ -172,12 +172,12 @@ __device__ float block_rms(const T* __restrict__ y, int ne, float* red) {
 
 // s_r = RMS over edges of y_{n-1} (one block of 256 threads per right-hand side)
 template <typename T>
-__global__ void k_mlp_rms(const T* __restrict__ ringbuf, int ring, int R, int ne, const Ctl* ctl,
+__global__ void k_mlp_rms(const T* __restrict__ ringbuf, int ring, int R, int ne, int ld, const Ctl* ctl,
                           float* __restrict__ scale) {
     __shared__ float red[256];
     const int r = blockIdx.x;
     const int64_t n = ctl->n;
-    const T* y = n > 1 ? ringbuf + ((n - 1) % ring) * (int64_t)R * ne + (int64_t)r * ne : nullptr;
+    const T* y = n > 1 ? ringbuf + (((n - 1) % ring) * R + r) * (int64_t)ld : nullptr;
     const float s = block_rms(y, ne, red);
     if (threadIdx.x == 0) scale[r] = s;
 }
@@ -209,7 +209,7 @@ __global__ void k_mlp_samples(const T* __restrict__ y, int R, int ne, int base, 
 // extrapolation 4 y_{n-1} - 6 y_{n-2} + 4 y_{n-3} - y_{n-4}; y_i = 0 for i <= 0.  The base is formed in
 // the path precision T, so a network that outputs zero reproduces it exactly.
 template <typename T>
-__global__ void k_mlp_guess(const __half* __restrict__ wh, const T* __restrict__ ringbuf, int ring, int R, int ne,
+__global__ void k_mlp_guess(const __half* __restrict__ wh, const T* __restrict__ ringbuf, int ring, int R, int ne, int ld,
                             const Ctl* ctl, const float* __restrict__ scale, int extrap, T* __restrict__ guess) {
     __shared__ float P[NP];
     for (int i = threadIdx.x; i < NP; i += blockDim.x) P[i] = __half2float(wh[i]);
@@ -224,14 +224,13 @@ __global__ void k_mlp_guess(const __half* __restrict__ wh, const T* __restrict__
     for (int k = 1; k <= NIN; ++k) {
         T v = 0;
         if (n - k >= 1) {
-            int64_t sl = (n - k) % ring;
-            v = ringbuf[sl * (int64_t)R * ne + (int64_t)r * ne + m];
+            v = ringbuf[(((n - k) % ring) * R + r) * (int64_t)ld + m];
         }
         if (k <= 4) yk[k - 1] = v;
         x[k - 1] = (float)v / s;
     }
     const T base = extrap ? (T)4 * yk[0] - (T)6 * yk[1] + (T)4 * yk[2] - yk[3] : yk[0];
-    guess[(int64_t)r * ne + m] = base + (T)(s * mlp_forward(P, x));   // base + predicted correction
+    guess[(int64_t)r * ld + m] = base + (T)(s * mlp_forward(P, x));   // base + predicted correction
 }
 
 // ---------------------------------------------------------------- march integration
@@ -249,16 +248,16 @@ void destroy_mlp(MlpState* m) {
 }
 
 template <typename T>
-void launch_mlp_guess(StepPlan* p, cudaStream_t s) {
+int launch_mlp_guess(StepPlan* p, cudaStream_t s) {
     MlpState* m = p->mlp;
-    k_mlp_rms<T><<<p->R, 256, 0, s>>>((const T*)p->ringbuf, p->ring, p->R, p->ne, p->ctl, m->scale);
+    k_mlp_rms<T><<<p->R, 256, 0, s>>>((const T*)p->ringbuf, p->ring, p->R, p->ne, p->ld, p->ctl, m->scale);
     k_mlp_guess<T><<<(p->R * p->ne + 127) / 128, 128, 0, s>>>(m->wh, (const T*)p->ringbuf, p->ring, p->R, p->ne,
-                                                                p->ctl, m->scale, p->guess_extrap ? 1 : 0,
+                                                                p->ld, p->ctl, m->scale, p->guess_extrap ? 1 : 0,
                                                                 (T*)p->guessbuf);
-    p->launches_per_step += 2;
+    return 2;
 }
-template void launch_mlp_guess<double>(StepPlan*, cudaStream_t);
-template void launch_mlp_guess<float>(StepPlan*, cudaStream_t);
+template int launch_mlp_guess<double>(StepPlan*, cudaStream_t);
+template int launch_mlp_guess<float>(StepPlan*, cudaStream_t);
 
 cudaError_t build_mlp(StepPlan* p) {
     auto* m = new MlpState();
@@ -384,7 +383,7 @@ extern "C" tdcfie_status tdcfie_mlp_samples(int precision, int base, const void*
 extern "C" tdcfie_status tdcfie_mlp_load(tdcfie_t h, const float* params) {
     if (!h || !params) return fail(h, TDCFIE_E_ARG, "NULL argument");
     if (!h->plan) return fail(h, TDCFIE_E_STATE, "call tdcfie_assemble first");
-    if (h->plan->ring < 8) return fail(h, TDCFIE_E_UNSUPPORTED, "the learned guess needs K - 1 >= 8 stored steps");
+    if (h->plan->K - 1 < 8) return fail(h, TDCFIE_E_UNSUPPORTED, "the learned guess needs K - 1 >= 8 stored steps");
     if (!h->plan->mlp) {
         const cudaError_t eb = build_mlp(h->plan);
         if (eb != cudaSuccess) return cuda_fail(h, eb, "learned-guess state");

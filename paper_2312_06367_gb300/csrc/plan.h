@@ -14,51 +14,70 @@ struct StepPlan {
     int prec = TDCFIE_FP64;
     int R = 1, ne = 0, nc = 0, K = 0, nblk = 0, ring = 0;
     size_t esz = 8;
-    void* blocks = nullptr;      // nblk x ne x ne (path precision): -A, alpha L2, -T_1 .. -T_{K-1}
-    void* t0inv = nullptr;       // ne x ne
+    int C = 1;                   // SIMT paths: steps per chunk (simt.h)
+    int ld = 0, ldc = 0;         // SIMT paths: row lengths of matrices and vectors (16-byte multiples)
+    int ngroups = 0, npts = 0;   // SIMT paths: groups of the pre-sums, distinct quadrature points
+    void* blocks = nullptr;      // nblk x ne x ld (path precision): -A, alpha L2, -T_1 .. -T_{K-1}
+    void* t0inv = nullptr;       // ne x ld
     void* t0mat = nullptr;       // ne x ne, T_0 itself (GMRES matvec)
-    void* guessbuf = nullptr;    // R x ne learned initial guess
+    void* guessbuf = nullptr;    // R x ld learned initial guess
     GmresPlan* gm = nullptr;
     MlpState* mlp = nullptr;     // learned-guess network (GMRES with TDCFIE_GUESS_MLP)
     bool gmres_on = false;       // per-step solve by GMRES (else the explicit T_0^-1)
     bool mlp_on = false;         // learned guess evaluated each step
     bool guess_extrap = false;   // learned guess on top of the cubic extrapolation (else y_{n-1})
-    void* pinv = nullptr;        // nc x nc
-    void* E = nullptr;           // R x ne  (e_n)
-    void* Hv = nullptr;          // R x ne  (h_n)
-    void* ringbuf = nullptr;     // ring x R x ne
-    void* b = nullptr;           // R x ne
-    void* partial = nullptr;     // nblk x R x ne
-    void* w = nullptr;           // R x ne
-    void* z = nullptr;           // R x nc
-    void* u = nullptr;           // R x nc
-    const void** xptr = nullptr; // device array (unused for SIMT: computed in kernel)
+    void* pinv = nullptr;        // nc x ldc
+    void* E = nullptr;           // C x R x ld  (e of the chunk's steps)
+    void* Hv = nullptr;          // C x R x ld  (h)
+    void* ringbuf = nullptr;     // ring x R x ld, then R x ld zeros
+    void* b = nullptr;           // R x ld
+    void* partial = nullptr;     // ngroups x C x R x ld pre-sums (8 bytes each: FP64, or an FP32 pair)
+    void* inner = nullptr;       // C x C x R x ld products of the lags inside a chunk
+    void* z = nullptr;           // C x R x ldc
+    void* u = nullptr;           // C x R x ldc
+    int* done = nullptr;
     Ctl* ctl = nullptr;
-    // rhs tables: per edge, quadrature points (x) and weighted basis vectors (c), e-points first
+    // plane-wave tests, SIMT paths: distinct points, and per edge (e-points first) point index and
+    // weighted basis vector
+    void* env = nullptr; void* pts = nullptr; void* ecoef = nullptr;
+    int* eptr = nullptr; int* enE = nullptr; int* eidx = nullptr;
+    // the same per entry for the tensor paths: quadrature points (x) and weighted basis vectors (c)
     int* pptr = nullptr; int* pnE = nullptr; void* px = nullptr; void* pc = nullptr;
     // factored history form (factored.cu); blocks and t0inv are then unused
     FactPlan* fact = nullptr;
     // tensor-core path
     TcStep* gemm = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    // step graphs.  Tensor paths: G_STEP is one step.  SIMT paths: G_PRE the tests and pre-sums of a
+    // chunk, G_STEP one step's history and solve, G_POST the post-processing of the finished steps,
+    // G_CHUNK a whole chunk.
+    enum { G_STEP = 0, G_PRE, G_POST, G_CHUNK, NGRAPH };
+    cudaGraph_t graph[NGRAPH] = {};
+    cudaGraphExec_t exec[NGRAPH] = {};
+    int nodes[NGRAPH] = {};                              // kernels per graph
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
-    cudaEvent_t evA = nullptr, evB = nullptr;            // captured around the history sum
+    cudaEvent_t evA = nullptr, evB = nullptr;            // tensor paths: captured around the history sum
     cudaGraphNode_t nodeA = nullptr, nodeB = nullptr;    // their record nodes in the step graph
     std::vector<cudaEvent_t> hA, hB;                     // per-step events of a tdcfie_step call
     int launches_per_step = 0;
 };
 
-// plane-wave tests e_n, h_n of one step into p.E, p.Hv (march.cu)
 template <typename T>
-void launch_rhs(tdcfie_t h, StepPlan& p, cudaStream_t s);
+struct SimtDev;
+// device view of the plan (march.cu)
+template <typename T>
+SimtDev<T> simt_view(tdcfie_t h, const StepPlan& p);
+// plane-wave tests of a chunk into p.E, p.Hv: nothing unless a chunk starts at the current step
+// (march.cu); returns the number of kernels
+template <typename T>
+int launch_tests(tdcfie_t h, StepPlan& p, cudaStream_t s);
 // factored history form (factored.cu)
 tdcfie_status build_fact(tdcfie_t h, StepPlan* p);
 tdcfie_status reset_fact(tdcfie_t h, StepPlan* p);
 void destroy_fact(FactPlan* f);
 double fact_step_bytes(const StepPlan* p);
 int64_t fact_nnz(const StepPlan* p, bool stored);
+// history, solve and post-processing of one step (the factored form needs j_n in its own history)
 template <typename T>
-cudaError_t launch_step_fact(tdcfie_t h, StepPlan& p, cudaStream_t s);
+int launch_step_fact(tdcfie_t h, StepPlan& p, cudaStream_t s);
 
 }  // namespace tdc

@@ -1,154 +1,382 @@
 // Device arithmetic of the SIMT (FP64 / FP32) step, shared by the per-handle step kernels
 // (march.cu) and the persistent uneven-batch kernel (batch.cu), so that both compute the same
 // values bit for bit.
+//
+// The march is blocked in time.  Step n belongs to the chunk of C steps that starts at the absolute
+// step n0 = n - i, i = (n - 1) mod C, so that the arithmetic of a step does not depend on how the
+// caller cuts the march into calls.  Everything of a chunk that is known before its first solve is
+// computed once for its C steps (columns) when n0 is reached:
+//   tests    e_n, h_n of the C steps (the incident field does not depend on the march);
+//   pre      the sums over the blocks -A e, alpha L2 h and over every lag k > i of column i, which
+//            reaches back before n0: each block is read once per chunk instead of once per step;
+// then step by step
+//   hist     b_n = (pre-sums of column i) - sum_{k = i..1} T_k y_{n-k}, the lags inside the chunk: only
+//            k = 1 waits for the solve before; the products T_k y_{n-1}, k >= 2, of the later columns
+//            are formed beside it, one per row and lag, so that the step's chain stays short;
+//   solve    y_n = T_0^-1 b_n (or GMRES);
+// and the post-processing of the finished steps together (its projector is not part of the
+// recurrence).  Matrix bytes per step at K = 42, C = 8: 43/8 + 3.5 + 1 + 1/8 blocks instead of 45.
+//
+// Rows of matrices and vectors are padded to 16 bytes (zeros), every load is a 16-byte vector.
 #pragma once
 #include "internal.h"
 
 namespace tdc {
 
-// ---------------------------------------------------------------- plane-wave tests
-// Per edge m a list of quadrature points with a weighted basis vector: 7 points on each
-// triangle of f_m (degree-5 rule, coefficient w A f_m(x)) for e_m and 3 points on each fine
-// triangle of g_m (degree-2 rule, coefficient w A g_m(x)) for h_m.  Per step n and wave P:
-//   e_m = sum_x c(x).p env(x, t_n),  h_m = sum_x c(x).(k x p) env(x, t_n),
-//   env(x, t) = amp exp(-((t - k.x - t0)/width)^2).
-template <typename T>
-__device__ __forceinline__ T mul_rn(T a, T b);
-template <>
-__device__ __forceinline__ float mul_rn<float>(float a, float b) { return __fmul_rn(a, b); }
-template <>
-__device__ __forceinline__ double mul_rn<double>(double a, double b) { return __dmul_rn(a, b); }
-template <typename T>
-__device__ __forceinline__ T add_rn(T a, T b);
-template <>
-__device__ __forceinline__ float add_rn<float>(float a, float b) { return __fadd_rn(a, b); }
-template <>
-__device__ __forceinline__ double add_rn<double>(double a, double b) { return __dadd_rn(a, b); }
+constexpr int GQ = 4;         // blocks per group of the pre-sums
 
-// Every multiply-add below is spelled out (fma or a rounded product), so that the per-handle
-// kernels and the persistent batch kernel, which inline this code into different kernels, round
-// identically.
+// Sums are carried in FP64 on the FP64 path and as unevaluated FP32 pairs (about 48 bits) on the FP32
+// path: the FP64 pipe would bound the warp reductions there.
+struct Pair32 { float h, l; };
+template <typename T> struct SumOf;
+template <> struct SumOf<double> { using S = double; };
+template <> struct SumOf<float> { using S = Pair32; };
+
 template <typename T>
-__device__ __forceinline__ void rhs_edge(const double* P, int64_t n, double dt, int mm, const int* __restrict__ pptr,
-                                         const T* __restrict__ px, const T* __restrict__ pc, const int* __restrict__ nE,
-                                         T& e_out, T& h_out) {
-    const T kx = (T)P[0], ky = (T)P[1], kz = (T)P[2], qx = (T)P[3], qy = (T)P[4], qz = (T)P[5];
+struct SimtDev {              // device view of one handle's step plan
+    int ne, nc, R, C, K, ring, ld, ldc, ngroups, npts;
+    const T *blocks, *t0inv, *pinv;     // (K + 1) x ne x ld (-A, alpha L2, -T_1 ..), ne x ld, nc x ldc
+    T *E, *H;                           // tests of the chunk [C R][ld], column i R + r
+    T *rbuf, *b;                        // ring [ring][R][ld], b_n [R][ld]
+    T *z, *u;                           // projector vectors of the steps to post-process [C R][ldc]
+    typename SumOf<T>::S* partial;      // pre-sums [ngroups][C R][ld]
+    typename SumOf<T>::S* inner;        // T_k y of lag k >= 2 for column i of the chunk [i][k][R][ld]
+    T* env;                             // envelopes [npts][R][C]
+    const T* pts;                       // distinct quadrature points, npts x 3
+    const int *eptr, *enE, *eidx;       // per edge: entries (e-points first), number of e-points, point index
+    const T* ecoef;                     // weighted basis vector per entry
+    const double* exc;
+    DevMesh m;
+    double dt, dtt;
+    Ctl* ctl;
+    int* done;
+};
+
+template <typename T> __device__ __forceinline__ T mul_rn(T a, T b);
+template <> __device__ __forceinline__ float mul_rn<float>(float a, float b) { return __fmul_rn(a, b); }
+template <> __device__ __forceinline__ double mul_rn<double>(double a, double b) { return __dmul_rn(a, b); }
+template <typename T> __device__ __forceinline__ T add_rn(T a, T b);
+template <> __device__ __forceinline__ float add_rn<float>(float a, float b) { return __fadd_rn(a, b); }
+template <> __device__ __forceinline__ double add_rn<double>(double a, double b) { return __dadd_rn(a, b); }
+
+__device__ __forceinline__ int64_t ring_slot(int64_t n, int ring) {
+    const int64_t s = n % ring;
+    return s < 0 ? s + ring : s;
+}
+
+// ---------------------------------------------------------------- plane-wave tests
+// e_m(t_n) = sum_x c(x).p env(x, t_n) over the 7-point rule of the RWG triangles, h_m the same with
+// c(x).(k x p) over the 3-point rule of the BC fine triangles; env(x, t) = amp exp(-((t - k.x - t0) /
+// width)^2).  A point belongs to three RWG or about twelve BC functions, so the envelopes are taken
+// once per point (one exponential each) and gathered per edge.  Every multiply-add is spelled out,
+// so that all kernels that inline this round identically.
+template <typename T>
+__device__ __forceinline__ T env_point(const double* P, int64_t n, double dt, T x, T y, T z) {
+    const T kx = (T)P[0], ky = (T)P[1], kz = (T)P[2];
     const T amp = (T)P[6], inv_w = (T)(1.0 / P[8]);
     const T tt = (T)((double)n * dt - P[7]);
+    const T arg = mul_rn(add_rn(tt, -fma(kx, x, fma(ky, y, mul_rn(kz, z)))), inv_w);
+    return mul_rn(amp, exp(-mul_rn(arg, arg)));
+}
+
+// e, h of edge m and wave r for the chunk's C steps (a divisor of 32): lane l takes column l % C and
+// every (32 / C)-th entry; the parts are added by a fixed tree
+template <typename T>
+__device__ __forceinline__ void gather_edge(const SimtDev<T>& d, int m, int r, int lane) {
+    const double* P = d.exc + 11 * r;
+    const T kx = (T)P[0], ky = (T)P[1], kz = (T)P[2], qx = (T)P[3], qy = (T)P[4], qz = (T)P[5];
     const T hx = fma(ky, qz, -mul_rn(kz, qy)), hy = fma(kz, qx, -mul_rn(kx, qz)), hz = fma(kx, qy, -mul_rn(ky, qx));   // k x p
+    const int i = lane % d.C, part = lane / d.C, parts = 32 / d.C;
+    const int b = d.eptr[m], me = b + d.enE[m], end = d.eptr[m + 1];
     T e = 0, h = 0;
-    const int b = pptr[mm], me = b + nE[mm], end = pptr[mm + 1];
-    for (int q = b; q < end; ++q) {
-        const T x = px[3 * q], y = px[3 * q + 1], z = px[3 * q + 2];
-        const T arg = mul_rn(add_rn(tt, -fma(kx, x, fma(ky, y, mul_rn(kz, z)))), inv_w);
-        const T env = mul_rn(amp, exp(-mul_rn(arg, arg)));
-        const T cx = pc[3 * q], cy = pc[3 * q + 1], cz = pc[3 * q + 2];
+#pragma unroll 4
+    for (int q = b + part; q < end; q += parts) {
+        const T cx = d.ecoef[3 * q], cy = d.ecoef[3 * q + 1], cz = d.ecoef[3 * q + 2];
+        const T env = d.env[((int64_t)d.eidx[q] * d.R + r) * d.C + i];
         if (q < me) e = fma(env, fma(cx, qx, fma(cy, qy, mul_rn(cz, qz))), e);
         else h = fma(env, fma(cx, hx, fma(cy, hy, mul_rn(cz, hz))), h);
     }
-    e_out = e;
-    h_out = h;
+    for (int o = 16; o >= d.C; o >>= 1) {
+        e = add_rn(e, __shfl_xor_sync(0xffffffffu, e, o));
+        h = add_rn(h, __shfl_xor_sync(0xffffffffu, h, o));
+    }
+    if (part == 0) {
+        d.E[(int64_t)(i * d.R + r) * d.ld + m] = e;
+        d.H[(int64_t)(i * d.R + r) * d.ld + m] = h;
+    }
 }
 
 // ---------------------------------------------------------------- row dot products (SIMT)
-// partial[q][r][i] = sum_j B_q[i][j] x_q[r][j] for one warp per (row i, block q); x_q is e_n, h_n
-// or a ring slot chosen from the device step counter.
-template <typename T> struct Vec2;
-template <> struct Vec2<double> { using type = double2; };
-template <> struct Vec2<float> { using type = float4; };
+// One warp, lane l takes the 16-byte vectors l, l + 32, ... of a row.  FP64: plain FP64
+// accumulation, one accumulator per vector component.  FP32: the products and their sums are carried
+// error-free (each product's rounding error from an FMA, each addition's from Knuth's TwoSum), so the
+// result equals the exact dot product of the FP32 inputs to about FP32 precision squared; the lanes
+// are combined as pairs too.  The MOT recurrence turns y into the current through (y_n - y_{n-1}) / dtt
+// (Eq. post_processing), which magnifies any per-step error of y by about |y| / |y_n - y_{n-1}|;
+// plain FP32 accumulation over rows of thousands of entries is then far above the reduced-precision
+// bar at small time steps.  The FP32 accumulators are packed pairs: ten two-lane instructions per two
+// products, half the issue slots of scalar code (issue bounds FP32 with several columns).
+template <typename T> struct VecOf;
+template <> struct VecOf<double> { using V = double2; static constexpr int W = 2; };
+template <> struct VecOf<float> { using V = float4; static constexpr int W = 4; };
 
-// Row dot products of one warp: acc[r] = B . x_r.  FP64: plain FP64 accumulation.  FP32: the
-// products and their sums are carried error-free (each product's rounding error from an FMA, each
-// addition's from Knuth's TwoSum), so the result equals the exact dot product of the FP32 inputs to
-// about FP32 precision squared; the lanes are combined in FP64.  The MOT recurrence turns y into the
-// current through (y_n - y_{n-1}) / dtt (Eq. post_processing), which magnifies any per-step error of
-// y by about |y| / |y_n - y_{n-1}|; plain FP32 accumulation over rows of thousands of entries is
-// then far above the reduced-precision bar at small time steps.
-template <typename T, int RMAX>
-struct RowDot {
-    __device__ static void run(const T* __restrict__ B, int ncols, const T* __restrict__ x, int R, int ldx,
-                               double* acc) {
-        const int lane = threadIdx.x & 31;
-        T s[RMAX];
-#pragma unroll
-        for (int r = 0; r < RMAX; ++r) s[r] = 0;
-        for (int j = lane; j < ncols; j += 32) {
-            const T a = B[j];
-#pragma unroll
-            for (int r = 0; r < RMAX; ++r)
-                if (r < R) s[r] = fma(a, x[(int64_t)r * ldx + j], s[r]);
-        }
-#pragma unroll
-        for (int r = 0; r < RMAX; ++r) {
-            double v = (double)s[r];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            acc[r] = v;
-        }
+template <typename T> struct Acc;
+template <>
+struct Acc<double> {
+    double s0 = 0.0, s1 = 0.0;
+    __device__ __forceinline__ void add(const double2& a, const double2&, const double2& x) {
+        s0 = fma(a.x, x.x, s0);
+        s1 = fma(a.y, x.y, s1);
     }
+    __device__ __forceinline__ double sum() const { return s0 + s1; }
 };
 
-__device__ __forceinline__ void ff_add(float& hi, float& lo, float a, float b) {
-    // rounded operations only: a contracted multiply-add here would break the error-free sums
-    const float p = __fmul_rn(a, b);
-    const float pe = fmaf(a, b, -p);        // a b = p + pe exactly
-    const float t = __fadd_rn(hi, p);        // TwoSum(hi, p) = t + te
-    const float bp = __fsub_rn(t, hi);
-    const float te = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bp)), __fsub_rn(p, bp));
+// sum of two sums; on pairs TwoSum of the leading parts (the same result for either order)
+__device__ __forceinline__ double add_sum(double a, double b) { return a + b; }
+__device__ __forceinline__ Pair32 add_sum(Pair32 a, Pair32 b) {
+    const float t = __fadd_rn(a.h, b.h);
+    const float bp = __fsub_rn(t, a.h);
+    const float te = __fadd_rn(__fsub_rn(a.h, __fsub_rn(t, bp)), __fsub_rn(b.h, bp));
+    return Pair32{t, __fadd_rn(__fadd_rn(a.l, b.l), te)};
+}
+__device__ __forceinline__ double shfl_sum(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ Pair32 shfl_sum(Pair32 a, int o) {
+    return Pair32{__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.l, o)};
+}
+__device__ __forceinline__ double sum_value(double a) { return a; }
+__device__ __forceinline__ double sum_value(Pair32 a) { return (double)a.h + (double)a.l; }
+
+// hi + lo += a b on two lanes; na = -a.  Rounded intrinsics only: nothing may be contracted.
+__device__ __forceinline__ void ff_add2(float2& hi, float2& lo, float2 a, float2 na, float2 b) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 p = __fmul2_rn(a, b);
+    const float2 pe = __ffma2_rn(na, b, p);     // p - a b: minus the product's rounding error, exact
+    const float2 t = __fadd2_rn(hi, p);         // TwoSum(hi, p) = t + te
+    const float2 bp = __ffma2_rn(hi, m1, t);    // t - hi
+    const float2 ap = __ffma2_rn(bp, m1, t);    // t - bp
+    const float2 te = __fadd2_rn(__ffma2_rn(ap, m1, hi), __ffma2_rn(bp, m1, p));
+    lo = __fadd2_rn(lo, __ffma2_rn(pe, m1, te));
     hi = t;
-    lo = __fadd_rn(lo, __fadd_rn(te, pe));
 }
-
-template <int RMAX>
-struct RowDot<float, RMAX> {
-    __device__ static void run(const float* __restrict__ B, int ncols, const float* __restrict__ x, int R, int ldx,
-                               double* acc) {
-        const int lane = threadIdx.x & 31;
-        // four independent compensated accumulators per right-hand side (one per float4 component)
-        float hi[RMAX][4], lo[RMAX][4];
-#pragma unroll
-        for (int r = 0; r < RMAX; ++r)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) hi[r][c] = lo[r][c] = 0.f;
-        const bool vec = ((ncols | ldx) & 3) == 0 && ((reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(x)) & 15) == 0;
-        if (vec) {
-            const float4* B4 = reinterpret_cast<const float4*>(B);
-            for (int j = lane; j < (ncols >> 2); j += 32) {
-                const float4 a = B4[j];
-#pragma unroll
-                for (int r = 0; r < RMAX; ++r)
-                    if (r < R) {
-                        const float4 v = reinterpret_cast<const float4*>(x + (int64_t)r * ldx)[j];
-                        ff_add(hi[r][0], lo[r][0], a.x, v.x);
-                        ff_add(hi[r][1], lo[r][1], a.y, v.y);
-                        ff_add(hi[r][2], lo[r][2], a.z, v.z);
-                        ff_add(hi[r][3], lo[r][3], a.w, v.w);
-                    }
-            }
-        } else {
-            for (int j = lane; j < ncols; j += 32) {
-                const float a = B[j];
-#pragma unroll
-                for (int r = 0; r < RMAX; ++r)
-                    if (r < R) ff_add(hi[r][0], lo[r][0], a, x[(int64_t)r * ldx + j]);
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < RMAX; ++r) {
-            double v = 0.0;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) v += (double)hi[r][c] + (double)lo[r][c];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            acc[r] = v;
-        }
+template <>
+struct Acc<float> {
+    float2 h0 = {0.f, 0.f}, h1 = {0.f, 0.f}, l0 = {0.f, 0.f}, l1 = {0.f, 0.f};
+    __device__ __forceinline__ void add(const float4& a, const float4& na, const float4& x) {
+        ff_add2(h0, l0, make_float2(a.x, a.y), make_float2(na.x, na.y), make_float2(x.x, x.y));
+        ff_add2(h1, l1, make_float2(a.z, a.w), make_float2(na.z, na.w), make_float2(x.z, x.w));
+    }
+    __device__ __forceinline__ Pair32 sum() const {
+        return add_sum(add_sum(Pair32{h0.x, l0.x}, Pair32{h0.y, l0.y}), add_sum(Pair32{h1.x, l1.x}, Pair32{h1.y, l1.y}));
     }
 };
+__device__ __forceinline__ double2 neg(double2 a) { return a; }    // unused by Acc<double>
+__device__ __forceinline__ float4 neg(float4 a) { return make_float4(-a.x, -a.y, -a.z, -a.w); }
 
-template <typename T, int RMAX>
-__device__ __forceinline__ void warp_rows(const T* __restrict__ B, int ncols, const T* __restrict__ x, int R,
-                                          int ldx, double* acc) {
-    RowDot<T, RMAX>::run(B, ncols, x, R, ldx, acc);
+// acc[i][c] += row_i . x_c for ROWS rows and COLS columns, nvec vectors per row.  No branch on a
+// column (one that is not wanted points at zeros or repeats another), so that all loads of a turn are
+// in flight together; the rows' next vectors are fetched a turn ahead.
+template <typename T, int ROWS, int COLS>
+__device__ __forceinline__ void tile_rows(const T* const (&row)[ROWS], const T* __restrict__ x, const int (&off)[COLS],
+                                          int nvec, int lane, Acc<T> (&acc)[ROWS][COLS]) {
+    using V = typename VecOf<T>::V;
+    if constexpr (ROWS * COLS >= 8) {
+        V nx[ROWS];
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) nx[i] = lane < nvec ? __ldg(reinterpret_cast<const V*>(row[i]) + lane) : V{};
+#pragma unroll 1
+        for (int j = lane; j < nvec; j += 32) {
+            V a[ROWS], na[ROWS], xv[COLS];
+#pragma unroll
+            for (int c = 0; c < COLS; ++c) xv[c] = reinterpret_cast<const V*>(x + off[c])[j];
+#pragma unroll
+            for (int i = 0; i < ROWS; ++i) {
+                a[i] = nx[i];
+                na[i] = neg(a[i]);
+                if (j + 32 < nvec) nx[i] = __ldg(reinterpret_cast<const V*>(row[i]) + j + 32);
+            }
+#pragma unroll
+            for (int c = 0; c < COLS; ++c)
+#pragma unroll
+                for (int i = 0; i < ROWS; ++i) acc[i][c].add(a[i], na[i], xv[c]);
+        }
+    } else {
+        constexpr int U = ROWS * COLS >= 4 ? 2 : 4;      // turns whose loads are issued together
+        for (int j0 = lane; j0 < nvec; j0 += 32 * U) {
+            V a[U][ROWS], xv[U][COLS];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int j = j0 + 32 * u;
+                const bool in = j < nvec;
+#pragma unroll
+                for (int i = 0; i < ROWS; ++i) a[u][i] = in ? __ldg(reinterpret_cast<const V*>(row[i]) + j) : V{};
+#pragma unroll
+                for (int c = 0; c < COLS; ++c) xv[u][c] = in ? reinterpret_cast<const V*>(x + off[c])[j] : V{};
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int i = 0; i < ROWS; ++i) {
+                    const V na = neg(a[u][i]);
+#pragma unroll
+                    for (int c = 0; c < COLS; ++c) acc[i][c].add(a[u][i], na, xv[u][c]);
+                }
+        }
+    }
 }
 
+// Sums over the warp of V values per lane (V a power of two up to 32): every sum is the same tree
+// over lanes (strides 16, 8, 4, 2, 1) whatever V is, and the first log2 V strides halve the number of
+// values a lane carries.  The lane returns the sum of value multi_index<V>(lane).
+template <int V, typename S>
+__device__ __forceinline__ S multi_reduce(S (&v)[V], int lane) {
+    int n = V;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = lane & o;
+#pragma unroll
+            for (int j = 0; j < V / 2; ++j)
+                if (j < n) {
+                    const S keep = up ? v[j + n] : v[j], send = up ? v[j] : v[j + n];
+                    v[j] = add_sum(keep, shfl_sum(send, o));
+                }
+        } else {
+            v[0] = add_sum(v[0], shfl_sum(v[0], o));
+        }
+    }
+    return v[0];
+}
+template <int V>
+__device__ __forceinline__ int multi_index(int lane) {
+    int id = 0, n = V;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        if (n > 1) {
+            n >>= 1;
+            if (lane & o) id += n;
+        }
+    return id;
+}
+// one lane per value: the one whose remaining bits are zero
+template <int V>
+__device__ __forceinline__ bool multi_owner(int lane) { return (lane & (32 / V - 1)) == 0; }
+
+// ---------------------------------------------------------------- pre-sums of a chunk
+constexpr int PRE_ROWS = 2, PRE_COLS = 8;      // 16 accumulators per lane
+
+// Rows row0, row0 + 1, columns col0 .. col0 + 7 and group g of the blocks in the order e, h, lag K-1,
+// ..., lag 1: accumulated over the group's blocks, then over the warp, into partial[g]
+template <typename T>
+__device__ __forceinline__ void pre_item(const SimtDev<T>& d, int64_t n0, int row0, int g, int col0, int lane) {
+    const int CR = d.C * d.R, nvec = d.ld / VecOf<T>::W;
+    Acc<T> acc[PRE_ROWS][PRE_COLS];
+#pragma unroll 1
+    for (int o = GQ * g; o < min(GQ * g + GQ, d.K + 1); ++o) {
+        const int k = o < 2 ? 0 : d.K + 1 - o, q = o < 2 ? o : 1 + k;      // lag and block
+        int off[PRE_COLS];
+        bool any = false;
+#pragma unroll
+        for (int c = 0; c < PRE_COLS; ++c) {
+            // columns whose lag lies inside the chunk read the zero vectors behind the ring
+            const int col = col0 + c, i = col / d.R, r = col - i * d.R;
+            const bool on = o < 2 || i < k;
+            any |= on;
+            off[c] = o < 2 ? col * d.ld : ((on ? (int)ring_slot(n0 + i - k, d.ring) : d.ring) * d.R + r) * d.ld;
+        }
+        if (!any) continue;
+        const T* base = d.blocks + (int64_t)q * d.ne * d.ld;
+        const T* row[PRE_ROWS];
+#pragma unroll
+        for (int i = 0; i < PRE_ROWS; ++i) row[i] = base + (int64_t)min(row0 + i, d.ne - 1) * d.ld;
+        tile_rows<T, PRE_ROWS, PRE_COLS>(row, o == 0 ? d.E : o == 1 ? d.H : d.rbuf, off, nvec, lane, acc);
+    }
+    typename SumOf<T>::S v[PRE_ROWS * PRE_COLS];
+#pragma unroll
+    for (int i = 0; i < PRE_ROWS; ++i)
+#pragma unroll
+        for (int c = 0; c < PRE_COLS; ++c) v[i * PRE_COLS + c] = acc[i][c].sum();
+    const auto s = multi_reduce<PRE_ROWS * PRE_COLS>(v, lane);
+    const int id = multi_index<PRE_ROWS * PRE_COLS>(lane), row = row0 + id / PRE_COLS, col = col0 + id % PRE_COLS;
+    if (multi_owner<PRE_ROWS * PRE_COLS>(lane) && row < d.ne && col < CR) d.partial[((int64_t)g * CR + col) * d.ld + row] = s;
+}
+
+// ---------------------------------------------------------------- one step
+template <int RM>
+constexpr int step_rows() { return RM <= 2 ? 2 : 1; }       // rows per unit (one warp)
+
+// lags k >= 2 whose product with y_{n-1} belongs to a later column of the chunk (n in column i)
+__device__ __forceinline__ int push_lags(int i, int C, int K) { return i == 0 ? 0 : max(0, min(C - i, K - 1) - 1); }
+
+// One unit of the history of step n (RM >= R columns): units 0 .. nu - 1 form b_n of their rows from the
+// pre-sums, the inner products kept by earlier steps and lag 1; the units after them form T_k y_{n-1}
+// for lag 2 + (u / nu - 1)
+template <typename T, int RM>
+__device__ __forceinline__ void hist_unit(const SimtDev<T>& d, int64_t n, int u, int lane) {
+    using S = typename SumOf<T>::S;
+    constexpr int ROWS = step_rows<RM>();
+    const int i = (int)((n - 1) % d.C), CR = d.C * d.R, nvec = d.ld / VecOf<T>::W, nu = (d.ne + ROWS - 1) / ROWS;
+    const int k = 1 + u / nu, row0 = u % nu * ROWS;
+    if (k - 1 > push_lags(i, d.C, d.K)) return;
+    Acc<T> acc[ROWS][RM];
+    if (i > 0 && k < d.K) {
+        int off[RM];
+        const int s0 = (int)ring_slot(n - 1, d.ring) * d.R;
+#pragma unroll
+        for (int r = 0; r < RM; ++r) off[r] = (s0 + min(r, d.R - 1)) * d.ld;
+        const T* row[ROWS];
+#pragma unroll
+        for (int q = 0; q < ROWS; ++q) row[q] = d.blocks + ((int64_t)(1 + k) * d.ne + min(row0 + q, d.ne - 1)) * d.ld;
+        tile_rows<T, ROWS, RM>(row, d.rbuf, off, nvec, lane, acc);
+    }
+    S v[ROWS * RM];
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q)
+#pragma unroll
+        for (int r = 0; r < RM; ++r) v[q * RM + r] = acc[q][r].sum();
+    if (k == 1) {
+        const int kept = d.ngroups + max(0, min(i, d.K - 1) - 1);
+        for (int t = lane; t < kept; t += 32) {
+            const S* src = t < d.ngroups ? d.partial + ((int64_t)t * CR + i * d.R) * d.ld
+                                         : d.inner + (((int64_t)i * d.C + 2 + t - d.ngroups) * d.R) * d.ld;
+#pragma unroll
+            for (int q = 0; q < ROWS; ++q)
+#pragma unroll
+                for (int r = 0; r < RM; ++r)
+                    if (r < d.R && row0 + q < d.ne) v[q * RM + r] = add_sum(v[q * RM + r], src[(int64_t)r * d.ld + row0 + q]);
+        }
+    }
+    const S s = multi_reduce<ROWS * RM>(v, lane);
+    const int id = multi_index<ROWS * RM>(lane), row = row0 + id / RM, r = id % RM;
+    if (!multi_owner<ROWS * RM>(lane) || r >= d.R || row >= d.ne) return;
+    if (k == 1) d.b[(int64_t)r * d.ld + row] = (T)sum_value(s);
+    else d.inner[(((int64_t)(i - 1 + k) * d.C + k) * d.R + r) * d.ld + row] = s;
+}
+
+// y_n: rows of T_0^-1 b_n into the ring
+template <typename T, int RM>
+__device__ __forceinline__ void solve_unit(const SimtDev<T>& d, int64_t n, int u, int lane) {
+    constexpr int ROWS = step_rows<RM>();
+    Acc<T> acc[ROWS][RM];
+    int off[RM];
+#pragma unroll
+    for (int r = 0; r < RM; ++r) off[r] = min(r, d.R - 1) * d.ld;
+    const T* rp[ROWS];
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) rp[q] = d.t0inv + (int64_t)min(u * ROWS + q, d.ne - 1) * d.ld;
+    tile_rows<T, ROWS, RM>(rp, d.b, off, d.ld / VecOf<T>::W, lane, acc);
+    typename SumOf<T>::S v[ROWS * RM];
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q)
+#pragma unroll
+        for (int r = 0; r < RM; ++r) v[q * RM + r] = acc[q][r].sum();
+    const auto s = multi_reduce<ROWS * RM>(v, lane);
+    const int id = multi_index<ROWS * RM>(lane), row = u * ROWS + id / RM, r = id % RM;
+    if (multi_owner<ROWS * RM>(lane) && r < d.R && row < d.ne)
+        d.rbuf[(ring_slot(n, d.ring) * d.R + r) * d.ld + row] = (T)sum_value(s);
+}
+
+// ---------------------------------------------------------------- post-processing of steps p0 .. p1 - 1
 // z_c = sum_j tsign[c][j] w[tedge[c][j]], w = (1/dtt - 1) y_n - y_{n-1}/dtt (y_{n-1} = 0 at n = 1)
 template <typename T>
 __device__ __forceinline__ double project_in_value(const DevMesh& m, int c, const T* __restrict__ yn,
@@ -160,6 +388,55 @@ __device__ __forceinline__ double project_in_value(const DevMesh& m, int c, cons
         s = fma(m.tsign[3 * c + j], w, s);
     }
     return s;
+}
+template <typename T>
+__device__ __forceinline__ void pin_value(const SimtDev<T>& d, int64_t n, int col, int r, int c) {
+    const T* yn = d.rbuf + (ring_slot(n, d.ring) * d.R + r) * d.ld;
+    const T* yp = d.rbuf + (ring_slot(n - 1, d.ring) * d.R + r) * d.ld;
+    d.z[(int64_t)col * d.ldc + c] = (T)project_in_value<T>(d.m, c, yn, yp, n == 1, d.dtt);
+}
+
+// u = (Sigma^T Sigma)^+ z for two rows and eight columns (col0 ..) of ncol
+template <typename T>
+__device__ __forceinline__ void pinv_item(const SimtDev<T>& d, int ncol, int row0, int col0, int lane) {
+    Acc<T> acc[PRE_ROWS][PRE_COLS];
+    int off[PRE_COLS];
+#pragma unroll
+    for (int c = 0; c < PRE_COLS; ++c) off[c] = min(col0 + c, ncol - 1) * d.ldc;
+    const T* row[PRE_ROWS];
+#pragma unroll
+    for (int i = 0; i < PRE_ROWS; ++i) row[i] = d.pinv + (int64_t)min(row0 + i, d.nc - 1) * d.ldc;
+    tile_rows<T, PRE_ROWS, PRE_COLS>(row, d.z, off, d.ldc / VecOf<T>::W, lane, acc);
+    typename SumOf<T>::S v[PRE_ROWS * PRE_COLS];
+#pragma unroll
+    for (int i = 0; i < PRE_ROWS; ++i)
+#pragma unroll
+        for (int c = 0; c < PRE_COLS; ++c) v[i * PRE_COLS + c] = acc[i][c].sum();
+    const auto s = multi_reduce<PRE_ROWS * PRE_COLS>(v, lane);
+    const int id = multi_index<PRE_ROWS * PRE_COLS>(lane), r = row0 + id / PRE_COLS, c = col0 + id % PRE_COLS;
+    if (multi_owner<PRE_ROWS * PRE_COLS>(lane) && r < d.nc && c < ncol) d.u[(int64_t)c * d.ldc + r] = (T)sum_value(s);
+}
+
+// j_n = y_n + Sigma u -> outputs; finiteness check (the first bad step is kept)
+template <typename T>
+__device__ __forceinline__ void pout_value(const SimtDev<T>& d, int64_t n, int col, int r, int e) {
+    const T y = d.rbuf[(ring_slot(n, d.ring) * d.R + r) * d.ld + e];
+    const T* u = d.u + (int64_t)col * d.ldc;
+    const T val = y + u[d.m.cplus_[e]] - u[d.m.cminus_[e]];
+    Ctl* ctl = d.ctl;
+    if (!isfinite((double)val)) {
+        atomicCAS(&ctl->status, 0, (int)TDCFIE_E_NONFINITE);
+        atomicMin(reinterpret_cast<unsigned long long*>(&ctl->bad_step), (unsigned long long)n);
+    }
+    const int64_t at = ((n - ctl->n0) * d.R + r) * (int64_t)d.ne + e;
+    if (ctl->out) reinterpret_cast<T*>(ctl->out)[at] = val;
+    if (ctl->yout) reinterpret_cast<T*>(ctl->yout)[at] = y;
+}
+
+__device__ __forceinline__ unsigned long long device_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
 }
 
 }  // namespace tdc
