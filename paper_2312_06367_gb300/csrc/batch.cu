@@ -42,13 +42,13 @@ static int phase_units(const StepPlan* p, int ph) {
     switch (ph) {
         case PH_ENV: return up((int64_t)p->npts * p->C, 32);
         case PH_GATHER: return p->ne;
-        case PH_PRE: return up(p->ne, PRE_ROWS) * p->ngroups * up(p->C, PRE_COLS);
+        case PH_PRE: return up(p->ne, pre_rows<float>()) * p->ngroups * up(p->C, PRE_COLS);
         case PH_PIN: return up(p->nc, 32);
-        case PH_PINV: return up(p->nc, PRE_ROWS);
+        case PH_PINV: return up(p->nc, pre_rows<float>());
         case PH_POUT: return up(p->ne, 32);
         // rows of the history, of every lag that may be pushed, and of the solve
         case PH_HIST: return up(p->ne, step_rows<1>()) * (1 + std::max(0, std::min(p->C - 1, p->K - 1) - 1));
-        default: return up(p->ne, step_rows<1>());
+        default: return p->ne;
     }
 }
 
@@ -89,15 +89,15 @@ __device__ __forceinline__ void batch_unit(int ph, const SimtDev<float>& d, int 
         gather_edge<float>(d, u, 0, lane);
     } else if (ph == PH_PRE) {
         const int ctiles = (d.C + PRE_COLS - 1) / PRE_COLS, t = u % ctiles, g = u / ctiles % d.ngroups;
-        pre_item<float>(d, n, u / ctiles / d.ngroups * PRE_ROWS, g, t * PRE_COLS, lane);
+        pre_item<float>(d, n, u / ctiles / d.ngroups * pre_rows<float>(), g, t * PRE_COLS, lane);
     } else if (ph == PH_HIST) {
-        hist_unit<float, 1>(d, n, u, lane);
+        hist_unit<float, 1>(d, n, u, lane, true, Nothing());
     } else if (ph == PH_SOLVE) {
-        solve_unit<float, 1>(d, n, u, lane);
+        solve_unit<float, 1>(d, n, u, lane, Nothing());
     } else if (ph == PH_PIN) {
         if (32 * u + lane < d.nc) pin_value<float>(d, n, 0, 0, 32 * u + lane);
     } else if (ph == PH_PINV) {
-        pinv_item<float>(d, 1, u * PRE_ROWS, 0, lane);
+        pinv_item<float>(d, 1, u * pre_rows<float>(), 0, lane);
     } else {
         if (32 * u + lane < d.ne) pout_value<float>(d, n, 0, 0, 32 * u + lane);
     }

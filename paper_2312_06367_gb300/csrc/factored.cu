@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(256) k_fact_apply(const T* __restrict__ Mtx, i
 #pragma unroll
     for (int r = 0; r < RM; ++r) off[r] = min(r, R - 1) * ncol;
     const T* rp[1] = {Mtx + (int64_t)row * ncol};
-    tile_rows<T, 1, RM>(rp, x, off, ncol / VecOf<T>::W, lane, acc);
+    tile_rows<T, 1, RM>(rp, x, off, RM, ncol / VecOf<T>::W, lane, acc);
     typename SumOf<T>::S v[RM];
 #pragma unroll
     for (int r = 0; r < RM; ++r) v[r] = acc[0][r].sum();

@@ -32,6 +32,7 @@ __device__ __forceinline__ bool chunk_start(const SimtDev<T>& d, int64_t n) { re
 
 template <typename T>
 __global__ void __launch_bounds__(128) k_env(const __grid_constant__ SimtDev<T> d) {
+    wait_prior();
     const int64_t n = d.ctl->n;
     if (!chunk_start(d, n)) return;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -42,6 +43,7 @@ __global__ void __launch_bounds__(128) k_env(const __grid_constant__ SimtDev<T> 
 
 template <typename T>
 __global__ void __launch_bounds__(128) k_gather(const __grid_constant__ SimtDev<T> d) {
+    wait_prior();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (w >= d.ne * d.R || !chunk_start(d, d.ctl->n)) return;
     gather_edge<T>(d, w / d.R, w % d.R, threadIdx.x & 31);
@@ -51,38 +53,46 @@ __global__ void __launch_bounds__(128) k_gather(const __grid_constant__ SimtDev<
 // run together
 template <typename T>
 __global__ void __launch_bounds__(128) k_pre(const __grid_constant__ SimtDev<T> d, int ctiles) {
+    wait_prior();
     const int64_t n = d.ctl->n;
     if (!chunk_start(d, n)) return;
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) d.ctl->t_mark = device_ns();
     const int tile = blockIdx.x % ctiles, rb = blockIdx.x / ctiles;
-    const int row0 = (rb * 4 + (threadIdx.x >> 5)) * PRE_ROWS;
+    const int row0 = (rb * 4 + (threadIdx.x >> 5)) * pre_rows<T>();
     if (row0 < d.ne) pre_item<T>(d, n, row0, blockIdx.y, tile * PRE_COLS, threadIdx.x & 31);
 }
 
-// b_n; step = ctl->n + off
+// b_n; step n = ctl->n + off.  sums_ready: the pre-sums are older than the kernel in front
 template <typename T, int RM>
-__global__ void __launch_bounds__(128) k_hist(const __grid_constant__ SimtDev<T> d, int off) {
+__global__ void __launch_bounds__(128) k_hist(const __grid_constant__ SimtDev<T> d, int off, bool sums_ready) {
     const int64_t n = d.ctl->n + off;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const unsigned long long t = device_ns();
-        if (chunk_start(d, n)) d.ctl->hist_ns += t - d.ctl->t_mark;     // the pre-sums ran just before
-        d.ctl->t_mark = t;
-    }
-    hist_unit<T, RM>(d, n, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31);
+    auto wait = [&] {
+        wait_prior();
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            const unsigned long long t = device_ns();
+            if (chunk_start(d, n)) d.ctl->hist_ns += t - d.ctl->t_mark;     // the pre-sums ran just before
+            d.ctl->t_mark = t;
+        }
+    };
+    hist_unit<T, RM>(d, n, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, sums_ready, wait);
 }
 
 template <typename T, int RM>
 __global__ void __launch_bounds__(128) k_solve(const __grid_constant__ SimtDev<T> d, int off) {
     const int64_t n = d.ctl->n + off;
-    if (blockIdx.x == 0 && threadIdx.x == 0) d.ctl->hist_ns += device_ns() - d.ctl->t_mark;
-    const int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (u * step_rows<RM>() < d.ne) solve_unit<T, RM>(d, n, u, threadIdx.x & 31);
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    auto wait = [&] {
+        wait_prior();
+        if (blockIdx.x == 0 && threadIdx.x == 0) d.ctl->hist_ns += device_ns() - d.ctl->t_mark;
+    };
+    if (row < d.ne) solve_unit<T, RM>(d, n, row, threadIdx.x & 31, wait);
 }
 
 // Post-processing of the steps p0 .. ctl->n + adv - 1 (at most C); the last kernel advances the step
 // counter by adv
 template <typename T>
 __global__ void __launch_bounds__(256) k_pin(const __grid_constant__ SimtDev<T> d, int adv) {
+    wait_prior();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     const int c = idx % d.nc, col = idx / d.nc;
     const int64_t n = d.ctl->p0 + col / d.R;
@@ -91,13 +101,15 @@ __global__ void __launch_bounds__(256) k_pin(const __grid_constant__ SimtDev<T> 
 
 template <typename T>
 __global__ void __launch_bounds__(128) k_pinv(const __grid_constant__ SimtDev<T> d, int adv, int ctiles) {
+    wait_prior();
     const int ncol = min((int)(d.ctl->n + adv - d.ctl->p0), d.C) * d.R;
-    const int col0 = blockIdx.x % ctiles * PRE_COLS, row0 = (blockIdx.x / ctiles * 4 + (threadIdx.x >> 5)) * PRE_ROWS;
+    const int col0 = blockIdx.x % ctiles * PRE_COLS, row0 = (blockIdx.x / ctiles * 4 + (threadIdx.x >> 5)) * pre_rows<T>();
     if (col0 < ncol && row0 < d.nc) pinv_item<T>(d, ncol, row0, col0, threadIdx.x & 31);
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_pout(const __grid_constant__ SimtDev<T> d, int adv) {
+    wait_prior();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     const int e = idx % d.ne, col = idx / d.ne;
     const int64_t end = d.ctl->n + adv, n = d.ctl->p0 + col / d.R;
@@ -114,7 +126,10 @@ __global__ void __launch_bounds__(256) k_pout(const __grid_constant__ SimtDev<T>
     }
 }
 
-__global__ void k_advance(Ctl* ctl) { ctl->n += 1; }
+__global__ void k_advance(Ctl* ctl) {
+    wait_prior();
+    ctl->n += 1;
+}
 
 // ---------------------------------------------------------------- launches
 static size_t esize(int prec) { return prec == TDCFIE_FP64 ? 8 : 4; }
@@ -136,11 +151,27 @@ template SimtDev<float> simt_view<float>(tdcfie_t, const StepPlan&);
 
 static unsigned div_up(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
+// launch with programmatic stream serialization: the kernel may be put on the SMs before the one ahead
+// of it has finished (it calls wait_prior before it touches anything that one writes)
+template <class... P, class... A>
+static void launch_chained(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 template <typename T>
 int launch_tests(tdcfie_t h, StepPlan& p, cudaStream_t s) {
     const SimtDev<T> d = simt_view<T>(h, p);
     k_env<T><<<div_up((int64_t)p.npts * p.R * p.C, 128), 128, 0, s>>>(d);
-    k_gather<T><<<div_up((int64_t)p.ne * p.R, 4), 128, 0, s>>>(d);
+    launch_chained(k_gather<T>, div_up((int64_t)p.ne * p.R, 4), 128, s, d);
     return 2;
 }
 template int launch_tests<double>(tdcfie_t, StepPlan&, cudaStream_t);
@@ -151,7 +182,7 @@ static int launch_pre(tdcfie_t h, StepPlan& p, cudaStream_t s) {
     int n = launch_tests<T>(h, p, s);
     if (p.fact) return n;
     const int ctiles = (int)div_up(p.C * p.R, PRE_COLS);
-    k_pre<T><<<dim3(ctiles * div_up(p.ne, 4 * PRE_ROWS), p.ngroups), 128, 0, s>>>(simt_view<T>(h, p), ctiles);
+    launch_chained(k_pre<T>, dim3(ctiles * div_up(p.ne, 4 * pre_rows<T>()), p.ngroups), 128, s, simt_view<T>(h, p), ctiles);
     return n + 1;
 }
 
@@ -168,11 +199,10 @@ static cudaError_t launch_inner(tdcfie_t h, StepPlan& p, bool chunk, int off, cu
     // step's column is known)
     const int lags = 1 + std::max(0, std::min(chunk ? p.C - off : p.C - 1, p.K - 1) - 1) * (chunk && off == 0 ? 0 : 1);
     unsigned g = div_up((int64_t)units * lags, 4);
-#define BY_R(K, ...) (p.R == 1 ? K<T, 1><<<g, 128, 0, s>>>(__VA_ARGS__) : p.R == 2 ? K<T, 2><<<g, 128, 0, s>>>(__VA_ARGS__) : \
-                      p.R <= 4 ? K<T, 4><<<g, 128, 0, s>>>(__VA_ARGS__) : K<T, 8><<<g, 128, 0, s>>>(__VA_ARGS__))
-    BY_R(k_hist, d, off);
+#define BY_R(K, ...) launch_chained(p.R == 1 ? K<T, 1> : p.R == 2 ? K<T, 2> : p.R <= 4 ? K<T, 4> : K<T, 8>, g, 128, s, __VA_ARGS__)
+    BY_R(k_hist, d, off, chunk && off > 0);
     kernels += 1;
-    g = div_up(units, 4);
+    g = div_up(p.ne, 4);
     if (p.mlp_on) kernels += launch_mlp_guess<T>(&p, s);
     if (p.gmres_on) {
         const cudaError_t e = launch_gmres<T>(h, &p, (const T*)p.b, (const T*)p.guessbuf, (const T*)p.t0mat,
@@ -191,9 +221,9 @@ static int launch_post(tdcfie_t h, StepPlan& p, int adv, cudaStream_t s) {
     if (p.fact) return 0;      // part of the step
     const SimtDev<T> d = simt_view<T>(h, p);
     const int CR = p.C * p.R, ctiles = (int)div_up(CR, PRE_COLS);
-    k_pin<T><<<div_up((int64_t)p.nc * CR, 256), 256, 0, s>>>(d, adv);
-    k_pinv<T><<<ctiles * div_up(p.nc, 4 * PRE_ROWS), 128, 0, s>>>(d, adv, ctiles);
-    k_pout<T><<<div_up((int64_t)p.ne * CR, 256), 256, 0, s>>>(d, adv);
+    launch_chained(k_pin<T>, div_up((int64_t)p.nc * CR, 256), 256, s, d, adv);
+    launch_chained(k_pinv<T>, ctiles * div_up(p.nc, 4 * pre_rows<T>()), 128, s, d, adv, ctiles);
+    launch_chained(k_pout<T>, div_up((int64_t)p.ne * CR, 256), 256, s, d, adv);
     return 3;
 }
 
@@ -206,7 +236,7 @@ static cudaError_t launch_graph(tdcfie_t h, StepPlan& p, int which, cudaStream_t
     if (which == StepPlan::G_STEP) {
         e = launch_inner<T>(h, p, false, 0, s, k);
         if (!p.fact) {                      // the factored step advances the counter itself
-            k_advance<<<1, 1, 0, s>>>(p.ctl);
+            launch_chained(k_advance, 1, 1, s, p.ctl);
             k += 1;
         }
     }

@@ -172,19 +172,22 @@ struct Acc<float> {
 __device__ __forceinline__ double2 neg(double2 a) { return a; }    // unused by Acc<double>
 __device__ __forceinline__ float4 neg(float4 a) { return make_float4(-a.x, -a.y, -a.z, -a.w); }
 
-// acc[i][c] += row_i . x_c for ROWS rows and COLS columns, nvec vectors per row.  No branch on a
-// column (one that is not wanted points at zeros or repeats another), so that all loads of a turn are
-// in flight together; the rows' next vectors are fetched a turn ahead.
-template <typename T, int ROWS, int COLS>
-__device__ __forceinline__ void tile_rows(const T* const (&row)[ROWS], const T* __restrict__ x, const int (&off)[COLS],
-                                          int nvec, int lane, Acc<T> (&acc)[ROWS][COLS]) {
+// acc[i][c] += row_i . x_c for ROWS rows and the first nv of COLS columns, nvec vectors per row.  The
+// loads do not branch on a column (one that is not wanted repeats another or points at zeros), so that
+// all loads of a turn are in flight together; the rows' next vectors are fetched a turn ahead.
+// before_x() runs between the first loads of the rows and the first loads of x (a kernel whose x comes
+// from the kernel before it waits there).
+struct Nothing { __device__ __forceinline__ void operator()() const {} };
+template <typename T, int ROWS, int COLS, class F = Nothing>
+__device__ __forceinline__ void tile_rows(const T* const (&row)[ROWS], const T* x, const int (&off)[COLS], int nv,
+                                          int nvec, int lane, Acc<T> (&acc)[ROWS][COLS], F before_x = F()) {
     using V = typename VecOf<T>::V;
     if constexpr (ROWS * COLS >= 8) {
         V nx[ROWS];
 #pragma unroll
         for (int i = 0; i < ROWS; ++i) nx[i] = lane < nvec ? __ldg(reinterpret_cast<const V*>(row[i]) + lane) : V{};
-#pragma unroll 1
-        for (int j = lane; j < nvec; j += 32) {
+        before_x();
+        auto turn = [&](int j, bool all) {
             V a[ROWS], na[ROWS], xv[COLS];
 #pragma unroll
             for (int c = 0; c < COLS; ++c) xv[c] = reinterpret_cast<const V*>(x + off[c])[j];
@@ -196,30 +199,46 @@ __device__ __forceinline__ void tile_rows(const T* const (&row)[ROWS], const T* 
             }
 #pragma unroll
             for (int c = 0; c < COLS; ++c)
+                if (all || c < nv)
 #pragma unroll
-                for (int i = 0; i < ROWS; ++i) acc[i][c].add(a[i], na[i], xv[c]);
+                    for (int i = 0; i < ROWS; ++i) acc[i][c].add(a[i], na[i], xv[c]);
+        };
+        if (nv >= COLS) {
+#pragma unroll 1
+            for (int j = lane; j < nvec; j += 32) turn(j, true);
+        } else {
+#pragma unroll 1
+            for (int j = lane; j < nvec; j += 32) turn(j, false);
         }
     } else {
-        constexpr int U = ROWS * COLS >= 4 ? 2 : 4;      // turns whose loads are issued together
-        for (int j0 = lane; j0 < nvec; j0 += 32 * U) {
-            V a[U][ROWS], xv[U][COLS];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int j = j0 + 32 * u;
-                const bool in = j < nvec;
-#pragma unroll
-                for (int i = 0; i < ROWS; ++i) a[u][i] = in ? __ldg(reinterpret_cast<const V*>(row[i]) + j) : V{};
-#pragma unroll
-                for (int c = 0; c < COLS; ++c) xv[u][c] = in ? reinterpret_cast<const V*>(x + off[c])[j] : V{};
-            }
+        // turns whose loads are issued together: a whole row up to about 1000 entries
+        constexpr int U = ROWS * COLS >= 4 ? 2 : ROWS * COLS == 2 ? 4 : 8;
+        V a[U][ROWS], xv[U][COLS];
+        auto load_rows = [&](int j0) {
 #pragma unroll
             for (int u = 0; u < U; ++u)
 #pragma unroll
-                for (int i = 0; i < ROWS; ++i) {
-                    const V na = neg(a[u][i]);
+                for (int i = 0; i < ROWS; ++i)
+                    a[u][i] = j0 + 32 * u < nvec ? __ldg(reinterpret_cast<const V*>(row[i]) + j0 + 32 * u) : V{};
+        };
+        load_rows(lane);
+        before_x();
+        for (int j0 = lane; j0 < nvec; j0 += 32 * U) {
+            if (j0 != lane) load_rows(j0);
 #pragma unroll
-                    for (int c = 0; c < COLS; ++c) acc[i][c].add(a[u][i], na, xv[u][c]);
-                }
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int c = 0; c < COLS; ++c)
+                    xv[u][c] = j0 + 32 * u < nvec ? reinterpret_cast<const V*>(x + off[c])[j0 + 32 * u] : V{};
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j0 - lane + 32 * u < nvec)
+#pragma unroll
+                    for (int i = 0; i < ROWS; ++i) {
+                        const V na = neg(a[u][i]);
+#pragma unroll
+                        for (int c = 0; c < COLS; ++c) acc[i][c].add(a[u][i], na, xv[u][c]);
+                    }
         }
     }
 }
@@ -263,33 +282,37 @@ template <int V>
 __device__ __forceinline__ bool multi_owner(int lane) { return (lane & (32 / V - 1)) == 0; }
 
 // ---------------------------------------------------------------- pre-sums of a chunk
-constexpr int PRE_ROWS = 2, PRE_COLS = 8;      // 16 accumulators per lane
+constexpr int PRE_COLS = 8;
+// rows per unit: two on the FP64 path (32 accumulator registers, the row's columns share the loads), one
+// on the FP32 path, whose pair accumulators would leave 8 warps per SM at two rows (fused multiply-add
+// pipe 62 % busy, 543 us for 8 columns at 1920 edges, K = 42)
+template <typename T> constexpr int pre_rows() { return sizeof(T) == 8 ? 2 : 1; }
 
-// Rows row0, row0 + 1, columns col0 .. col0 + 7 and group g of the blocks in the order e, h, lag K-1,
+// Rows row0 .. row0 + pre_rows - 1, columns col0 .. col0 + 7 and group g of the blocks in the order e, h, lag K-1,
 // ..., lag 1: accumulated over the group's blocks, then over the warp, into partial[g]
 template <typename T>
 __device__ __forceinline__ void pre_item(const SimtDev<T>& d, int64_t n0, int row0, int g, int col0, int lane) {
+    constexpr int PRE_ROWS = pre_rows<T>();
     const int CR = d.C * d.R, nvec = d.ld / VecOf<T>::W;
     Acc<T> acc[PRE_ROWS][PRE_COLS];
 #pragma unroll 1
     for (int o = GQ * g; o < min(GQ * g + GQ, d.K + 1); ++o) {
         const int k = o < 2 ? 0 : d.K + 1 - o, q = o < 2 ? o : 1 + k;      // lag and block
-        int off[PRE_COLS];
-        bool any = false;
+        int off[PRE_COLS], nv = 0;
 #pragma unroll
         for (int c = 0; c < PRE_COLS; ++c) {
             // columns whose lag lies inside the chunk read the zero vectors behind the ring
             const int col = col0 + c, i = col / d.R, r = col - i * d.R;
             const bool on = o < 2 || i < k;
-            any |= on;
+            nv += on;       // the first ones of the tile
             off[c] = o < 2 ? col * d.ld : ((on ? (int)ring_slot(n0 + i - k, d.ring) : d.ring) * d.R + r) * d.ld;
         }
-        if (!any) continue;
+        if (!nv) continue;
         const T* base = d.blocks + (int64_t)q * d.ne * d.ld;
         const T* row[PRE_ROWS];
 #pragma unroll
         for (int i = 0; i < PRE_ROWS; ++i) row[i] = base + (int64_t)min(row0 + i, d.ne - 1) * d.ld;
-        tile_rows<T, PRE_ROWS, PRE_COLS>(row, o == 0 ? d.E : o == 1 ? d.H : d.rbuf, off, nvec, lane, acc);
+        tile_rows<T, PRE_ROWS, PRE_COLS>(row, o == 0 ? d.E : o == 1 ? d.H : d.rbuf, off, nv, nvec, lane, acc);
     }
     typename SumOf<T>::S v[PRE_ROWS * PRE_COLS];
 #pragma unroll
@@ -302,8 +325,9 @@ __device__ __forceinline__ void pre_item(const SimtDev<T>& d, int64_t n0, int ro
 }
 
 // ---------------------------------------------------------------- one step
+// rows per unit (one warp) of the history; the solve takes one (its chain is the step's)
 template <int RM>
-constexpr int step_rows() { return RM <= 2 ? 2 : 1; }       // rows per unit (one warp)
+constexpr int step_rows() { return RM <= 2 ? 2 : 1; }
 
 // lags k >= 2 whose product with y_{n-1} belongs to a later column of the chunk (n in column i)
 __device__ __forceinline__ int push_lags(int i, int C, int K) { return i == 0 ? 0 : max(0, min(C - i, K - 1) - 1); }
@@ -311,31 +335,19 @@ __device__ __forceinline__ int push_lags(int i, int C, int K) { return i == 0 ? 
 // One unit of the history of step n (RM >= R columns): units 0 .. nu - 1 form b_n of their rows from the
 // pre-sums, the inner products kept by earlier steps and lag 1; the units after them form T_k y_{n-1}
 // for lag 2 + (u / nu - 1)
-template <typename T, int RM>
-__device__ __forceinline__ void hist_unit(const SimtDev<T>& d, int64_t n, int u, int lane) {
+// wait() returns when y_{n-1} is there; sums_ready: the pre-sums and inner products are there before it
+template <typename T, int RM, class F>
+__device__ __forceinline__ void hist_unit(const SimtDev<T>& d, int64_t n, int u, int lane, bool sums_ready, F wait) {
     using S = typename SumOf<T>::S;
     constexpr int ROWS = step_rows<RM>();
-    const int i = (int)((n - 1) % d.C), CR = d.C * d.R, nvec = d.ld / VecOf<T>::W, nu = (d.ne + ROWS - 1) / ROWS;
-    const int k = 1 + u / nu, row0 = u % nu * ROWS;
-    if (k - 1 > push_lags(i, d.C, d.K)) return;
-    Acc<T> acc[ROWS][RM];
-    if (i > 0 && k < d.K) {
-        int off[RM];
-        const int s0 = (int)ring_slot(n - 1, d.ring) * d.R;
-#pragma unroll
-        for (int r = 0; r < RM; ++r) off[r] = (s0 + min(r, d.R - 1)) * d.ld;
-        const T* row[ROWS];
-#pragma unroll
-        for (int q = 0; q < ROWS; ++q) row[q] = d.blocks + ((int64_t)(1 + k) * d.ne + min(row0 + q, d.ne - 1)) * d.ld;
-        tile_rows<T, ROWS, RM>(row, d.rbuf, off, nvec, lane, acc);
-    }
+    const int CR = d.C * d.R, nvec = d.ld / VecOf<T>::W, nu = (d.ne + ROWS - 1) / ROWS;
+    const int k = 1 + u / nu, row0 = u % nu * ROWS, i = (int)((n - 1) % d.C);
+    if (k > 1 && k - 1 > push_lags(i, d.C, d.K)) return;
     S v[ROWS * RM];
 #pragma unroll
-    for (int q = 0; q < ROWS; ++q)
-#pragma unroll
-        for (int r = 0; r < RM; ++r) v[q * RM + r] = acc[q][r].sum();
-    if (k == 1) {
-        const int kept = d.ngroups + max(0, min(i, d.K - 1) - 1);
+    for (int q = 0; q < ROWS * RM; ++q) v[q] = S{};
+    auto sums = [&] {
+        const int kept = k > 1 ? 0 : d.ngroups + max(0, min(i, d.K - 1) - 1);
         for (int t = lane; t < kept; t += 32) {
             const S* src = t < d.ngroups ? d.partial + ((int64_t)t * CR + i * d.R) * d.ld
                                          : d.inner + (((int64_t)i * d.C + 2 + t - d.ngroups) * d.R) * d.ld;
@@ -345,7 +357,26 @@ __device__ __forceinline__ void hist_unit(const SimtDev<T>& d, int64_t n, int u,
                 for (int r = 0; r < RM; ++r)
                     if (r < d.R && row0 + q < d.ne) v[q * RM + r] = add_sum(v[q * RM + r], src[(int64_t)r * d.ld + row0 + q]);
         }
+    };
+    if (sums_ready) sums();
+    Acc<T> acc[ROWS][RM];
+    if (i > 0) {
+        int off[RM];
+        const int s0 = (int)ring_slot(n - 1, d.ring) * d.R;
+#pragma unroll
+        for (int r = 0; r < RM; ++r) off[r] = (s0 + min(r, d.R - 1)) * d.ld;
+        const T* rp[ROWS];
+#pragma unroll
+        for (int q = 0; q < ROWS; ++q) rp[q] = d.blocks + ((int64_t)(1 + k) * d.ne + min(row0 + q, d.ne - 1)) * d.ld;
+        tile_rows<T, ROWS, RM>(rp, d.rbuf, off, RM, nvec, lane, acc, wait);
+    } else {
+        wait();
     }
+    if (!sums_ready) sums();
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q)
+#pragma unroll
+        for (int r = 0; r < RM; ++r) v[q * RM + r] = add_sum(v[q * RM + r], acc[q][r].sum());
     const S s = multi_reduce<ROWS * RM>(v, lane);
     const int id = multi_index<ROWS * RM>(lane), row = row0 + id / RM, r = id % RM;
     if (!multi_owner<ROWS * RM>(lane) || r >= d.R || row >= d.ne) return;
@@ -353,27 +384,21 @@ __device__ __forceinline__ void hist_unit(const SimtDev<T>& d, int64_t n, int u,
     else d.inner[(((int64_t)(i - 1 + k) * d.C + k) * d.R + r) * d.ld + row] = s;
 }
 
-// y_n: rows of T_0^-1 b_n into the ring
-template <typename T, int RM>
-__device__ __forceinline__ void solve_unit(const SimtDev<T>& d, int64_t n, int u, int lane) {
-    constexpr int ROWS = step_rows<RM>();
-    Acc<T> acc[ROWS][RM];
+// y_n of one row: T_0^-1 b_n into the ring; wait() returns when b_n is there
+template <typename T, int RM, class F>
+__device__ __forceinline__ void solve_unit(const SimtDev<T>& d, int64_t n, int row, int lane, F wait) {
+    Acc<T> acc[1][RM];
     int off[RM];
 #pragma unroll
     for (int r = 0; r < RM; ++r) off[r] = min(r, d.R - 1) * d.ld;
-    const T* rp[ROWS];
+    const T* rp[1] = {d.t0inv + (int64_t)row * d.ld};
+    tile_rows<T, 1, RM>(rp, d.b, off, RM, d.ld / VecOf<T>::W, lane, acc, wait);
+    typename SumOf<T>::S v[RM];
 #pragma unroll
-    for (int q = 0; q < ROWS; ++q) rp[q] = d.t0inv + (int64_t)min(u * ROWS + q, d.ne - 1) * d.ld;
-    tile_rows<T, ROWS, RM>(rp, d.b, off, d.ld / VecOf<T>::W, lane, acc);
-    typename SumOf<T>::S v[ROWS * RM];
-#pragma unroll
-    for (int q = 0; q < ROWS; ++q)
-#pragma unroll
-        for (int r = 0; r < RM; ++r) v[q * RM + r] = acc[q][r].sum();
-    const auto s = multi_reduce<ROWS * RM>(v, lane);
-    const int id = multi_index<ROWS * RM>(lane), row = u * ROWS + id / RM, r = id % RM;
-    if (multi_owner<ROWS * RM>(lane) && r < d.R && row < d.ne)
-        d.rbuf[(ring_slot(n, d.ring) * d.R + r) * d.ld + row] = (T)sum_value(s);
+    for (int r = 0; r < RM; ++r) v[r] = acc[0][r].sum();
+    const auto s = multi_reduce<RM>(v, lane);
+    const int r = multi_index<RM>(lane);
+    if (multi_owner<RM>(lane) && r < d.R) d.rbuf[(ring_slot(n, d.ring) * d.R + r) * d.ld + row] = (T)sum_value(s);
 }
 
 // ---------------------------------------------------------------- post-processing of steps p0 .. p1 - 1
@@ -396,9 +421,10 @@ __device__ __forceinline__ void pin_value(const SimtDev<T>& d, int64_t n, int co
     d.z[(int64_t)col * d.ldc + c] = (T)project_in_value<T>(d.m, c, yn, yp, n == 1, d.dtt);
 }
 
-// u = (Sigma^T Sigma)^+ z for two rows and eight columns (col0 ..) of ncol
+// u = (Sigma^T Sigma)^+ z for pre_rows rows and eight columns (col0 ..) of ncol
 template <typename T>
 __device__ __forceinline__ void pinv_item(const SimtDev<T>& d, int ncol, int row0, int col0, int lane) {
+    constexpr int PRE_ROWS = pre_rows<T>();
     Acc<T> acc[PRE_ROWS][PRE_COLS];
     int off[PRE_COLS];
 #pragma unroll
@@ -406,7 +432,7 @@ __device__ __forceinline__ void pinv_item(const SimtDev<T>& d, int ncol, int row
     const T* row[PRE_ROWS];
 #pragma unroll
     for (int i = 0; i < PRE_ROWS; ++i) row[i] = d.pinv + (int64_t)min(row0 + i, d.nc - 1) * d.ldc;
-    tile_rows<T, PRE_ROWS, PRE_COLS>(row, d.z, off, d.ldc / VecOf<T>::W, lane, acc);
+    tile_rows<T, PRE_ROWS, PRE_COLS>(row, d.z, off, min(ncol - col0, PRE_COLS), d.ldc / VecOf<T>::W, lane, acc);
     typename SumOf<T>::S v[PRE_ROWS * PRE_COLS];
 #pragma unroll
     for (int i = 0; i < PRE_ROWS; ++i)
@@ -431,6 +457,16 @@ __device__ __forceinline__ void pout_value(const SimtDev<T>& d, int64_t n, int c
     const int64_t at = ((n - ctl->n0) * d.R + r) * (int64_t)d.ne + e;
     if (ctl->out) reinterpret_cast<T*>(ctl->out)[at] = val;
     if (ctl->yout) reinterpret_cast<T*>(ctl->yout)[at] = y;
+}
+
+// Programmatic dependent launch: a kernel of a step's chain is put on the SMs while the kernel before
+// it finishes; wait_prior() returns when that kernel is complete and its results are visible (at once
+// in a kernel launched without the attribute), and the next kernel may be put on the SMs after it.
+// What a kernel reads ahead of it was complete before the kernel in front could pass its own wait:
+// matrices, the step counter (it only moves in the last kernel of a graph) and sums two kernels old.
+__device__ __forceinline__ void wait_prior() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 __device__ __forceinline__ unsigned long long device_ns() {
