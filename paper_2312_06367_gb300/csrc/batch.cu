@@ -89,17 +89,17 @@ __device__ __forceinline__ void batch_unit(int ph, const SimtDev<float>& d, int 
         gather_edge<float>(d, u, 0, lane);
     } else if (ph == PH_PRE) {
         const int ctiles = (d.C + PRE_COLS - 1) / PRE_COLS, t = u % ctiles, g = u / ctiles % d.ngroups;
-        pre_item<float>(d, n, u / ctiles / d.ngroups * pre_rows<float>(), g, t * PRE_COLS, lane);
+        pre_item<float>(d, d.ctl->slot, u / ctiles / d.ngroups * pre_rows<float>(), g, t * PRE_COLS, lane);
     } else if (ph == PH_HIST) {
-        hist_unit<float, 1>(d, n, u, lane, true, Nothing());
+        hist_unit<float, 1>(d, step_pos(d, 0), u, lane, true, Nothing());
     } else if (ph == PH_SOLVE) {
-        solve_unit<float, 1>(d, n, u, lane, Nothing());
+        solve_unit<float, 1>(d, step_pos(d, 0), u, lane, Nothing());
     } else if (ph == PH_PIN) {
-        if (32 * u + lane < d.nc) pin_value<float>(d, n, 0, 0, 32 * u + lane);
+        if (32 * u + lane < d.nc) pin_value<float>(d, n, d.ctl->slot, 0, 0, 32 * u + lane);
     } else if (ph == PH_PINV) {
         pinv_item<float>(d, 1, u * pre_rows<float>(), 0, lane);
     } else {
-        if (32 * u + lane < d.ne) pout_value<float>(d, n, 0, 0, 32 * u + lane);
+        if (32 * u + lane < d.ne) pout_value<float>(d, n, d.ctl->slot, 0, 0, 32 * u + lane);
     }
 }
 
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(256) k_batch_step(const __grid_constant__ BArg
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     bool start = false;      // some member starts a chunk (uniform: no counter moves before the end)
-    for (int s = 0; s < a.nmem; ++s) start |= (a.mem[s].ctl->n - 1) % a.mem[s].C == 0;
+    for (int s = 0; s < a.nmem; ++s) start |= a.mem[s].ctl->col == 0;
     for (int ph = start ? PH_ENV : PH_HIST; ph < NPH; ++ph) {
         const int* first = a.first[ph];
         const int total = first[a.nmem];
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(256) k_batch_step(const __grid_constant__ BArg
             for (int64_t u = u0; u < min(u0 + rows, (int64_t)total); ++u) {
                 while (u >= first[s + 1]) ++s;
                 const SimtDev<float>& d = a.mem[s];
-                if (ph <= PH_PRE && (d.ctl->n - 1) % d.C != 0) continue;
+                if (ph <= PH_PRE && d.ctl->col != 0) continue;
                 batch_unit(ph, d, (int)(u - first[s]), lane);
             }
         grid_barrier(a.sync);
@@ -126,9 +126,8 @@ __global__ void __launch_bounds__(256) k_batch_step(const __grid_constant__ BArg
     // every block has passed the last barrier: advance the members
     if (blockIdx.x == 0)
         for (int s = threadIdx.x; s < a.nmem; s += blockDim.x) {
-            Ctl* c = a.mem[s].ctl;
-            c->n += 1;
-            c->p0 = c->n;
+            advance(a.mem[s], 1);
+            a.mem[s].ctl->p0 = a.mem[s].ctl->n;
         }
 }
 

@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(256) k_shells(int ne, int nc, int K, int R, in
                                                 const int64_t* __restrict__ rowptr, const uint32_t* __restrict__ idx,
                                                 const T* __restrict__ val, const T* __restrict__ xring,
                                                 const T* __restrict__ qring, const T* __restrict__ E,
-                                                const T* __restrict__ Hv, int C, int ld, T* __restrict__ z) {
+                                                const T* __restrict__ Hv, int ld, T* __restrict__ z) {
     __shared__ double part[256 / 32][RMAX];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = blockIdx.x * (256 / 32 / WPR) + warp / WPR;
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(256) k_shells(int ne, int nc, int K, int R, in
         double v = 0.0;
         for (int q = 0; q < WPR; ++q) v += part[warp + q][lane];
         double base = 0.0;
-        const int col = (int)((ctl->n - 1) % C) * R + lane;      // the step's column of the chunk's tests
+        const int col = ctl->col * R + lane;      // the step's column of the chunk's tests
         if (row < ne) base = (double)E[(int64_t)col * ld + row];
         else if (row < 2 * ne) base = (double)Hv[(int64_t)col * ld + row - ne];
         z[(int64_t)lane * ldz + row] = (T)(base + v);
@@ -311,7 +311,10 @@ __global__ void __launch_bounds__(256) k_fact_apply(const T* __restrict__ Mtx, i
     if (multi_owner<RM>(lane) && r < R) y2[((ctl->n & 1) * R + r) * (int64_t)nrow + row] = (T)sum_value(s);
 }
 
-__global__ void k_fact_advance(Ctl* ctl) { ctl->n += 1; }
+__global__ void k_fact_advance(Ctl* ctl, int C) {
+    ctl->n += 1;
+    ctl->col = (ctl->col + 1) % C;
+}
 
 // ---------------------------------------------------------------- host side
 #define FK(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return cuda_fail(h, e_, #x); } while (0)
@@ -415,7 +418,7 @@ static void launch_fact_r(tdcfie_t h, StepPlan& p, cudaStream_t s) {
     k_shells<T, RMAX><<<(f.nrows + wpb / WPR - 1) / (wpb / WPR), 32 * wpb, 0, s>>>(ne, nc, f.K, R, f.ldz, p.ctl, f.rowptr, f.idx,
                                                                       (const T*)f.val, (const T*)f.xring,
                                                                       (const T*)f.qring, (const T*)p.E,
-                                                                      (const T*)p.Hv, p.C, p.ld, (T*)f.z);
+                                                                      (const T*)p.Hv, p.ld, (T*)f.z);
     k_fact_apply<T, RMAX><<<(ne + wpb - 1) / wpb, 32 * wpb, 0, s>>>((const T*)f.W, ne, f.ldz, R, (const T*)f.z,
                                                                      (T*)f.y2, p.ctl, true);
     k_fact_charges<T><<<(nc * R + tb - 1) / tb, tb, 0, s>>>(m, R, f.K, p.ldc, p.ctl, (const T*)f.y2, (T*)f.qring, (T*)f.qcur);
@@ -423,7 +426,7 @@ static void launch_fact_r(tdcfie_t h, StepPlan& p, cudaStream_t s) {
                                                                      (T*)f.v2, p.ctl, false);
     k_fact_post<T><<<(ne * R + tb - 1) / tb, tb, 0, s>>>(m, R, f.K, p.ctl, (const T*)f.y2, (const T*)f.v2,
                                                          (T*)f.xring, h->dtt);
-    k_fact_advance<<<1, 1, 0, s>>>(p.ctl);
+    k_fact_advance<<<1, 1, 0, s>>>(p.ctl, p.C);
 }
 
 template <typename T>

@@ -89,6 +89,7 @@ struct StepPlan;   // defined in march.cu
 
 struct Ctl {              // device-resident step state read by every kernel of a step
     int64_t n;            // current step (1-based)
+    int slot, col;        // SIMT paths: n mod ring, (n - 1) mod C
     int64_t n0;           // step of the first output row of this tdcfie_step call
     void* out;            // currents_out of this call (nullptr: discard)
     int status;           // 0 ok, else a tdcfie_status recorded with bad_step

@@ -28,13 +28,10 @@ namespace tdc {
 // ---------------------------------------------------------------- kernels (arithmetic in simt.h)
 // The tests and pre-sums of a chunk: no work unless the current step starts one
 template <typename T>
-__device__ __forceinline__ bool chunk_start(const SimtDev<T>& d, int64_t n) { return (n - 1) % d.C == 0; }
-
-template <typename T>
 __global__ void __launch_bounds__(128) k_env(const __grid_constant__ SimtDev<T> d) {
     wait_prior();
     const int64_t n = d.ctl->n;
-    if (!chunk_start(d, n)) return;
+    if (d.ctl->col) return;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)d.npts * d.R * d.C) return;
     const int i = (int)(idx % d.C), r = (int)(idx / d.C % d.R), pt = (int)(idx / d.C / d.R);
@@ -45,58 +42,65 @@ template <typename T>
 __global__ void __launch_bounds__(128) k_gather(const __grid_constant__ SimtDev<T> d) {
     wait_prior();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= d.ne * d.R || !chunk_start(d, d.ctl->n)) return;
+    if (w >= d.ne * d.R || d.ctl->col) return;
     gather_edge<T>(d, w / d.R, w % d.R, threadIdx.x & 31);
 }
 
 // grid: (column tiles x row blocks, groups), the column tiles fastest so that blocks that share rows
 // run together
 template <typename T>
-__global__ void __launch_bounds__(128) k_pre(const __grid_constant__ SimtDev<T> d, int ctiles) {
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 3) k_pre(const __grid_constant__ SimtDev<T> d, int ctiles) {
     wait_prior();
-    const int64_t n = d.ctl->n;
-    if (!chunk_start(d, n)) return;
+    if (d.ctl->col) return;
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) d.ctl->t_mark = device_ns();
     const int tile = blockIdx.x % ctiles, rb = blockIdx.x / ctiles;
     const int row0 = (rb * 4 + (threadIdx.x >> 5)) * pre_rows<T>();
-    if (row0 < d.ne) pre_item<T>(d, n, row0, blockIdx.y, tile * PRE_COLS, threadIdx.x & 31);
+    if (row0 < d.ne) pre_item<T>(d, d.ctl->slot, row0, blockIdx.y, tile * PRE_COLS, threadIdx.x & 31);
 }
 
 // b_n; step n = ctl->n + off.  sums_ready: the pre-sums are older than the kernel in front
 template <typename T, int RM>
-__global__ void __launch_bounds__(128) k_hist(const __grid_constant__ SimtDev<T> d, int off, bool sums_ready) {
-    const int64_t n = d.ctl->n + off;
+__global__ void __launch_bounds__(128, 4) k_hist(const __grid_constant__ SimtDev<T> d, int off, bool sums_ready) {
+    const StepPos pos = step_pos(d, off);
     auto wait = [&] {
         wait_prior();
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             const unsigned long long t = device_ns();
-            if (chunk_start(d, n)) d.ctl->hist_ns += t - d.ctl->t_mark;     // the pre-sums ran just before
+            if (pos.col == 0) d.ctl->hist_ns += t - d.ctl->t_mark;     // the pre-sums ran just before
             d.ctl->t_mark = t;
         }
     };
-    hist_unit<T, RM>(d, n, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, sums_ready, wait);
+    hist_unit<T, RM>(d, pos, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, sums_ready, wait);
 }
 
 template <typename T, int RM>
 __global__ void __launch_bounds__(128) k_solve(const __grid_constant__ SimtDev<T> d, int off) {
-    const int64_t n = d.ctl->n + off;
+    const StepPos pos = step_pos(d, off);
     const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     auto wait = [&] {
         wait_prior();
         if (blockIdx.x == 0 && threadIdx.x == 0) d.ctl->hist_ns += device_ns() - d.ctl->t_mark;
     };
-    if (row < d.ne) solve_unit<T, RM>(d, n, row, threadIdx.x & 31, wait);
+    if (row < d.ne) solve_unit<T, RM>(d, pos, row, threadIdx.x & 31, wait);
 }
 
 // Post-processing of the steps p0 .. ctl->n + adv - 1 (at most C); the last kernel advances the step
 // counter by adv
 template <typename T>
+__device__ __forceinline__ bool post_step(const SimtDev<T>& d, int adv, int col, int64_t& n, int& slot) {
+    const Ctl* c = d.ctl;
+    n = c->p0 + col / d.R;
+    slot = ring_at(c->slot, (int)(n - c->n), d.ring);
+    return n < c->n + adv && col < d.C * d.R;
+}
+template <typename T>
 __global__ void __launch_bounds__(256) k_pin(const __grid_constant__ SimtDev<T> d, int adv) {
     wait_prior();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     const int c = idx % d.nc, col = idx / d.nc;
-    const int64_t n = d.ctl->p0 + col / d.R;
-    if (n < d.ctl->n + adv && col < d.C * d.R) pin_value<T>(d, n, col, col % d.R, c);
+    int64_t n;
+    int slot;
+    if (post_step(d, adv, col, n, slot)) pin_value<T>(d, n, slot, col, col % d.R, c);
 }
 
 template <typename T>
@@ -112,23 +116,25 @@ __global__ void __launch_bounds__(256) k_pout(const __grid_constant__ SimtDev<T>
     wait_prior();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     const int e = idx % d.ne, col = idx / d.ne;
-    const int64_t end = d.ctl->n + adv, n = d.ctl->p0 + col / d.R;
-    if (n < end && col < d.C * d.R) pout_value<T>(d, n, col, col % d.R, e);
+    int64_t n;
+    int slot;
+    if (post_step(d, adv, col, n, slot)) pout_value<T>(d, n, slot, col, col % d.R, e);
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(d.done, 1) == (int)gridDim.x - 1) {     // every block has read n and p0
             *d.done = 0;
-            d.ctl->n = end;
-            d.ctl->p0 = end;
+            advance(d, adv);
+            d.ctl->p0 = d.ctl->n;
             __threadfence();
         }
     }
 }
 
-__global__ void k_advance(Ctl* ctl) {
+template <typename T>
+__global__ void k_advance(const __grid_constant__ SimtDev<T> d) {
     wait_prior();
-    ctl->n += 1;
+    advance(d, 1);
 }
 
 // ---------------------------------------------------------------- launches
@@ -236,7 +242,7 @@ static cudaError_t launch_graph(tdcfie_t h, StepPlan& p, int which, cudaStream_t
     if (which == StepPlan::G_STEP) {
         e = launch_inner<T>(h, p, false, 0, s, k);
         if (!p.fact) {                      // the factored step advances the counter itself
-            launch_chained(k_advance, 1, 1, s, p.ctl);
+            launch_chained(k_advance<T>, 1, 1, s, simt_view<T>(h, p));
             k += 1;
         }
     }
@@ -554,6 +560,7 @@ tdcfie_status plan_reset(tdcfie_t h) {
     Ctl c{};
     c.n = c.n0 = c.p0 = 1;
     c.bad_step = INT64_MAX;
+    c.slot = 1;      // n mod ring (ring > 1), column 0 of a chunk
     if (p->gm) CK(reset_gmres_stats(p->gm));
     CK(cudaMemcpyAsync(p->ctl, &c, sizeof(Ctl), cudaMemcpyHostToDevice, s));
     if (p->ringbuf) CK(cudaMemsetAsync(p->ringbuf, 0, p->esz * p->ring * p->R * p->ld, s));

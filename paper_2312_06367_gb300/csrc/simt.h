@@ -59,9 +59,26 @@ template <typename T> __device__ __forceinline__ T add_rn(T a, T b);
 template <> __device__ __forceinline__ float add_rn<float>(float a, float b) { return __fadd_rn(a, b); }
 template <> __device__ __forceinline__ double add_rn<double>(double a, double b) { return __dadd_rn(a, b); }
 
-__device__ __forceinline__ int64_t ring_slot(int64_t n, int ring) {
-    const int64_t s = n % ring;
-    return s < 0 ? s + ring : s;
+// Position of a step in the march: its ring slot and its column of the chunk.  Both ride in the step
+// state, so that no kernel of the chain starts with 64-bit divisions.
+struct StepPos { int64_t n; int slot, col; };
+__device__ __forceinline__ int ring_at(int slot, int delta, int ring) {      // |delta| <= ring
+    const int t = slot + delta;
+    return t < 0 ? t + ring : t >= ring ? t - ring : t;
+}
+// step ctl->n + off, which lies in the same chunk
+template <typename T>
+__device__ __forceinline__ StepPos step_pos(const SimtDev<T>& d, int off) {
+    const Ctl* c = d.ctl;
+    return StepPos{c->n + off, ring_at(c->slot, off, d.ring), c->col + off};
+}
+// the step counter moves by adv (at most C)
+template <typename T>
+__device__ __forceinline__ void advance(const SimtDev<T>& d, int adv) {
+    Ctl* c = d.ctl;
+    c->n += adv;
+    c->slot = ring_at(c->slot, adv, d.ring);
+    c->col = (c->col + adv) % d.C;
 }
 
 // ---------------------------------------------------------------- plane-wave tests
@@ -183,19 +200,33 @@ __device__ __forceinline__ void tile_rows(const T* const (&row)[ROWS], const T* 
                                           int nvec, int lane, Acc<T> (&acc)[ROWS][COLS], F before_x = F()) {
     using V = typename VecOf<T>::V;
     if constexpr (ROWS * COLS >= 8) {
+        // pointers and byte offsets advance by additions: index arithmetic by multiply-add would take
+        // the pipe that the packed FP32 instructions run on
+        const V* ap[ROWS];
         V nx[ROWS];
 #pragma unroll
-        for (int i = 0; i < ROWS; ++i) nx[i] = lane < nvec ? __ldg(reinterpret_cast<const V*>(row[i]) + lane) : V{};
+        for (int i = 0; i < ROWS; ++i) {
+            ap[i] = reinterpret_cast<const V*>(row[i]) + lane;
+            nx[i] = lane < nvec ? __ldg(ap[i]) : V{};
+        }
         before_x();
-        auto turn = [&](int j, bool all) {
+        const char* xb = reinterpret_cast<const char*>(x);
+        unsigned xo[COLS];
+#pragma unroll
+        for (int c = 0; c < COLS; ++c) xo[c] = (unsigned)off[c] * (unsigned)sizeof(T) + (unsigned)lane * 16u;
+        auto turn = [&](bool more, bool all) {
             V a[ROWS], na[ROWS], xv[COLS];
 #pragma unroll
-            for (int c = 0; c < COLS; ++c) xv[c] = reinterpret_cast<const V*>(x + off[c])[j];
+            for (int c = 0; c < COLS; ++c) {
+                xv[c] = *reinterpret_cast<const V*>(xb + xo[c]);
+                xo[c] += 512u;
+            }
 #pragma unroll
             for (int i = 0; i < ROWS; ++i) {
                 a[i] = nx[i];
                 na[i] = neg(a[i]);
-                if (j + 32 < nvec) nx[i] = __ldg(reinterpret_cast<const V*>(row[i]) + j + 32);
+                ap[i] += 32;
+                if (more) nx[i] = __ldg(ap[i]);
             }
 #pragma unroll
             for (int c = 0; c < COLS; ++c)
@@ -205,10 +236,10 @@ __device__ __forceinline__ void tile_rows(const T* const (&row)[ROWS], const T* 
         };
         if (nv >= COLS) {
 #pragma unroll 1
-            for (int j = lane; j < nvec; j += 32) turn(j, true);
+            for (int j = lane; j < nvec; j += 32) turn(j + 32 < nvec, true);
         } else {
 #pragma unroll 1
-            for (int j = lane; j < nvec; j += 32) turn(j, false);
+            for (int j = lane; j < nvec; j += 32) turn(j + 32 < nvec, false);
         }
     } else {
         // turns whose loads are issued together: a whole row up to about 1000 entries
@@ -288,24 +319,31 @@ constexpr int PRE_COLS = 8;
 // pipe 62 % busy, 543 us for 8 columns at 1920 edges, K = 42)
 template <typename T> constexpr int pre_rows() { return sizeof(T) == 8 ? 2 : 1; }
 
-// Rows row0 .. row0 + pre_rows - 1, columns col0 .. col0 + 7 and group g of the blocks in the order e, h, lag K-1,
-// ..., lag 1: accumulated over the group's blocks, then over the warp, into partial[g]
+// Rows row0 .. row0 + pre_rows - 1, columns col0 .. col0 + 7 and group g of the blocks in the order e, h,
+// lag K-1, ..., lag 1: accumulated over the group's blocks, then over the warp, into partial[g].  slot:
+// ring slot of the chunk's first step
 template <typename T>
-__device__ __forceinline__ void pre_item(const SimtDev<T>& d, int64_t n0, int row0, int g, int col0, int lane) {
+__device__ __forceinline__ void pre_item(const SimtDev<T>& d, int slot, int row0, int g, int col0, int lane) {
     constexpr int PRE_ROWS = pre_rows<T>();
     const int CR = d.C * d.R, nvec = d.ld / VecOf<T>::W;
+    int ci[PRE_COLS], co[PRE_COLS];      // step within the chunk, offset of the wave within a slot
+#pragma unroll
+    for (int c = 0; c < PRE_COLS; ++c) {
+        ci[c] = d.R == 1 ? col0 + c : (col0 + c) / d.R;
+        co[c] = (col0 + c - ci[c] * d.R) * d.ld;
+    }
     Acc<T> acc[PRE_ROWS][PRE_COLS];
 #pragma unroll 1
     for (int o = GQ * g; o < min(GQ * g + GQ, d.K + 1); ++o) {
         const int k = o < 2 ? 0 : d.K + 1 - o, q = o < 2 ? o : 1 + k;      // lag and block
+        const int sk = ring_at(slot, -k, d.ring);
         int off[PRE_COLS], nv = 0;
 #pragma unroll
         for (int c = 0; c < PRE_COLS; ++c) {
             // columns whose lag lies inside the chunk read the zero vectors behind the ring
-            const int col = col0 + c, i = col / d.R, r = col - i * d.R;
-            const bool on = o < 2 || i < k;
+            const bool on = o < 2 || ci[c] < k;
             nv += on;       // the first ones of the tile
-            off[c] = o < 2 ? col * d.ld : ((on ? (int)ring_slot(n0 + i - k, d.ring) : d.ring) * d.R + r) * d.ld;
+            off[c] = o < 2 ? (col0 + c) * d.ld : (on ? ring_at(sk, ci[c], d.ring) : d.ring) * d.R * d.ld + co[c];
         }
         if (!nv) continue;
         const T* base = d.blocks + (int64_t)q * d.ne * d.ld;
@@ -337,11 +375,11 @@ __device__ __forceinline__ int push_lags(int i, int C, int K) { return i == 0 ? 
 // for lag 2 + (u / nu - 1)
 // wait() returns when y_{n-1} is there; sums_ready: the pre-sums and inner products are there before it
 template <typename T, int RM, class F>
-__device__ __forceinline__ void hist_unit(const SimtDev<T>& d, int64_t n, int u, int lane, bool sums_ready, F wait) {
+__device__ __forceinline__ void hist_unit(const SimtDev<T>& d, const StepPos& pos, int u, int lane, bool sums_ready, F wait) {
     using S = typename SumOf<T>::S;
     constexpr int ROWS = step_rows<RM>();
     const int CR = d.C * d.R, nvec = d.ld / VecOf<T>::W, nu = (d.ne + ROWS - 1) / ROWS;
-    const int k = 1 + u / nu, row0 = u % nu * ROWS, i = (int)((n - 1) % d.C);
+    const int k = 1 + u / nu, row0 = (u - (k - 1) * nu) * ROWS, i = pos.col;
     if (k > 1 && k - 1 > push_lags(i, d.C, d.K)) return;
     S v[ROWS * RM];
 #pragma unroll
@@ -362,7 +400,7 @@ __device__ __forceinline__ void hist_unit(const SimtDev<T>& d, int64_t n, int u,
     Acc<T> acc[ROWS][RM];
     if (i > 0) {
         int off[RM];
-        const int s0 = (int)ring_slot(n - 1, d.ring) * d.R;
+        const int s0 = ring_at(pos.slot, -1, d.ring) * d.R;
 #pragma unroll
         for (int r = 0; r < RM; ++r) off[r] = (s0 + min(r, d.R - 1)) * d.ld;
         const T* rp[ROWS];
@@ -386,7 +424,7 @@ __device__ __forceinline__ void hist_unit(const SimtDev<T>& d, int64_t n, int u,
 
 // y_n of one row: T_0^-1 b_n into the ring; wait() returns when b_n is there
 template <typename T, int RM, class F>
-__device__ __forceinline__ void solve_unit(const SimtDev<T>& d, int64_t n, int row, int lane, F wait) {
+__device__ __forceinline__ void solve_unit(const SimtDev<T>& d, const StepPos& pos, int row, int lane, F wait) {
     Acc<T> acc[1][RM];
     int off[RM];
 #pragma unroll
@@ -398,7 +436,7 @@ __device__ __forceinline__ void solve_unit(const SimtDev<T>& d, int64_t n, int r
     for (int r = 0; r < RM; ++r) v[r] = acc[0][r].sum();
     const auto s = multi_reduce<RM>(v, lane);
     const int r = multi_index<RM>(lane);
-    if (multi_owner<RM>(lane) && r < d.R) d.rbuf[(ring_slot(n, d.ring) * d.R + r) * d.ld + row] = (T)sum_value(s);
+    if (multi_owner<RM>(lane) && r < d.R) d.rbuf[((int64_t)pos.slot * d.R + r) * d.ld + row] = (T)sum_value(s);
 }
 
 // ---------------------------------------------------------------- post-processing of steps p0 .. p1 - 1
@@ -415,9 +453,9 @@ __device__ __forceinline__ double project_in_value(const DevMesh& m, int c, cons
     return s;
 }
 template <typename T>
-__device__ __forceinline__ void pin_value(const SimtDev<T>& d, int64_t n, int col, int r, int c) {
-    const T* yn = d.rbuf + (ring_slot(n, d.ring) * d.R + r) * d.ld;
-    const T* yp = d.rbuf + (ring_slot(n - 1, d.ring) * d.R + r) * d.ld;
+__device__ __forceinline__ void pin_value(const SimtDev<T>& d, int64_t n, int slot, int col, int r, int c) {
+    const T* yn = d.rbuf + ((int64_t)slot * d.R + r) * d.ld;
+    const T* yp = d.rbuf + ((int64_t)ring_at(slot, -1, d.ring) * d.R + r) * d.ld;
     d.z[(int64_t)col * d.ldc + c] = (T)project_in_value<T>(d.m, c, yn, yp, n == 1, d.dtt);
 }
 
@@ -445,8 +483,8 @@ __device__ __forceinline__ void pinv_item(const SimtDev<T>& d, int ncol, int row
 
 // j_n = y_n + Sigma u -> outputs; finiteness check (the first bad step is kept)
 template <typename T>
-__device__ __forceinline__ void pout_value(const SimtDev<T>& d, int64_t n, int col, int r, int e) {
-    const T y = d.rbuf[(ring_slot(n, d.ring) * d.R + r) * d.ld + e];
+__device__ __forceinline__ void pout_value(const SimtDev<T>& d, int64_t n, int slot, int col, int r, int e) {
+    const T y = d.rbuf[((int64_t)slot * d.R + r) * d.ld + e];
     const T* u = d.u + (int64_t)col * d.ldc;
     const T val = y + u[d.m.cplus_[e]] - u[d.m.cminus_[e]];
     Ctl* ctl = d.ctl;
