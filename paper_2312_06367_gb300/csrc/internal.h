@@ -89,7 +89,7 @@ struct StepPlan;   // defined in march.cu
 
 struct Ctl {              // device-resident step state read by every kernel of a step
     int64_t n;            // current step (1-based)
-    int slot, col;        // SIMT paths: n mod ring, (n - 1) mod C
+    int slot, col;        // n mod ring (SIMT paths), (n - 1) mod C
     int64_t n0;           // step of the first output row of this tdcfie_step call
     void* out;            // currents_out of this call (nullptr: discard)
     int status;           // 0 ok, else a tdcfie_status recorded with bad_step
@@ -98,8 +98,8 @@ struct Ctl {              // device-resident step state read by every kernel of 
     void* yout;           // optional y_n output of this call (nullptr: none)
     int noconv;           // set when a GMRES solve stopped above its tolerance (gmres_maxit reached)
     int64_t noconv_step;  // the first such step
-    int64_t p0;           // SIMT paths: first step not yet post-processed
-    unsigned long long t_mark, hist_ns;   // SIMT paths: device time of the history kernels (ns)
+    int64_t p0;           // first step not yet post-processed
+    unsigned long long t_mark, hist_ns;   // device time of the history kernels (ns)
 };
 }  // namespace tdc
 

@@ -1,7 +1,5 @@
 // Per-handle step plan shared by the SIMT (march.cu) and tensor-core (umma.cu) paths.
 #pragma once
-#include <vector>
-
 #include "internal.h"
 
 namespace tdc {
@@ -14,7 +12,7 @@ struct StepPlan {
     int prec = TDCFIE_FP64;
     int R = 1, ne = 0, nc = 0, K = 0, nblk = 0, ring = 0;
     size_t esz = 8;
-    int C = 1;                   // SIMT paths: steps per chunk (simt.h)
+    int C = 1;                   // steps per chunk (simt.h)
     int ld = 0, ldc = 0;         // SIMT paths: row lengths of matrices and vectors (16-byte multiples)
     int ngroups = 0, npts = 0;   // SIMT paths: groups of the pre-sums, distinct quadrature points
     void* blocks = nullptr;      // nblk x ne x ld (path precision): -A, alpha L2, -T_1 .. -T_{K-1}
@@ -37,27 +35,21 @@ struct StepPlan {
     void* u = nullptr;           // C x R x ldc
     int* done = nullptr;
     Ctl* ctl = nullptr;
-    // plane-wave tests, SIMT paths: distinct points, and per edge (e-points first) point index and
-    // weighted basis vector
+    // plane-wave tests: distinct points, and per edge (e-points first) point index and weighted basis
+    // vector (tensor paths: as {c, index}); env: envelopes of a chunk (SIMT paths)
     void* env = nullptr; void* pts = nullptr; void* ecoef = nullptr;
     int* eptr = nullptr; int* enE = nullptr; int* eidx = nullptr;
-    // the same per entry for the tensor paths: quadrature points (x) and weighted basis vectors (c)
-    int* pptr = nullptr; int* pnE = nullptr; void* px = nullptr; void* pc = nullptr;
     // factored history form (factored.cu); blocks and t0inv are then unused
     FactPlan* fact = nullptr;
     // tensor-core path
     TcStep* gemm = nullptr;
-    // step graphs.  Tensor paths: G_STEP is one step.  SIMT paths: G_PRE the tests and pre-sums of a
-    // chunk, G_STEP one step's history and solve, G_POST the post-processing of the finished steps,
-    // G_CHUNK a whole chunk.
+    // graphs: G_PRE the tests (and, SIMT paths, pre-sums) of a chunk, G_STEP one step's history and
+    // solve, G_POST the post-processing of the finished steps, G_CHUNK a whole chunk
     enum { G_STEP = 0, G_PRE, G_POST, G_CHUNK, NGRAPH };
     cudaGraph_t graph[NGRAPH] = {};
     cudaGraphExec_t exec[NGRAPH] = {};
     int nodes[NGRAPH] = {};                              // kernels per graph
-    cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
-    cudaEvent_t evA = nullptr, evB = nullptr;            // tensor paths: captured around the history sum
-    cudaGraphNode_t nodeA = nullptr, nodeB = nullptr;    // their record nodes in the step graph
-    std::vector<cudaEvent_t> hA, hB;                     // per-step events of a tdcfie_step call
+    cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     int launches_per_step = 0;
 };
 

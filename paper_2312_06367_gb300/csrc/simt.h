@@ -507,6 +507,23 @@ __device__ __forceinline__ void wait_prior() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// launch with programmatic stream serialization: the kernel may be put on the SMs before the one ahead
+// of it has finished (it calls wait_prior before it touches anything that one writes)
+template <class... P, class... A>
+static void launch_chained(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t s, size_t smem, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 __device__ __forceinline__ unsigned long long device_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

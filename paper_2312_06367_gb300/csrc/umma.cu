@@ -18,21 +18,21 @@
 // the epilogue adds the tiles error-free (TwoSum pairs in registers), partial sums are reduced in
 // FP64 and the results (b_n, y_n, the projector's u) stay in FP64 until they are split again.
 //
-// Kernel layout (one CTA per SM, persistent, 576 threads):
+// Kernel layout (one CTA per SM, persistent, 320 threads):
 //   warp 0   TMA producer: A tiles (128 x 64, 128B swizzle) with L2 evict-first, x tiles
 //            (64 x 64 per slice) with L2 evict-last, into a 4-deep ring of shared-memory stages;
 //   warp 1   one elected thread issues tcgen05.mma (M = 128, N = 64, K = 16) and commits each
 //            stage back to the producer and each finished pair of accumulators to the epilogue;
-//   warps 2-17 epilogue (one row and 16 right-hand sides per thread): per k tile, tcgen05.ld of D0
-//            and D1 (two TMEM buffers, so the next tile's MMAs overlap), exact power-of-two
+//   warps 2-9 epilogue (one row and 32 right-hand sides per thread): per k tile, tcgen05.ld of D0
+//            and D1 (four TMEM buffers, so the next tiles' MMAs overlap), exact power-of-two
 //            rescaling, error-free accumulation, and at the end of the CTA's part of a row tile a
 //            coalesced store of the (hi, lo) partial sums.
-// Work split: stream-K over (row tile, q, k tile) iterations in row-tile-major order.  The CTA
-// that finishes a row tile last (per-tile arrival counter; no waiting) sums every partial of the
-// tile in a fixed order in FP64 and applies the consumer's epilogue: store (u, out), or split into
-// slices for the next product (b_n), or both (y_n: FP64 pair for the post-processing and the
-// slices of the history ring).  Every mbarrier wait is bounded (%globaltimer, 2 s) and reports a
-// timeout.
+// Work split: stream-K over (row tile, q, k tile) iterations in row-tile-major order.  A second kernel,
+// k_tc_fix, sums every tile's partials in a fixed order as FP32 pairs and applies the consumer's
+// epilogue: store (u, out), or split into slices for the next product (b_n), or both (y_n: FP64 for the
+// post-processing and the slices of the history ring).  (Left to the CTA that finished a tile last, the
+// sums of some ten partials ran in one SM per tile: 45 us of the 57 us solve at 1920 edges.)
+// Every mbarrier wait is bounded (%globaltimer, 2 s) and reports a timeout.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -42,6 +42,7 @@
 #include <vector>
 
 #include "plan.h"
+#include "simt.h"
 #include "umma.h"
 
 namespace tdc {
@@ -60,7 +61,6 @@ constexpr int EC = NR / (NEPI / 4);         // columns (right-hand sides) per ep
 #define TDC_LDC 16
 #endif
 constexpr int LDC = TDC_LDC < EC ? TDC_LDC : EC;   // TMEM columns per tcgen05.ld of the epilogue
-constexpr int FIXR = 4;      // right-hand sides per pass of the row-tile reduction
 #ifndef TDC_D0S
 #define TDC_D0S 1
 #endif
@@ -69,6 +69,7 @@ static_assert(D0S == 1 || D0S == 2 || D0S == 4, "D0S divides the four K = 16 ste
 constexpr int BUFC = (D0S + 1) * NR;                           // TMEM columns of one buffer (D0 parts, D1)
 constexpr int NBUF = BUFC <= 128 ? 4 : (BUFC <= 256 ? 2 : 1);  // accumulator buffers in tensor memory
 constexpr uint64_t WAIT_NS = 2000000000ull;
+constexpr int TC_C = 4;      // steps per chunk: tests and post-processing of so many steps share their kernels
 
 template <int XS>
 struct Cfg {
@@ -83,10 +84,11 @@ struct Cfg {
 
 enum { FIX_PLAIN = 0, FIX_SPLIT = 1, FIX_SOLVE = 2 };
 
-// what the CTA that completes a row tile does with the tile's sums s[r][row]
+// what k_tc_fix does with a row tile's sums s[r][row]
 struct FixOut {
     int mode;
-    double* out;          // PLAIN: out[r * ld_out + row]; SOLVE: dy_n to out[(NR + r) * ld_out + row], y_n += dy_n
+    double* out;          // PLAIN: out[(rep NR + r) * ld_out + row]; SOLVE: per column c of the chunk [y_n | dy_n],
+                          // y_n = y_{n-1} + dy_n with y_{n-1} in the column before (cyclic)
     int ld_out;
     uint16_t* xs[3];      // SPLIT/SOLVE: destination slices, each [slots][NR][ld_x]
     float* sx;            // inverse scales [slots][ld_x / 64][NR]
@@ -97,13 +99,16 @@ struct FixOut {
 struct GemmArgs {
     int rows, cols;       // M extent, K extent of one block
     int nblk, ktiles, rtiles;
-    int64_t total;        // rtiles * nblk * ktiles
+    int reps;             // independent products with the same matrix (vector slot and output by product)
+    int64_t total;        // reps * rtiles * nblk * ktiles
     int maxseg;
-    int slot_mode;        // 0: history (q=0 -> ring, q=1 -> ring+1, q>=2 -> (n-(q-1)) mod ring); 1: slot 0; 2: slot q
+    int slot_mode;        // 0: history (q = 0, 1 -> ring + 2 col + q, q >= 2 -> (n - (q - 1)) mod ring);
+                          // 1: slot rep; 2: slot q
     int ring;
+    int off;              // step = ctl->n + off, column of the chunk ctl->col + off
+    int mark;             // device time of the history: 1 starts it, 2 adds it up
     float* partial;       // [grid][maxseg][2][NR][BM]  (hi, lo)
-    int* cnt;             // [rtiles] arrivals of the current launch (reset by the last arrival)
-    const int* seg_ptr;   // [rtiles + 1]
+    const int* seg_ptr;   // [reps rtiles + 1]
     const int* seg_slot;  // partial slots of every row tile, in a fixed order
     Ctl* ctl;
     uint32_t idesc;       // instruction descriptor (operand format)
@@ -206,14 +211,13 @@ static uint32_t make_idesc(int n, bool bf16) {
     return (1u << 4) | (f << 7) | (f << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 
-__device__ __forceinline__ int slot_of(const GemmArgs& g, int q, int64_t n) {
-    if (g.slot_mode == 1) return 0;
+// vector slot of block q; base: n mod ring
+__device__ __forceinline__ int slot_of(const GemmArgs& g, int q, int rep, int base, int col) {
+    if (g.slot_mode == 1) return rep;
     if (g.slot_mode == 2) return q;
-    if (q == 0) return g.ring;
-    if (q == 1) return g.ring + 1;
-    int64_t sl = (n - (q - 1)) % g.ring;
-    if (sl < 0) sl += g.ring;
-    return (int)sl;
+    if (q < 2) return g.ring + 2 * col + q;
+    const int sl = base - (q - 1);      // q - 1 <= ring
+    return sl < 0 ? sl + g.ring : sl;
 }
 
 __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
@@ -260,9 +264,6 @@ __device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t* v) {
     else tmem_ld16(taddr, v);
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// named barrier of the epilogue warps
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * NEPI) : "memory"); }
 
 // TwoSum on packed pairs (two FP32 lanes per instruction, sm_100+): hi + lo += v with the rounding
 // error of each addition carried into lo.  x - y is written fma(y, -1, x): one rounding, exact
@@ -375,8 +376,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     uint64_t* acc_empty = acc_full + NBUF;   // [NBUF]
     uint64_t* sx_full = acc_empty + NBUF;    // [NBUF] the tile scales of a buffer have landed
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sx_full + NBUF);
-    int* last_flag = reinterpret_cast<int*>(tmem_slot + 1);
-    float* red = reinterpret_cast<float*>(misc + 256);    // [NEPI / 4 column groups][4 quads][FIXR] tile maxima
     float* sx_buf = reinterpret_cast<float*>(misc + 512);   // [NBUF][NR] x scales of an accumulator's tile
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -401,7 +400,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int64_t n = ctl->n;
+    wait_prior();       // what was set up above does not depend on the kernel before
+    const int64_t n = ctl->n + g.off;
+    const int col = ctl->col + g.off;
+    const int base = g.ring > 0 ? (int)(n % g.ring) : 0;
+    if (g.mark && blockIdx.x == 0 && threadIdx.x == 0) {
+        if (g.mark == 1) ctl->t_mark = device_ns();
+        else ctl->hist_ns += device_ns() - ctl->t_mark;
+    }
 
     if (warp == 0) {
         if (lane == 0) {
@@ -412,8 +418,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             int rt = (int)(begin / ipt);
             int q = (int)((begin - rt * ipt) / g.ktiles);
             int kt = (int)(begin - rt * ipt - (int64_t)q * g.ktiles);
+            int rep = rt / g.rtiles;
+            rt -= rep * g.rtiles;
             for (int64_t it = begin; it < end; ++it) {
-                const int slot = slot_of(g, q, n);
+                const int slot = slot_of(g, q, rep, base, col);
                 if (!mbar_wait(empty + stage, phase ^ 1u, ctl)) break;
                 // the tile's 64 x scales go to its accumulator buffer's slot, free once the epilogue
                 // has released that buffer (the tile NBUF earlier)
@@ -433,7 +441,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 buf = buf + 1 == NBUF ? 0 : buf + 1;
                 if (++kt == g.ktiles) {
                     kt = 0;
-                    if (++q == g.nblk) { q = 0; ++rt; }
+                    if (++q == g.nblk) {
+                        q = 0;
+                        if (++rt == g.rtiles) { rt = 0; ++rep; }
+                    }
                 }
             }
         }
@@ -486,7 +497,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         for (int c = 0; c < EC / 2; ++c) acc_hi[c] = acc_lo[c] = make_float2(0.f, 0.f);
         int seg = 0, buf = 0;
         bool ok = true;
-        int64_t rt = begin / ipt, pos = begin - rt * ipt;   // row tile and iteration within it
+        int64_t tile = begin / ipt, pos = begin - tile * ipt;   // (product, row tile) and iteration within it
         for (int64_t it = begin; it < end; ++it) {
             if (ok && !mbar_wait(acc_full + buf, (fphase >> buf) & 1u, ctl)) ok = false;
             if (ok && !mbar_wait(sx_full + buf, (fphase >> buf) & 1u, ctl)) ok = false;
@@ -495,6 +506,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 tc_fence_after();
                 const float* sx = sx_buf + buf * NR + cbase;
                 const uint32_t d0 = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BUFC + cbase);
+                float seal = 0.f;
 #pragma unroll
                 for (int c0 = 0; c0 < EC; c0 += LDC) {
                     uint32_t v0[D0S][LDC], v1[LDC];
@@ -506,6 +518,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     for (int c = 0; c < LDC; c += 4) {
                         const float4 s4 = *reinterpret_cast<const float4*>(sx + c0 + c);
                         const float2 sc[2] = {make_float2(s4.x, s4.y), make_float2(s4.z, s4.w)};
+                        seal = s4.w;
 #pragma unroll
                         for (int u = 0; u < 4; u += 2) {   // power-of-two scales: the products are exact
                             const int k = (c0 + c + u) >> 1;
@@ -520,15 +533,18 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     }
                 }
                 tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(acc_empty + buf);   // the warp's TMEM reads are complete
+                // The arrival lets the producer overwrite the tile's scales, and it does not wait for
+                // shared-memory loads still in flight: the vote on the last one read does (without it
+                // about one march in twenty took one tile's last scales from a later tile).
+                const bool seen = __all_sync(0xffffffffu, seal == seal);
+                if (lane == 0 && seen) mbar_arrive(acc_empty + buf);   // the warp's reads are complete
             }
             buf = buf + 1 == NBUF ? 0 : buf + 1;
             const bool tile_end = ++pos == ipt;
             if (it + 1 == end || tile_end) {   // end of this CTA's part of row tile rt
                 float* dst = g.partial + ((int64_t)blockIdx.x * g.maxseg + seg) * (int64_t)2 * NR * BM;
                 // one power-of-two row scale for all blocks: applied once here (exact)
-                const int grow = (int)rt * BM + row;
+                const int grow = (int)(tile % g.rtiles) * BM + row;
                 const float sa = grow < g.rows ? g.sA[grow] : 1.f;
 #pragma unroll
                 for (int c = 0; c < EC / 2; ++c) {
@@ -539,81 +555,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     acc_hi[c] = acc_lo[c] = make_float2(0.f, 0.f);
                 }
                 ++seg;
-                __threadfence();
-                epi_sync();
-                if (threadIdx.x == 64) {
-                    const int need = g.seg_ptr[rt + 1] - g.seg_ptr[rt];
-                    const int old = atomicAdd(&g.cnt[rt], 1);
-                    const int last = old == need - 1;
-                    if (last) g.cnt[rt] = 0;     // every arrival of this launch is in
-                    *last_flag = last;
-                    __threadfence();
-                }
-                epi_sync();
-                if (*last_flag) {
-                    // ---- row tile rt complete: FP64 sum of its partials, consumer epilogue
-                    __threadfence();
-                    const FixOut& fx = g.fx;
-                    const int grow = (int)rt * BM + row;
-                    const int half = row >> 6;                       // 64-row half = consumer k tile
-                    const bool split = fx.mode != FIX_PLAIN;
-                    const bool hvalid = split && (int)rt * BM + half * 64 < fx.ld_x;
-                    const int slot = fx.slot_ring > 0 ? (int)(n % fx.slot_ring) : 0;
-                    const int p0 = g.seg_ptr[rt], p1 = g.seg_ptr[rt + 1];
-                    for (int r0 = cbase; r0 < cbase + EC; r0 += FIXR) {
-                        float sh[FIXR], sl_[FIXR];
-#pragma unroll
-                        for (int j = 0; j < FIXR; ++j) sh[j] = sl_[j] = 0.f;
-                        for (int k = p0; k < p1; ++k) {      // the tile's partials in a fixed order
-                            const float* P = g.partial + (int64_t)g.seg_slot[k] * 2 * NR * BM;
-#pragma unroll
-                            for (int j = 0; j < FIXR; ++j) {
-                                two_sum_acc(sh[j], sl_[j], __ldcg(P + (int64_t)(r0 + j) * BM + row));
-                                sl_[j] += __ldcg(P + (int64_t)(NR + r0 + j) * BM + row);
-                            }
-                        }
-                        if (fx.mode != FIX_SPLIT && grow < g.rows) {
-#pragma unroll
-                            for (int j = 0; j < FIXR; ++j) {
-                                const double v = (double)sh[j] + (double)sl_[j];
-                                if (fx.mode == FIX_SOLVE) {     // increment dy_n, and y_n = y_{n-1} + dy_n
-                                    fx.out[(int64_t)(NR + r0 + j) * fx.ld_out + grow] = v;
-                                    fx.out[(int64_t)(r0 + j) * fx.ld_out + grow] += v;
-                                } else {
-                                    fx.out[(int64_t)(r0 + j) * fx.ld_out + grow] = v;
-                                }
-                            }
-                        }
-                        if (split) {
-                            // tile maxima over the 64 rows of each half: warps (2 half, 2 half + 1) of this column group
-#pragma unroll
-                            for (int j = 0; j < FIXR; ++j) {
-                                float m = fabsf(sh[j] + sl_[j]);
-                                if (!(m == m)) m = INFINITY;
-                                for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                                if (lane == 0) red[(ch * 4 + quad) * FIXR + j] = m;
-                            }
-                            epi_sync();
-                            if (hvalid) {
-#pragma unroll
-                                for (int j = 0; j < FIXR; ++j) {
-                                    const float mx = fmaxf(red[(ch * 4 + 2 * half) * FIXR + j], red[(ch * 4 + 2 * half + 1) * FIXR + j]);
-                                    const float sc = fill_scale(mx);
-                                    uint16_t sl[3];
-                                    split_pair<F16, XS>(sh[j] * sc, sl_[j] * sc, sl);
-                                    const int64_t off = ((int64_t)slot * NR + r0 + j) * fx.ld_x + grow;
-#pragma unroll
-                                    for (int i = 0; i < XS; ++i) fx.xs[i][off] = sl[i];
-                                    if ((row & 63) == 0)
-                                        fx.sx[((int64_t)slot * (fx.ld_x / 64) + (rt * 2 + half)) * NR + r0 + j] = 1.f / sc;
-                                }
-                            }
-                            epi_sync();
-                        }
-                    }
-                }
             }
-            if (tile_end) { ++rt; pos = 0; }
+            if (tile_end) { ++tile; pos = 0; }
         }
     }
     tc_fence_before();
@@ -622,6 +565,69 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)C::TMEM_COLS)
                      : "memory");
+    }
+}
+
+// ---------------------------------------------------------------- sums of the partials, consumer epilogue
+// One block per (64-row half of a tile, 8 right-hand sides): thread (row, two right-hand sides).  The
+// tile's partials are added in a fixed order (TwoSum pairs); 64 rows are one k tile of the consumer.
+constexpr int FIX_RB = 8;
+template <int XS, bool F16>
+__global__ void __launch_bounds__(256) k_tc_fix(GemmArgs g) {
+    __shared__ float red[2][FIX_RB];
+    wait_prior();
+    const FixOut& fx = g.fx;
+    const int tile = blockIdx.x >> 1, half = blockIdx.x & 1;
+    const int rep = tile / g.rtiles, rt = tile - rep * g.rtiles;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int row = half * 64 + (warp & 1) * 32 + lane, r0 = blockIdx.y * FIX_RB + (warp >> 1) * 2;
+    const int grow = rt * BM + row;
+    float sh[2] = {0.f, 0.f}, sl_[2] = {0.f, 0.f};
+    const int p1 = g.seg_ptr[tile + 1];
+#pragma unroll 4
+    for (int k = g.seg_ptr[tile]; k < p1; ++k) {
+        const float* P = g.partial + (int64_t)g.seg_slot[k] * 2 * NR * BM + (int64_t)r0 * BM + row;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            two_sum_acc(sh[j], sl_[j], __ldcg(P + (int64_t)j * BM));
+            sl_[j] += __ldcg(P + (int64_t)(NR + j) * BM);
+        }
+    }
+    const int64_t n = g.ctl->n + g.off;
+    const int col = g.ctl->col + g.off;
+    if (fx.mode != FIX_SPLIT && grow < g.rows) {
+        const int prev = col == 0 ? TC_C - 1 : col - 1;      // column of y_{n-1}
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const double v = (double)sh[j] + (double)sl_[j];
+            if (fx.mode == FIX_SOLVE) {     // increment dy_n, and y_n = y_{n-1} + dy_n
+                fx.out[(int64_t)((2 * col + 1) * NR + r0 + j) * fx.ld_out + grow] = v;
+                fx.out[(int64_t)(2 * col * NR + r0 + j) * fx.ld_out + grow] =
+                    fx.out[(int64_t)(2 * prev * NR + r0 + j) * fx.ld_out + grow] + v;
+            } else {
+                fx.out[(int64_t)(rep * NR + r0 + j) * fx.ld_out + grow] = v;
+            }
+        }
+    }
+    if (fx.mode == FIX_PLAIN || rt * BM + half * 64 >= fx.ld_x) return;
+    const int slot = fx.slot_ring > 0 ? (int)(n % fx.slot_ring) : 0;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {       // tile maxima over the 64 rows: two warps
+        float m = fabsf(sh[j] + sl_[j]);
+        if (!(m == m)) m = INFINITY;
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane == 0) red[warp & 1][(warp >> 1) * 2 + j] = m;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const float sc = fill_scale(fmaxf(red[0][(warp >> 1) * 2 + j], red[1][(warp >> 1) * 2 + j]));
+        uint16_t sl[3];
+        split_pair<F16, XS>(sh[j] * sc, sl_[j] * sc, sl);
+        const int64_t off = ((int64_t)slot * NR + r0 + j) * fx.ld_x + grow;
+#pragma unroll
+        for (int i = 0; i < XS; ++i) fx.xs[i][off] = sl[i];
+        if ((row & 63) == 0) fx.sx[((int64_t)slot * (fx.ld_x / 64) + (rt * 2 + half)) * NR + r0 + j] = 1.f / sc;
     }
 }
 
@@ -711,161 +717,222 @@ __global__ void __launch_bounds__(256) k_split_x(const double* __restrict__ x, i
 // Increments of the plane-wave tests (Sec. II-C): e_m(t_n) - e_m(t_{n-1}) = sum_x c(x).p
 // [env_r(x, t_n) - env_r(x, t_{n-1})] with env_r(x, t) = amp_r exp(-a^2), a = (t - k_r.x - t0_r) /
 // width_r, and the difference written as -amp_r exp(-a_n^2) expm1(d (2 a_n - d)), d = dt / width_r,
-// so that it keeps its relative precision; at n = 1 the test itself (r_0 = 0).  Same for h.  One
-// block per (64-edge tile, 16 waves): compensated FP32 sums over the quadrature points, then the
-// split into the e (slot ring) and h (slot ring + 1) slices of the history operand with one scale
-// per (slot, tile, wave).  t - t0 is carried as an FP32 pair so that late times lose no digits of
-// the pulse's argument.
-constexpr int RHS_RB = 16;
-// 8 warps x 2 edges x 16 waves per pass, 4 passes, so that the 480 blocks of the 7680-edge case are
-// resident at once (1024 threads with one pair each fit one block per SM and measured no faster)
-constexpr int RHS_NT = 256;
-constexpr int RHS_NW = RHS_NT / 32;
-constexpr int RHS_PASS = 64 / (2 * RHS_NW);
+// so that it keeps its relative precision; at n = 1 the test itself (r_0 = 0).  Same for h.  t - t0 is
+// carried as an FP32 pair so that late times lose no digits of the pulse's argument.
+// The tests of a chunk's TC_C steps are formed when it starts, in two kernels: the envelope increments
+// once per quadrature point, step and wave (a point belongs to three RWG or about twelve BC functions:
+// with one exponential pair per edge and point this took 106 us per step at 1920 edges), then one block
+// per (64-edge tile, step) gathers them, compensated FP32 sums over the points, and splits the tile into
+// the e and h slices of the step's slots with one scale per (slot, tile, wave).
+constexpr int ENV_PB = 32;       // points per block (the waves' FP64 parameters are formed once per block)
+__global__ void __launch_bounds__(NR * TC_C) k_env_tc(int npts, const double* __restrict__ exc, double dt, const Ctl* ctl,
+                                                      const float* __restrict__ pts, float* __restrict__ env) {
+    wait_prior();
+    if (ctl->col) return;
+    const int r = threadIdx.x % NR, i = threadIdx.x / NR;      // wave, step of the chunk
+    const double* P = exc + 11 * r;
+    const float kx = (float)P[0], ky = (float)P[1], kz = (float)P[2], amp = (float)P[6], inv_w = (float)(1.0 / P[8]);
+    const int64_t n = ctl->n + i;
+    const double tt = (double)n * dt - P[7];
+    const float tt_hi = (float)tt, tt_lo = (float)(tt - (double)tt_hi), d = (float)(dt / P[8]);
+    const int p1 = min(npts, (int)(blockIdx.x + 1) * ENV_PB);
+#pragma unroll 4
+    for (int pt = blockIdx.x * ENV_PB; pt < p1; ++pt) {
+        const float arg = ((tt_hi - fmaf(kx, pts[3 * pt], fmaf(ky, pts[3 * pt + 1], kz * pts[3 * pt + 2]))) + tt_lo) * inv_w;
+        float v = amp * expf(-arg * arg);
+        if (n != 1) v = -v * expm1f(d * (2.f * arg - d));     // env(t_n) - env(t_{n-1})
+        env[((int64_t)pt * TC_C + i) * NR + r] = v;
+    }
+}
+
+// Block (64-edge tile, step): 16 warps of 4 edges, two waves per lane in packed FP32x2 arithmetic;
+// entries {c, point index} as one 16-byte load
+constexpr int RHS_NW = 16;
+constexpr int RHS_LD = 65;
+constexpr int RHS_SMEM = 2 * 64 * RHS_LD * 8;
 template <bool F16, int XS>
-__global__ void __launch_bounds__(RHS_NT) k_rhs_tc(int ne, const double* __restrict__ exc, double dt, const Ctl* ctl,
-                                                const int* __restrict__ pptr, const float* __restrict__ px,
-                                                const float* __restrict__ pc, const int* __restrict__ nE,
+__global__ void __launch_bounds__(32 * RHS_NW) k_rhs_tc(int ne, const double* __restrict__ exc, const Ctl* ctl,
+                                                const int* __restrict__ eptr, const float* __restrict__ env,
+                                                const float4* __restrict__ ent, const int* __restrict__ nE,
                                                 uint16_t* __restrict__ X0, uint16_t* __restrict__ X1,
                                                 uint16_t* __restrict__ X2, float* __restrict__ sX, int ring, int ld) {
-    __shared__ double ev[2][64][RHS_RB + 1];
-    __shared__ float mred[2][RHS_NW][RHS_RB];
-    __shared__ float scl[2][RHS_RB];
-    const int tile = blockIdx.x, rb = blockIdx.y * RHS_RB;
+    extern __shared__ float2 ev[];      // [e, h][edge][wave], row length RHS_LD: sums as FP32 pairs
+    __shared__ float mred[2][RHS_NW][NR];
+    __shared__ float scl[2][NR];
+    wait_prior();
+    if (ctl->col) return;
+    const int tile = blockIdx.x, step = blockIdx.y;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int rl = lane & 15, r = rb + rl;
-    const double* P = exc + 11 * r;
-    const float kx = (float)P[0], ky = (float)P[1], kz = (float)P[2], qx = (float)P[3], qy = (float)P[4], qz = (float)P[5];
-    const float amp = (float)P[6], inv_w = (float)(1.0 / P[8]);
-    const int64_t n = ctl->n;
-    const double tt = (double)n * dt - P[7];
-    const float tt_hi = (float)tt, tt_lo = (float)(tt - (double)tt_hi);
-    const float d = (float)(dt / P[8]);
-    const bool first = n == 1;
-    const float hx = ky * qz - kz * qy, hy = kz * qx - kx * qz, hz = kx * qy - ky * qx;   // k x p
-    float me = 0.f, mh = 0.f;
-    for (int i = 0; i < RHS_PASS; ++i) {
-        const int el = 2 * warp + (lane >> 4) + 2 * RHS_NW * i;     // edge within the tile
-        const int mm = tile * 64 + el;
-        float e_hi = 0.f, e_lo = 0.f, h_hi = 0.f, h_lo = 0.f;
-        if (mm < ne) {
-            const int b = pptr[mm], me_ = b + nE[mm], end = pptr[mm + 1];
-            for (int qp = b; qp < end; ++qp) {
-                const float x = px[3 * qp], y = px[3 * qp + 1], z = px[3 * qp + 2];
-                const float arg = ((tt_hi - fmaf(kx, x, fmaf(ky, y, kz * z))) + tt_lo) * inv_w;
-                float env = amp * expf(-arg * arg);
-                if (!first) env = -env * expm1f(d * (2.f * arg - d));     // env(t_n) - env(t_{n-1})
-                const float cx = pc[3 * qp], cy = pc[3 * qp + 1], cz = pc[3 * qp + 2];
-                if (qp < me_) two_sum_acc(e_hi, e_lo, env * fmaf(cx, qx, fmaf(cy, qy, cz * qz)));
-                else two_sum_acc(h_hi, h_lo, env * fmaf(cx, hx, fmaf(cy, hy, cz * hz)));
-            }
+    float2 pol[2][3];       // p and k x p of the lane's two waves
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+        const double* P = exc + 11 * (2 * lane + w);
+        const float k[3] = {(float)P[0], (float)P[1], (float)P[2]}, q[3] = {(float)P[3], (float)P[4], (float)P[5]};
+        const float h[3] = {k[1] * q[2] - k[2] * q[1], k[2] * q[0] - k[0] * q[2], k[0] * q[1] - k[1] * q[0]};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            if (w == 0) { pol[0][c].x = q[c]; pol[1][c].x = h[c]; }
+            else { pol[0][c].y = q[c]; pol[1][c].y = h[c]; }
         }
-        const double ed = (double)e_hi + (double)e_lo, hd = (double)h_hi + (double)h_lo;
-        ev[0][el][rl] = ed;
-        ev[1][el][rl] = hd;
-        me = fmaxf(me, fabsf((float)ed));
-        mh = fmaxf(mh, fabsf((float)hd));
     }
-    // per-wave maxima over the 64 edges: lanes l and l + 16 share a wave
-    me = fmaxf(me, __shfl_xor_sync(0xffffffffu, me, 16));
-    mh = fmaxf(mh, __shfl_xor_sync(0xffffffffu, mh, 16));
-    if (lane < 16) { mred[0][warp][lane] = me; mred[1][warp][lane] = mh; }
+    const float2* en = reinterpret_cast<const float2*>(env) + step * (NR / 2) + lane;
+    float mx[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+    for (int el = warp; el < 64; el += RHS_NW) {
+        const int mm = tile * 64 + el;
+        int q = 0, end = 0;
+        if (mm < ne) q = eptr[mm];
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            float2 hi = make_float2(0.f, 0.f), lo = hi;
+            if (mm < ne) end = f == 0 ? q + nE[mm] : eptr[mm + 1];
+#pragma unroll 4
+            for (; q < end; ++q) {
+                const float4 c = ent[q];
+                const float2 v = en[(int64_t)__float_as_int(c.w) * (TC_C * NR / 2)];
+                const float2 cp = __ffma2_rn(make_float2(c.x, c.x), pol[f][0],
+                                             __ffma2_rn(make_float2(c.y, c.y), pol[f][1], __fmul2_rn(make_float2(c.z, c.z), pol[f][2])));
+                two_sum_acc2(hi, lo, __fmul2_rn(v, cp));
+            }
+            float2* dst = ev + (f * 64 + el) * RHS_LD + 2 * lane;
+            dst[0] = make_float2(hi.x, lo.x);
+            dst[1] = make_float2(hi.y, lo.y);
+            mx[f][0] = fmaxf(mx[f][0], fabsf(hi.x + lo.x));
+            mx[f][1] = fmaxf(mx[f][1], fabsf(hi.y + lo.y));
+        }
+    }
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+        mred[f][warp][2 * lane] = mx[f][0];
+        mred[f][warp][2 * lane + 1] = mx[f][1];
+    }
     __syncthreads();
-    if (t < 2 * RHS_RB) {
-        const int w = t / RHS_RB, j = t % RHS_RB;
+    const int slot0 = ring + 2 * step;
+    if (t < 2 * NR) {
+        const int w = t / NR, j = t % NR;
         float m = 0.f;
-        for (int k = 0; k < RHS_NW; ++k) m = fmaxf(m, mred[w][k][j]);
-        if (!(m == m)) m = INFINITY;
+        for (int k = 0; k < RHS_NW; ++k) {
+            const float v = mred[w][k][j];
+            m = v == v ? fmaxf(m, v) : INFINITY;
+        }
         scl[w][j] = fill_scale(m);
-        sX[((int64_t)(ring + w) * (ld / 64) + tile) * NR + rb + j] = 1.f / scl[w][j];
+        sX[((int64_t)(slot0 + w) * (ld / 64) + tile) * NR + j] = 1.f / scl[w][j];
     }
     __syncthreads();
     uint16_t* dst[3] = {X0, X1, X2};
-    for (int i = t; i < 2 * RHS_RB * 64; i += RHS_NT) {
-        const int w = i / (RHS_RB * 64), j = (i / 64) % RHS_RB, el = i & 63;
-        uint16_t sl[3];
-        split_vector<F16, XS>(ev[w][el][j] * (double)scl[w][j], sl);
-        const int64_t off = ((int64_t)(ring + w) * NR + rb + j) * ld + tile * 64 + el;
+    for (int i = t; i < 2 * NR * 32; i += 32 * RHS_NW) {      // two edges per thread and turn
+        const int w = i / (NR * 32), j = i / 32 % NR, el = 2 * (i & 31);
+        uint16_t sl[2][3];
 #pragma unroll
-        for (int k = 0; k < XS; ++k) dst[k][off] = sl[k];
+        for (int u = 0; u < 2; ++u) {
+            const float2 v = ev[(w * 64 + el + u) * RHS_LD + j];
+            split_pair<F16, XS>(v.x * scl[w][j], v.y * scl[w][j], sl[u]);
+        }
+        const int64_t off = ((int64_t)(slot0 + w) * NR + j) * ld + tile * 64 + el;
+#pragma unroll
+        for (int k = 0; k < XS; ++k)
+            *reinterpret_cast<uint32_t*>(dst[k] + off) = (uint32_t)sl[0][k] | ((uint32_t)sl[1][k] << 16);
     }
 }
 
 // ---------------------------------------------------------------- projector in / out
 // z[r][c] = sum_j tsign[c][j] w[r][tedge[c][j]], w = dy_n / dtt - y_n (= (1/dtt - 1) y_n - y_{n-1}/dtt)
-// from the FP64 y_n and dy_n; split into the z slices with one scale per (64-triangle tile, wave).
+// from the FP64 y_n and dy_n; split into the z slices with one scale per (64-triangle tile, wave).  Grid
+// z: the steps p0 .. ctl->n + adv - 1 still to post-process (at most TC_C), slot by slot.
+constexpr int PIN_RB = 16;      // waves per block
+__device__ __forceinline__ int post_count(const Ctl* ctl, int adv) { return (int)(ctl->n + adv - ctl->p0); }
+// column of the chunk of step p0 + k (ctl->col belongs to ctl->n)
+__device__ __forceinline__ int post_col(const Ctl* ctl, int k) {
+    const int c = ctl->col + (int)(ctl->p0 - ctl->n) + k;
+    return c < 0 ? c + TC_C : c;
+}
 template <bool F16, int XS>
-__global__ void __launch_bounds__(256) k_project_in_tc(DevMesh m, const Ctl* ctl, const double* __restrict__ y2,
-                                                       double dtt, uint16_t* __restrict__ Z0, uint16_t* __restrict__ Z1,
+__global__ void __launch_bounds__(256) k_project_in_tc(DevMesh m, const Ctl* ctl, int adv, const double* __restrict__ y2,
+                                                       double inv_dtt, uint16_t* __restrict__ Z0, uint16_t* __restrict__ Z1,
                                                        uint16_t* __restrict__ Z2, float* __restrict__ sZ, int ldc) {
-    __shared__ double zv[RHS_RB][65];
-    __shared__ float scl[RHS_RB];
-    const int tile = blockIdx.x, rb = blockIdx.y * RHS_RB;
+    __shared__ float2 zv[PIN_RB][65];      // FP64 values as FP32 pairs (their slices keep 33 bits)
+    __shared__ float scl[PIN_RB];
+    const int tile = blockIdx.x, rb = blockIdx.y * PIN_RB;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    (void)ctl;
-    const double* yn = y2;                          // y_n
-    const double* dy = y2 + (int64_t)NR * m.ne;     // dy_n
+    wait_prior();
+    const int k = blockIdx.z;
+    if (k >= post_count(ctl, adv)) return;
+    const double* yn = y2 + (int64_t)post_col(ctl, k) * 2 * NR * m.ne;      // y_n
+    const double* dy = yn + (int64_t)NR * m.ne;                             // dy_n
     float mx = 0.f;
     // thread -> (wave rb + (t >> 4) ... ): 16 waves x 64 triangles, 4 per thread, triangles fastest
-    for (int i = t; i < RHS_RB * 64; i += 256) {
+    for (int i = t; i < PIN_RB * 64; i += 256) {
         const int j = i >> 6, cl = i & 63, c = tile * 64 + cl, r = rb + j;
         double s = 0.0;
         if (c < m.nc) {
-            for (int k = 0; k < 3; ++k) {
-                const int e = m.tedge[3 * c + k];
-                const double w = dy[(int64_t)r * m.ne + e] / dtt - yn[(int64_t)r * m.ne + e];
-                s += m.tsign[3 * c + k] * w;
+            for (int l = 0; l < 3; ++l) {
+                const int e = m.tedge[3 * c + l];
+                s = fma(m.tsign[3 * c + l], fma(dy[(int64_t)r * m.ne + e], inv_dtt, -yn[(int64_t)r * m.ne + e]), s);
             }
         }
-        zv[j][cl] = s;
+        const float hi = (float)s;
+        zv[j][cl] = make_float2(hi, (float)(s - (double)hi));
     }
     __syncthreads();
     // maxima: warp w covers waves 2w, 2w+1 (lanes 0-15 / 16-31), 4 triangles per lane
     {
         const int j = 2 * warp + (lane >> 4), c4 = (lane & 15) * 4;
-        for (int k = 0; k < 4; ++k) mx = fmaxf(mx, fabsf((float)zv[j][c4 + k]));
+        for (int l = 0; l < 4; ++l) mx = fmaxf(mx, fabsf(zv[j][c4 + l].x));
         for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         if ((lane & 15) == 0) {
             if (!(mx == mx)) mx = INFINITY;
             scl[j] = fill_scale(mx);
-            sZ[((int64_t)tile) * NR + rb + j] = 1.f / scl[j];
+            sZ[((int64_t)k * (ldc / 64) + tile) * NR + rb + j] = 1.f / scl[j];
         }
     }
     __syncthreads();
     uint16_t* dst[3] = {Z0, Z1, Z2};
-    for (int i = t; i < RHS_RB * 64; i += 256) {
+    for (int i = t; i < PIN_RB * 64; i += 256) {
         const int j = i >> 6, cl = i & 63;
         uint16_t sl[3];
-        split_vector<F16, XS>(zv[j][cl] * (double)scl[j], sl);
-        const int64_t off = (int64_t)(rb + j) * ldc + tile * 64 + cl;
+        split_pair<F16, XS>(zv[j][cl].x * scl[j], zv[j][cl].y * scl[j], sl);
+        const int64_t off = ((int64_t)k * NR + rb + j) * ldc + tile * 64 + cl;
 #pragma unroll
-        for (int k = 0; k < XS; ++k) dst[k][off] = sl[k];
+        for (int l = 0; l < XS; ++l) dst[l][off] = sl[l];
     }
 }
 
-// j[r][m] = y_n[r][m] + u[r][c+(m)] - u[r][c-(m)] in FP64, stored in FP32; finiteness check; the
-// last block to finish advances the step counter (every block has read n before it arrives).
-__global__ void k_project_out_tc(DevMesh m, int R, Ctl* ctl, const double* __restrict__ y2, const double* __restrict__ u,
-                                 int* __restrict__ done) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t n = ctl->n;
-    if (idx < m.ne * R) {
+// j[r][m] = y_n[r][m] + u[r][c+(m)] - u[r][c-(m)] in FP64, stored in FP32; finiteness check (the first
+// bad step is kept); grid y: the steps to post-process; the last block to finish advances the step
+// counter by adv (every block has read it before it arrives).
+__global__ void k_project_out_tc(DevMesh m, Ctl* ctl, int adv, const double* __restrict__ y2,
+                                 const double* __restrict__ u, int* __restrict__ done) {
+    wait_prior();
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+    const int64_t n = ctl->p0 + k;
+    if (idx < m.ne * NR && k < post_count(ctl, adv)) {
         const int r = idx / m.ne, e = idx % m.ne;
-        const double yv = y2[(int64_t)r * m.ne + e];
-        const double val = yv + u[(int64_t)r * m.nc + m.cplus_[e]] - u[(int64_t)r * m.nc + m.cminus_[e]];
-        if (!isfinite(val) && atomicCAS(&ctl->status, 0, (int)TDCFIE_E_NONFINITE) == 0) ctl->bad_step = n;
-        if (ctl->out) reinterpret_cast<float*>(ctl->out)[((n - ctl->n0) * R + r) * (int64_t)m.ne + e] = (float)val;
-        if (ctl->yout) reinterpret_cast<float*>(ctl->yout)[((n - ctl->n0) * R + r) * (int64_t)m.ne + e] = (float)yv;
+        const double yv = y2[((int64_t)post_col(ctl, k) * 2 * NR + r) * m.ne + e];
+        const double* uk = u + ((int64_t)k * NR + r) * m.nc;
+        const double val = yv + uk[m.cplus_[e]] - uk[m.cminus_[e]];
+        if (!isfinite(val)) {
+            atomicCAS(&ctl->status, 0, (int)TDCFIE_E_NONFINITE);
+            atomicMin(reinterpret_cast<unsigned long long*>(&ctl->bad_step), (unsigned long long)n);
+        }
+        const int64_t at = ((n - ctl->n0) * NR + r) * (int64_t)m.ne + e;
+        if (ctl->out) reinterpret_cast<float*>(ctl->out)[at] = (float)val;
+        if (ctl->yout) reinterpret_cast<float*>(ctl->yout)[at] = (float)yv;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(done, 1) == (int)gridDim.x - 1) {
+        if (atomicAdd(done, 1) == (int)(gridDim.x * gridDim.y) - 1) {
             *done = 0;
-            ctl->n = n + 1;
+            ctl->n += adv;
+            ctl->col = (ctl->col + adv) % TC_C;
+            ctl->p0 = ctl->n;
             __threadfence();
         }
     }
+}
+__global__ void k_advance_tc(Ctl* ctl) {
+    wait_prior();
+    ctl->n += 1;
+    ctl->col = (ctl->col + 1) % TC_C;
 }
 
 // ---------------------------------------------------------------- host side
@@ -905,7 +972,6 @@ struct Gemm {
     int grid = 0;
     int* seg_ptr = nullptr;
     int* seg_slot = nullptr;
-    int* cnt = nullptr;
 };
 
 struct TcStep {
@@ -915,12 +981,13 @@ struct TcStep {
     uint16_t *Ah = nullptr, *Al = nullptr;          // history blocks [nblk][ne][ld]
     uint16_t *Th = nullptr, *Tl = nullptr;          // T_0^-1
     uint16_t *Ph = nullptr, *Pl = nullptr;          // (Sigma^T Sigma)^+
-    uint16_t* X[3] = {nullptr, nullptr, nullptr};   // history ring + e_n + h_n slots [ring+2][R][ld]
+    uint16_t* X[3] = {nullptr, nullptr, nullptr};   // history ring + e, h slots of a chunk [ring + 2 TC_C][R][ld]
     uint16_t* B[3] = {nullptr, nullptr, nullptr};   // b [R][ld]
-    uint16_t* Z[3] = {nullptr, nullptr, nullptr};   // z [R][ldc]
+    uint16_t* Z[3] = {nullptr, nullptr, nullptr};   // z [TC_C][R][ldc]
+    float* env = nullptr;                           // envelope increments [npts][TC_C][R]
     float *sAh = nullptr, *sAs = nullptr, *sAp = nullptr;   // inverse row scales
     float *sXh = nullptr, *sXb = nullptr, *sXz = nullptr;   // inverse tile scales of the vectors
-    double *y2 = nullptr, *u = nullptr;             // FP64 y_n and dy_n [2][R][ne], u [R][nc]
+    double *y2 = nullptr, *u = nullptr;             // FP64 y_n, dy_n [TC_C][2][R][ne], u [TC_C][R][nc]
     int* done = nullptr;
     float* partial = nullptr;
     Gemm hist, solve, proj;
@@ -930,7 +997,6 @@ struct TcStep {
         for (Gemm* g : {&hist, &solve, &proj}) {
             if (g->seg_ptr) cudaFree(g->seg_ptr);
             if (g->seg_slot) cudaFree(g->seg_slot);
-            if (g->cnt) cudaFree(g->cnt);
         }
     }
 };
@@ -944,14 +1010,14 @@ __global__ void k_fill(float* p, int64_t n, float v) {
 
 // history ring, e/h slots and the FP64 y pair start at zero (y_i = 0 for i <= 0)
 cudaError_t reset_tc(TcStep* g, int ring, int ne, cudaStream_t s) {
-    const size_t xs = sizeof(uint16_t) * (size_t)(ring + 2) * g->R * g->ld;
+    const size_t xs = sizeof(uint16_t) * (size_t)(ring + 2 * TC_C) * g->R * g->ld;
     cudaError_t e;
     for (int i = 0; i < g->xs; ++i)
         if ((e = cudaMemsetAsync(g->X[i], 0, xs, s)) != cudaSuccess) return e;
-    const int64_t ns = (int64_t)(ring + 2) * (g->ld / 64) * g->R;
+    const int64_t ns = (int64_t)(ring + 2 * TC_C) * (g->ld / 64) * g->R;
     k_fill<<<(unsigned)((ns + 255) / 256), 256, 0, s>>>(g->sXh, ns, 1.f);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return cudaMemsetAsync(g->y2, 0, sizeof(double) * 2 * (size_t)g->R * ne, s);
+    return cudaMemsetAsync(g->y2, 0, sizeof(double) * 2 * TC_C * (size_t)g->R * ne, s);
 }
 
 template <class T>
@@ -962,17 +1028,19 @@ static cudaError_t dalloc(TcStep* g, T** p, size_t count) {
 }
 
 // stream-K partition and the per-row-tile list of partial slots (same traversal as the kernel)
-static void plan_segments(GemmArgs& a, int& grid, int rows, int cols, int nblk, int sms, std::vector<int>& ptr,
+static void plan_segments(GemmArgs& a, int& grid, int rows, int cols, int nblk, int reps, int sms, std::vector<int>& ptr,
                           std::vector<int>& slot) {
     a.rows = rows;
     a.cols = cols;
     a.nblk = nblk;
+    a.reps = reps;
     a.ktiles = (cols + BK - 1) / BK;
     a.rtiles = (rows + BM - 1) / BM;
-    a.total = (int64_t)a.rtiles * nblk * a.ktiles;
+    const int tiles = a.rtiles * reps;
+    a.total = (int64_t)tiles * nblk * a.ktiles;
     grid = (int)std::min<int64_t>(sms, a.total);
     const int64_t ipt = (int64_t)nblk * a.ktiles;
-    std::vector<std::vector<std::pair<int, int>>> lists(a.rtiles);
+    std::vector<std::vector<std::pair<int, int>>> lists(tiles);
     int maxseg = 1;
     for (int c = 0; c < grid; ++c) {
         const int64_t b = (int64_t)c * a.total / grid, e = (int64_t)(c + 1) * a.total / grid;
@@ -985,27 +1053,24 @@ static void plan_segments(GemmArgs& a, int& grid, int rows, int cols, int nblk, 
         maxseg = std::max(maxseg, seg);
     }
     a.maxseg = maxseg;
-    ptr.assign(a.rtiles + 1, 0);
+    ptr.assign(tiles + 1, 0);
     slot.clear();
-    for (int t = 0; t < a.rtiles; ++t) {
+    for (int t = 0; t < tiles; ++t) {
         for (auto& cs : lists[t]) slot.push_back(cs.first * maxseg + cs.second);
         ptr[t + 1] = (int)slot.size();
     }
 }
 
-static cudaError_t plan_gemm(Gemm& G, int rows, int cols, int nblk, int sms) {
+static cudaError_t plan_gemm(Gemm& G, int rows, int cols, int nblk, int reps, int sms) {
     std::vector<int> ptr, slot;
-    plan_segments(G.a, G.grid, rows, cols, nblk, sms, ptr, slot);
+    plan_segments(G.a, G.grid, rows, cols, nblk, reps, sms, ptr, slot);
     cudaError_t e;
     if ((e = cudaMalloc(&G.seg_ptr, sizeof(int) * ptr.size())) != cudaSuccess) return e;
     if ((e = cudaMalloc(&G.seg_slot, sizeof(int) * slot.size())) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&G.cnt, sizeof(int) * G.a.rtiles)) != cudaSuccess) return e;
-    if ((e = cudaMemset(G.cnt, 0, sizeof(int) * G.a.rtiles)) != cudaSuccess) return e;
     if ((e = cudaMemcpy(G.seg_ptr, ptr.data(), sizeof(int) * ptr.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
     if ((e = cudaMemcpy(G.seg_slot, slot.data(), sizeof(int) * slot.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
     G.a.seg_ptr = G.seg_ptr;
     G.a.seg_slot = G.seg_slot;
-    G.a.cnt = G.cnt;
     return cudaSuccess;
 }
 
@@ -1013,9 +1078,11 @@ static size_t partial_floats(const Gemm& G) { return (size_t)G.grid * G.a.maxseg
 
 template <int XS, bool F16>
 static void launch_gemm(const Gemm& G, cudaStream_t s) {
-    k_tc_gemm<XS, F16><<<G.grid, NTHREADS, Cfg<XS>::SMEM, s>>>(G.ah, G.al, G.x[0], G.x[1], G.x[2], G.a);
+    launch_chained(k_tc_gemm<XS, F16>, G.grid, NTHREADS, s, Cfg<XS>::SMEM, G.ah, G.al, G.x[0], G.x[1], G.x[2], G.a);
+    launch_chained(k_tc_fix<XS, F16>, dim3(2 * G.a.rtiles * G.a.reps, NR / FIX_RB), 256, s, 0, G.a);
 }
 
+// the product and its sums: two kernels
 static void run_gemm(const TcStep* g, const Gemm& G, cudaStream_t s) {
     if (g->fp16) {
         if (g->xs == 3) launch_gemm<3, true>(G, s);
@@ -1032,6 +1099,10 @@ static cudaError_t set_smem_attrs() {
         return e;
     if ((e = cudaFuncSetAttribute(k_tc_gemm<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM)) !=
         cudaSuccess)
+        return e;
+    if ((e = cudaFuncSetAttribute(k_rhs_tc<true, FP16_XS>, cudaFuncAttributeMaxDynamicSharedMemorySize, RHS_SMEM)) != cudaSuccess)
+        return e;
+    if ((e = cudaFuncSetAttribute(k_rhs_tc<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, RHS_SMEM)) != cudaSuccess)
         return e;
     return cudaFuncSetAttribute(k_tc_gemm<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM);
 }
@@ -1083,11 +1154,11 @@ tdcfie_status build_tc(tdcfie_t h, StepPlan* p) {
     CKB(dalloc(g, &g->Ph, (size_t)nc * ldc));
     CKB(dalloc(g, &g->Pl, (size_t)nc * ldc));
     for (int i = 0; i < XS; ++i) {
-        CKB(dalloc(g, &g->X[i], (size_t)(ring + 2) * R * ld));
+        CKB(dalloc(g, &g->X[i], (size_t)(ring + 2 * TC_C) * R * ld));
         CKB(dalloc(g, &g->B[i], (size_t)R * ld));
-        CKB(dalloc(g, &g->Z[i], (size_t)R * ldc));
+        CKB(dalloc(g, &g->Z[i], (size_t)TC_C * R * ldc));
         CKB(cudaMemsetAsync(g->B[i], 0, sizeof(uint16_t) * R * ld, s));
-        CKB(cudaMemsetAsync(g->Z[i], 0, sizeof(uint16_t) * R * ldc, s));
+        CKB(cudaMemsetAsync(g->Z[i], 0, sizeof(uint16_t) * TC_C * R * ldc, s));
     }
     for (int i = XS; i < 3; ++i) { g->X[i] = g->X[0]; g->B[i] = g->B[0]; g->Z[i] = g->Z[0]; }   // unused maps
     CKB(dalloc(g, &g->sAh, (size_t)ne));
@@ -1095,11 +1166,13 @@ tdcfie_status build_tc(tdcfie_t h, StepPlan* p) {
     CKB(dalloc(g, &g->sAp, (size_t)nc));
     float* rowmax = nullptr;
     CKB(dalloc(g, &rowmax, (size_t)std::max(ne, nc)));
-    CKB(dalloc(g, &g->sXh, (size_t)(ring + 2) * (ld / 64) * R));
+    CKB(dalloc(g, &g->sXh, (size_t)(ring + 2 * TC_C) * (ld / 64) * R));
     CKB(dalloc(g, &g->sXb, (size_t)(ld / 64) * R));
-    CKB(dalloc(g, &g->sXz, (size_t)(ldc / 64) * R));
-    CKB(dalloc(g, &g->y2, (size_t)2 * R * ne));
-    CKB(dalloc(g, &g->u, (size_t)R * nc));
+    CKB(dalloc(g, &g->sXz, (size_t)TC_C * (ldc / 64) * R));
+    CKB(cudaMemsetAsync(g->sXz, 0, sizeof(float) * TC_C * (ldc / 64) * R, s));
+    CKB(dalloc(g, &g->y2, (size_t)2 * TC_C * R * ne));
+    CKB(dalloc(g, &g->u, (size_t)TC_C * R * nc));
+    CKB(dalloc(g, &g->env, (size_t)p->npts * TC_C * R));
     CKB(dalloc(g, &g->done, 1));
     CKB(cudaMemsetAsync(g->done, 0, sizeof(int), s));
     // matrices: -A, alpha L2, -T_1 .. -T_{K-1}, then T_0^-1 and the Laplacian pseudo-inverse
@@ -1118,9 +1191,9 @@ tdcfie_status build_tc(tdcfie_t h, StepPlan* p) {
     CKB(cudaStreamSynchronize(s));
     CKB(reset_tc(g, ring, ne, s));
     // GEMM plans and tensor maps
-    CKB(plan_gemm(g->hist, ne, ne, nblk, g->sms));
-    CKB(plan_gemm(g->solve, ne, ne, 1, g->sms));
-    CKB(plan_gemm(g->proj, nc, nc, 1, g->sms));
+    CKB(plan_gemm(g->hist, ne, ne, nblk, 1, g->sms));
+    CKB(plan_gemm(g->solve, ne, ne, 1, 1, g->sms));
+    CKB(plan_gemm(g->proj, nc, nc, 1, TC_C, g->sms));
     size_t pmax = 0;
     for (Gemm* G : {&g->hist, &g->solve, &g->proj}) pmax = std::max(pmax, partial_floats(*G));
     CKB(dalloc(g, &g->partial, pmax));
@@ -1128,9 +1201,9 @@ tdcfie_status build_tc(tdcfie_t h, StepPlan* p) {
               make_map(&g->solve.ah, g->Th, ne, ne, 1, ld, BM, f16) && make_map(&g->solve.al, g->Tl, ne, ne, 1, ld, BM, f16) &&
               make_map(&g->proj.ah, g->Ph, nc, nc, 1, ldc, BM, f16) && make_map(&g->proj.al, g->Pl, nc, nc, 1, ldc, BM, f16);
     for (int i = 0; i < 3; ++i)
-        ok = ok && make_map(&g->hist.x[i], g->X[i], ne, R, ring + 2, ld, R, f16) &&
+        ok = ok && make_map(&g->hist.x[i], g->X[i], ne, R, ring + 2 * TC_C, ld, R, f16) &&
              make_map(&g->solve.x[i], g->B[i], ne, R, 1, ld, R, f16) &&
-             make_map(&g->proj.x[i], g->Z[i], nc, R, 1, ldc, R, f16);
+             make_map(&g->proj.x[i], g->Z[i], nc, R, TC_C, ldc, R, f16);
     if (!ok) return fail(h, TDCFIE_E_CUDA, "cuTensorMapEncodeTiled failed");
     const uint32_t id = make_idesc(R, !f16);
     for (Gemm* G : {&g->hist, &g->solve, &g->proj}) {
@@ -1138,11 +1211,15 @@ tdcfie_status build_tc(tdcfie_t h, StepPlan* p) {
         G->a.ctl = p->ctl;
         G->a.ring = ring;
         G->a.slot_mode = 1;
+        G->a.off = 0;
+        G->a.mark = 0;
         G->a.idesc = id;
         G->a.fx = FixOut{};
     }
     // history: d_n -> slices of the solve's vector operand
     g->hist.a.slot_mode = 0;
+    g->hist.a.mark = 1;
+    g->solve.a.mark = 2;
     g->hist.a.sA = g->sAh;
     g->hist.a.sX = g->sXh;
     g->hist.a.fx.mode = FIX_SPLIT;
@@ -1174,32 +1251,52 @@ tdcfie_status build_tc(tdcfie_t h, StepPlan* p) {
     return TDCFIE_OK;
 }
 
-void launch_step_tc(tdcfie_t h, StepPlan* p, cudaStream_t s) {
+// tests of the chunk's steps (nothing unless a chunk starts at the current step) -> their e, h slots
+int launch_tests_tc(tdcfie_t h, StepPlan* p, cudaStream_t s) {
     TcStep* g = p->gemm;
-    const int R = p->R, ne = p->ne, ring = p->ring, ld = g->ld, ldc = g->ldc;
-    const dim3 grhs(ld / 64, R / RHS_RB), gproj(ldc / 64, R / RHS_RB);
-    // 1. increments of the plane-wave tests -> e, h slots of the history operand
+    const int ne = p->ne, ring = p->ring, ld = g->ld;
+    launch_chained(k_env_tc, (p->npts + ENV_PB - 1) / ENV_PB, NR * TC_C, s, 0, p->npts, h->dexc, h->dt, p->ctl, (const float*)p->pts, g->env);
+    const dim3 grhs(ld / 64, TC_C);
+    const float4* ent = (const float4*)p->ecoef;
     if (g->fp16)
-        k_rhs_tc<true, FP16_XS><<<grhs, RHS_NT, 0, s>>>(ne, h->dexc, h->dt, p->ctl, p->pptr, (const float*)p->px,
-                                                (const float*)p->pc, p->pnE, g->X[0], g->X[1], g->X[2], g->sXh, ring, ld);
+        launch_chained(k_rhs_tc<true, FP16_XS>, grhs, 32 * RHS_NW, s, RHS_SMEM, ne, h->dexc, p->ctl, p->eptr, g->env, ent, p->enE,
+                       g->X[0], g->X[1], g->X[2], g->sXh, ring, ld);
     else
-        k_rhs_tc<false, 2><<<grhs, RHS_NT, 0, s>>>(ne, h->dexc, h->dt, p->ctl, p->pptr, (const float*)p->px,
-                                                 (const float*)p->pc, p->pnE, g->X[0], g->X[1], g->X[2], g->sXh, ring, ld);
-    // 2. increment of the history sum d_n = -A de_n + alpha L2 dh_n - sum_k T_k dy_{n-k}  (events bracket the GEMM)
-    cudaEventRecordWithFlags(p->evA, s, cudaEventRecordExternal);
-    run_gemm(g, g->hist, s);
-    cudaEventRecordWithFlags(p->evB, s, cudaEventRecordExternal);
-    // 3. dy_n = T_0^-1 d_n, y_n = y_{n-1} + dy_n (FP64); dy_n's slices into history slot n % ring
-    run_gemm(g, g->solve, s);
-    // 4. projector: z = Sigma^T w_n, u = (Sigma^T Sigma)^+ z, j_n = y_n + Sigma u = P^LH y_n + P^S dy_n / dtt
-    if (g->fp16)
-        k_project_in_tc<true, FP16_XS><<<gproj, 256, 0, s>>>(h->dm, p->ctl, g->y2, h->dtt, g->Z[0], g->Z[1], g->Z[2], g->sXz, ldc);
-    else
-        k_project_in_tc<false, 2><<<gproj, 256, 0, s>>>(h->dm, p->ctl, g->y2, h->dtt, g->Z[0], g->Z[1], g->Z[2], g->sXz, ldc);
-    run_gemm(g, g->proj, s);
-    k_project_out_tc<<<(ne * R + 255) / 256, 256, 0, s>>>(h->dm, R, p->ctl, g->y2, g->u, g->done);
-    p->launches_per_step = 6;
+        launch_chained(k_rhs_tc<false, 2>, grhs, 32 * RHS_NW, s, RHS_SMEM, ne, h->dexc, p->ctl, p->eptr, g->env, ent, p->enE,
+                       g->X[0], g->X[1], g->X[2], g->sXh, ring, ld);
+    return 2;
 }
+
+// step ctl->n + off: d_n = -A de_n + alpha L2 dh_n - sum_k T_k dy_{n-k}, then dy_n = T_0^-1 d_n, y_n = y_{n-1} +
+// dy_n (FP64) and dy_n's slices into history slot n % ring; advance: the step counter moves on
+int launch_inner_tc(tdcfie_t h, StepPlan* p, int off, bool advance, cudaStream_t s) {
+    (void)h;
+    TcStep* g = p->gemm;
+    Gemm hist = g->hist, solve = g->solve;
+    hist.a.off = solve.a.off = off;
+    run_gemm(g, hist, s);
+    run_gemm(g, solve, s);
+    if (advance) launch_chained(k_advance_tc, 1, 1, s, 0, p->ctl);
+    return advance ? 5 : 4;
+}
+
+// projector of the finished steps: z = Sigma^T w_n, u = (Sigma^T Sigma)^+ z, j_n = y_n + Sigma u = P^LH y_n +
+// P^S dy_n / dtt; the step counter moves by adv
+int launch_post_tc(tdcfie_t h, StepPlan* p, int adv, cudaStream_t s) {
+    TcStep* g = p->gemm;
+    const int ne = p->ne, ldc = g->ldc;
+    const dim3 gproj(ldc / 64, NR / PIN_RB, TC_C);
+    if (g->fp16)
+        launch_chained(k_project_in_tc<true, FP16_XS>, gproj, 256, s, 0, h->dm, p->ctl, adv, g->y2, 1.0 / h->dtt, g->Z[0], g->Z[1],
+                       g->Z[2], g->sXz, ldc);
+    else
+        launch_chained(k_project_in_tc<false, 2>, gproj, 256, s, 0, h->dm, p->ctl, adv, g->y2, 1.0 / h->dtt, g->Z[0], g->Z[1], g->Z[2],
+                       g->sXz, ldc);
+    run_gemm(g, g->proj, s);
+    launch_chained(k_project_out_tc, dim3((ne * NR + 255) / 256, TC_C), 256, s, 0, h->dm, p->ctl, adv, g->y2, g->u, g->done);
+    return 4;
+}
+int tc_chunk() { return TC_C; }
 
 // ---------------------------------------------------------------- stand-alone product
 // out[r][i] = sum_q sum_j blocks[q][i][j] x[q][r][j] in the split format (see tdcfie.h)
@@ -1224,7 +1321,7 @@ tdcfie_status tc_gemm(int precision, const double* blocks, int64_t nblk, int64_t
     g.xs = XS;
     Gemm& G = g.hist;
     std::vector<int> ptr, slot;
-    plan_segments(G.a, G.grid, (int)rows, (int)cols, (int)nblk, sms, ptr, slot);
+    plan_segments(G.a, G.grid, (int)rows, (int)cols, (int)nblk, 1, sms, ptr, slot);
     CKB(dalloc(&g, &g.Ah, (size_t)nblk * rows * ld));
     CKB(dalloc(&g, &g.Al, (size_t)nblk * rows * ld));
     CKB(dalloc(&g, &g.sAh, (size_t)rows));
@@ -1236,11 +1333,9 @@ tdcfie_status tc_gemm(int precision, const double* blocks, int64_t nblk, int64_t
     CKB(dalloc(&g, &g.partial, partial_floats(G)));
     CKB(dalloc(&g, &G.seg_ptr, ptr.size()));
     CKB(dalloc(&g, &G.seg_slot, slot.size()));
-    CKB(dalloc(&g, &G.cnt, (size_t)G.a.rtiles));
-    g.owned.erase(g.owned.end() - 3, g.owned.end());   // freed by ~TcStep's per-Gemm loop
+    g.owned.erase(g.owned.end() - 2, g.owned.end());   // freed by ~TcStep's per-Gemm loop
     CKB(cudaMemcpyAsync(G.seg_ptr, ptr.data(), sizeof(int) * ptr.size(), cudaMemcpyHostToDevice, s));
     CKB(cudaMemcpyAsync(G.seg_slot, slot.data(), sizeof(int) * slot.size(), cudaMemcpyHostToDevice, s));
-    CKB(cudaMemsetAsync(G.cnt, 0, sizeof(int) * G.a.rtiles, s));
     {
         std::vector<SplitBlock> sb;
         for (int64_t q = 0; q < nblk; ++q) sb.push_back({blocks + q * rows * cols, 1.0, g.Ah + q * rows * ld, g.Al + q * rows * ld});
@@ -1258,10 +1353,11 @@ tdcfie_status tc_gemm(int precision, const double* blocks, int64_t nblk, int64_t
     CKB(cudaMemsetAsync(ctl, 0, sizeof(Ctl), s));
     G.a.seg_ptr = G.seg_ptr;
     G.a.seg_slot = G.seg_slot;
-    G.a.cnt = G.cnt;
     G.a.partial = g.partial;
     G.a.ctl = ctl;
     G.a.ring = 1;
+    G.a.off = 0;
+    G.a.mark = 0;
     G.a.slot_mode = 2;
     G.a.idesc = make_idesc(NR, !f16);
     G.a.sA = g.sAh;
