@@ -4,8 +4,8 @@
 // network 8 -> 64 -> 64 -> 1 with tanh hidden layers, prediction y_{n,m} = y_{n-1,m} + s_n f(x) (the
 // network learns the increment; a zero output is the previous-step guess).
 // Parameters (FP32 master, 4801 floats): W1 (64 x 8), b1 (64), W2 (64 x 64), b2 (64), W3 (64), b3.
-// Training: mini-batch squared error (1/2N) sum (f(x) - t)^2, gradient by these kernels (64-sample
-// tiles in shared memory, per-block partial gradients added with atomics), Adam update.
+// Training: mini-batch squared error (1/2N) sum (f(x) - t)^2, gradient by these kernels (32-sample
+// tiles, per-block gradients in registers added with atomics), Adam update in the next one's prologue.
 // Inference (march and tdcfie_mlp_predict) uses FP16 copies of the weights with FP32 arithmetic.
 #include <cuda_fp16.h>
 
@@ -15,103 +15,252 @@
 
 #include "gmres.h"
 #include "plan.h"
+#include "simt.h"
 
 namespace tdc {
 
 constexpr int NIN = 8, NH = 64, NP = 4801;
 constexpr int OW1 = 0, OB1 = 512, OW2 = 576, OB2 = 4672, OW3 = 4736, OB3 = 4800;
-constexpr int TS = 64;   // samples per training tile
+// ---------------------------------------------------------------- gradient
+// A block takes tiles of TS samples; its 256 threads hold the whole gradient in registers (19 parameters
+// each) and add it to the global one once.  Latency bounds it (a batch of 4096 samples is 60 M
+// multiply-adds), so every product is tiled in registers from shared memory with the operands in the
+// order that gives 16-byte loads: H1 and D2 in both orders, W2 too.  An update of 4096 samples: 17 us; 69 us
+// with one output per thread, a block per tile and Adam in a kernel of its own.
+constexpr int TS = 32;        // samples per tile
+constexpr int GT = 256;       // threads per block
+struct GradSh {      // every array's size is a multiple of 16 bytes
+    float W1[NH][NIN], b1[NH], b2[NH], w3[NH], b3[4];
+    float W2[NH][NH], W2t[NH][NH + 4];      // [i][j], [j][i]; padded against bank conflicts of the stores
+    float X[TS][NIN];
+    float H1[TS][NH], H1t[NH][TS + 2];      // [s][j], [j][s]
+    float H2[TS][NH];
+    float D2[TS][NH], D2t[NH][TS + 2];      // [s][i], [i][s]
+    float D1[TS][NH];
+    float o[TS], dv[TS];
+};
 
-// dynamic shared memory of k_mlp_grad (floats): params, X tile, H1, H2, dZ2, dZ1, d
-constexpr int GRAD_SMEM = (NP + 3) / 4 * 4 + TS * NIN + 4 * TS * NH + TS;
-
-__global__ void k_mlp_grad(const float* __restrict__ prm, const float* __restrict__ X, const float* __restrict__ Y,
-                           int64_t n, int64_t off, int64_t count, float inv_total, float* __restrict__ grad,
-                           float* __restrict__ loss) {
-    extern __shared__ float sm[];
-    float* P = sm;
-    float* Xs = P + (NP + 3) / 4 * 4;
-    float* H1 = Xs + TS * NIN;
-    float* H2 = H1 + TS * NH;
-    float* D2 = H2 + TS * NH;
-    float* D1 = D2 + TS * NH;
-    float* dv = D1 + TS * NH;
-    const int t = threadIdx.x;
-    for (int i = t; i < NP; i += blockDim.x) P[i] = prm[i];
-    const int64_t base = (int64_t)blockIdx.x * TS;
-    for (int i = t; i < TS * NIN; i += blockDim.x) {
-        const int64_t s = base + i / NIN;
-        Xs[i] = s < count ? X[((off + s) % n) * NIN + i % NIN] : 0.f;
-    }
-    __syncthreads();
-    for (int e = t; e < TS * NH; e += blockDim.x) {
-        const int s = e / NH, i = e % NH;
-        float z = P[OB1 + i];
-        for (int k = 0; k < NIN; ++k) z += P[OW1 + i * NIN + k] * Xs[s * NIN + k];
-        H1[e] = tanhf(z);
-    }
-    __syncthreads();
-    for (int e = t; e < TS * NH; e += blockDim.x) {
-        const int s = e / NH, i = e % NH;
-        float z = P[OB2 + i];
-        for (int j = 0; j < NH; ++j) z += P[OW2 + i * NH + j] * H1[s * NH + j];
-        H2[e] = tanhf(z);
-    }
-    __syncthreads();
-    if (t < TS) {
-        const int64_t s = base + t;
-        float o = P[OB3];
-        for (int i = 0; i < NH; ++i) o += P[OW3 + i] * H2[t * NH + i];
-        const float r = s < count ? o - Y[(off + s) % n] : 0.f;
-        dv[t] = r * inv_total;
-        atomicAdd(loss, 0.5f * r * r * inv_total);
-    }
-    __syncthreads();
-    for (int e = t; e < TS * NH; e += blockDim.x) {
-        const int s = e / NH, i = e % NH;
-        D2[e] = dv[s] * P[OW3 + i] * (1.f - H2[e] * H2[e]);
-    }
-    __syncthreads();
-    for (int e = t; e < TS * NH; e += blockDim.x) {
-        const int s = e / NH, j = e % NH;
-        float a = 0.f;
-        for (int i = 0; i < NH; ++i) a += D2[s * NH + i] * P[OW2 + i * NH + j];
-        D1[e] = a * (1.f - H1[e] * H1[e]);
-    }
-    __syncthreads();
-    // block partial gradients
-    for (int q = t; q < NP; q += blockDim.x) {
-        float a = 0.f;
-        if (q < OB1) {            // W1[i][k]
-            const int i = q / NIN, k = q % NIN;
-            for (int s = 0; s < TS; ++s) a += D1[s * NH + i] * Xs[s * NIN + k];
-        } else if (q < OW2) {     // b1
-            const int i = q - OB1;
-            for (int s = 0; s < TS; ++s) a += D1[s * NH + i];
-        } else if (q < OB2) {     // W2[i][j]
-            const int i = (q - OW2) / NH, j = (q - OW2) % NH;
-            for (int s = 0; s < TS; ++s) a += D2[s * NH + i] * H1[s * NH + j];
-        } else if (q < OW3) {     // b2
-            const int i = q - OB2;
-            for (int s = 0; s < TS; ++s) a += D2[s * NH + i];
-        } else if (q < OB3) {     // W3
-            const int i = q - OW3;
-            for (int s = 0; s < TS; ++s) a += dv[s] * H2[s * NH + i];
-        } else {                  // b3
-            for (int s = 0; s < TS; ++s) a += dv[s];
-        }
-        atomicAdd(grad + q, a);
-    }
+// parameters 4 q .. 4 q + 3 of the flat order into shared memory (a quad lies in one array)
+constexpr int NQ = (NP + 3) / 4, NPS = 4 * NQ;      // quads, and the stride of a padded vector
+__device__ __forceinline__ void put_quad(GradSh& sh, int q, float4 v) {
+    q *= 4;
+    if (q < OB1) *reinterpret_cast<float4*>(&sh.W1[q / NIN][q % NIN]) = v;
+    else if (q < OW2) *reinterpret_cast<float4*>(&sh.b1[q - OB1]) = v;
+    else if (q < OB2) {
+        const int i = (q - OW2) / NH, j = (q - OW2) % NH;
+        *reinterpret_cast<float4*>(&sh.W2[i][j]) = v;
+        sh.W2t[j][i] = v.x;
+        sh.W2t[j + 1][i] = v.y;
+        sh.W2t[j + 2][i] = v.z;
+        sh.W2t[j + 3][i] = v.w;
+    } else if (q < OW3) *reinterpret_cast<float4*>(&sh.b2[q - OB2]) = v;
+    else if (q < OB3) *reinterpret_cast<float4*>(&sh.w3[q - OW3]) = v;
+    else sh.b3[0] = v.x;
 }
 
-__global__ void k_mlp_adam(float* __restrict__ prm, const float* __restrict__ grad, float* __restrict__ m1,
-                           float* __restrict__ m2, float lr, float b1, float b2, float eps, float c1, float c2) {
+// This thread's entry of a tile's inputs, and of its targets (first TS threads)
+struct TileIn { float x, y; };
+__device__ __forceinline__ TileIn tile_in(const float* __restrict__ X, const float* __restrict__ Y, int64_t n, int64_t off,
+                                          int64_t count, int64_t base) {
+    const int t = threadIdx.x;
+    TileIn in{0.f, 0.f};
+    auto at = [&](int64_t q) { return off + q < n ? off + q : off + q - n; };      // off < n, count <= n
+    if (base + (t >> 3) < count) in.x = X[at(base + (t >> 3)) * NIN + (t & 7)];
+    if (t < TS && base + t < count) in.y = Y[at(base + t)];
+    return in;
+}
+
+// The gradient (added to grad) and the loss of samples off .. off + count - 1 (modulo n) with the
+// parameters in sh; all blocks share the tiles; `in` is this block's first.  VEC: grad is 16-byte aligned
+template <bool VEC>
+__device__ __forceinline__ void grad_tiles(GradSh& sh, TileIn in, const float* __restrict__ X, const float* __restrict__ Y,
+                                           int64_t n, int64_t off, int64_t count, float inv_total, float* grad, float* loss) {
+    const int t = threadIdx.x;
+    float g2[4][4] = {}, g1[2] = {}, gb = 0.f, g3 = 0.f;      // W2 tile, W1 pair, b1 | b2 | w3, b3
+    const int gi = (t >> 4) * 4, gj = (t & 15) * 4;                      // W2 rows gi.., columns gj..
+    for (int64_t base = (int64_t)blockIdx.x * TS; base < count; base += (int64_t)gridDim.x * TS) {
+        __syncthreads();      // the parameters are there, the tile before is done with
+        sh.X[t >> 3][t & 7] = in.x;
+        const float y = in.y;
+        if (base + (int64_t)gridDim.x * TS < count) in = tile_in(X, Y, n, off, count, base + (int64_t)gridDim.x * TS);
+        __syncthreads();
+        {      // H1: one unit per thread, eight samples
+            const int i = t & (NH - 1);
+            const float4 wa = *reinterpret_cast<const float4*>(&sh.W1[i][0]), wb = *reinterpret_cast<const float4*>(&sh.W1[i][4]);
+            const float bi = sh.b1[i];
+#pragma unroll
+            for (int u = 0; u < TS * NH / GT; ++u) {
+                const int s = (t >> 6) + u * (GT / NH);
+                const float4 xa = *reinterpret_cast<const float4*>(&sh.X[s][0]), xb = *reinterpret_cast<const float4*>(&sh.X[s][4]);
+                float z = fmaf(wa.x, xa.x, bi);
+                z = fmaf(wa.y, xa.y, z); z = fmaf(wa.z, xa.z, z); z = fmaf(wa.w, xa.w, z);
+                z = fmaf(wb.x, xb.x, z); z = fmaf(wb.y, xb.y, z); z = fmaf(wb.z, xb.z, z); z = fmaf(wb.w, xb.w, z);
+                const float h = tanhf(z);
+                sh.H1[s][i] = h;
+                sh.H1t[i][s] = h;
+            }
+        }
+        __syncthreads();
+        const int s0 = (t >> 4) * 2, i0 = (t & 15) * 4;      // two samples, four units
+        {
+            float z[2][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) z[0][u] = z[1][u] = sh.b2[i0 + u];
+#pragma unroll 8
+            for (int j = 0; j < NH; ++j) {
+                const float4 w = *reinterpret_cast<const float4*>(&sh.W2t[j][i0]);
+                const float2 h = *reinterpret_cast<const float2*>(&sh.H1t[j][s0]);
+                z[0][0] = fmaf(w.x, h.x, z[0][0]); z[0][1] = fmaf(w.y, h.x, z[0][1]);
+                z[0][2] = fmaf(w.z, h.x, z[0][2]); z[0][3] = fmaf(w.w, h.x, z[0][3]);
+                z[1][0] = fmaf(w.x, h.y, z[1][0]); z[1][1] = fmaf(w.y, h.y, z[1][1]);
+                z[1][2] = fmaf(w.z, h.y, z[1][2]); z[1][3] = fmaf(w.w, h.y, z[1][3]);
+            }
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                float o = 0.f;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    z[a][u] = tanhf(z[a][u]);
+                    o = fmaf(sh.w3[i0 + u], z[a][u], o);
+                }
+                *reinterpret_cast<float4*>(&sh.H2[s0 + a][i0]) = make_float4(z[a][0], z[a][1], z[a][2], z[a][3]);
+                for (int k = 8; k > 0; k >>= 1) o += __shfl_xor_sync(0xffffffffu, o, k);      // over the 16 lanes of a sample
+                if ((t & 15) == 0) sh.o[s0 + a] = o;
+            }
+        }
+        __syncthreads();
+        if (t < TS) {
+            const float r = base + t < count ? sh.o[t] + sh.b3[0] - y : 0.f;
+            sh.dv[t] = r * inv_total;
+            atomicAdd(loss, 0.5f * r * r * inv_total);
+        }
+        __syncthreads();
+        for (int e = t; e < TS * NH; e += GT) {
+            const int s = e / NH, i = e % NH;
+            const float h = sh.H2[s][i], d = sh.dv[s] * sh.w3[i] * (1.f - h * h);
+            sh.D2[s][i] = d;
+            sh.D2t[i][s] = d;
+        }
+        __syncthreads();
+        {
+            float a0[4] = {}, a1[4] = {};
+#pragma unroll 8
+            for (int i = 0; i < NH; ++i) {
+                const float4 w = *reinterpret_cast<const float4*>(&sh.W2[i][i0]);
+                const float2 d = *reinterpret_cast<const float2*>(&sh.D2t[i][s0]);
+                a0[0] = fmaf(w.x, d.x, a0[0]); a0[1] = fmaf(w.y, d.x, a0[1]); a0[2] = fmaf(w.z, d.x, a0[2]); a0[3] = fmaf(w.w, d.x, a0[3]);
+                a1[0] = fmaf(w.x, d.y, a1[0]); a1[1] = fmaf(w.y, d.y, a1[1]); a1[2] = fmaf(w.z, d.y, a1[2]); a1[3] = fmaf(w.w, d.y, a1[3]);
+            }
+            const float4 h0 = *reinterpret_cast<const float4*>(&sh.H1[s0][i0]);
+            const float4 h1 = *reinterpret_cast<const float4*>(&sh.H1[s0 + 1][i0]);
+            *reinterpret_cast<float4*>(&sh.D1[s0][i0]) =
+                make_float4(a0[0] * (1.f - h0.x * h0.x), a0[1] * (1.f - h0.y * h0.y), a0[2] * (1.f - h0.z * h0.z),
+                            a0[3] * (1.f - h0.w * h0.w));
+            *reinterpret_cast<float4*>(&sh.D1[s0 + 1][i0]) =
+                make_float4(a1[0] * (1.f - h1.x * h1.x), a1[1] * (1.f - h1.y * h1.y), a1[2] * (1.f - h1.z * h1.z),
+                            a1[3] * (1.f - h1.w * h1.w));
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int s = 0; s < TS; ++s) {
+            const float4 d = *reinterpret_cast<const float4*>(&sh.D2[s][gi]);
+            const float4 h = *reinterpret_cast<const float4*>(&sh.H1[s][gj]);
+            const float dd[4] = {d.x, d.y, d.z, d.w}, hh[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) g2[a][b] = fmaf(dd[a], hh[b], g2[a][b]);
+            // W1[i][k], i = t / 4, k = 2 (t % 4) + {0, 1}
+            const float d1 = sh.D1[s][t >> 2];
+            const float2 x = *reinterpret_cast<const float2*>(&sh.X[s][2 * (t & 3)]);
+            g1[0] = fmaf(d1, x.x, g1[0]);
+            g1[1] = fmaf(d1, x.y, g1[1]);
+            gb += t < NH ? sh.D1[s][t] : t < 2 * NH ? sh.D2[s][t - NH] : t < 3 * NH ? sh.dv[s] * sh.H2[s][t - 2 * NH] : 0.f;
+            if (t == GT - 1) g3 += sh.dv[s];
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        float* p = grad + OW2 + (gi + a) * NH + gj;
+        if constexpr (VEC) atomicAdd(reinterpret_cast<float4*>(p), make_float4(g2[a][0], g2[a][1], g2[a][2], g2[a][3]));
+        else
+#pragma unroll
+            for (int b = 0; b < 4; ++b) atomicAdd(p + b, g2[a][b]);
+    }
+    atomicAdd(grad + OW1 + (t >> 2) * NIN + 2 * (t & 3), g1[0]);
+    atomicAdd(grad + OW1 + (t >> 2) * NIN + 2 * (t & 3) + 1, g1[1]);
+    if (t < 3 * NH) atomicAdd(grad + (t < NH ? OB1 + t : t < 2 * NH ? OB2 + t - NH : OW3 + t - 2 * NH), gb);
+    if (t == GT - 1) atomicAdd(grad + OB3, g3);
+}
+
+__global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ prm, const float* __restrict__ X,
+                                                 const float* __restrict__ Y, int64_t n, float inv_total,
+                                                 float* __restrict__ grad, float* __restrict__ loss) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    GradSh& sh = *reinterpret_cast<GradSh*>(smem);
+    for (int q = threadIdx.x; q < NQ; q += GT)      // prm may have any alignment
+        put_quad(sh, q, 4 * q < OB3 ? make_float4(prm[4 * q], prm[4 * q + 1], prm[4 * q + 2], prm[4 * q + 3])
+                                    : make_float4(prm[OB3], 0.f, 0.f, 0.f));
+    grad_tiles<false>(sh, tile_in(X, Y, n, 0, n, (int64_t)blockIdx.x * TS), X, Y, n, 0, n, inv_total, grad, loss);
+}
+
+struct AdamStep { float lr, b1, b2, eps, c1, c2; };
+__device__ __forceinline__ float adam(const AdamStep& a, float p, float g, float& m1, float& m2) {
+    m1 = a.b1 * m1 + (1.f - a.b1) * g;
+    m2 = a.b2 * m2 + (1.f - a.b2) * g * g;
+    return p - a.lr * (m1 / a.c1) / (sqrtf(m2 / a.c2) + a.eps);
+}
+
+// One training update in one kernel: every block forms the parameters after the update before (from
+// that update's gradient; block 0 keeps them and the moments for the next kernel in the other of two
+// slots), then adds its samples' gradient to this update's buffer, one of three in turn (block 0 clears
+// the next one's).  Slot layout: params, m1, m2, each padded to NPS.
+struct TrainStep {
+    const float* cur;      // state before the update in front (this kernel's, if there is none)
+    float* next;
+    const float* gprev;    // its gradient (nullptr: none yet)
+    float* grad;
+    float* gclear;
+    float* loss;
+    AdamStep a;
+    int64_t n, off, count;
+};
+__global__ void __launch_bounds__(GT) k_mlp_step(const __grid_constant__ TrainStep ts, const float* __restrict__ X,
+                                                 const float* __restrict__ Y) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    GradSh& sh = *reinterpret_cast<GradSh*>(smem);
+    // the samples are the caller's: no kernel of the chain writes them
+    const TileIn in = tile_in(X, Y, ts.n, ts.off, ts.count, (int64_t)blockIdx.x * TS);
+    wait_prior();
+    const float4* cur = reinterpret_cast<const float4*>(ts.cur);
+    for (int q = threadIdx.x; q < NQ; q += GT) {
+        float4 p = cur[q];
+        if (ts.gprev) {
+            float4 m1 = cur[NQ + q], m2 = cur[2 * NQ + q];
+            const float4 g = reinterpret_cast<const float4*>(ts.gprev)[q];
+            p.x = adam(ts.a, p.x, g.x, m1.x, m2.x);
+            p.y = adam(ts.a, p.y, g.y, m1.y, m2.y);
+            p.z = adam(ts.a, p.z, g.z, m1.z, m2.z);
+            p.w = adam(ts.a, p.w, g.w, m1.w, m2.w);
+            if (blockIdx.x == 0) {
+                float4* next = reinterpret_cast<float4*>(ts.next);
+                next[q] = p;
+                next[NQ + q] = m1;
+                next[2 * NQ + q] = m2;
+            }
+        }
+        if (blockIdx.x == 0) reinterpret_cast<float4*>(ts.gclear)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        put_quad(sh, q, p);
+    }
+    grad_tiles<true>(sh, in, X, Y, ts.n, ts.off, ts.count, 1.f / (float)ts.count, ts.grad, ts.loss);
+}
+// the last update, into the caller's parameters
+__global__ void k_mlp_last(const float* cur, const float* g, AdamStep a, float* prm) {
+    wait_prior();
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= NP) return;
-    const float g = grad[q];
-    m1[q] = b1 * m1[q] + (1.f - b1) * g;
-    m2[q] = b2 * m2[q] + (1.f - b2) * g * g;
-    prm[q] -= lr * (m1[q] / c1) / (sqrtf(m2[q] / c2) + eps);
+    float m1 = cur[NPS + q], m2 = cur[2 * NPS + q];
+    prm[q] = adam(a, cur[q], g[q], m1, m2);
 }
 
 __global__ void k_to_half(const float* __restrict__ a, __half* __restrict__ b, int n) {
@@ -287,17 +436,12 @@ cudaError_t mlp_load(StepPlan* p, const float* host_params, cudaStream_t s) {
 
 using namespace tdc;
 
-static tdcfie_status launch_grad(const float* params, const float* X, const float* Y, int64_t n, int64_t off,
-                                 int64_t count, float* grad, float* loss, cudaStream_t s) {
-    // set on every call: the attribute is per device, and the call is cheap next to a training step
-    const cudaError_t ea = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                GRAD_SMEM * (int)sizeof(float));
-    if (ea != cudaSuccess) return cuda_fail(nullptr, ea, "cudaFuncSetAttribute (MLP gradient)");
-    const unsigned blocks = (unsigned)((count + TS - 1) / TS);
-    k_mlp_grad<<<blocks, 256, GRAD_SMEM * sizeof(float), s>>>(params, X, Y, n, off, count, 1.f / (float)count, grad,
-                                                              loss);
-    const cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? TDCFIE_OK : cuda_fail(nullptr, e, "MLP gradient launch");
+// blocks of a gradient over `count` samples: two per SM at most (they share the tiles)
+static int grad_blocks(int64_t count) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        sms = 148;
+    return (int)std::min<int64_t>((count + TS - 1) / TS, 2 * sms);
 }
 
 extern "C" tdcfie_status tdcfie_mlp_grad(const float* params, const float* X, const float* Y, int64_t n, float* grad,
@@ -305,10 +449,15 @@ extern "C" tdcfie_status tdcfie_mlp_grad(const float* params, const float* X, co
     if (!params || !X || !Y || !grad || !loss) return fail(nullptr, TDCFIE_E_ARG, "NULL device pointer");
     if (n < 1) return fail(nullptr, TDCFIE_E_ARG, "n must be >= 1");
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(grad, 0, sizeof(float) * NP, s);
+    // the attribute is set on every call: it is per device
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSh));
+    if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaFuncSetAttribute (MLP gradient)");
+    e = cudaMemsetAsync(grad, 0, sizeof(float) * NP, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(loss, 0, sizeof(float), s);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaMemsetAsync");
-    return launch_grad(params, X, Y, n, 0, n, grad, loss, s);
+    k_mlp_grad<<<grad_blocks(n), GT, sizeof(GradSh), s>>>(params, X, Y, n, 1.f / (float)n, grad, loss);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? TDCFIE_OK : cuda_fail(nullptr, e, "MLP gradient launch");
 }
 
 extern "C" tdcfie_status tdcfie_mlp_train(float* params, const float* X, const float* Y, int64_t n, int epochs,
@@ -316,34 +465,58 @@ extern "C" tdcfie_status tdcfie_mlp_train(float* params, const float* X, const f
     if (!params || !X || !Y) return fail(nullptr, TDCFIE_E_ARG, "NULL device pointer");
     if (n < 1 || epochs < 1 || batch < 1 || !(lr > 0.f)) return fail(nullptr, TDCFIE_E_ARG, "bad training sizes");
     cudaStream_t s = (cudaStream_t)stream;
-    float* buf = nullptr;   // grad, m1, m2, loss
-    cudaError_t e = cudaMallocAsync((void**)&buf, sizeof(float) * (3 * NP + 1), s);
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSh));
+    if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaFuncSetAttribute (MLP training)");
+    // two states (params, m1, m2), three gradients, the passes' losses
+    float* buf = nullptr;
+    const size_t bytes = sizeof(float) * (9 * (size_t)NPS + epochs);
+    e = cudaMallocAsync((void**)&buf, bytes, s);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaMallocAsync (MLP training state)");
-    float *grad = buf, *m1 = buf + NP, *m2 = buf + 2 * NP, *loss = buf + 3 * NP;
-    cudaMemsetAsync(buf, 0, sizeof(float) * (3 * NP + 1), s);
+    float* state[2] = {buf, buf + 3 * NPS};
+    float* grad = buf + 6 * NPS;
+    float* loss = buf + 9 * NPS;
+    e = cudaMemsetAsync(buf, 0, bytes, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(state[0], params, sizeof(float) * NP, cudaMemcpyDeviceToDevice, s);
     std::mt19937_64 rng(seed);
     const int64_t nb = (n + batch - 1) / batch;
     int64_t step = 0;
-    tdcfie_status st = TDCFIE_OK;
-    for (int ep = 0; ep < epochs && st == TDCFIE_OK; ++ep) {
+    TrainStep ts{};
+    ts.a = AdamStep{lr, 0.9f, 0.999f, 1e-8f, 1.f, 1.f};
+    ts.n = n;
+    auto corrections = [&](int64_t k) {      // of update k
+        ts.a.c1 = 1.f - std::pow(0.9f, (float)k);
+        ts.a.c2 = 1.f - std::pow(0.999f, (float)k);
+    };
+    const int blocks = grad_blocks(std::min(n, batch));
+    for (int ep = 0; ep < epochs && e == cudaSuccess; ++ep) {
         const int64_t rot = (int64_t)(rng() % (uint64_t)n);   // per-epoch rotation of the batch origin
-        cudaMemsetAsync(loss, 0, sizeof(float), s);
-        for (int64_t b = 0; b < nb && st == TDCFIE_OK; ++b) {
-            const int64_t off = (rot + b * batch) % n;
-            const int64_t cnt = std::min<int64_t>(batch, n - b * batch);
-            cudaMemsetAsync(grad, 0, sizeof(float) * NP, s);
-            st = launch_grad(params, X, Y, n, off, cnt, grad, loss, s);
-            ++step;
-            const float c1 = 1.f - std::pow(0.9f, (float)step), c2 = 1.f - std::pow(0.999f, (float)step);
-            k_mlp_adam<<<(NP + 255) / 256, 256, 0, s>>>(params, grad, m1, m2, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
+        for (int64_t b = 0; b < nb && e == cudaSuccess; ++b, ++step) {
+            // kernel `step` (from 0): state after step - 1 updates in slot (step + 1) & 1, from step 2 on
+            ts.off = (rot + b * batch) % n;
+            ts.count = std::min<int64_t>(batch, n - b * batch);
+            ts.cur = state[step < 2 ? 0 : (step - 1) & 1];
+            ts.next = state[step & 1];
+            ts.gprev = step ? grad + (step - 1) % 3 * NPS : nullptr;
+            ts.grad = grad + step % 3 * NPS;
+            ts.gclear = grad + (step + 1) % 3 * NPS;
+            ts.loss = loss + ep;
+            corrections(step);
+            launch_chained(k_mlp_step, blocks, GT, s, sizeof(GradSh), ts, X, Y);
+            e = cudaGetLastError();
         }
-        if (loss_history && st == TDCFIE_OK) {
-            float l = 0.f;
-            e = cudaMemcpyAsync(&l, loss, sizeof(float), cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            if (e != cudaSuccess) st = cuda_fail(nullptr, e, "MLP loss readback");
-            loss_history[ep] = l / (float)nb;
-        }
+    }
+    if (e == cudaSuccess) {
+        corrections(step);
+        launch_chained(k_mlp_last, (NP + 255) / 256, 256, s, 0, (const float*)state[step < 2 ? 0 : (step - 1) & 1],
+                       (const float*)(grad + (step - 1) % 3 * NPS), ts.a, params);
+        e = cudaGetLastError();
+    }
+    tdcfie_status st = e == cudaSuccess ? TDCFIE_OK : cuda_fail(nullptr, e, "MLP training launch");
+    if (loss_history && st == TDCFIE_OK) {
+        e = cudaMemcpyAsync(loss_history, loss, sizeof(float) * epochs, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) st = cuda_fail(nullptr, e, "MLP loss readback");
+        for (int ep = 0; ep < epochs; ++ep) loss_history[ep] /= (float)nb;
     }
     cudaFreeAsync(buf, s);
     return st;
