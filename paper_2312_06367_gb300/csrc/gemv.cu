@@ -1,60 +1,100 @@
 // Stand-alone history sum of the MOT recurrence (Sec. IV-B) on caller-held blocks:
 //   out[r][i] = sum_{q < nblk} sum_{j < n} blocks[q][i][j] x[q][r][j]
-// One warp per (row i, block q) writes the per-block partial sums; a second kernel adds the
+// A warp writes the per-block partial sums of a few rows of one block; a second kernel adds the
 // blocks in a fixed order (deterministic result).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <mutex>
 
-#include "internal.h"
+#include "simt.h"
 
 namespace tdc {
 
-template <typename T, int RMAX>
-__global__ void k_bg_partial(const T* __restrict__ blocks, int64_t nblk, int64_t n, const T* __restrict__ x, int R,
-                             T* __restrict__ partial) {
-    const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+// Streams the matrices once: bound by the memory.  A warp takes BG_ROWS rows, so that a value of x is
+// fetched once for all of them (with one row per warp the fetches of x at R = 8 took eight times the
+// matrix's), and keeps that many 16-byte loads in flight per turn.  41 blocks of 7680 rows, R = 1, FP32:
+// 1356 us (7.13 TB/s); 1614 us with 4-byte loads.
+template <typename T> struct Vec16;
+template <> struct Vec16<float> { using V = float4; };
+template <> struct Vec16<double> { using V = double2; };
+template <typename T> constexpr int BG_ROWS = sizeof(T) == 4 ? 4 : 2;
+
+// W: entries per load, 1 or (rows and pointers on 16-byte boundaries) a 16-byte vector
+template <typename T, int RMAX, int W>
+__global__ void __launch_bounds__(256) k_bg_partial(const T* __restrict__ blocks, int64_t n, const T* __restrict__ x, int R,
+                                                    T* __restrict__ partial) {
+    constexpr int NR = BG_ROWS<T>;
+    const int64_t row0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * NR;
     const int64_t q = blockIdx.y;
     const int lane = threadIdx.x & 31;
-    if (row >= n) return;
-    const T* a = blocks + (q * n + row) * n;
+    if (row0 >= n) return;
+    const T* a = blocks + (q * n + row0) * n;
     const T* xq = x + q * R * n;
-    T s[RMAX];
+    int64_t ro[NR];      // rows behind the last one read the last one
 #pragma unroll
-    for (int r = 0; r < RMAX; ++r) s[r] = 0;
-    for (int64_t j = lane; j < n; j += 32) {
-        const T v = a[j];
+    for (int i = 0; i < NR; ++i) ro[i] = (row0 + i < n ? i : n - 1 - row0) * n;
+    T s[NR][RMAX] = {};
+#pragma unroll(RMAX == 1 && W > 1 ? 4 : 2)
+    for (int64_t j = W * lane; j < n; j += 32 * W) {
+        T v[NR][W];
 #pragma unroll
-        for (int r = 0; r < RMAX; ++r)
-            if (r < R) s[r] += v * xq[(int64_t)r * n + j];
+        for (int i = 0; i < NR; ++i) {
+            if constexpr (W == 1) v[i][0] = __ldcs(a + ro[i] + j);
+            else *reinterpret_cast<typename Vec16<T>::V*>(v[i]) = __ldcs(reinterpret_cast<const typename Vec16<T>::V*>(a + ro[i] + j));
+        }
+#pragma unroll
+        for (int r = 0; r < RMAX; ++r) {
+            if (r >= R) break;
+            T u[W];
+            if constexpr (W == 1) u[0] = xq[r * n + j];
+            else *reinterpret_cast<typename Vec16<T>::V*>(u) = *reinterpret_cast<const typename Vec16<T>::V*>(xq + r * n + j);
+#pragma unroll
+            for (int i = 0; i < NR; ++i)
+#pragma unroll
+                for (int k = 0; k < W; ++k) s[i][r] += v[i][k] * u[k];
+        }
     }
 #pragma unroll
-    for (int r = 0; r < RMAX; ++r) {
-        T v = s[r];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0 && r < R) partial[(q * R + r) * n + row] = v;
-    }
+    for (int i = 0; i < NR; ++i)
+#pragma unroll
+        for (int r = 0; r < RMAX; ++r) {
+            T v = s[i][r];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0 && r < R && row0 + i < n) partial[(q * R + r) * n + row0 + i] = v;
+        }
 }
 
 template <typename T>
-__global__ void k_bg_reduce(const T* __restrict__ partial, int64_t nblk, int64_t n, int R, T* __restrict__ out) {
+__global__ void k_bg_reduce(const T* partial, int64_t nblk, int64_t n, int R, T* out) {
+    wait_prior();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n * R) return;
     T s = 0;
-    for (int64_t q = 0; q < nblk; ++q) s += partial[q * R * n + i];
+#pragma unroll 8
+    for (int64_t q = 0; q < nblk; ++q) s += __ldcg(partial + q * R * n + i);
     out[i] = s;
+}
+
+template <typename T, int RMAX>
+static void launch_bg_partial(const T* blocks, int64_t nblk, int64_t n, const T* x, int R, T* partial, cudaStream_t s) {
+    constexpr int W = 16 / (int)sizeof(T);
+    const int rows = 8 * BG_ROWS<T>;
+    const dim3 g((unsigned)((n + rows - 1) / rows), (unsigned)nblk);
+    if (n % W == 0 && (uintptr_t)blocks % 16 == 0 && (uintptr_t)x % 16 == 0)
+        k_bg_partial<T, RMAX, W><<<g, 256, 0, s>>>(blocks, n, x, R, partial);
+    else
+        k_bg_partial<T, RMAX, 1><<<g, 256, 0, s>>>(blocks, n, x, R, partial);
 }
 
 template <typename T>
 static cudaError_t launch_block_gemv(const T* blocks, int64_t nblk, int64_t n, const T* x, int R, T* out, T* partial,
                                      cudaStream_t s) {
-    const int wpb = 8;
-    const dim3 g((unsigned)((n + wpb - 1) / wpb), (unsigned)nblk);
-    if (R == 1) k_bg_partial<T, 1><<<g, 32 * wpb, 0, s>>>(blocks, nblk, n, x, R, partial);
-    else if (R <= 4) k_bg_partial<T, 4><<<g, 32 * wpb, 0, s>>>(blocks, nblk, n, x, R, partial);
-    else k_bg_partial<T, 8><<<g, 32 * wpb, 0, s>>>(blocks, nblk, n, x, R, partial);
-    k_bg_reduce<T><<<(unsigned)((n * R + 255) / 256), 256, 0, s>>>(partial, nblk, n, R, out);
+    if (R == 1) launch_bg_partial<T, 1>(blocks, nblk, n, x, R, partial, s);
+    else if (R == 2) launch_bg_partial<T, 2>(blocks, nblk, n, x, R, partial, s);
+    else if (R <= 4) launch_bg_partial<T, 4>(blocks, nblk, n, x, R, partial, s);
+    else launch_bg_partial<T, 8>(blocks, nblk, n, x, R, partial, s);
+    launch_chained(k_bg_reduce<T>, (unsigned)((n * R + 63) / 64), 64, s, 0, (const T*)partial, nblk, n, R, out);
     return cudaGetLastError();
 }
 
