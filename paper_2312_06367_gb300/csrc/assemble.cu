@@ -123,7 +123,7 @@ __device__ __forceinline__ double atanh_half(double w) {
 }
 
 // nodes of one radial piece with centre (rc, Rc) = |d| (sinh, cosh)(u_c) and half-width h in u:
-// acc.node(R, W / R, rho), W = cw h w_g rho R
+// acc.node(R, W / R, rho) (node2: two at a time), W = cw h w_g rho R
 template <class ACC>
 __device__ __forceinline__ void radial_nodes(double rc, double Rc, double h, double cw, ACC& acc) {
     static_assert(NRAD == 5, "symmetric five-point rule");
@@ -134,8 +134,7 @@ __device__ __forceinline__ void radial_nodes(double rc, double Rc, double h, dou
         double C, S;
         cosh_sinh(h * c_rx[g], C, S);
         const double a = rc * C, b = Rc * S, e = Rc * C, f = rc * S, w = ch * c_rw[g];
-        acc.node(e + f, w * (a + b), a + b);
-        acc.node(e - f, w * (a - b), a - b);
+        acc.node2(e + f, w * (a + b), a + b, e - f, w * (a - b), a - b);
     }
 }
 
@@ -280,11 +279,17 @@ __device__ __noinline__ void work_item(const BlockSh& sh, double* slots, int e, 
         const int j0 = sh.j0[e], j1 = j0 + st.ni;
         int j = max((int)(R0min * st.inv_dt), j0);
         double Ra = j * st.dt, ra = sqrt(fmax(fma(Ra, Ra, -d2), 0.0));
+        // the intervals at the near edge, those that all rays cross whole, the rest: a warp's lanes meet
+        // between the three, so that one ray's work is not done beside six rays'
+#pragma unroll 1
+        for (int ph = 0; ph < 3; ++ph)
 #pragma unroll 1
         for (; j < j1 && Ra < R1max; ++j) {
-            const double Rb = (j + 1) * st.dt, rb = sqrt(fmax(fma(Rb, Rb, -d2), 0.0)), Rs = fmax(Ra, ad);
-            acc.begin(j, st);
+            const double Rb = (j + 1) * st.dt;
             const bool whole = Rb <= R1min && (hn == 0.0 || R0max <= Ra);
+            if (ph < 2 && whole != (ph == 1)) break;
+            const double rb = sqrt(fmax(fma(Rb, Rb, -d2), 0.0)), Rs = fmax(Ra, ad);
+            acc.begin(j, st);
 #pragma unroll 1
             for (int k = 0; k < (whole ? 1 : 6); ++k) {
                 const bool in = !whole && R0[k] > Rs, out = !whole && R1[k] < Rb;
@@ -543,6 +548,10 @@ struct EfieAcc {
         r[0] = fma(Wr, rho, r[0]);
         if constexpr (NV == 2) r[1] = fma(Wr * rho, x, r[1]);
     }
+    __device__ __forceinline__ void node2(double Ra, double Wa, double rhoa, double Rb, double Wb, double rhob) {
+        node(Ra, Wa, rhoa);
+        node(Rb, Wb, rhob);
+    }
     __device__ __forceinline__ void turn(V3 om) {
 #pragma unroll
         for (int p = 0; p < NV; ++p) v[p] = v[p] + r[p] * om;
@@ -685,14 +694,20 @@ struct MfieAcc {
 #pragma unroll
         for (int p = 0; p < NB; ++p) r[p] = 0.0;
     }
-    __device__ __forceinline__ void node(double R, double Wr, double rho) {
-        double t = Wr / (R * R);
+    __device__ __forceinline__ void add(double R, double t, double rho) {
 #pragma unroll
         for (int p = 0; p < NB; ++p) {
             if (p) t *= fma(-R, inv_dt, jp);
             c[p] += t;
             r[p] = fma(t, rho, r[p]);
         }
+    }
+    __device__ __forceinline__ void node(double R, double Wr, double rho) { add(R, Wr / (R * R), rho); }
+    // one division for two nodes
+    __device__ __forceinline__ void node2(double Ra, double Wa, double rhoa, double Rb, double Wb, double rhob) {
+        const double qa = Ra * Ra, qb = Rb * Rb, inv = 1.0 / (qa * qb);
+        add(Ra, Wa * (qb * inv), rhoa);
+        add(Rb, Wb * (qa * inv), rhob);
     }
     __device__ __forceinline__ void turn(V3 om) {
 #pragma unroll
@@ -813,6 +828,10 @@ struct YukAcc {
         if constexpr (M) g *= fma(kappa, R, 1.0) / (R * R);
         c += g;
         r = fma(g, rho, r);
+    }
+    __device__ __forceinline__ void node2(double Ra, double Wa, double rhoa, double Rb, double Wb, double rhob) {
+        node(Ra, Wa, rhoa);
+        node(Rb, Wb, rhob);
     }
     __device__ __forceinline__ void turn(V3 om) { v = v + r * om; }
     __device__ __forceinline__ void flush(double* slot) const {
