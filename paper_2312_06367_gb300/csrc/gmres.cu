@@ -4,11 +4,13 @@
 //   cycle:   Arnoldi with the path-precision T_0 (FP32 or FP64 matvec), classical Gram-Schmidt
 //            applied twice (CGS2) in FP64, Givens rotations, up to m iterations or until the
 //            residual estimate drops below max(inner_tol beta, tol ||b|| / 2); then x += V_m y.
-// Each right-hand side runs its own state machine (residual -> Arnoldi iterations -> update ->
-// residual ...).  One pass of the loop body advances every open right-hand side by one Arnoldi
-// iteration (plus, where due, its restart or update); the body sits in a CUDA-graph WHILE node whose
-// condition the last kernel of the pass clears once every right-hand side has converged or given up
-// (a pass cap bounds the loop).  No kernel waits on another.
+// One cooperative kernel per step solves all right-hand sides, each by a group of co-resident blocks
+// of its own (grid.y) that hold the rows in equal shares.  A group meets at three barriers per Arnoldi
+// iteration (projections, their repetition, norm) and two per restart; between barriers a block only
+// touches its rows, and what the group sums passes through one partial per block, added by every
+// block in the same order: the Hessenberg column, the rotations and every decision are formed by all
+// blocks alike, and the results do not depend on timing.  Latency bounds it; 100 steps at 768 unknowns,
+// FP32, took 46.3 ms with an iteration as seven kernels in a graph loop, 23.9 ms so.
 #include <cmath>
 
 #include "gmres.h"
@@ -17,305 +19,324 @@
 
 namespace tdc {
 
-enum { F_DONE = 0, F_ST = 1, F_J = 2, F_ITERS = 3, NFLAGS = 4 };     // per right-hand side
-enum { ST_ARN = 0, ST_RESID = 1, ST_UPD = 2 };                         // F_ST
-enum { DONE_OPEN = 0, DONE_CONV = 1, DONE_GAVEUP = 2 };                // F_DONE
-enum { S_BN2 = 0, S_RN2 = 1, S_WN2 = 2, S_BETA = 3, S_HN = 4, NSCAL = 6 };
 // stats: [0] Arnoldi iterations this march, [1] steps, [2] max per step, [3] this step,
-//        [4] solves not converged, [5] loop passes this march, [6] passes this step
+//        [4] solves not converged, [5] groups done this step
 enum { NSTATS = 8 };
-constexpr int MV_WPB = 16;   // rows (warps) per block of the Arnoldi matvec
+constexpr int GM_T = 512, GM_W = GM_T / 32;       // threads and warps per block
+constexpr int GM_ROWS = 8;                        // rows per block, or more where the chip is full
+constexpr int GM_TILE = 8192;                     // entries of a vector staged at a time
 
 struct GmDev {
-    int R, ne, ld, m, maxit, pass_cap;     // ld: row length of the step's vectors (b, ring, guess)
+    int R, ne, ld, m, maxit;
+    int G, rpb, wpr;       // blocks per right-hand side, rows per block, warps per row of a product
+    int tile;              // doubles of the staging buffer
     double tol, inner_tol;
-    double *x, *r, *V, *w, *hdot, *H, *cs, *sn, *g, *yv, *scal;
-    int* flags;
+    double *x, *r, *V, *w, *H, *part;      // part: per right-hand side (2 (m + 1) + 2) x G
+    unsigned long long* sync;              // per right-hand side: arrivals so far; behind them: a wait ran out
     unsigned long long* stats;
 };
 
-__device__ __forceinline__ int fl(const GmDev& d, int r, int f) { return d.flags[r * NFLAGS + f]; }
-__device__ __forceinline__ bool arnoldi(const GmDev& d, int r) {
-    return fl(d, r, F_DONE) == DONE_OPEN && fl(d, r, F_ST) == ST_ARN;
-}
-
-// x = initial guess; ||b||^2; state reset; H cleared.  mode 0: zero, 1: y_{n-1} (ring slot
-// (n-1) % ring), 2 and 4: the learned guess buffer, 3: cubic extrapolation of y_{n-1..n-4}
-// (y_i = 0 for i <= 0)
-template <typename T>
-__global__ void k_gm_init(GmDev d, const T* __restrict__ b, int mode, const T* __restrict__ ringbuf, int ring,
-                          const T* __restrict__ learned, const Ctl* ctl) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = blockIdx.y;
-    const int64_t n = ctl->n;
-    const T* guess = nullptr;
-    if (mode == 1 && n > 1) guess = ringbuf + ((n - 1) % ring) * (int64_t)d.R * d.ld;
-    if ((mode == 2 || mode == 4) && n > 1) guess = learned;
-    if (i == 0) {
-        d.flags[r * NFLAGS + F_DONE] = DONE_OPEN;
-        d.flags[r * NFLAGS + F_ST] = ST_RESID;
-        d.flags[r * NFLAGS + F_J] = 0;
-        d.flags[r * NFLAGS + F_ITERS] = 0;
-        d.scal[r * NSCAL + S_RN2] = 0.0;
-        if (r == 0) { d.stats[3] = 0; d.stats[6] = 0; }
-    }
-    if (i < (d.m + 1) * d.m) d.H[(int64_t)r * (d.m + 1) * d.m + i] = 0.0;
-    if (i < 2 * (d.m + 1)) d.hdot[(int64_t)r * 2 * (d.m + 1) + i] = 0.0;
-    if (i >= d.ne) return;
-    const double bi = (double)b[(int64_t)r * d.ld + i];
-    double x0 = guess ? (double)guess[(int64_t)r * d.ld + i] : 0.0;
-    if (mode == 3) {
-        const double c[4] = {4.0, -6.0, 4.0, -1.0};
-        x0 = 0.0;
-        for (int k = 1; k <= 4 && k <= ring; ++k)
-            if (n - k >= 1) x0 += c[k - 1] * (double)ringbuf[(((n - k) % ring) * d.R + r) * (int64_t)d.ld + i];
-    }
-    d.x[(int64_t)r * d.ne + i] = x0;
-    atomicAdd(d.scal + r * NSCAL + S_BN2, bi * bi);
-}
-
-__global__ void k_gm_zero_scal(GmDev d, Ctl* ctl) {
-    const int t = threadIdx.x;
-    if (t == 0) ctl->hist_ns += device_ns() - ctl->t_mark;      // the history kernel ran just before
-    if (t < d.R * NSCAL) d.scal[t] = 0.0;
-}
-
-// r = b - T0 x (FP64 matrix), one warp per row, for a right-hand side at a restart (first pass of
-// the step, or a cycle updated in the previous pass); accumulates ||r||^2
-template <typename T>
-__global__ void k_gm_resid(GmDev d, const double* __restrict__ T0, const T* __restrict__ b) {
-    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    const int r = blockIdx.y;
-    if (row >= d.ne || fl(d, r, F_DONE) != DONE_OPEN || fl(d, r, F_ST) == ST_ARN) return;
-    const double* a = T0 + (int64_t)row * d.ne;
-    const double* xr = d.x + (int64_t)r * d.ne;
-    double s = 0.0;
-    for (int j = lane; j < d.ne; j += 32) s += a[j] * xr[j];
+__device__ __forceinline__ double warp_sum(double s) {
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-        const double v = (double)b[(int64_t)r * d.ld + row] - s;
-        d.r[(int64_t)r * d.ne + row] = v;
-        atomicAdd(d.scal + r * NSCAL + S_RN2, v * v);
-    }
+    return s;
 }
 
-// restart check: converged, out of iterations, or open a cycle with beta = ||r||
-__global__ void k_gm_check(GmDev d) {
-    const int r = threadIdx.x;
-    if (r >= d.R || fl(d, r, F_DONE) != DONE_OPEN || fl(d, r, F_ST) == ST_ARN) return;
-    double* sc = d.scal + r * NSCAL;
-    const double beta = sqrt(sc[S_RN2]);
-    const double bn = sqrt(sc[S_BN2]);
-    sc[S_RN2] = 0.0;
-    if (beta <= d.tol * bn || beta == 0.0) {
-        d.flags[r * NFLAGS + F_DONE] = DONE_CONV;
-        return;
-    }
-    if (fl(d, r, F_ITERS) >= d.maxit) {
-        d.flags[r * NFLAGS + F_DONE] = DONE_GAVEUP;
-        return;
-    }
-    sc[S_BETA] = beta;
-    d.flags[r * NFLAGS + F_ST] = ST_ARN;
-    d.flags[r * NFLAGS + F_J] = 0;
-    double* g = d.g + (int64_t)r * (d.m + 1);
-    g[0] = beta;
-    for (int k = 1; k <= d.m; ++k) g[k] = 0.0;
-}
-
-// The block's contributions to hdot[k] = V_k . w (k <= j) for its nloc entries starting at i0, w of
-// those entries in shared memory; one warp per k.
-__device__ __forceinline__ void block_dots(const GmDev& d, int r, int j, int64_t i0, int nloc, const double* wsh,
-                                           double* hdot) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int k = warp; k <= j; k += nw) {
-        const double* v = d.V + ((int64_t)k * d.R + r) * d.ne + i0;
-        double s = 0.0;
-        for (int t = lane; t < nloc; t += 32) s += v[t] * wsh[t];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) atomicAdd(hdot + k, s);
-    }
-}
-
-// Arnoldi iteration j, first part: w = T0p V_j (path precision matrix and accumulation, one warp per
-// row) and the first Gram-Schmidt projections hdot0[k] = V_k . w.  A cycle opened in this pass
-// (j = 0) takes V_0 = r / beta on the fly and stores it.
-template <typename T, int WPB>
-__global__ void __launch_bounds__(WPB * 32) k_gm_matvec(GmDev d, const T* __restrict__ T0p) {
-    __shared__ double wsh[WPB];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r = blockIdx.y;
-    if (!arnoldi(d, r)) return;
-    const int j = fl(d, r, F_J);
-    const int64_t row0 = (int64_t)blockIdx.x * WPB;
-    const int64_t row = row0 + warp;
-    const double* v = j == 0 ? d.r + (int64_t)r * d.ne : d.V + ((int64_t)j * d.R + r) * d.ne;
-    const double sc = j == 0 ? 1.0 / d.scal[r * NSCAL + S_BETA] : 1.0;
-    double wv = 0.0;
-    if (row < d.ne) {
-        const T* a = T0p + row * d.ne;
-        T s = 0;
-        for (int c = lane; c < d.ne; c += 32) s += a[c] * (T)(v[c] * sc);
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        wv = (double)s;
-        if (lane == 0) {
-            d.w[(int64_t)r * d.ne + row] = wv;
-            if (j == 0) d.V[(int64_t)r * d.ne + row] = v[row] * sc;
-        }
-    }
-    if (lane == 0) wsh[warp] = wv;
-    __syncthreads();   // also makes this block's V_0 stores visible to its warps
-    const int nloc = (int)min((int64_t)WPB, d.ne - row0);
-    block_dots(d, r, j, row0, nloc, wsh, d.hdot + (int64_t)r * 2 * (d.m + 1));
-}
-
-// w -= sum_k hdot[pass][k] V_k; pass 0 also accumulates the second projections hdot1 = V_k . w,
-// pass 1 the norm ||w||^2
-template <int PASS>
-__global__ void __launch_bounds__(256) k_gm_orth(GmDev d) {
-    __shared__ double hs[64];
-    __shared__ double wsh[256];
-    const int r = blockIdx.y;
-    if (!arnoldi(d, r)) return;
-    const int j = fl(d, r, F_J);
-    const double* h = d.hdot + (int64_t)r * 2 * (d.m + 1) + PASS * (d.m + 1);
-    for (int k = threadIdx.x; k <= j; k += blockDim.x) hs[k] = h[k];
-    __syncthreads();
-    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x;
-    const int64_t i = i0 + threadIdx.x;
-    double v = 0.0;
-    if (i < d.ne) {
-        v = d.w[(int64_t)r * d.ne + i];
-        for (int k = 0; k <= j; ++k) v -= hs[k] * d.V[((int64_t)k * d.R + r) * d.ne + i];
-        d.w[(int64_t)r * d.ne + i] = v;
-    }
-    if (PASS == 0) {
-        wsh[threadIdx.x] = v;
-        __syncthreads();
-        const int nloc = (int)min((int64_t)blockDim.x, d.ne - i0);
-        block_dots(d, r, j, i0, nloc, wsh, d.hdot + (int64_t)r * 2 * (d.m + 1) + (d.m + 1));
-    } else {
-        double s = v * v;
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if ((threadIdx.x & 31) == 0) atomicAdd(d.scal + r * NSCAL + S_WN2, s);
-    }
-}
-
-// One thread per right-hand side: fold both projections into H[:, j] (clearing them), Givens update,
-// residual estimate, cycle stop; at a stop, the back substitution H y = g.
-__global__ void k_gm_givens(GmDev d) {
-    const int r = threadIdx.x;
-    if (r >= d.R || !arnoldi(d, r)) return;
-    const int j = fl(d, r, F_J);
-    double* H = d.H + (int64_t)r * (d.m + 1) * d.m;
-    double* hd = d.hdot + (int64_t)r * 2 * (d.m + 1);
-    double* cs = d.cs + (int64_t)r * (d.m + 1);
-    double* sn = d.sn + (int64_t)r * (d.m + 1);
-    double* g = d.g + (int64_t)r * (d.m + 1);
-    double* sc = d.scal + r * NSCAL;
-    for (int k = 0; k <= j; ++k) {
-        H[(int64_t)k * d.m + j] = hd[k] + hd[d.m + 1 + k];
-        hd[k] = 0.0;
-        hd[d.m + 1 + k] = 0.0;
-    }
-    const double hn = sqrt(sc[S_WN2]);
-    sc[S_WN2] = 0.0;
-    H[(int64_t)(j + 1) * d.m + j] = hn;
-    for (int k = 0; k < j; ++k) {
-        const double a = H[(int64_t)k * d.m + j], b = H[(int64_t)(k + 1) * d.m + j];
-        H[(int64_t)k * d.m + j] = cs[k] * a + sn[k] * b;
-        H[(int64_t)(k + 1) * d.m + j] = -sn[k] * a + cs[k] * b;
-    }
-    const double a = H[(int64_t)j * d.m + j], b = H[(int64_t)(j + 1) * d.m + j];
-    const double rr = sqrt(a * a + b * b);
-    const double c = rr > 0.0 ? a / rr : 1.0, s = rr > 0.0 ? b / rr : 0.0;
-    cs[j] = c;
-    sn[j] = s;
-    H[(int64_t)j * d.m + j] = rr;
-    H[(int64_t)(j + 1) * d.m + j] = 0.0;
-    g[j + 1] = -s * g[j];
-    g[j] = c * g[j];
-    d.flags[r * NFLAGS + F_ITERS] += 1;
-    atomicAdd(d.stats + 0, 1ULL);
-    atomicAdd(d.stats + 3, 1ULL);
-    // a cycle gains inner_tol, but never solves past half the outer target (the true FP64 residual
-    // decides at the restart whether another cycle runs)
-    const double goal = fmax(d.inner_tol * sc[S_BETA], 0.5 * d.tol * sqrt(sc[S_BN2]));
-    const bool stop = fabs(g[j + 1]) <= goal || j + 1 == d.m || hn == 0.0 ||
-                      fl(d, r, F_ITERS) >= d.maxit;
-    sc[S_HN] = hn;    // kept for the next basis vector
-    d.flags[r * NFLAGS + F_J] = j + 1;
-    if (!stop) return;
-    const int J = j + 1;
-    double* y = d.yv + (int64_t)r * d.m;
-    for (int i = J - 1; i >= 0; --i) {
-        double t = g[i];
-        for (int k = i + 1; k < J; ++k) t -= H[(int64_t)i * d.m + k] * y[k];
-        y[i] = t / H[(int64_t)i * d.m + i];
-    }
-    d.flags[r * NFLAGS + F_ST] = ST_UPD;
-}
-
-// End of a pass, elementwise: V_{j+1} = w / h_{j+1,j} for a continuing cycle, x += V y and a
-// cleared H for a finished one (whose ST_UPD state sends it to the restart of the next pass).  Thread 0 of block (0, 0) then
-// sets the loop condition: another pass while some right-hand side is open, within the pass cap.
-__global__ void __launch_bounds__(256) k_gm_finish(GmDev d, cudaGraphConditionalHandle cond) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = blockIdx.y;
-    if (blockIdx.x == 0 && r == 0 && threadIdx.x == 0) {
-        bool open = false;
-        for (int q = 0; q < d.R; ++q) open |= fl(d, q, F_DONE) == DONE_OPEN;
-        const unsigned long long passes = ++d.stats[6];
-        d.stats[5] += 1;
-        cudaGraphSetConditional(cond, (open && passes < (unsigned long long)d.pass_cap) ? 1u : 0u);
-    }
-    if (fl(d, r, F_DONE) != DONE_OPEN) return;
-    const int st = fl(d, r, F_ST);
-    const int J = fl(d, r, F_J);
-    if (st == ST_ARN) {
-        if (i < d.ne) d.V[((int64_t)J * d.R + r) * d.ne + i] = d.w[(int64_t)r * d.ne + i] / d.scal[r * NSCAL + S_HN];
-    } else if (st == ST_UPD) {
-        if (i < d.ne) {
-            double v = d.x[(int64_t)r * d.ne + i];
-            for (int k = 0; k < J; ++k) v += d.yv[(int64_t)r * d.m + k] * d.V[((int64_t)k * d.R + r) * d.ne + i];
-            d.x[(int64_t)r * d.ne + i] = v;
-        }
-        if (i < (int64_t)(d.m + 1) * d.m) d.H[(int64_t)r * (d.m + 1) * d.m + i] = 0.0;
-    }
-}
-
-// y_n (ring slot n % ring, path type) = x; statistics of the step; the first step with a solve
-// left above the tolerance is recorded in the step state (returned as TDCFIE_E_NOCONV)
+// a . x over n entries by one warp; x in shared memory.  16-byte loads where the rows allow them
 template <typename T>
-__global__ void k_gm_store(GmDev d, T* __restrict__ ringbuf, int ring, Ctl* ctl) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = blockIdx.y;
-    if (i == 0 && r == 0) {
-        atomicAdd(d.stats + 1, 1ULL);
-        atomicMax(d.stats + 2, d.stats[3]);
-        for (int q = 0; q < d.R; ++q)
-            if (fl(d, q, F_DONE) != DONE_CONV) {
-                atomicAdd(d.stats + 4, 1ULL);
-                if (atomicCAS(&ctl->noconv, 0, 1) == 0) ctl->noconv_step = ctl->n;
+__device__ __forceinline__ T dot(const T* __restrict__ a, const T* x, int n, bool vec) {
+    const int lane = threadIdx.x & 31;
+    T s = 0;
+    if (vec) {
+        if constexpr (sizeof(T) == 4) {
+#pragma unroll 6
+            for (int c = 4 * lane; c < n; c += 128) {
+                const float4 u = *reinterpret_cast<const float4*>(a + c), v = *reinterpret_cast<const float4*>(x + c);
+                s += u.x * v.x; s += u.y * v.y; s += u.z * v.z; s += u.w * v.w;
             }
+        } else {
+#pragma unroll 6
+            for (int c = 2 * lane; c < n; c += 64) {
+                const double2 u = *reinterpret_cast<const double2*>(a + c), v = *reinterpret_cast<const double2*>(x + c);
+                s += u.x * v.x; s += u.y * v.y;
+            }
+        }
+    } else {
+#pragma unroll 8
+        for (int c = lane; c < n; c += 32) s += a[c] * x[c];
     }
-    if (i >= d.ne) return;
-    T* dst = ringbuf + (ctl->n % ring) * (int64_t)d.R * d.ld;
-    dst[(int64_t)r * d.ld + i] = (T)d.x[(int64_t)r * d.ne + i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// out[i] = A (sc src) over the block's rows; the vector is staged in shared memory (xs) in tiles, a row
+// is shared by d.wpr warps (psum: their parts).  Ends with a barrier of the block.
+template <typename T>
+__device__ __forceinline__ void block_product(const GmDev& d, const T* __restrict__ A, const double* src, double sc,
+                                              int row0, int nloc, double* xs_, double* psum, double* out) {
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    constexpr int Q = 16 / (int)sizeof(T);      // entries of a 16-byte load
+    T* xs = reinterpret_cast<T*>(xs_);
+    const bool vec = d.ne % Q == 0;
+    for (int c0 = 0; c0 < d.ne; c0 += GM_TILE) {
+        const int nc = min(GM_TILE, d.ne - c0);
+        if (c0) __syncthreads();
+        for (int c = t; c < nc; c += GM_T) xs[c] = (T)(__ldcg(src + c0 + c) * sc);
+        __syncthreads();
+        const int per = (nc + d.wpr * Q - 1) / (d.wpr * Q) * Q;      // columns per warp
+        for (int u = warp; u < nloc * d.wpr; u += GM_W) {
+            const int row = u / d.wpr, c1 = u % d.wpr * per, n = min(per, nc - c1);
+            const T v = n > 0 ? dot<T>(A + (int64_t)(row0 + row) * d.ne + c0 + c1, xs + c1, n, vec) : (T)0;
+            if (lane == 0) psum[u] = c0 ? psum[u] + (double)v : (double)v;
+        }
+    }
+    __syncthreads();
+    for (int i = t; i < nloc; i += GM_T) {
+        double s = psum[i * d.wpr];
+        for (int k = 1; k < d.wpr; ++k) s += psum[i * d.wpr + k];
+        out[i] = s;
+    }
+    __syncthreads();
+}
+
+// part[k][block] = V_k . w over the block's rows, k < cnt (w in shared memory)
+__device__ __forceinline__ void block_dots(const GmDev& d, const double* V, int cnt, int nloc, const double* w, double* part) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k = warp; k < cnt; k += GM_W) {
+        const double* v = V + (int64_t)k * d.R * d.ne;
+        double s = 0.0;
+        for (int i = lane; i < nloc; i += 32) s += v[i] * w[i];
+        s = warp_sum(s);
+        if (lane == 0) __stcg(part + k * d.G + blockIdx.x, s);
+    }
+}
+// part[block] = |v|^2 over the block's rows (first warp)
+__device__ __forceinline__ void block_norm(const double* v, int nloc, double* part) {
+    if (threadIdx.x >= 32) return;
+    double s = 0.0;
+    for (int i = threadIdx.x; i < nloc; i += 32) s += v[i] * v[i];
+    s = warp_sum(s);
+    if (threadIdx.x == 0) __stcg(part + blockIdx.x, s);
+}
+// out[k] = the sum of part[k][.], k < cnt.  Ends with a barrier of the block.
+__device__ __forceinline__ void group_sums(const GmDev& d, const double* part, int cnt, double* out) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k = warp; k < cnt; k += GM_W) {
+        double s = 0.0;
+        for (int q = lane; q < d.G; q += 32) s += __ldcg(part + k * d.G + q);
+        s = warp_sum(s);
+        if (lane == 0) out[k] = s;
+    }
+    __syncthreads();
+}
+// w[i] += sign sum_k c[k] V_k over the block's rows: one warp per row, lanes along the vectors
+__device__ __forceinline__ void add_vectors(const GmDev& d, const double* V, int cnt, int nloc, const double* c, double sign,
+                                            double* w) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = warp; i < nloc; i += GM_W) {
+        double s = 0.0;
+        for (int k = lane; k < cnt; k += 32) s += c[k] * V[(int64_t)k * d.R * d.ne + i];
+        s = warp_sum(s);
+        if (lane == 0) w[i] += sign * s;
+    }
+    __syncthreads();
+}
+
+// One step's solves; the solution goes to ring slot (ctl->n + off) % ring.  mode: the initial guess, 0
+// zero, 1 y_{n-1}, 2 and 4 the learned guess buffer, 3 cubic extrapolation of y_{n-1..n-4} (y_i = 0
+// for i <= 0).  The first step with a solve left above the tolerance is recorded in the step state
+// (returned as TDCFIE_E_NOCONV).
+template <typename T>
+__global__ void __launch_bounds__(GM_T, 1) k_gm_solve(const __grid_constant__ GmDev d, const double* __restrict__ T0,
+                                                   const T* __restrict__ T0p, const T* __restrict__ b, int mode,
+                                                   T* __restrict__ ringbuf, int ring, const T* __restrict__ learned, int off,
+                                                   Ctl* ctl) {
+    extern __shared__ __align__(16) double sm[];
+    __shared__ double sc[4];      // ||r||^2 (or ||w||^2), ||b||^2, h_{j+1,j}
+    __shared__ int failed, stop;
+    const int t = threadIdx.x, lane = t & 31, r = blockIdx.y, m = d.m;
+    const int row0 = blockIdx.x * d.rpb, nloc = min(d.rpb, d.ne - row0);
+    double* xs = sm;
+    double* cs = xs + d.tile;
+    double* sn = cs + m;
+    double* g = sn + m;
+    double* hc = g + m + 1;      // the current column of H
+    double* h1 = hc + m + 1;
+    double* wl = h1 + m + 1;     // the block's part of a vector
+    double* xl = wl + d.rpb;
+    double* psum = xl + d.rpb;
+    if (t == 0) failed = (int)__ldcg(d.sync + d.R);      // an earlier solve's wait ran out
+    if (t == 0 && blockIdx.x == 0 && r == 0) ctl->hist_ns += device_ns() - ctl->t_mark;      // the history kernel is done
+    __syncthreads();
+    if (failed) return;
+    const int64_t n = ctl->n + off;
+    const int64_t vec0 = (int64_t)r * d.ne;
+    double* x = d.x + vec0;
+    double* V = d.V + vec0 + row0;      // the block's rows of V_0
+    double* H = d.H + (int64_t)r * (m + 1) * m;
+    double* p0 = d.part + (int64_t)r * (2 * (m + 1) + 2) * d.G;
+    double* p1 = p0 + (m + 1) * d.G;
+    double* p2 = p1 + (m + 1) * d.G;
+    const T* br = b + (int64_t)r * d.ld + row0;
+#define MEET() if (!group_barrier(d.sync + r, d.G, d.sync + d.R, &failed)) { ctl->timeout = 1; return; }
+
+    for (int i = t; i < nloc; i += GM_T) {
+        const int64_t e = (int64_t)r * d.ld + row0 + i;
+        double x0 = 0.0;
+        if (mode == 1 && n > 1) x0 = (double)ringbuf[((n - 1) % ring) * (int64_t)d.R * d.ld + e];
+        if ((mode == 2 || mode == 4) && n > 1) x0 = (double)learned[e];
+        if (mode == 3) {
+            const double c[4] = {4.0, -6.0, 4.0, -1.0};
+            for (int k = 1; k <= 4 && k <= ring; ++k)
+                if (n - k >= 1) x0 += c[k - 1] * (double)ringbuf[((n - k) % ring) * (int64_t)d.R * d.ld + e];
+        }
+        __stcg(x + row0 + i, x0);
+        xl[i] = x0;
+        wl[i] = (double)br[i];
+    }
+    __syncthreads();
+    block_norm(wl, nloc, p2 + d.G);
+    MEET();
+    group_sums(d, p2 + d.G, 1, sc + 1);
+    const double bn = sqrt(sc[1]);
+    int iters = 0;
+    bool conv = false;
+    for (;;) {
+        // restart: converged, out of iterations, or open a cycle with beta = ||r||
+        block_product<double>(d, T0, x, 1.0, row0, nloc, xs, psum, wl);
+        for (int i = t; i < nloc; i += GM_T) {
+            wl[i] = (double)br[i] - wl[i];
+            __stcg(d.r + vec0 + row0 + i, wl[i]);
+        }
+        __syncthreads();
+        block_norm(wl, nloc, p2);
+        MEET();
+        group_sums(d, p2, 1, sc);
+        const double beta = sqrt(sc[0]);
+        conv = beta <= d.tol * bn || beta == 0.0;
+        if (conv || iters >= d.maxit) break;
+        if (t == 0) g[0] = beta;
+        const double* src = d.r + vec0;
+        double scale = 1.0 / beta;
+        int j = 0;
+        for (bool last = false; !last; ++j) {
+            // w = T0p V_j, V_j = scale * src taken on the fly; the rows of V_j kept; first projections
+            for (int i = t; i < nloc; i += GM_T) V[(int64_t)j * d.R * d.ne + i] = __ldcg(src + row0 + i) * scale;
+            block_product<T>(d, T0p, src, scale, row0, nloc, xs, psum, wl);
+            block_dots(d, V, j + 1, nloc, wl, p0);
+            MEET();
+            group_sums(d, p0, j + 1, hc);
+            add_vectors(d, V, j + 1, nloc, hc, -1.0, wl);
+            block_dots(d, V, j + 1, nloc, wl, p1);
+            MEET();
+            group_sums(d, p1, j + 1, h1);
+            add_vectors(d, V, j + 1, nloc, h1, -1.0, wl);
+            for (int i = t; i < nloc; i += GM_T) __stcg(d.w + vec0 + row0 + i, wl[i]);
+            block_norm(wl, nloc, p2 + d.G);
+            MEET();
+            group_sums(d, p2 + d.G, 1, sc);
+            ++iters;
+            if (t == 0) {      // Givens rotations, residual estimate
+                const double hn = sqrt(sc[0]);
+                double a = hc[0] + h1[0];
+                for (int k = 0; k < j; ++k) {
+                    const double q = hc[k + 1] + h1[k + 1];
+                    hc[k] = cs[k] * a + sn[k] * q;
+                    a = -sn[k] * a + cs[k] * q;
+                }
+                const double rr = sqrt(a * a + hn * hn);
+                const double c = rr > 0.0 ? a / rr : 1.0, s = rr > 0.0 ? hn / rr : 0.0;
+                cs[j] = c;
+                sn[j] = s;
+                hc[j] = rr;
+                g[j + 1] = -s * g[j];
+                g[j] = c * g[j];
+                // a cycle gains inner_tol, but never solves past half the outer target (the true FP64
+                // residual decides at the restart whether another cycle runs)
+                const double goal = fmax(d.inner_tol * beta, 0.5 * d.tol * bn);
+                stop = fabs(g[j + 1]) <= goal || j + 1 == m || hn == 0.0 || iters >= d.maxit;
+                sc[2] = 1.0 / hn;
+            }
+            __syncthreads();
+            last = stop != 0;
+            if (blockIdx.x == 0)
+                for (int k = t; k <= j; k += GM_T) __stcg(H + (int64_t)k * m + j, hc[k]);
+            src = d.w + vec0;
+            scale = sc[2];
+        }
+        // H y = g: the columns before the last were written ahead of a barrier, the last is in hc
+        for (int e = t; e < j * j; e += GM_T) {
+            const int i = e / j, k = e % j;
+            xs[e] = k < i ? 0.0 : k == j - 1 ? hc[i] : __ldcg(H + (int64_t)i * m + k);
+        }
+        __syncthreads();
+        if (t < 32) {      // by columns, two right-hand sides per lane (j <= 60); y replaces g
+            double u0 = lane < j ? g[lane] : 0.0, u1 = lane + 32 < j ? g[lane + 32] : 0.0;
+            for (int i = j - 1; i >= 0; --i) {
+                const double y = __shfl_sync(0xffffffffu, i < 32 ? u0 : u1, i & 31) / xs[i * j + i];
+                if (lane < i) u0 -= xs[lane * j + i] * y;
+                if (lane + 32 < i) u1 -= xs[(lane + 32) * j + i] * y;
+                if (lane == 0) g[i] = y;
+            }
+        }
+        __syncthreads();
+        add_vectors(d, V, j, nloc, g, 1.0, xl);
+        for (int i = t; i < nloc; i += GM_T) __stcg(x + row0 + i, xl[i]);
+        MEET();
+    }
+#undef MEET
+    for (int i = t; i < nloc; i += GM_T) ringbuf[(n % ring) * (int64_t)d.R * d.ld + (int64_t)r * d.ld + row0 + i] = (T)xl[i];
+    if (t == 0 && blockIdx.x == 0) {
+        atomicAdd(d.stats + 0, (unsigned long long)iters);
+        atomicAdd(d.stats + 3, (unsigned long long)iters);
+        if (!conv) {
+            atomicAdd(d.stats + 4, 1ULL);
+            if (atomicCAS(&ctl->noconv, 0, 1) == 0) ctl->noconv_step = n;
+        }
+        __threadfence();
+        if (atomicAdd(d.stats + 5, 1ULL) == (unsigned long long)(d.R - 1)) {      // the step's last group
+            __threadfence();
+            atomicAdd(d.stats + 1, 1ULL);
+            atomicMax(d.stats + 2, atomicExch(d.stats + 3, 0ULL));
+            atomicExch(d.stats + 5, 0ULL);
+        }
+    }
 }
 
 // ---------------------------------------------------------------- host side
 struct GmresPlan {
     GmDev d{};
-    cudaStream_t body_stream = nullptr;   // captures the loop body into the WHILE node's graph
+    size_t smem = 0;
     std::vector<void*> owned;
     ~GmresPlan() {
         for (void* p : owned) cudaFree(p);
-        if (body_stream) cudaStreamDestroy(body_stream);
     }
 };
 
 void destroy_gmres(GmresPlan* g) { delete g; }
+
+// The split of the rows.  GM_ROWS per block (two warps per row) until every SM has a block; then all
+// SMs, more rows each.
+template <typename T>
+static cudaError_t split_rows(GmresPlan* g) {
+    GmDev& d = g->d;
+    int dev = 0, sms = 0, occ = 0;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
+    auto shape = [&](int slots) {
+        const int per = std::max(1, slots / d.R);
+        d.rpb = std::max(GM_ROWS, (d.ne + per - 1) / per);
+        d.G = (d.ne + d.rpb - 1) / d.rpb;
+        d.wpr = d.rpb <= GM_W / 2 ? 2 : 1;
+        // the staged vector, or a cycle's triangle
+        d.tile = std::max(std::min(d.ne, GM_TILE), std::min(d.m, d.maxit) * std::min(d.m, d.maxit));
+        d.tile += d.tile & 1;
+        g->smem = sizeof(double) * (d.tile + 5 * d.m + 3 + (size_t)d.rpb * (2 + d.wpr));
+    };
+    shape(sms);
+    if ((e = cudaFuncSetAttribute(k_gm_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem))) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gm_solve<T>, GM_T, g->smem))) return e;
+    return (int64_t)d.G * d.R <= (int64_t)occ * sms ? cudaSuccess : cudaErrorCooperativeLaunchTooLarge;
+}
 
 cudaError_t build_gmres(tdcfie_t h, StepPlan* p) {
     auto* g = new GmresPlan();
@@ -327,105 +348,60 @@ cudaError_t build_gmres(tdcfie_t h, StepPlan* p) {
     d.tol = h->opts.gmres_tol;
     d.inner_tol = 1e-4;   // each cycle gains four digits; the restarts refine against the FP64 residual
     d.maxit = std::max(1, h->opts.gmres_maxit);
-    // every pass performs one Arnoldi iteration of each open right-hand side, and each cycle ends
-    // in one restart check that also starts the next cycle's first iteration
-    d.pass_cap = d.maxit + d.maxit / m + 3;
+    cudaError_t e = p->prec == TDCFIE_FP64 ? split_rows<double>(g) : split_rows<float>(g);
+    if (e != cudaSuccess) return e;
     auto al = [&](double** q, size_t n) -> cudaError_t {
         cudaError_t e = cudaMalloc((void**)q, sizeof(double) * (n ? n : 1));
         if (e == cudaSuccess) { g->owned.push_back(*q); e = cudaMemset(*q, 0, sizeof(double) * (n ? n : 1)); }
         return e;
     };
-    cudaError_t e;
     if ((e = al(&d.x, (size_t)R * ne)) || (e = al(&d.r, (size_t)R * ne)) || (e = al(&d.V, (size_t)(m + 1) * R * ne)) ||
-        (e = al(&d.w, (size_t)R * ne)) || (e = al(&d.hdot, (size_t)R * 2 * (m + 1))) ||
-        (e = al(&d.H, (size_t)R * (m + 1) * m)) || (e = al(&d.cs, (size_t)R * (m + 1))) ||
-        (e = al(&d.sn, (size_t)R * (m + 1))) || (e = al(&d.g, (size_t)R * (m + 1))) || (e = al(&d.yv, (size_t)R * m)) ||
-        (e = al(&d.scal, (size_t)R * NSCAL)))
+        (e = al(&d.w, (size_t)R * ne)) || (e = al(&d.H, (size_t)R * (m + 1) * m)) ||
+        (e = al(&d.part, (size_t)R * (2 * (m + 1) + 2) * d.G)))
         return e;
-    if ((e = cudaMalloc(&d.flags, sizeof(int) * R * NFLAGS)) != cudaSuccess) return e;
-    g->owned.push_back(d.flags);
-    if ((e = cudaMemset(d.flags, 0, sizeof(int) * R * NFLAGS)) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&d.stats, sizeof(unsigned long long) * NSTATS)) != cudaSuccess) return e;
-    g->owned.push_back(d.stats);
-    if ((e = cudaStreamCreateWithFlags(&g->body_stream, cudaStreamNonBlocking)) != cudaSuccess) return e;
-    return cudaMemset(d.stats, 0, sizeof(unsigned long long) * NSTATS);
+    // the barriers' counters and the statistics in one piece
+    if ((e = cudaMalloc(&d.sync, sizeof(unsigned long long) * (R + 1 + NSTATS))) != cudaSuccess) return e;
+    g->owned.push_back(d.sync);
+    d.stats = d.sync + R + 1;
+    return reset_gmres_stats(g);
 }
 
 void gmres_set_tol(GmresPlan* g, double tol) { g->d.tol = tol; }
 
-cudaError_t reset_gmres_stats(GmresPlan* g) { return cudaMemset(g->d.stats, 0, sizeof(unsigned long long) * NSTATS); }
+cudaError_t reset_gmres_stats(GmresPlan* g) {
+    return cudaMemset(g->d.sync, 0, sizeof(unsigned long long) * (g->d.R + 1 + NSTATS));
+}
 
-cudaError_t gmres_stats(GmresPlan* g, long long* out6) {
+cudaError_t gmres_stats(GmresPlan* g, long long* out5) {
     unsigned long long st[NSTATS];
     const cudaError_t e = cudaMemcpy(st, g->d.stats, sizeof(st), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return e;
-    for (int i = 0; i < 6; ++i) out6[i] = (long long)st[i];
+    for (int i = 0; i < 5; ++i) out5[i] = (long long)st[i];
     return cudaSuccess;
 }
 
-// Kernels of one loop pass: resid, check, matvec, orth x 2, givens, finish
-int gmres_body_launches() { return 7; }
-
-// Enqueue the step's solve on s, which must be capturing a graph: init, the WHILE node (its body
-// captured on the plan's own stream), then the store into the ring.
+// Enqueue the solve of step ctl->n + off on s
 template <typename T>
-cudaError_t launch_gmres(tdcfie_t h, StepPlan* p, const T* b, const T* learned, const T* T0p, T* ringbuf,
-                         cudaStream_t s, int& kernels) {
+cudaError_t launch_gmres(tdcfie_t h, StepPlan* p, const T* b, const T* learned, const T* T0p, T* ringbuf, int off,
+                         cudaStream_t s) {
     GmresPlan* g = p->gm;
-    const GmDev& d = g->d;
-    const int ne = d.ne, R = d.R, tb = 256, wpb = 8;
-    const int ninit = std::max(ne, (d.m + 1) * d.m + 1);
-    const dim3 gi((ninit + tb - 1) / tb, R), ge((ne + tb - 1) / tb, R), gw((ne + wpb - 1) / wpb, R),
-        gm((ne + MV_WPB - 1) / MV_WPB, R);
-    k_gm_zero_scal<<<1, 64, 0, s>>>(d, p->ctl);
-    k_gm_init<T><<<gi, tb, 0, s>>>(d, b, h->opts.guess, ringbuf, p->ring, learned, p->ctl);
-
-    cudaStreamCaptureStatus cs;
-    cudaGraph_t graph = nullptr;
-    const cudaGraphNode_t* deps = nullptr;
-    const cudaGraphEdgeData* edata = nullptr;
-    size_t ndeps = 0;
-    cudaError_t e = cudaStreamGetCaptureInfo(s, &cs, nullptr, &graph, &deps, &edata, &ndeps);
-    if (e != cudaSuccess) return e;
-    if (cs != cudaStreamCaptureStatusActive) return cudaErrorStreamCaptureUnmatched;
-    cudaGraphConditionalHandle cond;
-    if ((e = cudaGraphConditionalHandleCreate(&cond, graph, 1, cudaGraphCondAssignDefault)) != cudaSuccess) return e;
-    cudaGraphNodeParams np{};
-    np.type = cudaGraphNodeTypeConditional;
-    np.conditional.handle = cond;
-    np.conditional.type = cudaGraphCondTypeWhile;
-    np.conditional.size = 1;
-    cudaGraphNode_t node;
-    if ((e = cudaGraphAddNode(&node, graph, deps, edata, ndeps, &np)) != cudaSuccess) return e;
-    cudaGraph_t body = np.conditional.phGraph_out[0];
-    if ((e = cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1, cudaStreamSetCaptureDependencies)) !=
-        cudaSuccess)
-        return e;
-
-    cudaStream_t b2 = g->body_stream;
-    if ((e = cudaStreamBeginCaptureToGraph(b2, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed)) !=
-        cudaSuccess)
-        return e;
-    k_gm_resid<T><<<gw, 32 * wpb, 0, b2>>>(d, h->T, b);
-    k_gm_check<<<1, 32 * ((R + 31) / 32), 0, b2>>>(d);
-    k_gm_matvec<T, MV_WPB><<<gm, 32 * MV_WPB, 0, b2>>>(d, T0p);
-    k_gm_orth<0><<<ge, tb, 0, b2>>>(d);
-    k_gm_orth<1><<<ge, tb, 0, b2>>>(d);
-    k_gm_givens<<<1, 32 * ((R + 31) / 32), 0, b2>>>(d);
-    k_gm_finish<<<gi, tb, 0, b2>>>(d, cond);
-    cudaGraph_t captured = nullptr;
-    const cudaError_t le = cudaGetLastError();
-    if ((e = cudaStreamEndCapture(b2, &captured)) != cudaSuccess) return e;
-    if (le != cudaSuccess) return le;
-
-    k_gm_store<T><<<ge, tb, 0, s>>>(d, ringbuf, p->ring, p->ctl);
-    kernels += 3;   // zero_scal, init, store; the loop passes are counted on the device
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(g->d.G, g->d.R);
+    cfg.blockDim = dim3(GM_T);
+    cfg.dynamicSmemBytes = g->smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_gm_solve<T>, g->d, (const double*)h->T, T0p, b, h->opts.guess, ringbuf, p->ring, learned,
+                              off, p->ctl);
 }
 
-template cudaError_t launch_gmres<double>(tdcfie_t, StepPlan*, const double*, const double*, const double*, double*,
-                                          cudaStream_t, int&);
-template cudaError_t launch_gmres<float>(tdcfie_t, StepPlan*, const float*, const float*, const float*, float*,
-                                         cudaStream_t, int&);
+template cudaError_t launch_gmres<double>(tdcfie_t, StepPlan*, const double*, const double*, const double*, double*, int,
+                                          cudaStream_t);
+template cudaError_t launch_gmres<float>(tdcfie_t, StepPlan*, const float*, const float*, const float*, float*, int,
+                                         cudaStream_t);
 
 }  // namespace tdc

@@ -149,7 +149,7 @@ void free_plan(tdcfie_t h);
 void to_path(cudaStream_t s, int prec, const double* src, void* dst, int64_t rows, int cols, int ld, double scale);
 tdcfie_status plan_reset(tdcfie_t h);
 tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout = nullptr);
-tdcfie_status plan_gmres_stats(tdcfie_t h, long long* out6);
+tdcfie_status plan_gmres_stats(tdcfie_t h, long long* out5);
 tdcfie_status plan_set_solver(tdcfie_t h, int solver, int guess, double tol);
 cudaError_t capture_step(tdcfie_t h, cudaStream_t s);   // one whole step of any path and position in a chunk
 tdcfie_status plan_set_outputs(tdcfie_t h, void* out, void* yout);

@@ -193,11 +193,12 @@ static cudaError_t launch_inner(tdcfie_t h, StepPlan& p, bool chunk, int off, cu
     BY_R(k_hist, d, off, chunk && off > 0);
     kernels += 1;
     g = div_up(p.ne, 4);
-    if (p.mlp_on) kernels += launch_mlp_guess<T>(&p, s);
+    if (p.mlp_on) kernels += launch_mlp_guess<T>(&p, off, s);
     if (p.gmres_on) {
         const cudaError_t e = launch_gmres<T>(h, &p, (const T*)p.b, (const T*)p.guessbuf, (const T*)p.t0mat,
-                                              (T*)p.ringbuf, s, kernels);
+                                              (T*)p.ringbuf, off, s);
         if (e != cudaSuccess) return e;
+        kernels += 1;
     } else {
         BY_R(k_solve, d, off);
         kernels += 1;
@@ -245,10 +246,10 @@ static cudaError_t launch_graph_tc(tdcfie_t h, StepPlan& p, int which, cudaStrea
     return cudaGetLastError();
 }
 
-tdcfie_status plan_gmres_stats(tdcfie_t h, long long* out6) {
+tdcfie_status plan_gmres_stats(tdcfie_t h, long long* out5) {
     StepPlan* p = h->plan;
     if (!p || !p->gm) return fail(h, TDCFIE_E_STATE, "GMRES solver not active on this handle");
-    const cudaError_t e = gmres_stats(p->gm, out6);
+    const cudaError_t e = gmres_stats(p->gm, out5);
     if (e != cudaSuccess) return cuda_fail(h, e, "gmres_stats");
     return TDCFIE_OK;
 }
@@ -615,7 +616,7 @@ tdcfie_status plan_set_outputs(tdcfie_t h, void* out, void* yout) {
 // stopped above its tolerance (each with the first step it happened at)
 tdcfie_status plan_status(tdcfie_t h, const Ctl& c) {
     if (c.timeout)
-        return fail(h, TDCFIE_E_TIMEOUT, "a bounded device-side wait ran out (tensor-core pipeline)");
+        return fail(h, TDCFIE_E_TIMEOUT, "a bounded device-side wait ran out (tensor-core pipeline, or the GMRES solve)");
     if (c.status != 0)
         return fail(h, TDCFIE_E_NONFINITE, "non-finite current at step " + std::to_string(c.bad_step));
     if (c.noconv)
@@ -651,8 +652,6 @@ tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout) {
     c.yout = yout;
     c.hist_ns = 0;
     CK(cudaMemcpyAsync(p->ctl, &c, sizeof(Ctl), cudaMemcpyHostToDevice, s));
-    long long g0[6] = {0, 0, 0, 0, 0, 0}, g1[6] = {0, 0, 0, 0, 0, 0};
-    if (p->gm) CK(gmres_stats(p->gm, g0));
     int64_t kernels = 0;
     auto run = [&](int which) -> tdcfie_status {
         const tdcfie_status st = plan_graph(h, which);
@@ -662,13 +661,13 @@ tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout) {
         return TDCFIE_OK;
     };
 #define RUN(g) do { const tdcfie_status st_ = run(g); if (st_ != TDCFIE_OK) return st_; } while (0)
-    // whole chunks by one graph (the GMRES loop nodes only step by step), the rest step by step; the
-    // post-processing runs when a chunk ends and when the call does
+    // whole chunks by one graph, the rest step by step; the post-processing runs when a chunk ends and
+    // when the call does
     const int64_t C = p->C;
     CK(cudaEventRecord(p->ev0, s));
     for (int64_t n = c.n, end = c.n + nsteps; n < end;) {
         const int64_t i = (n - 1) % C, m = std::min(C - i, end - n);
-        if (m == C && !p->gmres_on) {
+        if (m == C) {
             RUN(StepPlan::G_CHUNK);
         } else {
             if (i == 0) RUN(StepPlan::G_PRE);
@@ -686,10 +685,6 @@ tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout) {
     h->last_step_ms = ms / (nsteps > 0 ? nsteps : 1);
     h->last_hist_ms = 1e-6 * (double)c.hist_ns / (double)nsteps;
     h->last_launches = kernels;
-    if (p->gm) {
-        CK(gmres_stats(p->gm, g1));
-        h->last_launches += (g1[5] - g0[5]) * gmres_body_launches();
-    }
     return plan_status(h, c);
 }
 

@@ -321,11 +321,11 @@ __device__ float block_rms(const T* __restrict__ y, int ne, float* red) {
 
 // s_r = RMS over edges of y_{n-1} (one block of 256 threads per right-hand side)
 template <typename T>
-__global__ void k_mlp_rms(const T* __restrict__ ringbuf, int ring, int R, int ne, int ld, const Ctl* ctl,
+__global__ void k_mlp_rms(const T* __restrict__ ringbuf, int ring, int R, int ne, int ld, const Ctl* ctl, int off,
                           float* __restrict__ scale) {
     __shared__ float red[256];
     const int r = blockIdx.x;
-    const int64_t n = ctl->n;
+    const int64_t n = ctl->n + off;
     const T* y = n > 1 ? ringbuf + (((n - 1) % ring) * R + r) * (int64_t)ld : nullptr;
     const float s = block_rms(y, ne, red);
     if (threadIdx.x == 0) scale[r] = s;
@@ -359,14 +359,14 @@ __global__ void k_mlp_samples(const T* __restrict__ y, int R, int ne, int base, 
 // the path precision T, so a network that outputs zero reproduces it exactly.
 template <typename T>
 __global__ void k_mlp_guess(const __half* __restrict__ wh, const T* __restrict__ ringbuf, int ring, int R, int ne, int ld,
-                            const Ctl* ctl, const float* __restrict__ scale, int extrap, T* __restrict__ guess) {
+                            const Ctl* ctl, int off, const float* __restrict__ scale, int extrap, T* __restrict__ guess) {
     __shared__ float P[NP];
     for (int i = threadIdx.x; i < NP; i += blockDim.x) P[i] = __half2float(wh[i]);
     __syncthreads();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= R * ne) return;
     const int r = idx / ne, m = idx % ne;
-    const int64_t n = ctl->n;
+    const int64_t n = ctl->n + off;
     const float s = scale[r];
     float x[NIN];
     T yk[4] = {0, 0, 0, 0};
@@ -397,16 +397,16 @@ void destroy_mlp(MlpState* m) {
 }
 
 template <typename T>
-int launch_mlp_guess(StepPlan* p, cudaStream_t s) {
+int launch_mlp_guess(StepPlan* p, int off, cudaStream_t s) {
     MlpState* m = p->mlp;
-    k_mlp_rms<T><<<p->R, 256, 0, s>>>((const T*)p->ringbuf, p->ring, p->R, p->ne, p->ld, p->ctl, m->scale);
+    k_mlp_rms<T><<<p->R, 256, 0, s>>>((const T*)p->ringbuf, p->ring, p->R, p->ne, p->ld, p->ctl, off, m->scale);
     k_mlp_guess<T><<<(p->R * p->ne + 127) / 128, 128, 0, s>>>(m->wh, (const T*)p->ringbuf, p->ring, p->R, p->ne,
-                                                                p->ld, p->ctl, m->scale, p->guess_extrap ? 1 : 0,
+                                                                p->ld, p->ctl, off, m->scale, p->guess_extrap ? 1 : 0,
                                                                 (T*)p->guessbuf);
     return 2;
 }
-template int launch_mlp_guess<double>(StepPlan*, cudaStream_t);
-template int launch_mlp_guess<float>(StepPlan*, cudaStream_t);
+template int launch_mlp_guess<double>(StepPlan*, int, cudaStream_t);
+template int launch_mlp_guess<float>(StepPlan*, int, cudaStream_t);
 
 cudaError_t build_mlp(StepPlan* p) {
     auto* m = new MlpState();

@@ -530,4 +530,35 @@ __device__ __forceinline__ unsigned long long device_ns() {
     return t;
 }
 
+constexpr uint64_t WAIT_NS = 2000000000ull;      // limit of every device-side wait
+
+// Barrier of the nb co-resident blocks (cooperative launch) that share the counter c, which only ever
+// grows; false when a wait ran out.  One atomic and one load that waits; the timer is read once in a
+// thousand turns.
+__device__ __forceinline__ bool group_barrier(unsigned long long* c, unsigned long long nb, unsigned long long* err,
+                                              int* failed) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned long long target = (atomicAdd(c, 1ULL) / nb + 1) * nb;
+        unsigned long long v, t0 = 0;
+        for (unsigned spin = 1;; ++spin) {
+            asm volatile("ld.acquire.gpu.u64 %0, [%1];" : "=l"(v) : "l"(c) : "memory");
+            if (v >= target) break;
+            if (spin % 1024 == 0) {
+                const unsigned long long t = device_ns();
+                if (t0 == 0) t0 = t;
+                if (t - t0 > WAIT_NS) {
+                    atomicExch(err, 1ULL);
+                    *failed = 1;
+                    break;
+                }
+            }
+        }
+        __threadfence();
+    }
+    __syncthreads();
+    return !*failed;
+}
+
 }  // namespace tdc

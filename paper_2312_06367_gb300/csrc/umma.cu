@@ -68,7 +68,6 @@ constexpr int D0S = TDC_D0S;  // accumulators of the leading product per k tile 
 static_assert(D0S == 1 || D0S == 2 || D0S == 4, "D0S divides the four K = 16 steps of a k tile");
 constexpr int BUFC = (D0S + 1) * NR;                           // TMEM columns of one buffer (D0 parts, D1)
 constexpr int NBUF = BUFC <= 128 ? 4 : (BUFC <= 256 ? 2 : 1);  // accumulator buffers in tensor memory
-constexpr uint64_t WAIT_NS = 2000000000ull;
 constexpr int TC_C = 4;      // steps per chunk: tests and post-processing of so many steps share their kernels
 
 template <int XS>
@@ -752,7 +751,7 @@ constexpr int RHS_LD = 65;
 constexpr int RHS_SMEM = 2 * 64 * RHS_LD * 8;
 template <bool F16, int XS>
 __global__ void __launch_bounds__(32 * RHS_NW) k_rhs_tc(int ne, const double* __restrict__ exc, const Ctl* ctl,
-                                                const int* __restrict__ eptr, const float* __restrict__ env,
+                                                const int* __restrict__ eptr, const float* env,
                                                 const float4* __restrict__ ent, const int* __restrict__ nE,
                                                 uint16_t* __restrict__ X0, uint16_t* __restrict__ X1,
                                                 uint16_t* __restrict__ X2, float* __restrict__ sX, int ring, int ld) {
@@ -846,7 +845,7 @@ __device__ __forceinline__ int post_col(const Ctl* ctl, int k) {
     return c < 0 ? c + TC_C : c;
 }
 template <bool F16, int XS>
-__global__ void __launch_bounds__(256) k_project_in_tc(DevMesh m, const Ctl* ctl, int adv, const double* __restrict__ y2,
+__global__ void __launch_bounds__(256) k_project_in_tc(DevMesh m, const Ctl* ctl, int adv, const double* y2,
                                                        double inv_dtt, uint16_t* __restrict__ Z0, uint16_t* __restrict__ Z1,
                                                        uint16_t* __restrict__ Z2, float* __restrict__ sZ, int ldc) {
     __shared__ float2 zv[PIN_RB][65];      // FP64 values as FP32 pairs (their slices keep 33 bits)
@@ -899,8 +898,8 @@ __global__ void __launch_bounds__(256) k_project_in_tc(DevMesh m, const Ctl* ctl
 // j[r][m] = y_n[r][m] + u[r][c+(m)] - u[r][c-(m)] in FP64, stored in FP32; finiteness check (the first
 // bad step is kept); grid y: the steps to post-process; the last block to finish advances the step
 // counter by adv (every block has read it before it arrives).
-__global__ void k_project_out_tc(DevMesh m, Ctl* ctl, int adv, const double* __restrict__ y2,
-                                 const double* __restrict__ u, int* __restrict__ done) {
+__global__ void k_project_out_tc(DevMesh m, Ctl* ctl, int adv, const double* y2,
+                                 const double* u, int* __restrict__ done) {
     wait_prior();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
     const int64_t n = ctl->p0 + k;
