@@ -331,7 +331,8 @@ def run_guess_study(args, w):
         "roofline": {"bound": "hbm", "achieved": hb / (m["history_ms"] / 1e3) / 1e9 if m["history_ms"] else None,
                      "peak": pk.get("hbm_gbs"), "unit": "GB/s",
                      "frac": (hb / (m["history_ms"] / 1e3) / 1e9 / pk["hbm_gbs"]) if m["history_ms"] else None,
-                     "traffic": None, "kernel": "history sum (k_history + k_reduce)",
+                     "traffic": None,
+                     "kernel": "history sum (k_pre + k_hist; the bytes are those of a sum per step, a pass over older lags serves a chunk)",
                      "algorithmic_bytes_per_launch": hb},
         "guess_study": rows, "training": info,
     }
@@ -439,7 +440,7 @@ def run_batch(args, probs, name):
                    "dt": probs[0]["dt"], "assemble_s": round(t_asm, 1), "tune_s": round(t_tune, 2), "launch": cfg,
                    "cache": f"history operands of all scatterers ({hb / 1e9:.2f} GB) stream each step",
                    "finite": finite},
-        "gpu_launches": int(t["launches"]) * args.steps,
+        "gpu_launches": -(-args.steps // 32) if cfg["persistent"] else int(t["launches"]) * args.steps,
         "sequential": {"ms_per_step": seq_ms, "steps_s": 1e3 / seq_ms, "how": "each handle's own step graph, one after another"},
         "speedup_vs_sequential": seq_ms / t["step_ms"],
         "roofline": {"bound": "hbm", "achieved": hb / (t["step_ms"] / 1e3) / 1e9, "peak": pk.get("hbm_gbs"), "unit": "GB/s",
@@ -488,7 +489,7 @@ def accuracy_in_run(s, w, nt, stream):
 
 def factored_study(s, w, steps, warmup, nt_acc, stream):
     """The two forms of the history sum on the workload's mesh with one incident wave, same FP64
-    assembly: the dense T_k stream (k_history + k_reduce) against the shell-sparse factored form
+    assembly: the dense T_k stream (k_pre + k_hist) against the shell-sparse factored form
     (k_shells, then one dense product with T_0^-1 [-A | alpha L2 | -L1 Sigma]); per path precision
     the step rate, the history kernels' time and algorithmic bytes, the matrix bytes per step, and
     the rel-L2 of the factored currents against the dense ones over nt_acc steps."""
@@ -640,8 +641,9 @@ def run_ours(args, w):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": pk.get("hbm_gbs"), "unit": "GB/s",
                      "frac": (achieved / pk["hbm_gbs"]) if achieved else None, "traffic": traffic,
                      "kernel": ("factored history sum over all lags of S_k, MM'_k, Phi_k (k_shells)" if factored else
-                                "history sum (k_history + k_reduce)" if prec in ("fp64", "fp32") else
-                                "tcgen05 split-precision history GEMM (k_tc_gemm, fixup in-kernel)"),
+                                "history sum (k_pre + k_hist; the bytes are those of a sum per step, a pass over older lags serves a chunk)"
+                                if prec in ("fp64", "fp32") else
+                                "tcgen05 split-precision history GEMM (k_tc_gemm + k_tc_fix)"),
                      "algorithmic_bytes_per_launch": work_bytes, "history_ms": h_ms,
                      "peak_source": "measured" if not pk.get("fallback") else "fallback"},
         "clocks": clk.summary(),

@@ -217,14 +217,13 @@ tdcfie_status tdcfie_history_stats(tdcfie_t h, int32_t* form, int64_t* nnz, doub
 
 /*
  * Several scatterers marched together (the uneven-batch case; the paper marches one scatterer).
- * Every tdcfie_batch_step advances all handles by one launch of a CUDA graph captured at the first
- * step, and each handle computes exactly what tdcfie_step computes on it (bit for bit).
+ * Every handle computes exactly what tdcfie_step computes on it (bit for bit).
  *   Persistent form, used when every handle is FP32 with one incident wave and the direct solve:
- *   the graph holds ONE cooperative kernel that walks a work list of all handles' items
- *   (plane-wave tests, per-block history partial sums of 8 rows x 4 blocks, their reduction in
- *   block order, T_0^-1 rows, projector gathers, pseudo-inverse rows, post-processing), longest
- *   items first, with a bounded grid-wide barrier between the seven phases.
- *   Graph-branch form, for any other mix: one step of every handle on its own stream branch.
+ *   ONE cooperative kernel makes up to 32 steps of all handles.  Per step it walks the history rows
+ *   and the T_0^-1 rows of every handle; where a handle's chunk of steps starts, the plane-wave tests
+ *   and pre-sums of the chunk; where a chunk or the kernel ends, the post-processing of its steps;
+ *   with a bounded grid-wide barrier between the phases.
+ *   Graph-branch form, for any other mix: one CUDA graph per step, every handle on its own branch.
  *
  * tdcfie_batch_create: handles (host array of n assembled handles on one device, each at most once)
  * are borrowed, not owned: destroy the batch before any of them, and re-create it after
@@ -232,13 +231,14 @@ tdcfie_status tdcfie_history_stats(tdcfie_t h, int32_t* form, int64_t* nnz, doub
  * tdcfie_batch_step: every handle must have its excitation set; currents_out is NULL (discard) or a
  * host array of n DEVICE pointers laid out as in tdcfie_step for each handle (entries may be NULL).
  * Synchronous; a member's non-finite current or device timeout is returned with its index.
- * tdcfie_batch_tune (persistent form): times every candidate launch shape (rows per warp 1/2/4,
- * 128/256/512 threads per block, 1/2/4 blocks per SM within the occupancy limit) for
- * steps_per_candidate steps each and keeps the fastest; the candidates march the members, which
+ * tdcfie_batch_tune (persistent form): times every candidate launch shape (units per turn of a warp
+ * 1/2/4, 64/128/256 threads per block, 1/2/4 blocks per SM within the occupancy limit) for
+ * steps_per_candidate steps each (rounded up to a multiple of 16) and keeps the fastest; the candidates march the members, which
  * are then reset to the start of their march (as tdcfie_set_excitation does).  config (host, 4
- * int32, may be NULL) receives {persistent 1/0, rows per warp, threads per block, blocks per SM}.
+ * int32, may be NULL) receives {persistent 1/0, units per turn, threads per block, blocks per SM}.
  * For the graph-branch form it only reports {0, ...}.
- * tdcfie_batch_timing: device time per batch step of the last call and kernel launches per step.
+ * tdcfie_batch_timing: device time per batch step of the last call and kernel launches per step
+ * (rounded up: 1 in the persistent form).
  */
 typedef struct tdcfie_batch_s* tdcfie_batch_t;
 tdcfie_status tdcfie_batch_create(const tdcfie_t* handles, int64_t n, tdcfie_batch_t* out);
@@ -295,8 +295,10 @@ tdcfie_status tdcfie_bc_table(tdcfie_t h, int64_t* nentries, int32_t* fine_tri, 
  *   11: Phi_k (nc x nc, the charge-potential matrix with H_k = Sigma Phi_k Sigma^T). */
 tdcfie_status tdcfie_get_matrix(tdcfie_t h, int which, int64_t k, double* host_out);
 
-/* Device time (ms, CUDA events on the handle's stream) of the last tdcfie_step call and of its
- * history-sum kernels alone; history_bytes = algorithmic bytes those kernels stream per step. */
+/* Device time (ms per step) of the last tdcfie_step call (CUDA events on the handle's stream) and of its
+ * history-sum kernels alone (device timer); history_bytes = algorithmic bytes of the history sum per
+ * step.  The dense FP64 and FP32 paths take the older lags of several steps in one pass over the
+ * blocks, so what they stream per step is less than that. */
 tdcfie_status tdcfie_last_timing(tdcfie_t h, double* step_ms, double* history_ms, double* history_bytes,
                                  int64_t* kernel_launches);
 

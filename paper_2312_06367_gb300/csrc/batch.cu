@@ -1,17 +1,17 @@
 // Several scatterers marched together (the uneven batch).  Two forms, chosen at creation:
 //
 //  * Persistent (every member FP32, one incident wave, direct solve: the uneven-batch workload):
-//    ONE cooperative kernel per step runs the phases of the step of every member -- where a chunk
-//    starts, the envelopes, tests and pre-sums of its steps; the history rows inside the chunk, T_0^-1
-//    rows, projector gathers, pseudo-inverse rows, post-processing -- with grid-wide barriers in
-//    between.  The units of a phase (rows, edges, triangles of all members) are dealt to the warps in
+//    ONE cooperative kernel runs the phases of up to B_STEPS steps of every member -- where a chunk
+//    starts, the envelopes, tests and pre-sums of its steps; the history rows inside the chunk and the
+//    T_0^-1 rows of every step; where a chunk or the call ends, the post-processing of its steps
+//    together -- with grid-wide barriers in between.  The units of a phase (rows, edges, triangles of all members) are dealt to the warps in
 //    turn, so that every member spreads over the whole grid; no unit waits for a counter.  The
 //    arithmetic is that of the per-handle step (simt.h), so every member's currents equal those of
 //    tdcfie_step bit for bit.  Units per turn, warps per block and blocks per SM come from a
 //    measuring autotuner (tdcfie_batch_tune).
 //  * Graph branches (any other mix of precisions, waves or solvers): one CUDA graph holds one step
 //    of every handle, each on its own forked stream.
-// Either way a single graph launch advances all members; the handles keep their own blocks,
+// Either way a single launch advances all members; the handles keep their own blocks,
 // rings and step counters.  Every grid-wide wait is bounded (%globaltimer, 2 s) and reports
 // TDCFIE_E_TIMEOUT.
 #include <algorithm>
@@ -27,13 +27,13 @@ using namespace tdc;
 namespace tdc {
 
 enum { PH_ENV = 0, PH_GATHER, PH_PRE, PH_HIST, PH_SOLVE, PH_PIN, PH_PINV, PH_POUT, NPH };
-constexpr uint64_t BWAIT_NS = 2000000000ull;
+constexpr int64_t B_STEPS = 32;      // steps per kernel
 
 struct BArgs {
     const SimtDev<float>* mem;
     int nmem;
     const int* first[NPH];   // first unit of every member in a phase, [nmem + 1]
-    unsigned* sync;          // arrival count, generation, timeout flag
+    unsigned long long* sync;      // arrivals so far, timeout flag
 };
 
 // units of a phase for one member (one warp works on a unit)
@@ -43,91 +43,93 @@ static int phase_units(const StepPlan* p, int ph) {
         case PH_ENV: return up((int64_t)p->npts * p->C, 32);
         case PH_GATHER: return p->ne;
         case PH_PRE: return up(p->ne, pre_rows<float>()) * p->ngroups * up(p->C, PRE_COLS);
-        case PH_PIN: return up(p->nc, 32);
-        case PH_PINV: return up(p->nc, pre_rows<float>());
-        case PH_POUT: return up(p->ne, 32);
+        // post-processing: all columns of a chunk
+        case PH_PIN: return up(p->nc, 32) * p->C;
+        case PH_PINV: return up(p->nc, pre_rows<float>()) * up(p->C, PRE_COLS);
+        case PH_POUT: return up(p->ne, 32) * p->C;
         // rows of the history, of every lag that may be pushed, and of the solve
         case PH_HIST: return up(p->ne, step_rows<1>()) * (1 + std::max(0, std::min(p->C - 1, p->K - 1) - 1));
         default: return p->ne;
     }
 }
 
-// grid-wide barrier of the co-resident blocks (cooperative launch); bounded spin
-__device__ __forceinline__ void grid_barrier(unsigned* sync) {
-    volatile unsigned* gen = sync + 1;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const unsigned g = *gen;
-        __threadfence();
-        if (atomicAdd(sync, 1u) == gridDim.x - 1) {
-            *sync = 0;
-            __threadfence();
-            atomicAdd(sync + 1, 1u);
-        } else {
-            const uint64_t t0 = device_ns();
-            while (*gen == g) {
-                if (device_ns() - t0 > BWAIT_NS) {
-                    atomicExch(sync + 2, 1u);
-                    break;
-                }
-            }
-        }
-        __threadfence();
-    }
-    __syncthreads();
-}
-
-__device__ __forceinline__ void batch_unit(int ph, const SimtDev<float>& d, int u, int lane) {
-    const int64_t n = d.ctl->n;
+// u: the unit; t: steps since the kernel's first (the step counters stay until its end); np: steps to
+// post-process, the last of them this one
+__device__ __forceinline__ void batch_unit(int ph, const SimtDev<float>& d, int t, int np, int u, int lane) {
+    const Ctl* c = d.ctl;
+    StepPos pos{c->n + t, (c->slot + t) % d.ring, (c->col + t) % d.C};
     if (ph == PH_ENV) {
         const int idx = 32 * u + lane;
         if (idx < d.npts * d.C) {
             const int i = idx % d.C, pt = idx / d.C;
-            d.env[idx] = env_point<float>(d.exc, n + i, d.dt, d.pts[3 * pt], d.pts[3 * pt + 1], d.pts[3 * pt + 2]);
+            d.env[idx] = env_point<float>(d.exc, pos.n + i, d.dt, d.pts[3 * pt], d.pts[3 * pt + 1], d.pts[3 * pt + 2]);
         }
     } else if (ph == PH_GATHER) {
         gather_edge<float>(d, u, 0, lane);
     } else if (ph == PH_PRE) {
-        const int ctiles = (d.C + PRE_COLS - 1) / PRE_COLS, t = u % ctiles, g = u / ctiles % d.ngroups;
-        pre_item<float>(d, d.ctl->slot, u / ctiles / d.ngroups * pre_rows<float>(), g, t * PRE_COLS, lane);
+        const int ctiles = (d.C + PRE_COLS - 1) / PRE_COLS, q = u % ctiles, g = u / ctiles % d.ngroups;
+        pre_item<float>(d, pos.slot, u / ctiles / d.ngroups * pre_rows<float>(), g, q * PRE_COLS, lane);
     } else if (ph == PH_HIST) {
-        hist_unit<float, 1>(d, step_pos(d, 0), u, lane, true, Nothing());
+        hist_unit<float, 1>(d, pos, u, lane, true, Nothing());
     } else if (ph == PH_SOLVE) {
-        solve_unit<float, 1>(d, step_pos(d, 0), u, lane, Nothing());
-    } else if (ph == PH_PIN) {
-        if (32 * u + lane < d.nc) pin_value<float>(d, n, d.ctl->slot, 0, 0, 32 * u + lane);
+        solve_unit<float, 1>(d, pos, u, lane, Nothing());
     } else if (ph == PH_PINV) {
-        pinv_item<float>(d, 1, u * pre_rows<float>(), 0, lane);
+        const int ctiles = (d.C + PRE_COLS - 1) / PRE_COLS, col0 = u % ctiles * PRE_COLS;
+        if (col0 < np) pinv_item<float>(d, np, u / ctiles * pre_rows<float>(), col0, lane);
     } else {
-        if (32 * u + lane < d.ne) pout_value<float>(d, n, d.ctl->slot, 0, 0, 32 * u + lane);
+        const int len = ph == PH_PIN ? d.nc : d.ne, per = (len + 31) / 32, q = u / per, i = (u - q * per) * 32 + lane;
+        if (q >= np || i >= len) return;
+        const int back = np - 1 - q, slot = ring_at(pos.slot, -back, d.ring);
+        if (ph == PH_PIN) pin_value<float>(d, pos.n - back, slot, q, 0, i);
+        else pout_value<float>(d, pos.n - back, slot, q, 0, i);
     }
 }
 
-// one MOT step of every member; rows: consecutive units per turn of a warp
-__global__ void __launch_bounds__(256) k_batch_step(const __grid_constant__ BArgs a, int rows) {
+// `steps` MOT steps of every member; rows: consecutive units per turn of a warp.  Launches and barriers
+// bound it: five members of uneven size took 44 us a step with a kernel per step and the post-processing
+// in each (six barriers), 28 us with two phases a step.
+__global__ void __launch_bounds__(256) k_batch_step(const __grid_constant__ BArgs a, int rows, int steps) {
+    extern __shared__ int2 mcol[];      // (column of the first step, C) of every member
+    __shared__ int failed;
+    if (threadIdx.x == 0) failed = (int)a.sync[1];      // an earlier kernel's wait ran out
+    for (int s = threadIdx.x; s < a.nmem; s += blockDim.x) mcol[s] = make_int2(a.mem[s].ctl->col, a.mem[s].C);
+    __syncthreads();
+    if (failed) return;
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    bool start = false;      // some member starts a chunk (uniform: no counter moves before the end)
-    for (int s = 0; s < a.nmem; ++s) start |= a.mem[s].ctl->col == 0;
-    for (int ph = start ? PH_ENV : PH_HIST; ph < NPH; ++ph) {
-        const int* first = a.first[ph];
-        const int total = first[a.nmem];
-        int s = 0;
-        for (int64_t u0 = warp * rows; u0 < total; u0 += nwarps * rows)
-            for (int64_t u = u0; u < min(u0 + rows, (int64_t)total); ++u) {
-                while (u >= first[s + 1]) ++s;
-                const SimtDev<float>& d = a.mem[s];
-                if (ph <= PH_PRE && d.ctl->col != 0) continue;
-                batch_unit(ph, d, (int)(u - first[s]), lane);
-            }
-        grid_barrier(a.sync);
+    for (int t = 0; t < steps; ++t) {
+        bool starts = false, ends = t == steps - 1;      // some member starts, ends a chunk
+        for (int s = threadIdx.x; s < a.nmem; s += blockDim.x) {
+            const int col = (mcol[s].x + t) % mcol[s].y;
+            starts |= col == 0;
+            ends |= col == mcol[s].y - 1;
+        }
+        starts = __syncthreads_or(starts);
+        ends = __syncthreads_or(ends);
+        for (int ph = starts ? PH_ENV : PH_HIST; ph < (ends ? NPH : PH_PIN); ++ph) {
+            const int* first = a.first[ph];
+            const int total = first[a.nmem];
+            int s = 0;
+            for (int64_t u0 = warp * rows; u0 < total; u0 += nwarps * rows)
+                for (int64_t u = u0; u < min(u0 + rows, (int64_t)total); ++u) {
+                    while (u >= first[s + 1]) ++s;
+                    const int C = mcol[s].y, col = (mcol[s].x + t) % C;
+                    if (ph <= PH_PRE && col != 0) continue;
+                    if (ph >= PH_PIN && col != C - 1 && t != steps - 1) continue;
+                    batch_unit(ph, a.mem[s], t, min(t, col) + 1, (int)(u - first[s]), lane);
+                }
+            if (!group_barrier(a.sync, gridDim.x, a.sync + 1, &failed)) return;
+        }
     }
     // every block has passed the last barrier: advance the members
     if (blockIdx.x == 0)
         for (int s = threadIdx.x; s < a.nmem; s += blockDim.x) {
-            advance(a.mem[s], 1);
-            a.mem[s].ctl->p0 = a.mem[s].ctl->n;
+            const SimtDev<float>& d = a.mem[s];
+            d.ctl->n += steps;
+            d.ctl->slot = (d.ctl->slot + steps) % d.ring;
+            d.ctl->col = (d.ctl->col + steps) % d.C;
+            d.ctl->p0 = d.ctl->n;
         }
 }
 
@@ -160,7 +162,7 @@ struct tdcfie_batch_s {
     bool persistent = false;
     SimtDev<float>* dmem = nullptr;
     int* dfirst = nullptr;
-    unsigned* dsync = nullptr;
+    unsigned long long* dsync = nullptr;
     void** douts = nullptr;       // the members' output pointers of a call
     Ctl* dstat = nullptr;         // the members' step states after a call
     BArgs args{};
@@ -188,23 +190,37 @@ static bool persistent_member(tdcfie_t h) {
     return h->plan && h->plan->prec == TDCFIE_FP32 && h->plan->R == 1 && !h->plan->gmres_on && h->plan->blocks;
 }
 
-static cudaError_t launch_persistent(tdcfie_batch_t b, cudaStream_t s) {
+// nsteps steps of the members with the batch's configuration
+static cudaError_t launch_persistent(tdcfie_batch_t b, int64_t nsteps, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(b->grid);
     cfg.blockDim = dim3(b->threads);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = b->hs.size() * sizeof(int2);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_batch_step, b->args, b->rows);
+    cudaError_t e = cudaSuccess;
+    for (; nsteps > 0 && e == cudaSuccess; nsteps -= B_STEPS)
+        e = cudaLaunchKernelEx(&cfg, k_batch_step, b->args, b->rows, (int)std::min(nsteps, B_STEPS));
+    return e;
 }
 
-static int max_blocks_per_sm(int threads) {
+static int max_blocks_per_sm(tdcfie_batch_t b, int threads) {
     int nb = 0;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_step, threads, 0) == cudaSuccess ? nb : 0;
+    const size_t smem = b->hs.size() * sizeof(int2);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_step, threads, smem) == cudaSuccess ? nb : 0;
+}
+
+// the kernel's launch shape; the barrier's count starts again, it is a multiple of the grid
+static cudaError_t set_shape(tdcfie_batch_t b, int rows, int threads, int blocks_per_sm) {
+    b->rows = rows;
+    b->threads = threads;
+    b->blocks_per_sm = blocks_per_sm;
+    b->grid = b->sms * blocks_per_sm;
+    return cudaMemsetAsync(b->dsync, 0, sizeof(unsigned long long), b->main);
 }
 
 // members' views and the units of every phase
@@ -222,12 +238,12 @@ static cudaError_t build_persistent(tdcfie_batch_t b) {
     cudaError_t e;
     if ((e = cudaMalloc(&b->dmem, sizeof(SimtDev<float>) * n)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->dfirst, sizeof(int) * first.size())) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&b->dsync, sizeof(unsigned) * 3)) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&b->dsync, sizeof(unsigned long long) * 2)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->douts, sizeof(void*) * n)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->dstat, sizeof(Ctl) * n)) != cudaSuccess) return e;
     if ((e = cudaMemcpy(b->dmem, mem.data(), sizeof(SimtDev<float>) * n, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
     if ((e = cudaMemcpy(b->dfirst, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
-    if ((e = cudaMemset(b->dsync, 0, sizeof(unsigned) * 3)) != cudaSuccess) return e;
+    if ((e = cudaMemset(b->dsync, 0, sizeof(unsigned long long) * 2)) != cudaSuccess) return e;
     b->args.mem = b->dmem;
     b->args.nmem = n;
     for (int ph = 0; ph < NPH; ++ph) b->args.first[ph] = b->dfirst + ph * (n + 1);
@@ -235,11 +251,7 @@ static cudaError_t build_persistent(tdcfie_batch_t b) {
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    b->rows = 1;
-    b->threads = 256;
-    b->blocks_per_sm = 1;
-    b->grid = b->sms;
-    return cudaSuccess;
+    return set_shape(b, 1, 256, 1);
 }
 }  // namespace tdc
 
@@ -303,25 +315,21 @@ extern "C" tdcfie_status tdcfie_batch_step(tdcfie_batch_t b, int64_t nsteps, voi
             if (st != TDCFIE_OK) return fail(nullptr, st, "batch handle " + std::to_string(i) + ": " + b->hs[i]->err);
         }
     }
-    if (!b->exec) {
+    if (b->persistent) {
+        b->launches_per_step = 1;      // one launch steps every member, and up to B_STEPS steps
+    } else if (!b->exec) {
         e = cudaStreamBeginCapture(b->main, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaStreamBeginCapture");
         cudaError_t ce = cudaSuccess;
-        if (b->persistent) {
-            // one cooperative launch steps every member
-            ce = launch_persistent(b, b->main);
-            b->launches_per_step = 1;
-        } else {
-            // one step of every handle, each on its own branch of the graph
-            ce = cudaEventRecord(b->fork, b->main);
-            b->launches_per_step = 0;
-            for (int64_t i = 0; i < n && ce == cudaSuccess; ++i) {
-                ce = cudaStreamWaitEvent(b->branch[i], b->fork, 0);
-                if (ce == cudaSuccess) ce = capture_step(b->hs[i], b->branch[i]);
-                if (ce == cudaSuccess) ce = cudaEventRecord(b->joined[i], b->branch[i]);
-                if (ce == cudaSuccess) ce = cudaStreamWaitEvent(b->main, b->joined[i], 0);
-                b->launches_per_step += plan_launches_per_step(b->hs[i]);
-            }
+        // one step of every handle, each on its own branch of the graph
+        ce = cudaEventRecord(b->fork, b->main);
+        b->launches_per_step = 0;
+        for (int64_t i = 0; i < n && ce == cudaSuccess; ++i) {
+            ce = cudaStreamWaitEvent(b->branch[i], b->fork, 0);
+            if (ce == cudaSuccess) ce = capture_step(b->hs[i], b->branch[i]);
+            if (ce == cudaSuccess) ce = cudaEventRecord(b->joined[i], b->branch[i]);
+            if (ce == cudaSuccess) ce = cudaStreamWaitEvent(b->main, b->joined[i], 0);
+            b->launches_per_step += plan_launches_per_step(b->hs[i]);
         }
         const cudaError_t ee = cudaStreamEndCapture(b->main, &b->graph);
         if (ce != cudaSuccess || ee != cudaSuccess) {
@@ -332,14 +340,15 @@ extern "C" tdcfie_status tdcfie_batch_step(tdcfie_batch_t b, int64_t nsteps, voi
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaGraphInstantiate (batch)");
     }
     std::vector<Ctl> ctl(n);
-    unsigned timeout = 0;
+    unsigned long long timeout = 0;
     e = cudaEventRecord(b->t0, b->main);
-    for (int64_t i = 0; i < nsteps && e == cudaSuccess; ++i) e = cudaGraphLaunch(b->exec, b->main);
+    if (b->persistent && e == cudaSuccess) e = launch_persistent(b, nsteps, b->main);
+    for (int64_t i = 0; !b->persistent && i < nsteps && e == cudaSuccess; ++i) e = cudaGraphLaunch(b->exec, b->main);
     if (e == cudaSuccess) e = cudaEventRecord(b->t1, b->main);
     if (e == cudaSuccess && b->persistent) {
         k_batch_status<<<1, 256, 0, b->main>>>(b->args, b->dstat);
         e = cudaMemcpyAsync(ctl.data(), b->dstat, sizeof(Ctl) * n, cudaMemcpyDeviceToHost, b->main);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&timeout, b->dsync + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, b->main);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&timeout, b->dsync + 1, sizeof timeout, cudaMemcpyDeviceToHost, b->main);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->main);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch step");
@@ -373,13 +382,13 @@ extern "C" tdcfie_status tdcfie_batch_tune(tdcfie_batch_t b, int64_t steps_per_c
         int br = b->rows, bt = b->threads, bb = b->blocks_per_sm;
         for (int rows : {1, 2, 4})
             for (int threads : {64, 128, 256}) {
-                const int maxb = max_blocks_per_sm(threads);
+                const int maxb = max_blocks_per_sm(b, threads);
                 for (int bps : {1, 2, 4}) {
                     if (bps > maxb) continue;
-                    b->rows = rows; b->threads = threads; b->blocks_per_sm = bps; b->grid = b->sms * bps;
-                    e = launch_persistent(b, b->main);                        // warm-up
+                    e = set_shape(b, rows, threads, bps);
+                    if (e == cudaSuccess) e = launch_persistent(b, 1, b->main);                        // warm-up
                     if (e == cudaSuccess) e = cudaEventRecord(b->t0, b->main);
-                    for (int64_t i = 0; i < steps_per_candidate && e == cudaSuccess; ++i) e = launch_persistent(b, b->main);
+                    if (e == cudaSuccess) e = launch_persistent(b, steps_per_candidate, b->main);
                     if (e == cudaSuccess) e = cudaEventRecord(b->t1, b->main);
                     if (e == cudaSuccess) e = cudaStreamSynchronize(b->main);
                     if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch autotuner");
@@ -388,11 +397,10 @@ extern "C" tdcfie_status tdcfie_batch_tune(tdcfie_batch_t b, int64_t steps_per_c
                     if (ms < best) { best = ms; br = rows; bt = threads; bb = bps; }
                 }
             }
-        b->rows = br; b->threads = bt; b->blocks_per_sm = bb; b->grid = b->sms * bb;
-        if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
-        if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
-        unsigned timeout = 0;
-        e = cudaMemcpy(&timeout, b->dsync + 2, sizeof(unsigned), cudaMemcpyDeviceToHost);
+        e = set_shape(b, br, bt, bb);
+        if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch autotuner");
+        unsigned long long timeout = 0;
+        e = cudaMemcpy(&timeout, b->dsync + 1, sizeof timeout, cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch status");
         if (timeout) return fail(nullptr, TDCFIE_E_TIMEOUT, "a bounded grid-wide wait of the batch kernel ran out");
         // the candidates marched the members: back to the start of the march
