@@ -1,0 +1,191 @@
+"""GPU: the blocked march, the group GMRES, the quadrature's windows, the history sum's row tiles and the
+training step at the sizes where their splits can go wrong: chunks that start or stop anywhere, fewer
+lags than a chunk has steps, rows that no vector load fits, waves that fill no tile.
+
+Tolerances are those of the paths elsewhere in the suite (FP64 1e-10 against the oracle, FP32 and FP16X3
+1e-5, BF16X3 not used here); results that depend on no rounding order are compared bit for bit."""
+import numpy as np
+import pytest
+
+from synth import excitation, meshes
+
+pytestmark = pytest.mark.gpu
+
+
+def rel(a, b):
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+def _oracle(mesh, dt, nt, pw):
+    """The oracle's march on the library's FP64 matrices.  (The matrices have their own tests, on spheres
+    for the 1e-10 bar: on this coarse torus the oracle's quadrature itself is good to some 1e-10.)"""
+    from oracle import mot, rhs
+    from oracle.assemble import Operators
+    from oracle.formulation import Formulation
+    ops = Operators(*mesh, dt=dt)
+    s = _solver(mesh, dt, nt, 1, "fp64")
+    for name in ("G", "Zs", "Zh", "M"):
+        setattr(ops, name, s.matrix(name, 0))
+    for name in ("S", "H", "MM"):
+        setattr(ops, name, np.stack([s.matrix(name, k) for k in range(ops.K)]))
+    s.close()
+    fm = Formulation(ops)
+    e, h = rhs.incident_tests(ops, pw, dt * np.arange(1, nt + 1))
+    return fm.postprocess(mot.march_factored(fm, fm.rhs(e, h)))
+
+
+def _solver(mesh, dt, nt, R, precision, **kw):
+    from paper_2312_06367_gb300 import Solver
+    return Solver(*mesh, dt=dt, nt=nt, R=R, precision=precision, **kw).assemble()
+
+
+SMALL = meshes.torus(1.0, 0.4, 5, 3)      # 45 edges: odd rows, fewer than a block of any kernel
+BOUND = {"fp64": 1e-10, "fp32": 1e-5}
+# (dt, steps): more lags than a chunk has steps; as few lags as there can be; a chunk and one step
+SPLITS = [(0.15, 35), (4.0, 18), (0.8, 17)]
+
+
+@pytest.fixture(scope="module")
+def waves():
+    return excitation.random_batch(8, seed=31, t0=3.0, sigma=0.8)
+
+
+@pytest.fixture(scope="module")
+def refs(waves):
+    return {dt: _oracle(SMALL, dt, nt, waves) for dt, nt in SPLITS}
+
+
+@pytest.mark.parametrize("dt,nt", SPLITS)
+@pytest.mark.parametrize("precision,R", [("fp64", 1), ("fp64", 8), ("fp32", 2), ("fp32", 3), ("fp32", 8)])
+def test_march_in_chunks(waves, refs, precision, R, dt, nt):
+    """Against the oracle, and any partition of the steps gives the same bits."""
+    import torch
+    pw = {k: v[:R] for k, v in waves.items()}
+    s = _solver(SMALL, dt, nt, R, precision)
+    out = torch.zeros((nt, R, s.ne), dtype=s.dtype, device="cuda")
+    s.march(pw, out)
+    parts = torch.zeros_like(out)
+    s.set_excitation(pw)
+    at = 0
+    for m in (1, 7, 9, 2, nt):
+        m = min(m, nt - at)
+        s.step(m, parts[at:at + m])
+        at += m
+    torch.cuda.synchronize()
+    assert torch.equal(out, parts)
+    if precision == "fp64" or dt > 0.15:      # FP32 at 0.15 on this mesh: 2e-5 to 4e-5 by the path's rounding
+        assert rel(out.double().cpu().numpy().transpose(0, 2, 1), refs[dt][:, :, :R]) < BOUND[precision]
+
+
+@pytest.mark.parametrize("precision,R", [("fp64", 1), ("fp64", 3), ("fp32", 1), ("fp32", 8)])
+def test_group_gmres(waves, refs, precision, R):
+    """Restarts after three iterations, one group of blocks per wave; partitions give the same bits."""
+    import torch
+    dt, nt = SPLITS[0 if precision == "fp64" else 2]
+    pw = {k: v[:R] for k, v in waves.items()}
+    s = _solver(SMALL, dt, nt, R, precision, solver="gmres", guess="extrap", gmres_restart=3, gmres_maxit=300,
+                gmres_tol=1e-13 if precision == "fp64" else 1e-9)
+    out = torch.zeros((nt, R, s.ne), dtype=s.dtype, device="cuda")
+    s.march(pw, out)
+    st = s.gmres_stats()
+    parts = torch.zeros_like(out)
+    s.set_excitation(pw)
+    s.step(11, parts[:11])
+    s.step(nt - 11, parts[11:])
+    torch.cuda.synchronize()
+    assert st["steps"] == nt and st["not_converged"] == 0
+    assert torch.equal(out, parts)
+    assert rel(out.double().cpu().numpy().transpose(0, 2, 1), refs[dt][:, :, :R]) < BOUND[precision]
+
+
+@pytest.mark.parametrize("precision", ["fp16x3", "bf16x3"])
+def test_tensor_chunks(precision):
+    """45 edges (one ragged tile): partitions of the steps, and repetitions, give the same bits."""
+    import torch
+    nt = 14
+    pw = excitation.fibonacci_batch(64, seed=5, t0=3.0, sigma=0.8)
+    s = _solver(meshes.icosphere(0), 0.4, nt, 64, precision)
+    out = torch.zeros((nt, 64, s.ne), dtype=s.dtype, device="cuda")
+    s.march(pw, out)
+    for split in ((1, 2, 3, 4, 4), (5, 9), (14,), (14,)):
+        parts = torch.zeros_like(out)
+        s.set_excitation(pw)
+        at = 0
+        for m in split:
+            s.step(m, parts[at:at + m])
+            at += m
+        torch.cuda.synchronize()
+        assert torch.isfinite(out).all() and torch.equal(out, parts), split
+
+
+@pytest.mark.parametrize("time_order", [1, 2])
+@pytest.mark.parametrize("dt", [0.02, 0.11, 5.0])
+def test_quadrature_windows(dt, time_order):
+    """Lags per pair from one to several windows, on 30 edges."""
+    from oracle.assemble import Operators
+    V, F = meshes.icosphere(0)
+    ops = Operators(V, F, dt=dt, time_order=time_order)
+    s = _solver((V, F), dt, 4, 1, "fp64", time_order=time_order)
+    for k in range(0, ops.K, max(1, ops.K // 6)):
+        for name, ref in (("S", ops.S[k]), ("H", ops.H[k]), ("MM", ops.MM[k])):
+            got = s.matrix(name, k)
+            scale = max(np.linalg.norm(x) for x in {"S": ops.S, "H": ops.H, "MM": ops.MM}[name])
+            # an almost empty block at the end of the lags is held to the largest block's scale
+            assert np.linalg.norm(got - ref) <= 1e-10 * max(np.linalg.norm(ref), 1e-3 * scale), (name, k)
+
+
+@pytest.mark.parametrize("dtype,tol", [("float64", 1e-13), ("float32", 1e-5)])
+@pytest.mark.parametrize("nblk,n,R,off", [(2, 4, 1, 0), (3, 130, 2, 0), (3, 132, 2, 1), (2, 65, 4, 0), (9, 516, 5, 0), (9, 257, 8, 0)])
+def test_block_gemv_row_tiles(dtype, tol, nblk, n, R, off):
+    """Vector and scalar loads (odd rows, blocks off the 16-byte boundary), rows that fill no tile."""
+    import torch
+    from paper_2312_06367_gb300 import block_gemv
+    g = torch.Generator(device="cuda").manual_seed(nblk * n + R)
+    dt = getattr(torch, dtype)
+    B = torch.randn(nblk * n * n + off, generator=g, dtype=dt, device="cuda")[off:].view(nblk, n, n)
+    X = torch.randn((nblk, R, n), generator=g, dtype=dt, device="cuda")
+    ref = torch.einsum("qij,qrj->ri", B.double(), X.double())
+    got = block_gemv(B, X)
+    torch.cuda.synchronize()
+    assert float((got.double() - ref).norm() / ref.norm()) < tol
+
+
+@pytest.mark.parametrize("n,epochs", [(1, 1), (31, 2), (1000, 5)])
+def test_training_updates(n, epochs):
+    """One batch per pass: the parameters after 1, 2 and 5 updates against Adam on the oracle's
+    gradient.  An update moves a parameter by lr g / |g| at most, with g good to 1e-4."""
+    import torch
+    from oracle import mlp
+    from paper_2312_06367_gb300 import mlp_train
+    rng = np.random.default_rng(n)
+    X = rng.standard_normal((n, 8)).astype(np.float32)
+    Y = np.tanh(X @ rng.standard_normal(8)).astype(np.float32)
+    p = torch.tensor(mlp.init_params(2), dtype=torch.float32, device="cuda")
+    q = p.double().cpu().numpy()
+    hist = mlp_train(p, torch.tensor(X, device="cuda"), torch.tensor(Y, device="cuda"), epochs=epochs, batch=4096, lr=1e-3)
+    m1, m2 = np.zeros_like(q), np.zeros_like(q)
+    for k in range(1, epochs + 1):
+        loss, g = mlp.loss_and_grad(q, X.astype(np.float64), Y.astype(np.float64))
+        assert abs(hist[k - 1] - loss) <= 1e-4 * loss
+        m1, m2 = 0.9 * m1 + 0.1 * g, 0.999 * m2 + 0.001 * g * g
+        q = q - 1e-3 * (m1 / (1 - 0.9 ** k)) / (np.sqrt(m2 / (1 - 0.999 ** k)) + 1e-8)
+    assert rel(p.double().cpu().numpy(), q) < 1e-4
+
+
+def test_batch_before_excitation(waves):
+    """A batch made of handles without an excitation yet."""
+    import torch
+    from paper_2312_06367_gb300 import Batch
+    pw = {k: v[:1] for k, v in waves.items()}
+    ss = [_solver(SMALL, 0.15, 20, 1, "fp32"), _solver(meshes.icosphere(0), 0.3, 20, 1, "fp32")]
+    b = Batch(ss)
+    for s in ss:
+        s.set_excitation(pw)
+    outs = [torch.zeros((20, 1, s.ne), dtype=torch.float32, device="cuda") for s in ss]
+    b.step(20, outs)
+    b.close()
+    for s, o in zip(ss, outs):
+        ref = torch.zeros_like(o)
+        s.march(pw, ref)
+        torch.cuda.synchronize()
+        assert torch.equal(o, ref)
