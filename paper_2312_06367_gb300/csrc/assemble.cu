@@ -606,7 +606,9 @@ struct EfieAcc {
 // pair has about 30 of them), so the lanes have to be full and nothing may be computed twice; the
 // queue of sub-pieces above is for that.  The sums of an interval of length dt are moments in v,
 // turned into lags at the end, so that a node costs its own few multiply-adds whatever the number of
-// lags.  Pairs that meet more than lagw lags take them in several windows.
+// lags.  Pairs that meet more than lagw lags take them in several windows.  480-edge sphere, 7 lags: the
+// whole assembly 1524 -> 178 ms against one thread per pair, with the rays' intervals one by one and library
+// functions at every node.
 template <int ORDER>
 __global__ void __launch_bounds__(AB) k_retarded_efie(DevMesh m, double dt, int K, int lagw, double T0, double* __restrict__ S,
                                                       double* __restrict__ Phi) {

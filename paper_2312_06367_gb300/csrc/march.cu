@@ -317,7 +317,8 @@ tdcfie_status build_plan(tdcfie_t h) {
     // Steps per chunk.  Matrix blocks read per step: (K + 1) / C + (C - 1) / 2 + 1 + 1 / C, least near
     // C = sqrt(2 (K + 2)) = 9 at K = 42; where everything sits in L2 (up to about 1000 edges) the
     // kernels per chunk count, not the bytes, and 16 steps share them.  The tests' kernel needs a
-    // divisor of 32.
+    // divisor of 32.  Against every block in every step: 480 edges FP64 232 -> 20 us per step, 1920 edges
+    // FP32 243 -> 74 us, with eight waves 990 -> 490 us.
     p->C = tensor ? tc_chunk() : (ne <= 1024 && R <= 2 ? 16 : 8);
     p->ring = tensor ? h->K - 1 : h->K - 1 + p->C;
     const int vw = (int)(16 / es);      // elements per 16-byte vector

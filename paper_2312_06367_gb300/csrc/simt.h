@@ -316,7 +316,7 @@ __device__ __forceinline__ bool multi_owner(int lane) { return (lane & (32 / V -
 constexpr int PRE_COLS = 8;
 // rows per unit: two on the FP64 path (32 accumulator registers, the row's columns share the loads), one
 // on the FP32 path, whose pair accumulators would leave 8 warps per SM at two rows (fused multiply-add
-// pipe 62 % busy, 543 us for 8 columns at 1920 edges, K = 42)
+// pipe 62 % busy, 543 us for 8 columns at 1920 edges, K = 42; 433 us with one)
 template <typename T> constexpr int pre_rows() { return sizeof(T) == 8 ? 2 : 1; }
 
 // Rows row0 .. row0 + pre_rows - 1, columns col0 .. col0 + 7 and group g of the blocks in the order e, h,
