@@ -278,6 +278,17 @@ __device__ __forceinline__ void two_sum_acc2(float2& hi, float2& lo, float2 v) {
     hi = t;
 }
 
+// the same for the product a b, unrounded
+__device__ __forceinline__ void two_sum_fma2(float2& hi, float2& lo, float2 a, float2 b) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 t = __ffma2_rn(a, b, hi);
+    const float2 bp = __ffma2_rn(hi, m1, t);                                    // t - hi
+    const float2 e1 = __ffma2_rn(__ffma2_rn(bp, m1, t), m1, hi);                // hi - (t - bp)
+    const float2 e2 = __ffma2_rn(a, b, make_float2(-bp.x, -bp.y));              // a b - bp
+    lo = __fadd2_rn(lo, __fadd2_rn(e1, e2));
+    hi = t;
+}
+
 __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float v) {
     const float t = hi + v;
     const float bp = t - hi;
@@ -791,7 +802,7 @@ __global__ void __launch_bounds__(32 * RHS_NW) k_rhs_tc(int ne, const double* __
                 const float2 v = en[(int64_t)__float_as_int(c.w) * (TC_C * NR / 2)];
                 const float2 cp = __ffma2_rn(make_float2(c.x, c.x), pol[f][0],
                                              __ffma2_rn(make_float2(c.y, c.y), pol[f][1], __fmul2_rn(make_float2(c.z, c.z), pol[f][2])));
-                two_sum_acc2(hi, lo, __fmul2_rn(v, cp));
+                two_sum_fma2(hi, lo, v, cp);
             }
             float2* dst = ev + (f * 64 + el) * RHS_LD + 2 * lane;
             dst[0] = make_float2(hi.x, lo.x);
