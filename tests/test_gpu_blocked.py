@@ -2,8 +2,8 @@
 training step at the sizes where their splits can go wrong: chunks that start or stop anywhere, fewer
 lags than a chunk has steps, rows that no vector load fits, waves that fill no tile.
 
-Tolerances are those of the paths elsewhere in the suite (FP64 1e-10 against the oracle, FP32 and FP16X3
-1e-5, BF16X3 not used here); results that depend on no rounding order are compared bit for bit."""
+Tolerances are those of the paths elsewhere in the suite (FP64 1e-10 against the oracle, FP32
+1e-5); results that depend on no rounding order are compared bit for bit."""
 import numpy as np
 import pytest
 
@@ -100,7 +100,7 @@ def test_group_gmres(waves, refs, precision, R):
 
 @pytest.mark.parametrize("precision", ["fp16x3", "bf16x3"])
 def test_tensor_chunks(precision):
-    """45 edges (one ragged tile): partitions of the steps, and repetitions, give the same bits."""
+    """30 edges (one ragged tile): partitions of the steps, and repetitions, give the same bits."""
     import torch
     nt = 14
     pw = excitation.fibonacci_batch(64, seed=5, t0=3.0, sigma=0.8)
