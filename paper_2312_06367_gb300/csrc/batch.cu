@@ -185,6 +185,22 @@ static void destroy_batch(tdcfie_batch_t b) {
 }
 
 namespace tdc {
+// The batch's stream starts after what is queued on the members' streams (a handle's device work is
+// ordered with its opts.stream; for a stream of the library's own, with the legacy default stream, as in
+// plan_step): fills and last readers of the output buffers above all.
+static cudaError_t wait_members(tdcfie_batch_t b) {
+    cudaError_t e = cudaSuccess;
+    bool legacy = false;
+    for (size_t i = 0; i < b->hs.size() && e == cudaSuccess; ++i) {
+        tdcfie_t h = b->hs[i];
+        if (h->own_stream && legacy) continue;
+        legacy = legacy || h->own_stream;
+        e = cudaEventRecord(h->ev_in, h->own_stream ? cudaStreamLegacy : h->stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(b->main, h->ev_in, 0);
+    }
+    return e;
+}
+
 // a handle the persistent kernel can step: FP32, one wave, direct solve
 static bool persistent_member(tdcfie_t h) {
     return h->plan && h->plan->prec == TDCFIE_FP32 && h->plan->R == 1 && !h->plan->gmres_on && h->plan->blocks;
@@ -301,6 +317,8 @@ extern "C" tdcfie_status tdcfie_batch_step(tdcfie_batch_t b, int64_t nsteps, voi
     if (nsteps == 0) return TDCFIE_OK;
     cudaError_t e = cudaSetDevice(b->hs[0]->opts.device);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaSetDevice");
+    e = wait_members(b);
+    if (e != cudaSuccess) return cuda_fail(nullptr, e, "waiting for the members' streams");
     if (b->persistent) {
         // one kernel sets every member's output base
         if (currents_out) e = cudaMemcpyAsync(b->douts, currents_out, sizeof(void*) * n, cudaMemcpyHostToDevice, b->main);
