@@ -257,9 +257,9 @@ static cudaError_t build_persistent(tdcfie_batch_t b) {
     if ((e = cudaMalloc(&b->dsync, sizeof(unsigned long long) * 2)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->douts, sizeof(void*) * n)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&b->dstat, sizeof(Ctl) * n)) != cudaSuccess) return e;
-    if ((e = cudaMemcpy(b->dmem, mem.data(), sizeof(SimtDev<float>) * n, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
-    if ((e = cudaMemcpy(b->dfirst, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
-    if ((e = cudaMemset(b->dsync, 0, sizeof(unsigned long long) * 2)) != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(b->dmem, mem.data(), sizeof(SimtDev<float>) * n, cudaMemcpyHostToDevice, b->main)) != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(b->dfirst, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice, b->main)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(b->dsync, 0, sizeof(unsigned long long) * 2, b->main)) != cudaSuccess) return e;
     b->args.mem = b->dmem;
     b->args.nmem = n;
     for (int ph = 0; ph < NPH; ++ph) b->args.first[ph] = b->dfirst + ph * (n + 1);
@@ -418,7 +418,8 @@ extern "C" tdcfie_status tdcfie_batch_tune(tdcfie_batch_t b, int64_t steps_per_c
         e = set_shape(b, br, bt, bb);
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch autotuner");
         unsigned long long timeout = 0;
-        e = cudaMemcpy(&timeout, b->dsync + 1, sizeof timeout, cudaMemcpyDeviceToHost);
+        e = cudaMemcpyAsync(&timeout, b->dsync + 1, sizeof timeout, cudaMemcpyDeviceToHost, b->main);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(b->main);
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch status");
         if (timeout) return fail(nullptr, TDCFIE_E_TIMEOUT, "a bounded grid-wide wait of the batch kernel ran out");
         // the candidates marched the members: back to the start of the march

@@ -167,7 +167,10 @@ __global__ void __launch_bounds__(GM_T, 1) k_gm_solve(const __grid_constant__ Gm
     if (t == 0) failed = (int)__ldcg(d.sync + d.R);      // an earlier solve's wait ran out
     if (t == 0 && blockIdx.x == 0 && r == 0) ctl->hist_ns += device_ns() - ctl->t_mark;      // the history kernel is done
     __syncthreads();
-    if (failed) return;
+    if (failed) {
+        ctl->timeout = 1;
+        return;
+    }
     const int64_t n = ctl->n + off;
     const int64_t vec0 = (int64_t)r * d.ne;
     double* x = d.x + vec0;
@@ -352,7 +355,7 @@ cudaError_t build_gmres(tdcfie_t h, StepPlan* p) {
     if (e != cudaSuccess) return e;
     auto al = [&](double** q, size_t n) -> cudaError_t {
         cudaError_t e = cudaMalloc((void**)q, sizeof(double) * (n ? n : 1));
-        if (e == cudaSuccess) { g->owned.push_back(*q); e = cudaMemset(*q, 0, sizeof(double) * (n ? n : 1)); }
+        if (e == cudaSuccess) { g->owned.push_back(*q); e = cudaMemsetAsync(*q, 0, sizeof(double) * (n ? n : 1), h->stream); }
         return e;
     };
     if ((e = al(&d.x, (size_t)R * ne)) || (e = al(&d.r, (size_t)R * ne)) || (e = al(&d.V, (size_t)(m + 1) * R * ne)) ||
@@ -363,13 +366,14 @@ cudaError_t build_gmres(tdcfie_t h, StepPlan* p) {
     if ((e = cudaMalloc(&d.sync, sizeof(unsigned long long) * (R + 1 + NSTATS))) != cudaSuccess) return e;
     g->owned.push_back(d.sync);
     d.stats = d.sync + R + 1;
-    return reset_gmres_stats(g);
+    return reset_gmres_stats(g, h->stream);
 }
 
 void gmres_set_tol(GmresPlan* g, double tol) { g->d.tol = tol; }
 
-cudaError_t reset_gmres_stats(GmresPlan* g) {
-    return cudaMemset(g->d.sync, 0, sizeof(unsigned long long) * (g->d.R + 1 + NSTATS));
+// on the handle's stream, ahead of its next solve: the counters must stand while a solve runs
+cudaError_t reset_gmres_stats(GmresPlan* g, cudaStream_t s) {
+    return cudaMemsetAsync(g->d.sync, 0, sizeof(unsigned long long) * (g->d.R + 1 + NSTATS), s);
 }
 
 cudaError_t gmres_stats(GmresPlan* g, long long* out5) {

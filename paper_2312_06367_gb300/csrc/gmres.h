@@ -7,7 +7,7 @@ struct StepPlan;
 struct GmresPlan;
 cudaError_t build_gmres(tdcfie_t h, StepPlan* p);
 void destroy_gmres(GmresPlan* g);
-cudaError_t reset_gmres_stats(GmresPlan* g);
+cudaError_t reset_gmres_stats(GmresPlan* g, cudaStream_t s);
 void gmres_set_tol(GmresPlan* g, double tol);
 // out5: Arnoldi iterations, steps, max per step, (unused), solves not converged
 cudaError_t gmres_stats(GmresPlan* g, long long* out5);
@@ -19,7 +19,7 @@ cudaError_t launch_gmres(tdcfie_t h, StepPlan* p, const T* b, const T* learned, 
 
 // Learned initial guess (mlp.cu): FP16 weights on the device, filled into p->guessbuf each step.
 struct MlpState;
-cudaError_t build_mlp(StepPlan* p);
+cudaError_t build_mlp(StepPlan* p, cudaStream_t s);
 void destroy_mlp(MlpState* m);
 cudaError_t mlp_load(StepPlan* p, const float* host_params, cudaStream_t s);
 template <typename T>

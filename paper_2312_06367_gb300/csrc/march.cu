@@ -325,7 +325,8 @@ tdcfie_status build_plan(tdcfie_t h) {
     p->ld = (int)(ne + vw - 1) / vw * vw;
     p->ldc = (int)(nc + vw - 1) / vw * vw;
     p->ngroups = (h->K + 1 + 3) / 4;
-    // rhs quadrature tables (host, FP64), uploaded in the path precision
+    // rhs quadrature tables (host, FP64), uploaded in the path precision on the handle's stream (the legacy
+    // stream has no order to it)
     {
         const double s15 = std::sqrt(15.0);
         const double a1 = (9.0 - 2.0 * s15) / 21.0, b1 = (6.0 + s15) / 21.0, w1 = (155.0 + s15) / 1200.0;
@@ -398,11 +399,11 @@ tdcfie_status build_plan(tdcfie_t h) {
             if (!f64) vf.assign(v.begin(), v.end());
             const size_t bytes = v.size() * (f64 ? 8 : 4);
             const cudaError_t e = cudaMalloc(dst, bytes);
-            return e != cudaSuccess ? e : cudaMemcpy(*dst, f64 ? (const void*)v.data() : vf.data(), bytes, cudaMemcpyHostToDevice);
+            return e != cudaSuccess ? e : cudaMemcpyAsync(*dst, f64 ? (const void*)v.data() : vf.data(), bytes, cudaMemcpyHostToDevice, s);
         };
         auto puti = [&](int** dst, const std::vector<int>& v) -> cudaError_t {
             const cudaError_t e = cudaMalloc(dst, sizeof(int) * v.size());
-            return e != cudaSuccess ? e : cudaMemcpy(*dst, v.data(), sizeof(int) * v.size(), cudaMemcpyHostToDevice);
+            return e != cudaSuccess ? e : cudaMemcpyAsync(*dst, v.data(), sizeof(int) * v.size(), cudaMemcpyHostToDevice, s);
         };
         p->npts = (int)(X.size() / 3);
         CK(puti(&p->eptr, ptr));
@@ -415,7 +416,7 @@ tdcfie_status build_plan(tdcfie_t h) {
                 std::memcpy(&ent[4 * q + 3], &I[q], sizeof(int));
             }
             CK(cudaMalloc(&p->ecoef, sizeof(float) * ent.size()));
-            CK(cudaMemcpy(p->ecoef, ent.data(), sizeof(float) * ent.size(), cudaMemcpyHostToDevice));
+            CK(cudaMemcpyAsync(p->ecoef, ent.data(), sizeof(float) * ent.size(), cudaMemcpyHostToDevice, s));
         } else {
             CK(puti(&p->eidx, I));
             CK(put(&p->ecoef, C));
@@ -525,11 +526,11 @@ tdcfie_status plan_set_solver(tdcfie_t h, int solver, int guess, double tol) {
             to_path(s, p->prec, h->T, p->t0mat, ne, (int)ne, (int)ne, 1.0);
             CK(cudaMalloc(&p->guessbuf, es * R * p->ld));
             CK(cudaMemsetAsync(p->guessbuf, 0, es * R * p->ld, s));
-            CK(cudaStreamSynchronize(s));
         }
         if (!p->gm) CK(build_gmres(h, p));
         gmres_set_tol(p->gm, tol);
-        if (learned && !p->mlp) CK(build_mlp(p));
+        if (learned && !p->mlp) CK(build_mlp(p, s));
+        CK(cudaStreamSynchronize(s));
     }
     p->gmres_on = solver == TDCFIE_SOLVE_GMRES;
     p->mlp_on = p->gmres_on && learned;
@@ -545,7 +546,7 @@ tdcfie_status plan_reset(tdcfie_t h) {
     c.n = c.n0 = c.p0 = 1;
     c.bad_step = INT64_MAX;
     c.slot = 1;      // n mod ring (ring > 1), column 0 of a chunk
-    if (p->gm) CK(reset_gmres_stats(p->gm));
+    if (p->gm) CK(reset_gmres_stats(p->gm, s));
     CK(cudaMemcpyAsync(p->ctl, &c, sizeof(Ctl), cudaMemcpyHostToDevice, s));
     if (p->ringbuf) CK(cudaMemsetAsync(p->ringbuf, 0, p->esz * p->ring * p->R * p->ld, s));
     if (p->fact) {

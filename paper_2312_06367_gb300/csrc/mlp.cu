@@ -408,12 +408,12 @@ int launch_mlp_guess(StepPlan* p, int off, cudaStream_t s) {
 template int launch_mlp_guess<double>(StepPlan*, int, cudaStream_t);
 template int launch_mlp_guess<float>(StepPlan*, int, cudaStream_t);
 
-cudaError_t build_mlp(StepPlan* p) {
+cudaError_t build_mlp(StepPlan* p, cudaStream_t s) {
     auto* m = new MlpState();
     p->mlp = m;
     cudaError_t e;
     if ((e = cudaMalloc(&m->wh, sizeof(__half) * NP)) != cudaSuccess) return e;
-    if ((e = cudaMemset(m->wh, 0, sizeof(__half) * NP)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(m->wh, 0, sizeof(__half) * NP, s)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&m->scale, sizeof(float) * p->R)) != cudaSuccess) return e;
     return cudaSuccess;
 }
@@ -558,7 +558,7 @@ extern "C" tdcfie_status tdcfie_mlp_load(tdcfie_t h, const float* params) {
     if (!h->plan) return fail(h, TDCFIE_E_STATE, "call tdcfie_assemble first");
     if (h->plan->K - 1 < 8) return fail(h, TDCFIE_E_UNSUPPORTED, "the learned guess needs K - 1 >= 8 stored steps");
     if (!h->plan->mlp) {
-        const cudaError_t eb = build_mlp(h->plan);
+        const cudaError_t eb = build_mlp(h->plan, h->stream);
         if (eb != cudaSuccess) return cuda_fail(h, eb, "learned-guess state");
     }
     const cudaError_t e = mlp_load(h->plan, params, h->stream);

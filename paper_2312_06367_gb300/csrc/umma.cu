@@ -1072,14 +1072,14 @@ static void plan_segments(GemmArgs& a, int& grid, int rows, int cols, int nblk, 
     }
 }
 
-static cudaError_t plan_gemm(Gemm& G, int rows, int cols, int nblk, int reps, int sms) {
+static cudaError_t plan_gemm(Gemm& G, int rows, int cols, int nblk, int reps, int sms, cudaStream_t s) {
     std::vector<int> ptr, slot;
     plan_segments(G.a, G.grid, rows, cols, nblk, reps, sms, ptr, slot);
     cudaError_t e;
     if ((e = cudaMalloc(&G.seg_ptr, sizeof(int) * ptr.size())) != cudaSuccess) return e;
     if ((e = cudaMalloc(&G.seg_slot, sizeof(int) * slot.size())) != cudaSuccess) return e;
-    if ((e = cudaMemcpy(G.seg_ptr, ptr.data(), sizeof(int) * ptr.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
-    if ((e = cudaMemcpy(G.seg_slot, slot.data(), sizeof(int) * slot.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(G.seg_ptr, ptr.data(), sizeof(int) * ptr.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(G.seg_slot, slot.data(), sizeof(int) * slot.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
     G.a.seg_ptr = G.seg_ptr;
     G.a.seg_slot = G.seg_slot;
     return cudaSuccess;
@@ -1202,9 +1202,9 @@ tdcfie_status build_tc(tdcfie_t h, StepPlan* p) {
     CKB(cudaStreamSynchronize(s));
     CKB(reset_tc(g, ring, ne, s));
     // GEMM plans and tensor maps
-    CKB(plan_gemm(g->hist, ne, ne, nblk, 1, g->sms));
-    CKB(plan_gemm(g->solve, ne, ne, 1, 1, g->sms));
-    CKB(plan_gemm(g->proj, nc, nc, 1, TC_C, g->sms));
+    CKB(plan_gemm(g->hist, ne, ne, nblk, 1, g->sms, s));
+    CKB(plan_gemm(g->solve, ne, ne, 1, 1, g->sms, s));
+    CKB(plan_gemm(g->proj, nc, nc, 1, TC_C, g->sms, s));
     size_t pmax = 0;
     for (Gemm* G : {&g->hist, &g->solve, &g->proj}) pmax = std::max(pmax, partial_floats(*G));
     CKB(dalloc(g, &g->partial, pmax));

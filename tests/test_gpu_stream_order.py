@@ -40,3 +40,42 @@ def test_batch_waits_for_the_members_streams(own, precisions):
     b.close()
     for o, ref in zip(outs, refs):
         assert torch.equal(o, ref)
+
+
+@pytest.mark.parametrize("precision,R,kw", [("fp64", 1, {}), ("fp32", 3, {"solver": "gmres", "guess": "extrap"}), ("fp16x3", 64, {})])
+def test_plan_state_does_not_wait_for_the_legacy_stream(precision, R, kw):
+    """Plan, solver state and their resets are on the handle's stream: work pending on the legacy stream
+    meanwhile neither delays them into a running march nor leaves them out."""
+    import torch
+    from paper_2312_06367_gb300 import Solver
+    V, F = meshes.icosphere(1)
+    pw = excitation.fibonacci_batch(R, seed=3, t0=3.0, sigma=0.8)
+    st = torch.cuda.Stream()
+
+    def march(busy):
+        def hold():
+            if busy:
+                with torch.cuda.stream(torch.cuda.default_stream()):
+                    torch.cuda._sleep(SLOW)
+        out = torch.zeros((NT, R, 120), dtype=torch.float64 if precision == "fp64" else torch.float32, device="cuda")
+        s = Solver(V, F, dt=0.4, nt=NT, precision=precision, R=R, stream=st.cuda_stream)
+        torch.cuda.synchronize()
+        s.assemble()
+        if kw:
+            hold()
+            s.set_solver(kw["solver"], kw["guess"], 1e-9)
+        else:
+            hold()
+            s.replan(precision, R)
+        s.set_excitation(pw)
+        s.step(7, out[:7])
+        hold()
+        s.set_excitation(pw)
+        s.step(NT, out)
+        torch.cuda.synchronize()
+        return out
+
+    ref = march(False)
+    assert torch.isfinite(ref).all()
+    # (the FP64 assembly adds with atomics, so two assemblies agree to rounding only)
+    assert float((march(True) - ref).double().norm() / ref.double().norm()) < 1e-5
