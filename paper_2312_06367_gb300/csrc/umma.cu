@@ -727,7 +727,8 @@ __global__ void __launch_bounds__(256) k_split_x(const double* __restrict__ x, i
 // Increments of the plane-wave tests (Sec. II-C): e_m(t_n) - e_m(t_{n-1}) = sum_x c(x).p
 // [env_r(x, t_n) - env_r(x, t_{n-1})] with env_r(x, t) = amp_r exp(-a^2), a = (t - k_r.x - t0_r) /
 // width_r, and the difference written as -amp_r exp(-a_n^2) expm1(d (2 a_n - d)), d = dt / width_r,
-// so that it keeps its relative precision; at n = 1 the test itself (r_0 = 0).  Same for h.  t - t0 is
+// so that it keeps its relative precision (-amp_r exp(-(a_n - d)^2) where the argument is above 64: the
+// factor would overflow); at n = 1 the test itself (r_0 = 0).  Same for h.  t - t0 is
 // carried as an FP32 pair so that late times lose no digits of the pulse's argument.
 // The tests of a chunk's TC_C steps are formed when it starts, in two kernels: the envelope increments
 // once per quadrature point, step and wave (a point belongs to three RWG or about twelve BC functions:
@@ -751,7 +752,11 @@ __global__ void __launch_bounds__(NR * TC_C) k_env_tc(int npts, const double* __
     for (int pt = blockIdx.x * ENV_PB; pt < p1; ++pt) {
         const float arg = ((tt_hi - fmaf(kx, pts[3 * pt], fmaf(ky, pts[3 * pt + 1], kz * pts[3 * pt + 2]))) + tt_lo) * inv_w;
         float v = amp * expf(-arg * arg);
-        if (n != 1) v = -v * expm1f(d * (2.f * arg - d));     // env(t_n) - env(t_{n-1})
+        if (n != 1) {       // env(t_n) - env(t_{n-1})
+            const float x = d * (2.f * arg - d), b = arg - d;
+            // e^x would overflow behind the pulse, where v underflows; there e^-x is nothing beside 1
+            v = x > 64.f ? -amp * expf(-b * b) : -v * expm1f(x);
+        }
         env[((int64_t)pt * TC_C + i) * NR + r] = v;
     }
 }

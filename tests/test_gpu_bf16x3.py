@@ -51,3 +51,23 @@ def test_tensor_core_path_matches_oracle(level, dt, nt, precision, bound):
     print(f"{precision} level {level}: rel-L2 {err:.3e}")
     assert np.all(np.isfinite(j))
     assert err < bound
+
+
+@pytest.mark.parametrize("precision,bound", [("fp16x3", 1e-5), ("bf16x3", 1e-2)])
+@pytest.mark.parametrize("dt,sigma,t0,nt", [(0.8, 0.8, 4.0, 80), (4.0, 0.3, 8.2, 12)])
+def test_march_past_the_pulse(precision, bound, dt, sigma, t0, nt):
+    """Long after the pulse, and with steps of many widths, the increment of its envelope is a product of
+    an underflow and an overflow unless it is formed otherwise: the march stays finite and equals the
+    FP64 path's (bounds of the two paths at large steps)."""
+    import torch
+    from paper_2312_06367_gb300 import Solver
+    V, F = meshes.icosphere(1)
+    pw = excitation.fibonacci_batch(64, seed=5, t0=t0, sigma=sigma)
+    s = Solver(V, F, dt=dt, nt=nt, precision="fp64", R=8).assemble()
+    ref = torch.zeros((nt, 8, s.ne), dtype=torch.float64, device="cuda")
+    s.march({k: v[:8] for k, v in pw.items()}, ref)
+    s.replan(precision, 64)
+    out = torch.zeros((nt, 64, s.ne), dtype=torch.float32, device="cuda")
+    s.march(pw, out)
+    torch.cuda.synchronize()
+    assert float((out[:, :8].double() - ref).norm() / ref.norm()) < bound
