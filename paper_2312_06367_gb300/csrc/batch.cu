@@ -53,22 +53,23 @@ static int phase_units(const StepPlan* p, int ph) {
     }
 }
 
-// u: the unit; t: steps since the kernel's first (the step counters stay until its end); np: steps to
-// post-process, the last of them this one
-__device__ __forceinline__ void batch_unit(int ph, const SimtDev<float>& d, int t, int np, int u, int lane) {
+// u: the unit; t: steps since the kernel's first (the step counters stay until its end), left: steps from
+// this one on; np: steps to post-process, the last of them this one
+__device__ __forceinline__ void batch_unit(int ph, const SimtDev<float>& d, int t, int left, int np, int u, int lane) {
     const Ctl* c = d.ctl;
     StepPos pos{c->n + t, (c->slot + t) % d.ring, (c->col + t) % d.C};
+    const Cols cs = ph <= PH_PRE ? new_cols(d, pos.n, pos.col, left) : Cols{};
     if (ph == PH_ENV) {
-        const int idx = 32 * u + lane;
-        if (idx < d.npts * d.C) {
-            const int i = idx % d.C, pt = idx / d.C;
-            d.env[idx] = env_point<float>(d.exc, pos.n + i, d.dt, d.pts[3 * pt], d.pts[3 * pt + 1], d.pts[3 * pt + 2]);
+        const int idx = 32 * u + lane, nc = cs.hi - cs.lo;
+        if (idx < d.npts * nc) {
+            const int i = cs.lo + idx % nc, pt = idx / nc;
+            d.env[pt * d.C + i] = env_point<float>(d.exc, pos.n - pos.col + i, d.dt, d.pts[3 * pt], d.pts[3 * pt + 1], d.pts[3 * pt + 2]);
         }
     } else if (ph == PH_GATHER) {
-        gather_edge<float>(d, u, 0, lane);
+        gather_edge<float>(d, cs, u, 0, lane);
     } else if (ph == PH_PRE) {
         const int ctiles = (d.C + PRE_COLS - 1) / PRE_COLS, q = u % ctiles, g = u / ctiles % d.ngroups;
-        pre_item<float>(d, pos.slot, u / ctiles / d.ngroups * pre_rows<float>(), g, q * PRE_COLS, lane);
+        pre_item<float>(d, cs, ring_at(pos.slot, -pos.col, d.ring), u / ctiles / d.ngroups * pre_rows<float>(), g, q, lane);
     } else if (ph == PH_HIST) {
         hist_unit<float, 1>(d, pos, u, lane, true, Nothing());
     } else if (ph == PH_SOLVE) {
@@ -89,10 +90,13 @@ __device__ __forceinline__ void batch_unit(int ph, const SimtDev<float>& d, int 
 // bound it: five members of uneven size took 44 us a step with a kernel per step and the post-processing
 // in each (six barriers), 28 us with two phases a step.
 __global__ void __launch_bounds__(256) k_batch_step(const __grid_constant__ BArgs a, int rows, int steps) {
-    extern __shared__ int2 mcol[];      // (column of the first step, C) of every member
+    extern __shared__ int2 mcol[];      // every member's column of the kernel's first step, and C (negative: its march's first chunk)
     __shared__ int failed;
     if (threadIdx.x == 0) failed = (int)a.sync[1];      // an earlier kernel's wait ran out
-    for (int s = threadIdx.x; s < a.nmem; s += blockDim.x) mcol[s] = make_int2(a.mem[s].ctl->col, a.mem[s].C);
+    for (int s = threadIdx.x; s < a.nmem; s += blockDim.x) {
+        const Ctl* c = a.mem[s].ctl;
+        mcol[s] = make_int2(c->col, c->n - c->col == 1 ? -a.mem[s].C : a.mem[s].C);
+    }
     __syncthreads();
     if (failed) return;
     const int lane = threadIdx.x & 31;
@@ -101,9 +105,9 @@ __global__ void __launch_bounds__(256) k_batch_step(const __grid_constant__ BArg
     for (int t = 0; t < steps; ++t) {
         bool starts = false, ends = t == steps - 1;      // some member starts, ends a chunk
         for (int s = threadIdx.x; s < a.nmem; s += blockDim.x) {
-            const int col = (mcol[s].x + t) % mcol[s].y;
-            starts |= col == 0;
-            ends |= col == mcol[s].y - 1;
+            const int C = abs(mcol[s].y), col = (mcol[s].x + t) % C;
+            starts |= col == 0 || (t == 0 && mcol[s].y < 0);      // (new_cols)
+            ends |= col == C - 1;
         }
         starts = __syncthreads_or(starts);
         ends = __syncthreads_or(ends);
@@ -114,10 +118,10 @@ __global__ void __launch_bounds__(256) k_batch_step(const __grid_constant__ BArg
             for (int64_t u0 = warp * rows; u0 < total; u0 += nwarps * rows)
                 for (int64_t u = u0; u < min(u0 + rows, (int64_t)total); ++u) {
                     while (u >= first[s + 1]) ++s;
-                    const int C = mcol[s].y, col = (mcol[s].x + t) % C;
-                    if (ph <= PH_PRE && col != 0) continue;
+                    const int C = abs(mcol[s].y), col = (mcol[s].x + t) % C;
+                    if (ph <= PH_PRE && col != 0 && (t != 0 || mcol[s].y > 0)) continue;
                     if (ph >= PH_PIN && col != C - 1 && t != steps - 1) continue;
-                    batch_unit(ph, a.mem[s], t, min(t, col) + 1, (int)(u - first[s]), lane);
+                    batch_unit(ph, a.mem[s], t, steps - t, min(t, col) + 1, (int)(u - first[s]), lane);
                 }
             if (!group_barrier(a.sync, gridDim.x, a.sync + 1, &failed)) return;
         }

@@ -91,6 +91,7 @@ struct Ctl {              // device-resident step state read by every kernel of 
     int64_t n;            // current step (1-based)
     int slot, col;        // n mod ring (SIMT paths), (n - 1) mod C
     int64_t n0;           // step of the first output row of this tdcfie_step call
+    int64_t last;         // its last step
     void* out;            // currents_out of this call (nullptr: discard)
     int status;           // 0 ok, else a tdcfie_status recorded with bad_step
     int64_t bad_step;     // first step with a non-finite current (INT64_MAX: none)

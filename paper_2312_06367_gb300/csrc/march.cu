@@ -26,36 +26,41 @@
 namespace tdc {
 
 // ---------------------------------------------------------------- kernels (arithmetic in simt.h)
-// The tests and pre-sums of a chunk: no work unless the current step starts one
+// The tests and pre-sums of a chunk: no work where new_cols gives no columns
 template <typename T>
-__global__ void __launch_bounds__(128) k_env(const __grid_constant__ SimtDev<T> d) {
+__global__ void __launch_bounds__(128) k_env(const __grid_constant__ SimtDev<T> d, int most) {
     wait_prior();
     const int64_t n = d.ctl->n;
-    if (d.ctl->col) return;
+    const int col = d.ctl->col;
+    const Cols cs = new_cols(d, n, col, most);
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)d.npts * d.R * d.C) return;
-    const int i = (int)(idx % d.C), r = (int)(idx / d.C % d.R), pt = (int)(idx / d.C / d.R);
-    d.env[idx] = env_point<T>(d.exc + 11 * r, n + i, d.dt, d.pts[3 * pt], d.pts[3 * pt + 1], d.pts[3 * pt + 2]);
+    const int nc = cs.hi - cs.lo;
+    if (idx >= (int64_t)d.npts * d.R * nc) return;
+    const int i = cs.lo + (int)(idx % nc), r = (int)(idx / nc % d.R), pt = (int)(idx / nc / d.R);
+    d.env[((int64_t)pt * d.R + r) * d.C + i] = env_point<T>(d.exc + 11 * r, n - col + i, d.dt, d.pts[3 * pt], d.pts[3 * pt + 1], d.pts[3 * pt + 2]);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(128) k_gather(const __grid_constant__ SimtDev<T> d) {
+__global__ void __launch_bounds__(128) k_gather(const __grid_constant__ SimtDev<T> d, int most) {
     wait_prior();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= d.ne * d.R || d.ctl->col) return;
-    gather_edge<T>(d, w / d.R, w % d.R, threadIdx.x & 31);
+    const Cols cs = new_cols(d, d.ctl->n, d.ctl->col, most);
+    if (w >= d.ne * d.R || cs.lo == cs.hi) return;
+    gather_edge<T>(d, cs, w / d.R, w % d.R, threadIdx.x & 31);
 }
 
 // grid: (column tiles x row blocks, groups), the column tiles fastest so that blocks that share rows
 // run together
 template <typename T>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 3) k_pre(const __grid_constant__ SimtDev<T> d, int ctiles) {
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 3) k_pre(const __grid_constant__ SimtDev<T> d, int ctiles, int most) {
     wait_prior();
-    if (d.ctl->col) return;
+    const int col = d.ctl->col;
+    const Cols cs = new_cols(d, d.ctl->n, col, most);
+    if (cs.lo == cs.hi) return;
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) d.ctl->t_mark = device_ns();
     const int tile = blockIdx.x % ctiles, rb = blockIdx.x / ctiles;
     const int row0 = (rb * 4 + (threadIdx.x >> 5)) * pre_rows<T>();
-    if (row0 < d.ne) pre_item<T>(d, d.ctl->slot, row0, blockIdx.y, tile * PRE_COLS, threadIdx.x & 31);
+    if (row0 < d.ne) pre_item<T>(d, cs, ring_at(d.ctl->slot, -col, d.ring), row0, blockIdx.y, tile, threadIdx.x & 31);
 }
 
 // b_n; step n = ctl->n + off.  sums_ready: the pre-sums are older than the kernel in front
@@ -66,7 +71,7 @@ __global__ void __launch_bounds__(128, 4) k_hist(const __grid_constant__ SimtDev
         wait_prior();
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             const unsigned long long t = device_ns();
-            if (pos.col == 0) d.ctl->hist_ns += t - d.ctl->t_mark;     // the pre-sums ran just before
+            if (pos.col == 0) d.ctl->hist_ns += t - d.ctl->t_mark;     // the chunk's pre-sums ran just before
             d.ctl->t_mark = t;
         }
     };
@@ -158,21 +163,21 @@ template SimtDev<float> simt_view<float>(tdcfie_t, const StepPlan&);
 static unsigned div_up(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
 template <typename T>
-int launch_tests(tdcfie_t h, StepPlan& p, cudaStream_t s) {
+int launch_tests(tdcfie_t h, StepPlan& p, int most, cudaStream_t s) {
     const SimtDev<T> d = simt_view<T>(h, p);
-    k_env<T><<<div_up((int64_t)p.npts * p.R * p.C, 128), 128, 0, s>>>(d);
-    launch_chained(k_gather<T>, div_up((int64_t)p.ne * p.R, 4), 128, s, 0, d);
+    k_env<T><<<div_up((int64_t)p.npts * p.R * p.C, 128), 128, 0, s>>>(d, most);
+    launch_chained(k_gather<T>, div_up((int64_t)p.ne * p.R, 4), 128, s, 0, d, most);
     return 2;
 }
-template int launch_tests<double>(tdcfie_t, StepPlan&, cudaStream_t);
-template int launch_tests<float>(tdcfie_t, StepPlan&, cudaStream_t);
+template int launch_tests<double>(tdcfie_t, StepPlan&, int, cudaStream_t);
+template int launch_tests<float>(tdcfie_t, StepPlan&, int, cudaStream_t);
 
 template <typename T>
-static int launch_pre(tdcfie_t h, StepPlan& p, cudaStream_t s) {
-    int n = launch_tests<T>(h, p, s);
+static int launch_pre(tdcfie_t h, StepPlan& p, int most, cudaStream_t s) {
+    int n = launch_tests<T>(h, p, most, s);
     if (p.fact) return n;
     const int ctiles = (int)div_up(p.C * p.R, PRE_COLS);
-    launch_chained(k_pre<T>, dim3(ctiles * div_up(p.ne, 4 * pre_rows<T>()), p.ngroups), 128, s, 0, simt_view<T>(h, p), ctiles);
+    launch_chained(k_pre<T>, dim3(ctiles * div_up(p.ne, 4 * pre_rows<T>()), p.ngroups), 128, s, 0, simt_view<T>(h, p), ctiles, most);
     return n + 1;
 }
 
@@ -223,26 +228,24 @@ template <typename T>
 static cudaError_t launch_graph(tdcfie_t h, StepPlan& p, int which, cudaStream_t s, int& k) {
     cudaError_t e = cudaSuccess;
     const bool chunk = which == StepPlan::G_CHUNK;
-    if (which == StepPlan::G_PRE || chunk) k += launch_pre<T>(h, p, s);
-    if (which == StepPlan::G_STEP) {
-        e = launch_inner<T>(h, p, false, 0, s, k);
-        if (!p.fact) {                      // the factored step advances the counter itself
-            launch_chained(k_advance<T>, 1, 1, s, 0, simt_view<T>(h, p));
-            k += 1;
-        }
+    if (which == StepPlan::G_PRE || chunk) k += launch_pre<T>(h, p, chunk ? p.C : 0, s);
+    if (which == StepPlan::G_STEP || which == StepPlan::G_LAST) e = launch_inner<T>(h, p, false, 0, s, k);
+    if (which == StepPlan::G_STEP && !p.fact) {      // the factored step advances the counter itself
+        launch_chained(k_advance<T>, 1, 1, s, 0, simt_view<T>(h, p));
+        k += 1;
     }
     if (chunk)
         for (int i = 0; i < p.C && e == cudaSuccess; ++i) e = launch_inner<T>(h, p, true, p.fact ? 0 : i, s, k);
-    if (which == StepPlan::G_POST || chunk) k += launch_post<T>(h, p, chunk ? p.C : 0, s);
+    if (which == StepPlan::G_LAST || chunk) k += launch_post<T>(h, p, chunk ? p.C : 1, s);
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 static cudaError_t launch_graph_tc(tdcfie_t h, StepPlan& p, int which, cudaStream_t s, int& k) {
     const bool chunk = which == StepPlan::G_CHUNK;
     if (which == StepPlan::G_PRE || chunk) k += launch_tests_tc(h, &p, s);
-    if (which == StepPlan::G_STEP) k += launch_inner_tc(h, &p, 0, true, s);
+    if (which == StepPlan::G_STEP || which == StepPlan::G_LAST) k += launch_inner_tc(h, &p, 0, which == StepPlan::G_STEP, s);
     if (chunk)
         for (int i = 0; i < p.C; ++i) k += launch_inner_tc(h, &p, i, false, s);
-    if (which == StepPlan::G_POST || chunk) k += launch_post_tc(h, &p, chunk ? p.C : 0, s);
+    if (which == StepPlan::G_LAST || chunk) k += launch_post_tc(h, &p, chunk ? p.C : 1, s);
     return cudaGetLastError();
 }
 
@@ -559,12 +562,12 @@ tdcfie_status plan_reset(tdcfie_t h) {
 }
 
 // Enqueue one whole step of h on s (s must be capturing a graph): the tests and pre-sums (which return
-// at once unless a chunk starts), the step, its post-processing.
+// at once unless a chunk starts or it is the march's first), the step, its post-processing.
 cudaError_t capture_step(tdcfie_t h, cudaStream_t s) {
     StepPlan* p = h->plan;
     auto simt = [&](auto t) -> cudaError_t {
         using T = decltype(t);
-        int k = launch_pre<T>(h, *p, s);
+        int k = launch_pre<T>(h, *p, 1, s);
         const cudaError_t e = launch_inner<T>(h, *p, false, 0, s, k);
         k += launch_post<T>(h, *p, 1, s);
         p->launches_per_step = k;
@@ -650,6 +653,7 @@ tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout) {
     CK(cudaMemcpyAsync(&c, p->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     c.n0 = c.n;
+    c.last = c.n + nsteps - 1;
     c.out = out;
     c.yout = yout;
     c.hist_ns = 0;
@@ -664,7 +668,7 @@ tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout) {
     };
 #define RUN(g) do { const tdcfie_status st_ = run(g); if (st_ != TDCFIE_OK) return st_; } while (0)
     // whole chunks by one graph, the rest step by step; the post-processing runs when a chunk ends and
-    // when the call does
+    // when the call does (with its last step)
     const int64_t C = p->C;
     CK(cudaEventRecord(p->ev0, s));
     for (int64_t n = c.n, end = c.n + nsteps; n < end;) {
@@ -672,9 +676,9 @@ tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout) {
         if (m == C) {
             RUN(StepPlan::G_CHUNK);
         } else {
-            if (i == 0) RUN(StepPlan::G_PRE);
-            for (int64_t q = 0; q < m; ++q) RUN(StepPlan::G_STEP);
-            if (!p->fact) RUN(StepPlan::G_POST);
+            if (i == 0 || (n - i == 1 && !p->gemm)) RUN(StepPlan::G_PRE);      // (new_cols)
+            for (int64_t q = 1; q < m; ++q) RUN(StepPlan::G_STEP);
+            RUN(p->fact ? StepPlan::G_STEP : StepPlan::G_LAST);
         }
         n += m;
     }

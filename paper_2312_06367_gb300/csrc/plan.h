@@ -44,8 +44,8 @@ struct StepPlan {
     // tensor-core path
     TcStep* gemm = nullptr;
     // graphs: G_PRE the tests (and, SIMT paths, pre-sums) of a chunk, G_STEP one step's history and
-    // solve, G_POST the post-processing of the finished steps, G_CHUNK a whole chunk
-    enum { G_STEP = 0, G_PRE, G_POST, G_CHUNK, NGRAPH };
+    // solve, G_LAST the same and the post-processing of the finished steps, G_CHUNK a whole chunk
+    enum { G_STEP = 0, G_PRE, G_LAST, G_CHUNK, NGRAPH };
     cudaGraph_t graph[NGRAPH] = {};
     cudaGraphExec_t exec[NGRAPH] = {};
     int nodes[NGRAPH] = {};                              // kernels per graph
@@ -58,10 +58,10 @@ struct SimtDev;
 // device view of the plan (march.cu)
 template <typename T>
 SimtDev<T> simt_view(tdcfie_t h, const StepPlan& p);
-// plane-wave tests of a chunk into p.E, p.Hv: nothing unless a chunk starts at the current step
-// (march.cu); returns the number of kernels
+// plane-wave tests into p.E, p.Hv, of the columns that new_cols gives (march.cu); returns the number of
+// kernels
 template <typename T>
-int launch_tests(tdcfie_t h, StepPlan& p, cudaStream_t s);
+int launch_tests(tdcfie_t h, StepPlan& p, int most, cudaStream_t s);
 // factored history form (factored.cu)
 tdcfie_status build_fact(tdcfie_t h, StepPlan* p);
 tdcfie_status reset_fact(tdcfie_t h, StepPlan* p);

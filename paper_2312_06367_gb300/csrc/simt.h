@@ -15,7 +15,7 @@
 //            are formed beside it, one per row and lag, so that the step's chain stays short;
 //   solve    y_n = T_0^-1 b_n (or GMRES);
 // and the post-processing of the finished steps together (its projector is not part of the
-// recurrence).  Matrix bytes per step at K = 42, C = 8: 43/8 + 3.5 + 1 + 1/8 blocks instead of 45.
+// recurrence).  The first chunk of a march is the exception, see new_cols.  Matrix bytes per step at K = 42, C = 8: 43/8 + 3.5 + 1 + 1/8 blocks instead of 45.
 //
 // Rows of matrices and vectors are padded to 16 bytes (zeros), every load is a 16-byte vector.
 #pragma once
@@ -81,6 +81,20 @@ __device__ __forceinline__ void advance(const SimtDev<T>& d, int adv) {
     c->col = (c->col + adv) % d.C;
 }
 
+// Columns lo .. hi - 1 of the current chunk whose tests and pre-sums are formed at this step: all of them
+// where a chunk starts.  In the march's first chunk (the steps 1 .. C), where the lags that reach back before
+// it meet y_i = 0 and only the tests' blocks count, each call forms those of its own steps: a march may
+// end there, and one of a few steps does not pay for C (a march of one step, 1920 edges, K = 42, FP64: 2.33 ms
+// with the chunk formed whole, 0.33 ms so; with eight waves 15.8 and 0.74 ms).  most: the call's steps from this one on, 0: up to
+// ctl->last.
+struct Cols { int lo, hi; bool first; };
+template <typename T>
+__device__ __forceinline__ Cols new_cols(const SimtDev<T>& d, int64_t n, int col, int most) {
+    if (n - col != 1) return Cols{0, col ? 0 : d.C, false};
+    const int64_t left = most ? most : d.ctl->last - n + 1;
+    return Cols{col, (int)(left < d.C - col ? col + left : d.C), true};
+}
+
 // ---------------------------------------------------------------- plane-wave tests
 // e_m(t_n) = sum_x c(x).p env(x, t_n) over the 7-point rule of the RWG triangles, h_m the same with
 // c(x).(k x p) over the 3-point rule of the BC fine triangles; env(x, t) = amp exp(-((t - k.x - t0) /
@@ -96,15 +110,16 @@ __device__ __forceinline__ T env_point(const double* P, int64_t n, double dt, T 
     return mul_rn(amp, exp(-mul_rn(arg, arg)));
 }
 
-// e, h of edge m and wave r for the chunk's C steps (a divisor of 32): lane l takes column l % C and
-// every (32 / C)-th entry; the parts are added by a fixed tree
+// e, h of edge m and wave r for the columns `cs` of the chunk's C (a divisor of 32): lane l takes column
+// l % C and every (32 / C)-th entry; the parts are added by a fixed tree
 template <typename T>
-__device__ __forceinline__ void gather_edge(const SimtDev<T>& d, int m, int r, int lane) {
+__device__ __forceinline__ void gather_edge(const SimtDev<T>& d, const Cols& cs, int m, int r, int lane) {
     const double* P = d.exc + 11 * r;
     const T kx = (T)P[0], ky = (T)P[1], kz = (T)P[2], qx = (T)P[3], qy = (T)P[4], qz = (T)P[5];
     const T hx = fma(ky, qz, -mul_rn(kz, qy)), hy = fma(kz, qx, -mul_rn(kx, qz)), hz = fma(kx, qy, -mul_rn(ky, qx));   // k x p
     const int i = lane % d.C, part = lane / d.C, parts = 32 / d.C;
-    const int b = d.eptr[m], me = b + d.enE[m], end = d.eptr[m + 1];
+    const bool mine = i >= cs.lo && i < cs.hi;
+    const int b = d.eptr[m], me = b + d.enE[m], end = mine ? d.eptr[m + 1] : b;
     T e = 0, h = 0;
 #pragma unroll 4
     for (int q = b + part; q < end; q += parts) {
@@ -117,7 +132,7 @@ __device__ __forceinline__ void gather_edge(const SimtDev<T>& d, int m, int r, i
         e = add_rn(e, __shfl_xor_sync(0xffffffffu, e, o));
         h = add_rn(h, __shfl_xor_sync(0xffffffffu, h, o));
     }
-    if (part == 0) {
+    if (part == 0 && mine) {
         d.E[(int64_t)(i * d.R + r) * d.ld + m] = e;
         d.H[(int64_t)(i * d.R + r) * d.ld + m] = h;
     }
@@ -319,13 +334,14 @@ constexpr int PRE_COLS = 8;
 // pipe 62 % busy, 543 us for 8 columns at 1920 edges, K = 42; 433 us with one)
 template <typename T> constexpr int pre_rows() { return sizeof(T) == 8 ? 2 : 1; }
 
-// Rows row0 .. row0 + pre_rows - 1, columns col0 .. col0 + 7 and group g of the blocks in the order e, h,
-// lag K-1, ..., lag 1: accumulated over the group's blocks, then over the warp, into partial[g].  slot:
-// ring slot of the chunk's first step
+// Rows row0 .. row0 + pre_rows - 1, the tile-th eight columns of `cs` and group g of the blocks in the
+// order e, h, lag K-1, ..., lag 1: accumulated over the group's blocks, then over the warp, into partial[g].
+// slot: ring slot of the chunk's first step
 template <typename T>
-__device__ __forceinline__ void pre_item(const SimtDev<T>& d, int slot, int row0, int g, int col0, int lane) {
+__device__ __forceinline__ void pre_item(const SimtDev<T>& d, const Cols& cs, int slot, int row0, int g, int tile, int lane) {
     constexpr int PRE_ROWS = pre_rows<T>();
-    const int CR = d.C * d.R, nvec = d.ld / VecOf<T>::W;
+    const int CR = d.C * d.R, nvec = d.ld / VecOf<T>::W, end = cs.hi * d.R, col0 = cs.lo * d.R + tile * PRE_COLS;
+    if (col0 >= end) return;
     int ci[PRE_COLS], co[PRE_COLS];      // step within the chunk, offset of the wave within a slot
 #pragma unroll
     for (int c = 0; c < PRE_COLS; ++c) {
@@ -334,16 +350,18 @@ __device__ __forceinline__ void pre_item(const SimtDev<T>& d, int slot, int row0
     }
     Acc<T> acc[PRE_ROWS][PRE_COLS];
 #pragma unroll 1
-    for (int o = GQ * g; o < min(GQ * g + GQ, d.K + 1); ++o) {
+    for (int o = GQ * g; o < min(GQ * g + GQ, cs.first ? 2 : d.K + 1); ++o) {
         const int k = o < 2 ? 0 : d.K + 1 - o, q = o < 2 ? o : 1 + k;      // lag and block
         const int sk = ring_at(slot, -k, d.ring);
         int off[PRE_COLS], nv = 0;
 #pragma unroll
         for (int c = 0; c < PRE_COLS; ++c) {
-            // columns whose lag lies inside the chunk read the zero vectors behind the ring
-            const bool on = o < 2 || ci[c] < k;
+            // columns whose lag lies inside the chunk read the zero vectors behind the ring, those behind
+            // the last one that is wanted repeat it
+            const bool on = col0 + c < end && (o < 2 || ci[c] < k);
             nv += on;       // the first ones of the tile
-            off[c] = o < 2 ? (col0 + c) * d.ld : (on ? ring_at(sk, ci[c], d.ring) : d.ring) * d.R * d.ld + co[c];
+            off[c] = o < 2 ? min(col0 + c, end - 1) * d.ld
+                           : (on ? ring_at(sk, ci[c], d.ring) * d.R * d.ld + co[c] : d.ring * d.R * d.ld);
         }
         if (!nv) continue;
         const T* base = d.blocks + (int64_t)q * d.ne * d.ld;
@@ -359,7 +377,7 @@ __device__ __forceinline__ void pre_item(const SimtDev<T>& d, int slot, int row0
         for (int c = 0; c < PRE_COLS; ++c) v[i * PRE_COLS + c] = acc[i][c].sum();
     const auto s = multi_reduce<PRE_ROWS * PRE_COLS>(v, lane);
     const int id = multi_index<PRE_ROWS * PRE_COLS>(lane), row = row0 + id / PRE_COLS, col = col0 + id % PRE_COLS;
-    if (multi_owner<PRE_ROWS * PRE_COLS>(lane) && row < d.ne && col < CR) d.partial[((int64_t)g * CR + col) * d.ld + row] = s;
+    if (multi_owner<PRE_ROWS * PRE_COLS>(lane) && row < d.ne && col < end) d.partial[((int64_t)g * CR + col) * d.ld + row] = s;
 }
 
 // ---------------------------------------------------------------- one step

@@ -189,3 +189,55 @@ def test_batch_before_excitation(waves):
         s.march(pw, ref)
         torch.cuda.synchronize()
         assert torch.equal(o, ref)
+
+
+@pytest.mark.parametrize("precision,R", [("fp64", 1), ("fp64", 3), ("fp32", 1), ("fp32", 8)])
+@pytest.mark.parametrize("form", ["dense", "factored"])
+def test_first_chunk_in_calls(waves, precision, R, form):
+    """The first chunk of a march is formed call by call: any calls, also a batch's, give the same bits."""
+    import torch
+    from paper_2312_06367_gb300 import Batch
+    pw = {k: v[:R] for k, v in waves.items()}
+    s, other = _solver(SMALL, 0.15, 20, R, precision), _solver(meshes.icosphere(0), 0.3, 20, R, precision)
+    for t in (s, other):
+        t.set_history_form(form)
+        t.set_excitation(pw)
+    out = torch.zeros((20, R, s.ne), dtype=s.dtype, device="cuda")
+    s.march(pw, out)
+    b = Batch([s, other])
+    for calls in ((1, -1, 1, -2, 15), (-1, 3, -4, 12), (2, -18), (-17, 3)):      # negative: steps of the batch
+        parts = torch.zeros_like(out)
+        s.set_excitation(pw)
+        other.set_excitation(pw)
+        torch.cuda.synchronize()
+        at = 0
+        for m in calls:
+            if m > 0:
+                s.step(m, parts[at:at + m])
+            else:
+                b.step(-m, [parts[at:at - m], None])
+            at += abs(m)
+        torch.cuda.synchronize()
+        assert at == 20 and torch.equal(out, parts), calls
+    b.close()
+
+
+def test_one_step_does_not_pay_for_a_chunk():
+    """A new march of one step costs well under one of eight (before the first chunk was formed call by
+    call it cost 0.8 of it: the sums over all lags of eight columns)."""
+    import time
+    import torch
+    pw = excitation.random_batch(8, seed=3, t0=3.0, sigma=0.8)
+    s = _solver(meshes.icosphere(2), 0.05, 8, 8, "fp64")
+    times = {}
+    for nt in (1, 8):
+        best = []
+        for _ in range(7):
+            s.set_excitation(pw)
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            s.step(nt)
+            best.append(time.perf_counter() - t0)
+        times[nt] = min(best)
+    print(times)
+    assert times[1] < 0.6 * times[8]
