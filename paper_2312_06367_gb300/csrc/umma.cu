@@ -345,6 +345,23 @@ __device__ __forceinline__ void split_pair(float H, float L, uint16_t* out) {
     }
 }
 
+// the slices that the FP64 value of H + L has: the sum is normalised first and the rounding error of the
+// first remainder is carried to the next slice
+template <bool F16, int XS>
+__device__ __forceinline__ void split_sum(float H, float L, uint16_t* out) {
+    const float h = H + L, l = L - (h - H);
+    const uint16_t b0 = to16<F16>(h);
+    out[0] = b0;
+    float r = h - from16<F16>(b0), e = 0.f;
+    two_sum_acc(r, e, l);
+#pragma unroll
+    for (int i = 1; i < XS; ++i) {
+        const uint16_t b = to16<F16>(r);
+        out[i] = b;
+        r = (r - from16<F16>(b)) + e;
+    }
+}
+
 #ifndef TDC_XHI_BITS
 #define TDC_XHI_BITS 11
 #endif
@@ -841,7 +858,7 @@ __global__ void __launch_bounds__(32 * RHS_NW) k_rhs_tc(int ne, const double* __
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const float2 v = ev[(w * 64 + el + u) * RHS_LD + j];
-            split_pair<F16, XS>(v.x * scl[w][j], v.y * scl[w][j], sl[u]);
+            split_sum<F16, XS>(v.x * scl[w][j], v.y * scl[w][j], sl[u]);
         }
         const int64_t off = ((int64_t)(slot0 + w) * NR + j) * ld + tile * 64 + el;
 #pragma unroll
@@ -865,7 +882,7 @@ template <bool F16, int XS>
 __global__ void __launch_bounds__(256) k_project_in_tc(DevMesh m, const Ctl* ctl, int adv, const double* y2,
                                                        double inv_dtt, uint16_t* __restrict__ Z0, uint16_t* __restrict__ Z1,
                                                        uint16_t* __restrict__ Z2, float* __restrict__ sZ, int ldc) {
-    __shared__ float2 zv[PIN_RB][65];      // FP64 values as FP32 pairs (their slices keep 33 bits)
+    __shared__ double zv[PIN_RB][65];
     __shared__ float scl[PIN_RB];
     const int tile = blockIdx.x, rb = blockIdx.y * PIN_RB;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -885,14 +902,13 @@ __global__ void __launch_bounds__(256) k_project_in_tc(DevMesh m, const Ctl* ctl
                 s = fma(m.tsign[3 * c + l], fma(dy[(int64_t)r * m.ne + e], inv_dtt, -yn[(int64_t)r * m.ne + e]), s);
             }
         }
-        const float hi = (float)s;
-        zv[j][cl] = make_float2(hi, (float)(s - (double)hi));
+        zv[j][cl] = s;
     }
     __syncthreads();
     // maxima: warp w covers waves 2w, 2w+1 (lanes 0-15 / 16-31), 4 triangles per lane
     {
         const int j = 2 * warp + (lane >> 4), c4 = (lane & 15) * 4;
-        for (int l = 0; l < 4; ++l) mx = fmaxf(mx, fabsf(zv[j][c4 + l].x));
+        for (int l = 0; l < 4; ++l) mx = fmaxf(mx, fabsf((float)zv[j][c4 + l]));
         for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         if ((lane & 15) == 0) {
             if (!(mx == mx)) mx = INFINITY;
@@ -905,7 +921,7 @@ __global__ void __launch_bounds__(256) k_project_in_tc(DevMesh m, const Ctl* ctl
     for (int i = t; i < PIN_RB * 64; i += 256) {
         const int j = i >> 6, cl = i & 63;
         uint16_t sl[3];
-        split_pair<F16, XS>(zv[j][cl].x * scl[j], zv[j][cl].y * scl[j], sl);
+        split_vector<F16, XS>(zv[j][cl] * (double)scl[j], sl);
         const int64_t off = ((int64_t)k * NR + rb + j) * ldc + tile * 64 + cl;
 #pragma unroll
         for (int l = 0; l < XS; ++l) dst[l][off] = sl[l];
