@@ -32,7 +32,7 @@
 
 namespace tdc {
 
-constexpr int MAXB = 64;   // breakpoint circles that may cross one edge of a source triangle
+constexpr int MAXB = 64;   // breakpoint circles across one edge whose cuts are kept in a list (more: MANY)
 __constant__ double c_ax[NANG], c_aw[NANG], c_rx[NRAD], c_rw[NRAD];
 __constant__ double c_r7[7][4];   // barycentric a, b, c, weight
 __constant__ double c_r3[3][4];
@@ -341,10 +341,36 @@ __device__ __forceinline__ void insert_sorted(double* a, int& n, double v) {
     a[j] = v;
 }
 
+// MANY (time steps below a 62nd of the longest edge): the circles R = j dt across an edge one after another
+// in the edge's direction, inwards to its foot, then outwards, without a list.  It finds each circle twice and
+// pushes pieces as it goes: on meshes that need no more than the list holds, 5 % slower than the list.
+struct Circles {
+    int j, jin, jend;       // next circle, innermost, behind the last one outwards
+    bool out;
+    // distances of the outer point from the edge's start, the point nearest to it and the end; whether
+    // that point is the start or the end
+    __device__ void set(double R0, double Rmin, double R1, bool start, bool end, double inv_dt) {
+        out = start;
+        jin = (int)(Rmin * inv_dt);
+        j = start ? jin : (int)(R0 * inv_dt) + 1;
+        jend = end ? jin : (int)(R1 * inv_dt) + 2;
+    }
+    // false: no more; inwards: the crossing lies before the foot
+    __device__ bool next(int& circle, bool& inwards) {
+        if (!out && j < jin) {
+            out = true;
+            j = jin;
+        }
+        if (out && j >= jend) return false;
+        inwards = !out;
+        circle = out ? j++ : j--;
+        return true;
+    }
+};
+
 // Polar rule about p: one signed sub-triangle (fan) per edge; round s is edge s
-template <class ACC>
+template <class ACC, bool MANY>
 __device__ void push_near(BlockSh& sh, double* slots, int s, const Pair& P, Steps st, double kappa) {
-    double sp[2 * MAXB + 2];
     const V3 a = P.v[s], b = P.v[s == 2 ? 0 : s + 1];
     const V3 ab = b - a;
     const double L = nrm(ab);
@@ -356,11 +382,30 @@ __device__ void push_near(BlockSh& sh, double* slots, int s, const Pair& P, Step
     const double h = nrm(nu);
     if (h <= 1e-14 * L) return;
     store_fan(sh, Fan{(1.0 / h) * nu, e, 0.0, h, sig > 0.0 ? 1.0 : -1.0, 1.0});
-    const double psa = asinh(-t / h), psb = asinh((L - t) / h);
+    const double psa = asinh(-t / h), psb = asinh((L - t) / h), d2 = P.d * P.d;
+    double P0 = psa;
+    if constexpr (ACC::RETARDED && MANY) {
+        const double m2 = fma(h, h, d2), R0 = sqrt(fma(t, t, m2)), R1 = sqrt(fma(L - t, L - t, m2));
+        Circles cir;
+        cir.set(R0, t < 0.0 ? R0 : t > L ? R1 : sqrt(m2), R1, t < 0.0, t > L, st.inv_dt);
+        int j;
+        for (bool inwards; cir.next(j, inwards);) {
+            const double R = j * st.dt, r2 = fma(R, R, -d2);
+            if (!(r2 > h * h)) continue;
+            const double c = acosh(sqrt(r2) / h), P1 = inwards ? -c : c;
+            if (P1 > P0 && P1 < psb) {
+                push_piece<ACC>(sh, slots, P0, P1, st, kappa);
+                P0 = P1;
+            }
+        }
+        if (psb > P0) push_piece<ACC>(sh, slots, P0, psb, st, kappa);
+        return;
+    }
+    double sp[2 * MAXB + 2];
     int nsp = 0;
     if constexpr (ACC::RETARDED) {
         // breakpoint circles that cross the edge: between its foot and its farther end
-        const double d2 = P.d * P.d, m = fmax(fabs(t), fabs(L - t));
+        const double m = fmax(fabs(t), fabs(L - t));
         const double hi = sqrt(fma(m, m, fma(h, h, d2)));
         int j = (int)(sqrt(fma(h, h, d2)) * st.inv_dt);
         for (int nb = 0; nb < MAXB && j * st.dt < hi; ++j) {
@@ -372,7 +417,6 @@ __device__ void push_near(BlockSh& sh, double* slots, int s, const Pair& P, Step
             if (c > psa && c < psb) insert_sorted(sp, nsp, c);
         }
     }
-    double P0 = psa;
     for (int pc = 0; pc <= nsp; ++pc) {
         const double P1 = pc < nsp ? sp[pc] : psb;
         if (P1 > P0) push_piece<ACC>(sh, slots, P0, P1, st, kappa);
@@ -386,7 +430,7 @@ __device__ __forceinline__ double cr2(double ax, double ay, double bx, double by
 // cancellation), one fan per half.  Angles are measured from the foot of the half's near edge and
 // carried as asinh(tan(angle)) = asinh(cross / dot), so that no angle itself is formed.  Round
 // half is one half.
-template <class ACC>
+template <class ACC, bool MANY>
 __device__ void push_far(BlockSh& sh, double* slots, int half, const Pair& P, Steps st) {
     V3 g = (1.0 / 3.0) * (P.v[0] + P.v[1] + P.v[2]) - P.p;
     const V3 u = (1.0 / nrm(g)) * g, w = cross(P.n, u);
@@ -403,7 +447,6 @@ __device__ void push_far(BlockSh& sh, double* slots, int half, const Pair& P, St
                 t = Y[k]; Y[k] = Y[k - 1]; Y[k - 1] = t;
             }
     const double d2 = P.d * P.d;
-    double sp[4 * MAXB + 2];
     // the half between vertex half and vertex half + 1; its edges: that pair's and the long one (0, 2)
     const double x0 = X[half], y0 = Y[half], x1 = X[half + 1], y1 = Y[half + 1];
     if (!(cr2(x0, y0, x1, y1) > 0.0)) return;
@@ -421,6 +464,47 @@ __device__ void push_far(BlockSh& sh, double* slots, int half, const Pair& P, St
     const double cf = fx / hn, sf = fy / hn;
     auto angle = [&](double vx, double vy) { return asinh((cf * vy - sf * vx) / (cf * vx + sf * vy)); };
     const double S0 = angle(x0, y0), S1 = angle(x1, y1);
+    const double fdx = lnear ? sx : lx, fdy = lnear ? sy : ly;       // far edge
+    store_fan(sh, Fan{cf * u + sf * w, cf * w - sf * u, hn, lnear ? nsh : nl, cf * fdx + sf * fdy, cf * fdy - sf * fdx});
+    double P0 = S0;
+    if constexpr (MANY) {
+        // both edges run by ascending angle: a cut is the nearer of their next crossings
+        Circles cir[2];
+        for (int ei = 0; ei < 2; ++ei) {
+            const double bx = ei ? x0 : X[0], by = ei ? y0 : Y[0], dx = ei ? sx : lx, dy = ei ? sy : ly;
+            const double dd = dx * dx + dy * dy, bq = bx * dx + by * dy, aa = bx * bx + by * by, ee = aa + 2.0 * bq + dd;
+            const double foot = bq < 0.0 && -bq < dd ? aa - bq * bq / dd : fmin(aa, ee);
+            cir[ei].set(sqrt(aa + d2), sqrt(fmax(foot, 0.0) + d2), sqrt(fmax(ee, 0.0) + d2), bq >= 0.0, -bq >= dd, st.inv_dt);
+        }
+        auto crossing = [&](int ei) {       // the edge's next one inside the half, S1 if there is none
+            const double bx = ei ? x0 : X[0], by = ei ? y0 : Y[0], dx = ei ? sx : lx, dy = ei ? sy : ly;
+            const double dd = dx * dx + dy * dy, bq = bx * dx + by * dy, aa = bx * bx + by * by;
+            int j;
+            for (bool inwards; cir[ei].next(j, inwards);) {
+                const double R = j * st.dt, r2 = fma(R, R, -d2);
+                if (!(r2 > 0.0)) continue;
+                const double disc = bq * bq - dd * (aa - r2);
+                if (disc <= 0.0) continue;
+                const double sq = sqrt(disc), ts = (inwards ? -bq - sq : sq - bq) / dd;
+                if (ts <= 0.0 || ts >= 1.0) continue;
+                const double S = angle(bx + ts * dx, by + ts * dy);
+                if (S > S0 && S < S1) return S;
+            }
+            return S1;
+        };
+        for (double s0 = crossing(0), s1 = crossing(1); P0 < S1;) {
+            const double P1 = fmin(s0, s1);
+            if (P1 > P0) {
+                push_piece<ACC>(sh, slots, P0, P1, st, 0.0);
+                P0 = P1;
+            }
+            if (!(P1 < S1)) break;
+            if (s0 <= s1) s0 = crossing(0);
+            else s1 = crossing(1);
+        }
+        return;
+    }
+    double sp[4 * MAXB + 2];
     int nsp = 0;
 #pragma unroll 1
     for (int ei = 0; ei < 2; ++ei) {
@@ -444,9 +528,6 @@ __device__ void push_far(BlockSh& sh, double* slots, int half, const Pair& P, St
             }
         }
     }
-    const double fdx = lnear ? sx : lx, fdy = lnear ? sy : ly;       // far edge
-    store_fan(sh, Fan{cf * u + sf * w, cf * w - sf * u, hn, lnear ? nsh : nl, cf * fdx + sf * fdy, cf * fdy - sf * fdx});
-    double P0 = S0;
     for (int pc = 0; pc <= nsp; ++pc) {
         const double P1 = pc < nsp ? sp[pc] : S1;
         if (P1 > P0) push_piece<ACC>(sh, slots, P0, P1, st, 0.0);
@@ -455,14 +536,14 @@ __device__ void push_far(BlockSh& sh, double* slots, int half, const Pair& P, St
 }
 
 // the block's rounds for one window: kind 0 near, 1 far, other: no pair on this thread
-template <class ACC>
+template <class ACC, bool MANY>
 __device__ __forceinline__ void run_rounds(BlockSh& sh, double* slots, int kind, const Pair& P, Steps st, double kappa) {
     const int rounds = __syncthreads_or(kind == 0) ? 3 : 2;
     for (int s = 0; s < rounds; ++s) {
         if (threadIdx.x == 0) sh.qn = 0;
         __syncthreads();
-        if (kind == 0) push_near<ACC>(sh, slots, s, P, st, kappa);
-        else if (ACC::RETARDED && kind == 1 && s < 2) push_far<ACC>(sh, slots, s, P, st);
+        if (kind == 0) push_near<ACC, MANY>(sh, slots, s, P, st, kappa);
+        else if (ACC::RETARDED && kind == 1 && s < 2) push_far<ACC, MANY>(sh, slots, s, P, st);
         __syncthreads();
         const int n = min(sh.qn, QCAP);
         for (int i = threadIdx.x; i < n; i += AB) work_item<ACC>(sh, slots, sh.qe[i], sh.qc[i], sh.qh[i], st, kappa);
@@ -609,7 +690,7 @@ struct EfieAcc {
 // lags.  Pairs that meet more than lagw lags take them in several windows.  480-edge sphere, 7 lags: the
 // whole assembly 1524 -> 178 ms against one thread per pair, with the rays' intervals one by one and library
 // functions at every node.
-template <int ORDER>
+template <int ORDER, bool MANY>
 __global__ void __launch_bounds__(AB) k_retarded_efie(DevMesh m, double dt, int K, int lagw, double T0, double* __restrict__ S,
                                                       double* __restrict__ Phi) {
     using ACC = EfieAcc<ORDER>;
@@ -654,7 +735,7 @@ __global__ void __launch_bounds__(AB) k_retarded_efie(DevMesh m, double dt, int 
         const int kd = k0 <= khi ? kind : 2;
         sh.j0[tid] = k0 - ORDER - 1;
         for (int i = 0; i < st.ni * ACC::NCOMP; ++i) slots[i * AB + tid] = 0.0;
-        run_rounds<ACC>(sh, slots, kd, P, st, 0.0);
+        run_rounds<ACC, MANY>(sh, slots, kd, P, st, 0.0);
         if (kd == 2) continue;
         const int nk = min(lagw, khi - k0 + 1);
         for (int l = 0; l < nk; ++l) {
@@ -748,7 +829,7 @@ struct MfieAcc {
     }
 };
 
-template <int ORDER>
+template <int ORDER, bool MANY>
 __global__ void __launch_bounds__(AB) k_retarded_mfie(DevMesh m, double dt, int K, int lagw, double* __restrict__ MM) {
     using ACC = MfieAcc<ORDER>;
     BlockSh& sh = block_sh();
@@ -791,7 +872,7 @@ __global__ void __launch_bounds__(AB) k_retarded_mfie(DevMesh m, double dt, int 
         const int kd = k0 <= khi ? kind : 2;
         sh.j0[tid] = k0 - ORDER;
         for (int i = 0; i < st.ni * ACC::NCOMP; ++i) slots[i * AB + tid] = 0.0;
-        run_rounds<ACC>(sh, slots, kd, P, st, 0.0);
+        run_rounds<ACC, MANY>(sh, slots, kd, P, st, 0.0);
         if (kd == 2) continue;
         const int nk = min(lagw, khi - k0 + 1);
         for (int l = 0; l < nk; ++l) {
@@ -850,7 +931,7 @@ struct YukAcc {
         if (valid) sh.d[t] = P.d;
 #pragma unroll
         for (int i = 0; i < NCOMP; ++i) slots[i * AB + t] = 0.0;
-        run_rounds<YukAcc>(sh, slots, valid ? 0 : 2, P, Steps{0.0, 0.0, 1}, kappa);
+        run_rounds<YukAcc, false>(sh, slots, valid ? 0 : 2, P, Steps{0.0, 0.0, 1}, kappa);
         const double f = 1.0 / (4.0 * M_PI);
         z0 = f * slots[t];
         z1 = f * (V3{slots[AB + t], slots[2 * AB + t], slots[3 * AB + t]} - (slots[t] * P.d) * P.n);
@@ -1045,27 +1126,37 @@ static void launch_pairs(K kernel, int64_t n, size_t smem, cudaStream_t s, A... 
 }
 
 // lags per window: what a pair of the mesh can meet (its distances span at most twice the longest
-// edge), at most LAGW so that two blocks of 128 pairs fit the shared memory of an SM
+// edge), at most LAGW, so that blocks of 128 pairs fit the shared memory of an SM: two (EFIE, 83 KB) and
+// three (MFIE, 58 KB) at order 1, one at order 2 (134 and 144 KB)
 static int lag_window(double lmax, double dt, int order) {
     const double span = std::ceil(2.0 * lmax / dt) + order + 4.0;
     return span < LAGW ? (int)span : LAGW;
 }
 
+// a circle and a half of room for the ends' rounding
+static bool many_circles(double lmax, double dt) { return lmax / dt + 2.5 > MAXB; }
+
+template <int ORDER>
+static void launch_efie(const DevMesh& m, double dt, int K, double T0, double lmax, double* S, double* Phi, cudaStream_t s) {
+    const int w = lag_window(lmax, dt, ORDER);
+    launch_pairs(many_circles(lmax, dt) ? k_retarded_efie<ORDER, true> : k_retarded_efie<ORDER, false>, (int64_t)m.nc * 7 * m.nc,
+                 pair_smem(EfieAcc<ORDER>::NCOMP, w + ORDER + 1), s, m, dt, K, w, T0, S, Phi);
+}
 void launch_retarded_efie(const DevMesh& m, double dt, int K, double T0, double lmax, double* S, double* Phi, int order,
                           cudaStream_t s) {
-    const int64_t n = (int64_t)m.nc * 7 * m.nc;
-    const int w = lag_window(lmax, dt, order);
-    if (order == 1)
-        launch_pairs(k_retarded_efie<1>, n, pair_smem(EfieAcc<1>::NCOMP, w + 2), s, m, dt, K, w, T0, S, Phi);
-    else
-        launch_pairs(k_retarded_efie<2>, n, pair_smem(EfieAcc<2>::NCOMP, w + 3), s, m, dt, K, w, T0, S, Phi);
+    if (order == 1) launch_efie<1>(m, dt, K, T0, lmax, S, Phi, s);
+    else launch_efie<2>(m, dt, K, T0, lmax, S, Phi, s);
 }
 
+template <int ORDER>
+static void launch_mfie(const DevMesh& m, double dt, int K, double lmax, double* MM, cudaStream_t s) {
+    const int w = lag_window(lmax, dt, ORDER);
+    launch_pairs(many_circles(lmax, dt) ? k_retarded_mfie<ORDER, true> : k_retarded_mfie<ORDER, false>, (int64_t)m.nf * 3 * m.nc,
+                 pair_smem(MfieAcc<ORDER>::NCOMP, w + ORDER), s, m, dt, K, w, MM);
+}
 void launch_retarded_mfie(const DevMesh& m, double dt, int K, double lmax, double* MM, int order, cudaStream_t s) {
-    const int64_t n = (int64_t)m.nf * 3 * m.nc;
-    const int w = lag_window(lmax, dt, order);
-    if (order == 1) launch_pairs(k_retarded_mfie<1>, n, pair_smem(MfieAcc<1>::NCOMP, w + 1), s, m, dt, K, w, MM);
-    else launch_pairs(k_retarded_mfie<2>, n, pair_smem(MfieAcc<2>::NCOMP, w + 2), s, m, dt, K, w, MM);
+    if (order == 1) launch_mfie<1>(m, dt, K, lmax, MM, s);
+    else launch_mfie<2>(m, dt, K, lmax, MM, s);
 }
 
 void launch_static(const DevMesh& m, double kappa, double* Zs, double* Psi, double* M, double* G, cudaStream_t s) {

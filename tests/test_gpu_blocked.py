@@ -241,3 +241,55 @@ def test_one_step_does_not_pay_for_a_chunk():
         times[nt] = min(best)
     print(times)
     assert times[1] < 0.6 * times[8]
+
+
+def _prism(sections, length, radius):
+    """A slightly irregular triangular prism of `sections` sections with a triangle at either end."""
+    rng = np.random.default_rng(5)
+    V = [((radius + 0.05 * rng.uniform()) * np.cos(2.1 * i + 0.1 * s), (radius + 0.05 * rng.uniform()) * np.sin(2.1 * i + 0.1 * s), length * s)
+         for s in range(sections + 1) for i in range(3)]
+    F = [(0, 2, 1), (3 * sections, 3 * sections + 1, 3 * sections + 2)]
+    for s in range(sections):
+        for i in range(3):
+            a, b = 3 * s + i, 3 * s + (i + 1) % 3
+            F += [(a, b, b + 3), (a, b + 3, a + 3)]
+    return np.array(V), np.array(F, dtype=np.int32)
+
+
+@pytest.mark.parametrize("circles", [60, 63, 90])
+def test_quadrature_many_circles(circles):
+    """As many breakpoint circles across an edge as the list of cuts holds, and more: every one of them
+    splits, in both forms of the rule.  The scalar potential's blocks of a pair against the oracle's rule with all breakpoints."""
+    from oracle import cquad
+    V, F = _prism(5, 1.0, 0.5)
+    tri = V[F]
+    L = max(np.linalg.norm(tri[:, i] - tri[:, (i + 1) % 3], axis=1).max() for i in range(3))
+    dt = L / circles
+    s = _solver((V, F), dt, 1, 1, "fp64")
+    T0, K = s.D, s.K
+    Phi = np.stack([s.matrix("Phi", k) for k in range(K)])
+    s.close()
+    s15 = np.sqrt(15.0)
+    rule = [((1 / 3, 1 / 3, 1 / 3), 9 / 40)]
+    for sg in (-1, 1):
+        a, b, w = (9 + sg * 2 * s15) / 21, (6 - sg * s15) / 21, (155 - sg * s15) / 1200
+        rule += [((a, b, b), w), ((b, a, b), w), ((b, b, a), w)]
+    brk = [j * dt for j in range(1, K)]
+    area = 0.5 * np.linalg.norm(np.cross(tri[:, 1] - tri[:, 0], tri[:, 2] - tri[:, 0]), axis=1)
+    far = 0
+    for c, c2 in ((0, 2), (4, 6), (4, 3), (4, 28), (30, 3), (3, 31)):
+        n = np.cross(tri[c2, 1] - tri[c2, 0], tri[c2, 2] - tri[c2, 0])
+        n /= np.linalg.norm(n)
+        lags = np.argsort(-np.abs(Phi[:, c, c2]))[:60:4]
+        ref = np.zeros(len(lags))
+        for bary, w in rule:
+            x = np.array(bary) @ tri[c]
+            p = x - np.dot(x - tri[c2, 0], n) * n
+            edges = np.linalg.norm(tri[c2] - np.roll(tri[c2], 1, axis=0), axis=1).max()
+            is_far = np.linalg.norm(tri[c2] - p, axis=1).min() >= 2 * edges
+            far += is_far
+            for i, k in enumerate(lags):
+                m = cquad.triangle_moments(x, *tri[c2], kind=4, p1=k * dt, p2=dt, brk=brk, coplanar=2)
+                ref[i] += -T0 * w / (4 * np.pi * area[c2]) * m[0]
+        assert np.abs(Phi[lags, c, c2] - ref).max() <= 1e-10 * np.abs(ref).max(), (c, c2)
+    assert far >= 14
