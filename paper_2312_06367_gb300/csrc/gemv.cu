@@ -11,20 +11,32 @@
 
 namespace tdc {
 
-// Streams the matrices once: bound by the memory.  A warp takes BG_ROWS rows, so that a value of x is
-// fetched once for all of them (with one row per warp the fetches of x at R = 8 took eight times the
-// matrix's), and keeps that many 16-byte loads in flight per turn.  41 blocks of 7680 rows, R = 1, FP32:
-// 1356 us (7.13 TB/s); 1614 us with 4-byte loads.
+// Streams the matrices once.  FP32 is bound by the memory: several loads per row are in flight, and with
+// R > 1 a warp takes two rows, so that a value of x is fetched once for both (with one row per warp the
+// fetches of x at R = 8 took eight times the matrix's).  41 blocks of 7680 rows, R = 1, FP32: 1300 us
+// (7.4 TB/s); 1614 us with 4-byte loads.  FP64 is bound by its pipe from R = 3 on (0.62e12 multiply-adds/s),
+// where vector loads only lengthen a row's last turn.  Every R has its own kernel: a bound on r that is not a
+// constant costs a branch or an idle issue slot per product (R = 5, FP64, 7680 rows: 2.0 ms, 3.6 ms with room for 8).
 template <typename T> struct Vec16;
 template <> struct Vec16<float> { using V = float4; };
 template <> struct Vec16<double> { using V = double2; };
-template <typename T> constexpr int BG_ROWS = sizeof(T) == 4 ? 4 : 2;
 
-// W: entries per load, 1 or (rows and pointers on 16-byte boundaries) a 16-byte vector
-template <typename T, int RMAX, int W>
-__global__ void __launch_bounds__(256) k_bg_partial(const T* __restrict__ blocks, int64_t n, const T* __restrict__ x, int R,
-                                                    T* __restrict__ partial) {
-    constexpr int NR = BG_ROWS<T>;
+// Rows per warp and turns unrolled, W entries per load: 1, or (rows and pointers on 16-byte boundaries)
+// a 16-byte vector.  Measured over 1, 2, 4 rows x 1, 2, 4, 8 turns at 120 to 7680 rows per block:
+//   FP32  vectors  R = 1: 1 row x 4 (41 blocks of 7680: 1296 us; 4 x 4 1390); R > 1: 2 x 1 (R = 8, 4 blocks: 219 us; 4 x 2 305)
+//         scalars  R = 1: 1 x 8 (4 blocks of 7679: 167 us; 4 x 2 272); R > 1: 2 x 2 (R = 8: 391 us; 4 x 2 386, 1 x 2 725)
+//   FP64  1 row (R = 8, 7679: 3.24 ms; 2 rows 3.27, 4 rows 3.7), 4 turns up to R = 4, above 1
+template <typename T, int R, int W>
+struct BgShape {
+    static constexpr bool F32 = sizeof(T) == 4;
+    static constexpr int ROWS = F32 && R > 1 ? 2 : 1;
+    static constexpr int TURNS = !F32 ? (R <= 4 ? 4 : 1) : R > 1 ? (W > 1 ? 1 : 2) : W > 1 ? 4 : 8;
+};
+
+template <typename T, int R, int W>
+__global__ void k_bg_partial(const T* __restrict__ blocks, int64_t n, const T* __restrict__ x,
+                             T* __restrict__ partial) {
+    constexpr int NR = BgShape<T, R, W>::ROWS;
     const int64_t row0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * NR;
     const int64_t q = blockIdx.y;
     const int lane = threadIdx.x & 31;
@@ -34,8 +46,8 @@ __global__ void __launch_bounds__(256) k_bg_partial(const T* __restrict__ blocks
     int64_t ro[NR];      // rows behind the last one read the last one
 #pragma unroll
     for (int i = 0; i < NR; ++i) ro[i] = (row0 + i < n ? i : n - 1 - row0) * n;
-    T s[NR][RMAX] = {};
-#pragma unroll(RMAX == 1 && W > 1 ? 4 : 2)
+    T s[NR][R] = {};
+#pragma unroll(BgShape<T, R, W>::TURNS)
     for (int64_t j = W * lane; j < n; j += 32 * W) {
         T v[NR][W];
 #pragma unroll
@@ -44,8 +56,7 @@ __global__ void __launch_bounds__(256) k_bg_partial(const T* __restrict__ blocks
             else *reinterpret_cast<typename Vec16<T>::V*>(v[i]) = __ldcs(reinterpret_cast<const typename Vec16<T>::V*>(a + ro[i] + j));
         }
 #pragma unroll
-        for (int r = 0; r < RMAX; ++r) {
-            if (r >= R) break;
+        for (int r = 0; r < R; ++r) {
             T u[W];
             if constexpr (W == 1) u[0] = xq[r * n + j];
             else *reinterpret_cast<typename Vec16<T>::V*>(u) = *reinterpret_cast<const typename Vec16<T>::V*>(xq + r * n + j);
@@ -58,10 +69,10 @@ __global__ void __launch_bounds__(256) k_bg_partial(const T* __restrict__ blocks
 #pragma unroll
     for (int i = 0; i < NR; ++i)
 #pragma unroll
-        for (int r = 0; r < RMAX; ++r) {
+        for (int r = 0; r < R; ++r) {
             T v = s[i][r];
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0 && r < R && row0 + i < n) partial[(q * R + r) * n + row0 + i] = v;
+            if (lane == 0 && row0 + i < n) partial[(q * R + r) * n + row0 + i] = v;
         }
 }
 
@@ -76,24 +87,23 @@ __global__ void k_bg_reduce(const T* partial, int64_t nblk, int64_t n, int R, T*
     out[i] = s;
 }
 
-template <typename T, int RMAX>
-static void launch_bg_partial(const T* blocks, int64_t nblk, int64_t n, const T* x, int R, T* partial, cudaStream_t s) {
-    constexpr int W = 16 / (int)sizeof(T);
-    const int rows = 8 * BG_ROWS<T>;
-    const dim3 g((unsigned)((n + rows - 1) / rows), (unsigned)nblk);
-    if (n % W == 0 && (uintptr_t)blocks % 16 == 0 && (uintptr_t)x % 16 == 0)
-        k_bg_partial<T, RMAX, W><<<g, 256, 0, s>>>(blocks, n, x, R, partial);
+template <typename T, int R>
+static void launch_bg_partial(const T* blocks, int64_t nblk, int64_t n, const T* x, T* partial, cudaStream_t s) {
+    constexpr int V = 16 / (int)sizeof(T), W = sizeof(T) == 8 && R > 3 ? 1 : V;
+    const auto grid = [&](int rows) { return dim3((unsigned)((n + 8 * rows - 1) / (8 * rows)), (unsigned)nblk); };
+    if (W > 1 && n % W == 0 && (uintptr_t)blocks % 16 == 0 && (uintptr_t)x % 16 == 0)
+        k_bg_partial<T, R, W><<<grid(BgShape<T, R, W>::ROWS), 256, 0, s>>>(blocks, n, x, partial);
     else
-        k_bg_partial<T, RMAX, 1><<<g, 256, 0, s>>>(blocks, n, x, R, partial);
+        k_bg_partial<T, R, 1><<<grid(BgShape<T, R, 1>::ROWS), 256, 0, s>>>(blocks, n, x, partial);
 }
 
 template <typename T>
 static cudaError_t launch_block_gemv(const T* blocks, int64_t nblk, int64_t n, const T* x, int R, T* out, T* partial,
                                      cudaStream_t s) {
-    if (R == 1) launch_bg_partial<T, 1>(blocks, nblk, n, x, R, partial, s);
-    else if (R == 2) launch_bg_partial<T, 2>(blocks, nblk, n, x, R, partial, s);
-    else if (R <= 4) launch_bg_partial<T, 4>(blocks, nblk, n, x, R, partial, s);
-    else launch_bg_partial<T, 8>(blocks, nblk, n, x, R, partial, s);
+    using Launch = void (*)(const T*, int64_t, int64_t, const T*, T*, cudaStream_t);
+    static const Launch by_r[] = {launch_bg_partial<T, 1>, launch_bg_partial<T, 2>, launch_bg_partial<T, 3>, launch_bg_partial<T, 4>,
+                                  launch_bg_partial<T, 5>, launch_bg_partial<T, 6>, launch_bg_partial<T, 7>, launch_bg_partial<T, 8>};
+    by_r[R - 1](blocks, nblk, n, x, partial, s);
     launch_chained(k_bg_reduce<T>, (unsigned)((n * R + 63) / 64), 64, s, 0, (const T*)partial, nblk, n, R, out);
     return cudaGetLastError();
 }

@@ -293,3 +293,20 @@ def test_quadrature_many_circles(circles):
                 ref[i] += -T0 * w / (4 * np.pi * area[c2]) * m[0]
         assert np.abs(Phi[lags, c, c2] - ref).max() <= 1e-10 * np.abs(ref).max(), (c, c2)
     assert far >= 14
+
+
+@pytest.mark.parametrize("R", range(1, 9))
+@pytest.mark.parametrize("dtype,tol", [("float64", 1e-13), ("float32", 1e-5)])
+def test_block_gemv_every_wave_count(dtype, tol, R):
+    """Each number of vectors has its own kernel, for rows that vector loads fit and others."""
+    import torch
+    from paper_2312_06367_gb300 import block_gemv
+    g = torch.Generator(device="cuda").manual_seed(R)
+    dt = getattr(torch, dtype)
+    for n in (132, 131):
+        B = torch.randn((3, n, n), generator=g, dtype=dt, device="cuda")
+        X = torch.randn((3, R, n), generator=g, dtype=dt, device="cuda")
+        ref = torch.einsum("qij,qrj->ri", B.double(), X.double())
+        got = block_gemv(B, X)
+        torch.cuda.synchronize()
+        assert float((got.double() - ref).norm() / ref.norm()) < tol
