@@ -1,4 +1,4 @@
-"""GPU: several uneven scatterers stepped by one graph launch per step (tdcfie_batch_*).
+"""GPU: several uneven scatterers stepped together (tdcfie_batch_*).
 
 Each member computes exactly what tdcfie_step computes on its own handle, so the batched currents
 must equal the individually marched ones bit for bit, for mixed sizes, time steps, path precisions
@@ -89,7 +89,7 @@ def test_batch_rejects_bad_input():
 
 
 # ---------------------------------------------------------------- persistent form
-# every member FP32 with one wave and the direct solve: one cooperative kernel per step
+# every member FP32 with one wave and the direct solve: one cooperative kernel for up to 32 steps
 PCASES = [  # mesh, dt (uneven sizes and lags; a torus; one mesh whose edge count is not a multiple of 4)
     (meshes.icosphere(2), 0.2),
     (meshes.torus(1.0, 0.3, 16, 8), 0.3),
@@ -162,3 +162,39 @@ def test_persistent_batch_member_matches_oracle():
     j_ref = fm.postprocess(mot.march_factored(fm, fm.rhs(e, h)))
     j = outs[1].double().cpu().numpy().transpose(0, 2, 1)
     assert np.linalg.norm(j - j_ref) / np.linalg.norm(j_ref) < 1e-5
+
+
+# ---------------------------------------------------------------- graph branches with every kind of member
+def test_batch_of_gmres_and_tensor_members():
+    """GMRES members on parallel branches (each solve a cooperative kernel whose blocks wait for one
+    another; together they have more blocks than the GPU holds at once), a tensor-core member, a factored
+    and a direct one."""
+    import torch
+    from paper_2312_06367_gb300 import Batch, Solver
+    nt = 24
+    kinds = [(meshes.icosphere(2), 0.2, "fp32", 1, "gmres"), (meshes.icosphere(2), 0.3, "fp64", 1, "gmres"),
+             (meshes.icosphere(1), 0.3, "fp32", 8, "gmres"), (meshes.icosphere(2), 0.25, "fp32", 2, "gmres"),
+             (meshes.icosphere(1), 0.4, "fp16x3", 64, "direct"), (meshes.torus(1.0, 0.4, 10, 5), 0.5, "fp64", 2, "factored"),
+             (meshes.torus(1.0, 0.4, 5, 3), 0.5, "fp32", 1, "direct")]
+    ss, outs, refs = [], [], []
+    for i, ((V, F), dt, prec, R, kind) in enumerate(kinds):
+        s = Solver(V, F, dt=dt, nt=nt, precision=prec, R=R).assemble()
+        if kind == "gmres":
+            s.set_solver("gmres", "extrap", 1e-8)
+        if kind == "factored":
+            s.set_history_form("factored")
+        refs.append(torch.zeros((nt, R, s.ne), dtype=s.dtype, device="cuda"))
+        outs.append(torch.zeros_like(refs[-1]))
+        s.march(_pw(200 + i, R), refs[-1])
+        s.set_excitation(_pw(200 + i, R))
+        ss.append(s)
+    b = Batch(ss)
+    b.step(7, [o[:7] for o in outs])
+    b.step(nt - 7, [o[7:] for o in outs])
+    b.close()
+    torch.cuda.synchronize()
+    for i, (o, ref) in enumerate(zip(outs, refs)):
+        assert torch.isfinite(o).all() and torch.equal(o, ref), kinds[i][2:]
+    for s, k in zip(ss, kinds):
+        if k[4] == "gmres":
+            assert s.gmres_stats()["steps"] == nt and s.gmres_stats()["not_converged"] == 0

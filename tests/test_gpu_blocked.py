@@ -310,3 +310,22 @@ def test_block_gemv_every_wave_count(dtype, tol, R):
         got = block_gemv(B, X)
         torch.cuda.synchronize()
         assert float((got.double() - ref).norm() / ref.norm()) < tol
+
+
+@pytest.mark.parametrize("R", [2, 3, 8])
+def test_fp32_waves_against_fp64(waves, R):
+    """More lags (21) than a chunk has steps, every wave by itself against the FP64 path on the same
+    matrices.  The path's own rounding is 2e-5 to 4e-5 of the currents on this mesh; a wrong lag, column
+    or wave is of their size."""
+    import torch
+    dt, nt = SPLITS[0]
+    pw = {k: v[:R] for k, v in waves.items()}
+    s = _solver(SMALL, dt, nt, R, "fp64")
+    ref = torch.zeros((nt, R, s.ne), dtype=torch.float64, device="cuda")
+    s.march(pw, ref)
+    s.replan("fp32", R)
+    out = torch.zeros((nt, R, s.ne), dtype=torch.float32, device="cuda")
+    s.march(pw, out)
+    torch.cuda.synchronize()
+    for r in range(R):
+        assert float((out[:, r].double() - ref[:, r]).norm() / ref[:, r].norm()) < 1e-4, r
