@@ -59,6 +59,10 @@ def peaks():
         return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "fallback": True}
 
 
+# the dense FP64 / FP32 history: its bytes per step over its time are not a bandwidth
+SIMT_HISTORY = "history sum (k_pre + k_hist): a pass over the blocks of the older lags serves a chunk of steps"
+
+
 class Clocks:
     """nvidia-smi sampler running during the timed region."""
 
@@ -328,12 +332,8 @@ def run_guess_study(args, w):
                    "solver": "gmres", "guess": best, "gmres_tol": w["gmres_tol"], "assemble_s": round(t_asm, 1),
                    "cache": "inputs larger than L2"},
         "gpu_launches": int(m["launches"]),
-        "roofline": {"bound": "hbm", "achieved": hb / (m["history_ms"] / 1e3) / 1e9 if m["history_ms"] else None,
-                     "peak": pk.get("hbm_gbs"), "unit": "GB/s",
-                     "frac": (hb / (m["history_ms"] / 1e3) / 1e9 / pk["hbm_gbs"]) if m["history_ms"] else None,
-                     "traffic": None,
-                     "kernel": "history sum (k_pre + k_hist; the bytes are those of a sum per step, a pass over older lags serves a chunk)",
-                     "algorithmic_bytes_per_launch": hb},
+        "roofline": {"bound": "hbm", "achieved": None, "peak": pk.get("hbm_gbs"), "unit": "GB/s", "frac": None, "traffic": None,
+                     "kernel": SIMT_HISTORY, "history_ms": m["history_ms"], "algorithmic_bytes_per_step": hb},
         "guess_study": rows, "training": info,
     }
     print(json.dumps(line), flush=True)
@@ -391,8 +391,8 @@ def run_accuracy(args, w):
 
 
 def run_batch(args, probs, name):
-    """Uneven batch: every scatterer FP32 with one wave, all advanced by one graph launch per step
-    (tdcfie_batch_step: the persistent cooperative kernel, launch shape from tdcfie_batch_tune),
+    """Uneven batch: every scatterer FP32 with one wave, all advanced together (tdcfie_batch_step: the
+    persistent cooperative kernel, up to 32 steps per launch, launch shape from tdcfie_batch_tune),
     against the same handles stepped one after another (tdcfie_step each)."""
     import torch
 
@@ -438,14 +438,13 @@ def run_batch(args, probs, name):
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": name, "scatterers": len(ss), "edges": [s.ne for s in ss], "K": [s.K for s in ss],
                    "dt": probs[0]["dt"], "assemble_s": round(t_asm, 1), "tune_s": round(t_tune, 2), "launch": cfg,
-                   "cache": f"history operands of all scatterers ({hb / 1e9:.2f} GB) stream each step",
+                   "cache": f"history operands of all scatterers: {hb / 1e9:.2f} GB",
                    "finite": finite},
         "gpu_launches": -(-args.steps // 32) if cfg["persistent"] else int(t["launches"]) * args.steps,
-        "sequential": {"ms_per_step": seq_ms, "steps_s": 1e3 / seq_ms, "how": "each handle's own step graph, one after another"},
+        "sequential": {"ms_per_step": seq_ms, "steps_s": 1e3 / seq_ms, "how": "each handle's own march, one after another"},
         "speedup_vs_sequential": seq_ms / t["step_ms"],
-        "roofline": {"bound": "hbm", "achieved": hb / (t["step_ms"] / 1e3) / 1e9, "peak": pk.get("hbm_gbs"), "unit": "GB/s",
-                     "frac": hb / (t["step_ms"] / 1e3) / 1e9 / pk["hbm_gbs"], "traffic": None,
-                     "kernel": "whole batch step (k_batch_step; history rows dominate)", "algorithmic_bytes_per_launch": hb},
+        "roofline": {"bound": "hbm", "achieved": None, "peak": pk.get("hbm_gbs"), "unit": "GB/s", "frac": None, "traffic": None,
+                     "kernel": "whole batch step (k_batch_step: " + SIMT_HISTORY + ")", "algorithmic_bytes_per_step": hb},
         "clocks": clk.summary(),
     }
     print(json.dumps(line), flush=True)
@@ -518,7 +517,8 @@ def factored_study(s, w, steps, warmup, nt_acc, stream):
             t = s.timing()
             cur[form] = acc.double().cpu().numpy()
             h_ms = t["history_ms"]
-            gbs = st["history_bytes"] / (h_ms / 1e3) / 1e9 if h_ms > 0 else None
+            # (no bandwidth for the dense form: see SIMT_HISTORY)
+            gbs = st["history_bytes"] / (h_ms / 1e3) / 1e9 if h_ms > 0 and form == "factored" else None
             row[form] = {"steps_s": 1e3 / t["step_ms"], "step_ms": t["step_ms"], "history_ms": h_ms,
                          "history_bytes": st["history_bytes"], "step_bytes": st["step_bytes"],
                          "history_gbs": gbs, "history_frac_hbm": gbs / pk["hbm_gbs"] if gbs else None,
@@ -617,7 +617,7 @@ def run_ours(args, w):
     # roofline of the dominant kernel (history sum: streams every history and right-hand-side block)
     pk = peaks()
     h_ms = statistics.mean(hist_ms) if hist_ms and hist_ms[0] > 0 else None
-    achieved = work_bytes / (h_ms / 1e3) / 1e9 if h_ms else None
+    achieved = work_bytes / (h_ms / 1e3) / 1e9 if h_ms and (tensor or factored) else None
     traffic = None
     prof = os.path.join(ROOT, "profiles", f"history_{w['name']}.json")
     if os.path.exists(prof):
@@ -641,8 +641,7 @@ def run_ours(args, w):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": pk.get("hbm_gbs"), "unit": "GB/s",
                      "frac": (achieved / pk["hbm_gbs"]) if achieved else None, "traffic": traffic,
                      "kernel": ("factored history sum over all lags of S_k, MM'_k, Phi_k (k_shells)" if factored else
-                                "history sum (k_pre + k_hist; the bytes are those of a sum per step, a pass over older lags serves a chunk)"
-                                if prec in ("fp64", "fp32") else
+                                SIMT_HISTORY if prec in ("fp64", "fp32") else
                                 "tcgen05 split-precision history GEMM (k_tc_gemm + k_tc_fix)"),
                      "algorithmic_bytes_per_launch": work_bytes, "history_ms": h_ms,
                      "peak_source": "measured" if not pk.get("fallback") else "fallback"},
