@@ -19,6 +19,8 @@
 //
 // Rows of matrices and vectors are padded to 16 bytes (zeros), every load is a 16-byte vector.
 #pragma once
+#include <type_traits>
+
 #include "internal.h"
 
 namespace tdc {
@@ -204,9 +206,11 @@ struct Acc<float> {
 __device__ __forceinline__ double2 neg(double2 a) { return a; }    // unused by Acc<double>
 __device__ __forceinline__ float4 neg(float4 a) { return make_float4(-a.x, -a.y, -a.z, -a.w); }
 
-// acc[i][c] += row_i . x_c for ROWS rows and the first nv of COLS columns, nvec vectors per row.  The
-// loads do not branch on a column (one that is not wanted repeats another or points at zeros), so that
-// all loads of a turn are in flight together; the rows' next vectors are fetched a turn ahead.
+// acc[i][c] += row_i . x_c for ROWS rows and (at least) the first nv of COLS columns, nvec vectors per row.
+// The loads do not branch on a column (one that is not wanted repeats another, whose sum nobody reads, or
+// points at zeros), so that all loads of a turn are in flight together; the rows' next vectors are fetched a
+// turn ahead.  A loop each for 1, 2, 4, 8 columns: a bound inside it is predicated and costs the pipe all of
+// them (two blocks of 3072 rows, FP64: 302 us with one column as with eight, 69 us so).
 // before_x() runs between the first loads of the rows and the first loads of x (a kernel whose x comes
 // from the kernel before it waits there).
 struct Nothing { __device__ __forceinline__ void operator()() const {} };
@@ -229,10 +233,11 @@ __device__ __forceinline__ void tile_rows(const T* const (&row)[ROWS], const T* 
         unsigned xo[COLS];
 #pragma unroll
         for (int c = 0; c < COLS; ++c) xo[c] = (unsigned)off[c] * (unsigned)sizeof(T) + (unsigned)lane * 16u;
-        auto turn = [&](bool more, bool all) {
-            V a[ROWS], na[ROWS], xv[COLS];
+        auto turn = [&](bool more, auto cols) {
+            constexpr int N = decltype(cols)::value;
+            V a[ROWS], na[ROWS], xv[N];
 #pragma unroll
-            for (int c = 0; c < COLS; ++c) {
+            for (int c = 0; c < N; ++c) {
                 xv[c] = *reinterpret_cast<const V*>(xb + xo[c]);
                 xo[c] += 512u;
             }
@@ -244,18 +249,18 @@ __device__ __forceinline__ void tile_rows(const T* const (&row)[ROWS], const T* 
                 if (more) nx[i] = __ldg(ap[i]);
             }
 #pragma unroll
-            for (int c = 0; c < COLS; ++c)
-                if (all || c < nv)
+            for (int c = 0; c < N; ++c)
 #pragma unroll
-                    for (int i = 0; i < ROWS; ++i) acc[i][c].add(a[i], na[i], xv[c]);
+                for (int i = 0; i < ROWS; ++i) acc[i][c].add(a[i], na[i], xv[c]);
         };
-        if (nv >= COLS) {
+        auto loop = [&](auto cols) {
 #pragma unroll 1
-            for (int j = lane; j < nvec; j += 32) turn(j + 32 < nvec, true);
-        } else {
-#pragma unroll 1
-            for (int j = lane; j < nvec; j += 32) turn(j + 32 < nvec, false);
-        }
+            for (int j = lane; j < nvec; j += 32) turn(j + 32 < nvec, cols);
+        };
+        if (2 * nv > COLS) loop(std::integral_constant<int, COLS>());
+        else if (4 * nv > COLS) loop(std::integral_constant<int, COLS / 2>());
+        else if (nv > 1) loop(std::integral_constant<int, COLS / 4>());
+        else loop(std::integral_constant<int, 1>());
     } else {
         // turns whose loads are issued together: a whole row up to about 1000 entries
         constexpr int U = ROWS * COLS >= 4 ? 2 : ROWS * COLS == 2 ? 4 : 8;
