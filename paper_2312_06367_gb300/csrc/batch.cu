@@ -58,7 +58,7 @@ static int phase_units(const StepPlan* p, int ph) {
 __device__ __forceinline__ void batch_unit(int ph, const SimtDev<float>& d, int t, int left, int np, int u, int lane) {
     const Ctl* c = d.ctl;
     StepPos pos{c->n + t, (c->slot + t) % d.ring, (c->col + t) % d.C};
-    const Cols cs = ph <= PH_PRE ? new_cols(d, pos.n, pos.col, left) : Cols{};
+    const Cols cs = ph <= PH_PRE ? new_cols(d.ctl, d.C, pos.n, pos.col, left) : Cols{};
     if (ph == PH_ENV) {
         const int idx = 32 * u + lane, nc = cs.hi - cs.lo;
         if (idx < d.npts * nc) {

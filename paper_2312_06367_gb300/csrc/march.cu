@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(128) k_env(const __grid_constant__ SimtDev<T> 
     wait_prior();
     const int64_t n = d.ctl->n;
     const int col = d.ctl->col;
-    const Cols cs = new_cols(d, n, col, most);
+    const Cols cs = new_cols(d.ctl, d.C, n, col, most);
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int nc = cs.hi - cs.lo;
     if (idx >= (int64_t)d.npts * d.R * nc) return;
@@ -44,7 +44,7 @@ template <typename T>
 __global__ void __launch_bounds__(128) k_gather(const __grid_constant__ SimtDev<T> d, int most) {
     wait_prior();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const Cols cs = new_cols(d, d.ctl->n, d.ctl->col, most);
+    const Cols cs = new_cols(d.ctl, d.C, d.ctl->n, d.ctl->col, most);
     if (w >= d.ne * d.R || cs.lo == cs.hi) return;
     gather_edge<T>(d, cs, w / d.R, w % d.R, threadIdx.x & 31);
 }
@@ -55,7 +55,7 @@ template <typename T>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 3) k_pre(const __grid_constant__ SimtDev<T> d, int ctiles, int most) {
     wait_prior();
     const int col = d.ctl->col;
-    const Cols cs = new_cols(d, d.ctl->n, col, most);
+    const Cols cs = new_cols(d.ctl, d.C, d.ctl->n, col, most);
     if (cs.lo == cs.hi) return;
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) d.ctl->t_mark = device_ns();
     const int tile = blockIdx.x % ctiles, rb = blockIdx.x / ctiles;
@@ -240,12 +240,13 @@ static cudaError_t launch_graph(tdcfie_t h, StepPlan& p, int which, cudaStream_t
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 static cudaError_t launch_graph_tc(tdcfie_t h, StepPlan& p, int which, cudaStream_t s, int& k) {
-    const bool chunk = which == StepPlan::G_CHUNK;
-    if (which == StepPlan::G_PRE || chunk) k += launch_tests_tc(h, &p, s);
-    if (which == StepPlan::G_STEP || which == StepPlan::G_LAST) k += launch_inner_tc(h, &p, 0, which == StepPlan::G_STEP, s);
+    const bool chunk = which == StepPlan::G_CHUNK, last = which >= StepPlan::G_LAST;
+    if (which == StepPlan::G_PRE || chunk) k += launch_tests_tc(h, &p, chunk ? p.C : 0, s);
+    if (which == StepPlan::G_STEP || last) k += launch_inner_tc(h, &p, 0, which == StepPlan::G_STEP, s);
     if (chunk)
         for (int i = 0; i < p.C; ++i) k += launch_inner_tc(h, &p, i, false, s);
-    if (which == StepPlan::G_LAST || chunk) k += launch_post_tc(h, &p, chunk ? p.C : 1, s);
+    if (chunk) k += launch_post_tc(h, &p, p.C, p.C, s);
+    if (last) k += launch_post_tc(h, &p, 1, which - StepPlan::G_LAST + 1, s);
     return cudaGetLastError();
 }
 
@@ -318,9 +319,12 @@ tdcfie_status build_plan(tdcfie_t h) {
     if (tensor) p->esz = 4;   // the tensor-core paths keep FP32 vectors, 16-bit hi/lo matrices
     const size_t es = p->esz;
     // Steps per chunk.  Matrix blocks read per step: (K + 1) / C + (C - 1) / 2 + 1 + 1 / C, least near
-    // C = sqrt(2 (K + 2)) = 9 at K = 42; where everything sits in L2 (up to about 1000 edges) the
-    // kernels per chunk count, not the bytes, and 16 steps share them.  The tests' kernel needs a
-    // divisor of 32.  Against every block in every step: 480 edges FP64 232 -> 20 us per step, 1920 edges
+    // C = sqrt(2 (K + 2)) = 9 at K = 42; where the C matrices that a step re-reads sit in L2 the kernels
+    // per chunk count, not the bytes, and 16 steps share them.  The tests' kernel needs a divisor of 32.
+    // us per step with 8 and 16, R = 1, FP64 / FP32: 480 edges 22.6 and 19.2 / 8.9 and 7.8; 990 edges 66.2
+    // and 64.5 / 19.7 and 17.6; 1920 edges, K = 42, 319 and 310 / 72.9 and 73.4; 3072 edges 469 and 455 /
+    // 109 and 112.  R = 3: 990 edges 173 and 173 / 42.9 and 42.7; 1320 edges 284 and 289 / 68 and 71.  So 16 pays
+    // clearly below the line, and beyond it little (FP64) or nothing.  Against every block in every step: 480 edges FP64 232 -> 20 us per step, 1920 edges
     // FP32 243 -> 74 us, with eight waves 990 -> 490 us.
     p->C = tensor ? tc_chunk() : (ne <= 1024 && R <= 2 ? 16 : 8);
     p->ring = tensor ? h->K - 1 : h->K - 1 + p->C;
@@ -575,9 +579,9 @@ cudaError_t capture_step(tdcfie_t h, cudaStream_t s) {
     };
     if (p->prec == TDCFIE_FP64) return simt(0.0);
     if (p->prec == TDCFIE_FP32) return simt(0.f);
-    p->launches_per_step = launch_tests_tc(h, p, s);
+    p->launches_per_step = launch_tests_tc(h, p, 1, s);
     p->launches_per_step += launch_inner_tc(h, p, 0, false, s);
-    p->launches_per_step += launch_post_tc(h, p, 1, s);
+    p->launches_per_step += launch_post_tc(h, p, 1, 1, s);
     return cudaGetLastError();
 }
 
@@ -676,9 +680,9 @@ tdcfie_status plan_step(tdcfie_t h, int64_t nsteps, void* out, void* yout) {
         if (m == C) {
             RUN(StepPlan::G_CHUNK);
         } else {
-            if (i == 0 || (n - i == 1 && !p->gemm)) RUN(StepPlan::G_PRE);      // (new_cols)
+            if (i == 0 || n - i == 1) RUN(StepPlan::G_PRE);      // (new_cols)
             for (int64_t q = 1; q < m; ++q) RUN(StepPlan::G_STEP);
-            RUN(p->fact ? StepPlan::G_STEP : StepPlan::G_LAST);
+            RUN(p->fact ? StepPlan::G_STEP : StepPlan::G_LAST + (p->gemm ? (int)m - 1 : 0));
         }
         n += m;
     }

@@ -44,8 +44,9 @@ struct StepPlan {
     // tensor-core path
     TcStep* gemm = nullptr;
     // graphs: G_PRE the tests (and, SIMT paths, pre-sums) of a chunk, G_STEP one step's history and
-    // solve, G_LAST the same and the post-processing of the finished steps, G_CHUNK a whole chunk
-    enum { G_STEP = 0, G_PRE, G_LAST, G_CHUNK, NGRAPH };
+    // solve, G_LAST the same and the post-processing of the finished steps (tensor paths: of k steps in
+    // G_LAST + k - 1), G_CHUNK a whole chunk
+    enum { G_STEP = 0, G_PRE, G_CHUNK, G_LAST, NGRAPH = G_LAST + 3 };
     cudaGraph_t graph[NGRAPH] = {};
     cudaGraphExec_t exec[NGRAPH] = {};
     int nodes[NGRAPH] = {};                              // kernels per graph

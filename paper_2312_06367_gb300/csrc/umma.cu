@@ -15,8 +15,8 @@
 // to step (vector rounding, accumulation) by about |y| / |y_n - y_{n-1}|, so those are kept near
 // or below FP32 level: the leading product A_hi x_hi has its own tensor-memory accumulator (D0),
 // separate from the four smaller ones (D1), and each accumulator covers one 64-wide k tile only;
-// the epilogue adds the tiles error-free (TwoSum pairs in registers), partial sums are reduced in
-// FP64 and the results (b_n, y_n, the projector's u) stay in FP64 until they are split again.
+// the epilogue adds the tiles error-free (TwoSum pairs in registers), partial sums are reduced as such
+// pairs, and y_n, dy_n and the projector's u are kept in FP64; b_n goes from its pair to its slices.
 //
 // Kernel layout (one CTA per SM, persistent, 320 threads):
 //   warp 0   TMA producer: A tiles (128 x 64, 128B swizzle) with L2 evict-first, x tiles
@@ -27,7 +27,9 @@
 //            and D1 (four TMEM buffers, so the next tiles' MMAs overlap), exact power-of-two
 //            rescaling, error-free accumulation, and at the end of the CTA's part of a row tile a
 //            coalesced store of the (hi, lo) partial sums.
-// Work split: stream-K over (row tile, q, k tile) iterations in row-tile-major order.  A second kernel,
+// Work split: stream-K over (row tile, q, k tile) iterations in row-tile-major order; of several products
+// with the same matrix (the projector's steps) each has blocks of its own, so that a step's sums do not
+// depend on how many are taken together.  A second kernel,
 // k_tc_fix, sums every tile's partials in a fixed order as FP32 pairs and applies the consumer's
 // epilogue: store (u, out), or split into slices for the next product (b_n), or both (y_n: FP64 for the
 // post-processing and the slices of the history ring).  (Left to the CTA that finished a tile last, the
@@ -99,16 +101,17 @@ struct GemmArgs {
     int rows, cols;       // M extent, K extent of one block
     int nblk, ktiles, rtiles;
     int reps;             // independent products with the same matrix (vector slot and output by product)
-    int64_t total;        // reps * rtiles * nblk * ktiles
+    int64_t total;        // iterations of one product: rtiles * nblk * ktiles
     int maxseg;
     int slot_mode;        // 0: history (q = 0, 1 -> ring + 2 col + q, q >= 2 -> (n - (q - 1)) mod ring);
                           // 1: slot rep; 2: slot q
     int ring;
     int off;              // step = ctl->n + off, column of the chunk ctl->col + off
     int mark;             // device time of the history: 1 starts it, 2 adds it up
-    float* partial;       // [grid][maxseg][2][NR][BM]  (hi, lo)
-    const int* seg_ptr;   // [reps rtiles + 1]
-    const int* seg_slot;  // partial slots of every row tile, in a fixed order
+    int grid;             // blocks of one product
+    float* partial;       // [reps grid][maxseg][2][NR][BM]  (hi, lo)
+    const int* seg_ptr;   // [rtiles + 1]
+    const int* seg_slot;  // partial slots of every row tile (of the first product), in a fixed order
     Ctl* ctl;
     uint32_t idesc;       // instruction descriptor (operand format)
     const float* sA;      // [rows] inverse row scales of A (one per row, common to all blocks)
@@ -407,8 +410,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     const int64_t ipt = (int64_t)g.nblk * g.ktiles;     // iterations per row tile
-    const int64_t begin = (int64_t)blockIdx.x * g.total / gridDim.x;
-    const int64_t end = (int64_t)(blockIdx.x + 1) * g.total / gridDim.x;
+    const int rep = (int)blockIdx.x / g.grid, cta = (int)blockIdx.x - rep * g.grid;
+    const int64_t begin = (int64_t)cta * g.total / g.grid;
+    const int64_t end = (int64_t)(cta + 1) * g.total / g.grid;
     Ctl* ctl = g.ctl;
 
     if (threadIdx.x == 0) {
@@ -445,8 +449,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             int rt = (int)(begin / ipt);
             int q = (int)((begin - rt * ipt) / g.ktiles);
             int kt = (int)(begin - rt * ipt - (int64_t)q * g.ktiles);
-            int rep = rt / g.rtiles;
-            rt -= rep * g.rtiles;
             for (int64_t it = begin; it < end; ++it) {
                 const int slot = slot_of(g, q, rep, base, col);
                 if (!mbar_wait(empty + stage, phase ^ 1u, ctl)) break;
@@ -470,7 +472,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     kt = 0;
                     if (++q == g.nblk) {
                         q = 0;
-                        if (++rt == g.rtiles) { rt = 0; ++rep; }
+                        ++rt;
                     }
                 }
             }
@@ -524,7 +526,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         for (int c = 0; c < EC / 2; ++c) acc_hi[c] = acc_lo[c] = make_float2(0.f, 0.f);
         int seg = 0, buf = 0;
         bool ok = true;
-        int64_t tile = begin / ipt, pos = begin - tile * ipt;   // (product, row tile) and iteration within it
+        int64_t tile = begin / ipt, pos = begin - tile * ipt;   // row tile and iteration within it
         for (int64_t it = begin; it < end; ++it) {
             if (ok && !mbar_wait(acc_full + buf, (fphase >> buf) & 1u, ctl)) ok = false;
             if (ok && !mbar_wait(sx_full + buf, (fphase >> buf) & 1u, ctl)) ok = false;
@@ -568,10 +570,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             }
             buf = buf + 1 == NBUF ? 0 : buf + 1;
             const bool tile_end = ++pos == ipt;
-            if (it + 1 == end || tile_end) {   // end of this CTA's part of row tile rt
+            if (it + 1 == end || tile_end) {   // end of this CTA's part of the row tile
                 float* dst = g.partial + ((int64_t)blockIdx.x * g.maxseg + seg) * (int64_t)2 * NR * BM;
                 // one power-of-two row scale for all blocks: applied once here (exact)
-                const int grow = (int)(tile % g.rtiles) * BM + row;
+                const int grow = (int)tile * BM + row;
                 const float sa = grow < g.rows ? g.sA[grow] : 1.f;
 #pragma unroll
                 for (int c = 0; c < EC / 2; ++c) {
@@ -610,10 +612,11 @@ __global__ void __launch_bounds__(256) k_tc_fix(GemmArgs g) {
     const int row = half * 64 + (warp & 1) * 32 + lane, r0 = blockIdx.y * FIX_RB + (warp >> 1) * 2;
     const int grow = rt * BM + row;
     float sh[2] = {0.f, 0.f}, sl_[2] = {0.f, 0.f};
-    const int p1 = g.seg_ptr[tile + 1];
+    const int p1 = g.seg_ptr[rt + 1];
+    const float* part = g.partial + ((int64_t)rep * g.grid * g.maxseg * 2 * NR + r0) * BM + row;
 #pragma unroll 4
-    for (int k = g.seg_ptr[tile]; k < p1; ++k) {
-        const float* P = g.partial + (int64_t)g.seg_slot[k] * 2 * NR * BM + (int64_t)r0 * BM + row;
+    for (int k = g.seg_ptr[rt]; k < p1; ++k) {
+        const float* P = part + (int64_t)g.seg_slot[k] * 2 * NR * BM;
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             two_sum_acc(sh[j], sl_[j], __ldcg(P + (int64_t)j * BM));
@@ -747,21 +750,24 @@ __global__ void __launch_bounds__(256) k_split_x(const double* __restrict__ x, i
 // so that it keeps its relative precision (-amp_r exp(-(a_n - d)^2) where the argument is above 64: the
 // factor would overflow); at n = 1 the test itself (r_0 = 0).  Same for h.  t - t0 is
 // carried as an FP32 pair so that late times lose no digits of the pulse's argument.
-// The tests of a chunk's TC_C steps are formed when it starts, in two kernels: the envelope increments
+// The tests of a chunk's TC_C steps are formed when it starts (in the march's first chunk: of the steps that
+// the calls make, new_cols), in two kernels: the envelope increments
 // once per quadrature point, step and wave (a point belongs to three RWG or about twelve BC functions:
 // with one exponential pair per edge and point this took 106 us per step at 1920 edges, now 27 + 82 us per
 // four steps), then one block
 // per (64-edge tile, step) gathers them, compensated FP32 sums over the points, and splits the tile into
 // the e and h slices of the step's slots with one scale per (slot, tile, wave).
 constexpr int ENV_PB = 32;       // points per block (the waves' FP64 parameters are formed once per block)
-__global__ void __launch_bounds__(NR * TC_C) k_env_tc(int npts, const double* __restrict__ exc, double dt, const Ctl* ctl,
+__global__ void __launch_bounds__(NR * TC_C) k_env_tc(int npts, const double* __restrict__ exc, double dt, const Ctl* ctl, int most,
                                                       const float* __restrict__ pts, float* __restrict__ env) {
     wait_prior();
-    if (ctl->col) return;
     const int r = threadIdx.x % NR, i = threadIdx.x / NR;      // wave, step of the chunk
+    const int col = ctl->col;
+    const Cols cs = new_cols(ctl, TC_C, ctl->n, col, most);
+    if (i < cs.lo || i >= cs.hi) return;
     const double* P = exc + 11 * r;
     const float kx = (float)P[0], ky = (float)P[1], kz = (float)P[2], amp = (float)P[6], inv_w = (float)(1.0 / P[8]);
-    const int64_t n = ctl->n + i;
+    const int64_t n = ctl->n - col + i;
     const double tt = (double)n * dt - P[7];
     const float tt_hi = (float)tt, tt_lo = (float)(tt - (double)tt_hi), d = (float)(dt / P[8]);
     const int p1 = min(npts, (int)(blockIdx.x + 1) * ENV_PB);
@@ -784,7 +790,7 @@ constexpr int RHS_NW = 16;
 constexpr int RHS_LD = 65;
 constexpr int RHS_SMEM = 2 * 64 * RHS_LD * 8;
 template <bool F16, int XS>
-__global__ void __launch_bounds__(32 * RHS_NW) k_rhs_tc(int ne, const double* __restrict__ exc, const Ctl* ctl,
+__global__ void __launch_bounds__(32 * RHS_NW) k_rhs_tc(int ne, const double* __restrict__ exc, const Ctl* ctl, int most,
                                                 const int* __restrict__ eptr, const float* env,
                                                 const float4* __restrict__ ent, const int* __restrict__ nE,
                                                 uint16_t* __restrict__ X0, uint16_t* __restrict__ X1,
@@ -793,8 +799,9 @@ __global__ void __launch_bounds__(32 * RHS_NW) k_rhs_tc(int ne, const double* __
     __shared__ float mred[2][RHS_NW][NR];
     __shared__ float scl[2][NR];
     wait_prior();
-    if (ctl->col) return;
     const int tile = blockIdx.x, step = blockIdx.y;
+    const Cols cs = new_cols(ctl, TC_C, ctl->n, ctl->col, most);
+    if (step < cs.lo || step >= cs.hi) return;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     float2 pol[2][3];       // p and k x p of the lane's two waves
 #pragma unroll
@@ -870,7 +877,8 @@ __global__ void __launch_bounds__(32 * RHS_NW) k_rhs_tc(int ne, const double* __
 // ---------------------------------------------------------------- projector in / out
 // z[r][c] = sum_j tsign[c][j] w[r][tedge[c][j]], w = dy_n / dtt - y_n (= (1/dtt - 1) y_n - y_{n-1}/dtt)
 // from the FP64 y_n and dy_n; split into the z slices with one scale per (64-triangle tile, wave).  Grid
-// z: the steps p0 .. ctl->n + adv - 1 still to post-process (at most TC_C), slot by slot.
+// z: the steps p0 .. ctl->n + adv - 1 still to post-process (at most TC_C), slot by slot.  (A march of one
+// step, 7680 edges, K = 4, with the products of four steps: 666 us, 617 us with one.)
 constexpr int PIN_RB = 16;      // waves per block
 __device__ __forceinline__ int post_count(const Ctl* ctl, int adv) { return (int)(ctl->n + adv - ctl->p0); }
 // column of the chunk of step p0 + k (ctl->col belongs to ctl->n)
@@ -1068,9 +1076,9 @@ static void plan_segments(GemmArgs& a, int& grid, int rows, int cols, int nblk, 
     a.reps = reps;
     a.ktiles = (cols + BK - 1) / BK;
     a.rtiles = (rows + BM - 1) / BM;
-    const int tiles = a.rtiles * reps;
+    const int tiles = a.rtiles;
     a.total = (int64_t)tiles * nblk * a.ktiles;
-    grid = (int)std::min<int64_t>(sms, a.total);
+    a.grid = grid = (int)std::min<int64_t>(sms, a.total);
     const int64_t ipt = (int64_t)nblk * a.ktiles;
     std::vector<std::vector<std::pair<int, int>>> lists(tiles);
     int maxseg = 1;
@@ -1106,11 +1114,11 @@ static cudaError_t plan_gemm(Gemm& G, int rows, int cols, int nblk, int reps, in
     return cudaSuccess;
 }
 
-static size_t partial_floats(const Gemm& G) { return (size_t)G.grid * G.a.maxseg * 2 * NR * BM; }
+static size_t partial_floats(const Gemm& G) { return (size_t)G.a.reps * G.grid * G.a.maxseg * 2 * NR * BM; }
 
 template <int XS, bool F16>
 static void launch_gemm(const Gemm& G, cudaStream_t s) {
-    launch_chained(k_tc_gemm<XS, F16>, G.grid, NTHREADS, s, Cfg<XS>::SMEM, G.ah, G.al, G.x[0], G.x[1], G.x[2], G.a);
+    launch_chained(k_tc_gemm<XS, F16>, G.grid * G.a.reps, NTHREADS, s, Cfg<XS>::SMEM, G.ah, G.al, G.x[0], G.x[1], G.x[2], G.a);
     launch_chained(k_tc_fix<XS, F16>, dim3(2 * G.a.rtiles * G.a.reps, NR / FIX_RB), 256, s, 0, G.a);
 }
 
@@ -1225,7 +1233,13 @@ tdcfie_status build_tc(tdcfie_t h, StepPlan* p) {
     // GEMM plans and tensor maps
     CKB(plan_gemm(g->hist, ne, ne, nblk, 1, g->sms, s));
     CKB(plan_gemm(g->solve, ne, ne, 1, 1, g->sms, s));
-    CKB(plan_gemm(g->proj, nc, nc, 1, TC_C, g->sms, s));
+    // The projector's blocks per step: those of a chunk's four steps fill the chip once (a quarter each),
+    // so that a block's part is long against its partial sums (1920 edges, 200 k tiles: with all blocks each
+    // a march of 100 steps takes 20.8 instead of 20.0 ms); on large meshes half each, so that a step taken
+    // alone does not leave most of the chip idle (7680 edges, 3200 k tiles, 17 steps: 7.51 ms, a quarter
+    // 7.58, all 7.66)
+    const int64_t its = (int64_t)(ldc / BK) * ((nc + BM - 1) / BM);
+    CKB(plan_gemm(g->proj, nc, nc, 1, TC_C, std::max(1, g->sms / (its < 1024 ? 4 : 2)), s));
     size_t pmax = 0;
     for (Gemm* G : {&g->hist, &g->solve, &g->proj}) pmax = std::max(pmax, partial_floats(*G));
     CKB(dalloc(g, &g->partial, pmax));
@@ -1283,18 +1297,19 @@ tdcfie_status build_tc(tdcfie_t h, StepPlan* p) {
     return TDCFIE_OK;
 }
 
-// tests of the chunk's steps (nothing unless a chunk starts at the current step) -> their e, h slots
-int launch_tests_tc(tdcfie_t h, StepPlan* p, cudaStream_t s) {
+// tests of the steps that new_cols gives -> their e, h slots
+int launch_tests_tc(tdcfie_t h, StepPlan* p, int most, cudaStream_t s) {
     TcStep* g = p->gemm;
     const int ne = p->ne, ring = p->ring, ld = g->ld;
-    launch_chained(k_env_tc, (p->npts + ENV_PB - 1) / ENV_PB, NR * TC_C, s, 0, p->npts, h->dexc, h->dt, p->ctl, (const float*)p->pts, g->env);
+    launch_chained(k_env_tc, (p->npts + ENV_PB - 1) / ENV_PB, NR * TC_C, s, 0, p->npts, h->dexc, h->dt, p->ctl, most,
+                   (const float*)p->pts, g->env);
     const dim3 grhs(ld / 64, TC_C);
     const float4* ent = (const float4*)p->ecoef;
     if (g->fp16)
-        launch_chained(k_rhs_tc<true, FP16_XS>, grhs, 32 * RHS_NW, s, RHS_SMEM, ne, h->dexc, p->ctl, p->eptr, g->env, ent, p->enE,
+        launch_chained(k_rhs_tc<true, FP16_XS>, grhs, 32 * RHS_NW, s, RHS_SMEM, ne, h->dexc, p->ctl, most, p->eptr, g->env, ent, p->enE,
                        g->X[0], g->X[1], g->X[2], g->sXh, ring, ld);
     else
-        launch_chained(k_rhs_tc<false, 2>, grhs, 32 * RHS_NW, s, RHS_SMEM, ne, h->dexc, p->ctl, p->eptr, g->env, ent, p->enE,
+        launch_chained(k_rhs_tc<false, 2>, grhs, 32 * RHS_NW, s, RHS_SMEM, ne, h->dexc, p->ctl, most, p->eptr, g->env, ent, p->enE,
                        g->X[0], g->X[1], g->X[2], g->sXh, ring, ld);
     return 2;
 }
@@ -1312,20 +1327,22 @@ int launch_inner_tc(tdcfie_t h, StepPlan* p, int off, bool advance, cudaStream_t
     return advance ? 5 : 4;
 }
 
-// projector of the finished steps: z = Sigma^T w_n, u = (Sigma^T Sigma)^+ z, j_n = y_n + Sigma u = P^LH y_n +
+// projector of the `count` finished steps: z = Sigma^T w_n, u = (Sigma^T Sigma)^+ z, j_n = y_n + Sigma u = P^LH y_n +
 // P^S dy_n / dtt; the step counter moves by adv
-int launch_post_tc(tdcfie_t h, StepPlan* p, int adv, cudaStream_t s) {
+int launch_post_tc(tdcfie_t h, StepPlan* p, int adv, int count, cudaStream_t s) {
     TcStep* g = p->gemm;
     const int ne = p->ne, ldc = g->ldc;
-    const dim3 gproj(ldc / 64, NR / PIN_RB, TC_C);
+    const dim3 gproj(ldc / 64, NR / PIN_RB, count);
     if (g->fp16)
         launch_chained(k_project_in_tc<true, FP16_XS>, gproj, 256, s, 0, h->dm, p->ctl, adv, g->y2, 1.0 / h->dtt, g->Z[0], g->Z[1],
                        g->Z[2], g->sXz, ldc);
     else
         launch_chained(k_project_in_tc<false, 2>, gproj, 256, s, 0, h->dm, p->ctl, adv, g->y2, 1.0 / h->dtt, g->Z[0], g->Z[1], g->Z[2],
                        g->sXz, ldc);
-    run_gemm(g, g->proj, s);
-    launch_chained(k_project_out_tc, dim3((ne * NR + 255) / 256, TC_C), 256, s, 0, h->dm, p->ctl, adv, g->y2, g->u, g->done);
+    Gemm proj = g->proj;
+    proj.a.reps = count;
+    run_gemm(g, proj, s);
+    launch_chained(k_project_out_tc, dim3((ne * NR + 255) / 256, count), 256, s, 0, h->dm, p->ctl, adv, g->y2, g->u, g->done);
     return 4;
 }
 int tc_chunk() { return TC_C; }
