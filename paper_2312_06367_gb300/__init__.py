@@ -313,7 +313,8 @@ class Solver:
 
 
 class Batch:
-    """Several assembled Solvers stepped by one graph launch per step (tdcfie_batch_*).
+    """Several assembled Solvers stepped together (tdcfie_batch_*): FP32 members with one wave and the
+    direct solve by one cooperative kernel for up to 32 steps, any other mix by one graph per step.
 
     The solvers are borrowed: keep them alive and close the batch first."""
 
@@ -333,7 +334,8 @@ class Batch:
 
     def tune(self, steps_per_candidate: int = 3):
         """Measure the persistent kernel's launch shapes and keep the fastest (tdcfie_batch_tune);
-        the members are reset to the start of their march.  Returns the chosen configuration."""
+        the members are reset to the start of their march.  Returns the chosen configuration
+        ("rows_per_warp": consecutive units of work per turn of a warp)."""
         cfg = np.zeros(4, dtype=np.int32)
         _lib.check(_lib.load().tdcfie_batch_tune(self._b, int(steps_per_candidate), _lib._ptr(cfg)))
         return dict(zip(("persistent", "rows_per_warp", "threads", "blocks_per_sm"), cfg.tolist()))

@@ -23,7 +23,10 @@ namespace tdc {
 //        [4] solves not converged, [5] groups done this step
 enum { NSTATS = 8 };
 constexpr int GM_T = 512, GM_W = GM_T / 32;       // threads and warps per block
-constexpr int GM_ROWS = 8;                        // rows per block, or more where the chip is full
+// Rows per block, or more where the chip is full.  us per step at 4, 8, 16, 32: 120 unknowns FP64 204, 216,
+// 229, 274; 480 FP32 196, 197, 203, 244; 768 FP32 226, 235, 253, 287; from 1920 on the chip is full.  Fewer rows
+// are more partial sums to add per block, more rows a longer product; 4 and 8 are within 6 %.
+constexpr int GM_ROWS = 8;
 constexpr int GM_TILE = 8192;                     // entries of a vector staged at a time
 
 struct GmDev {

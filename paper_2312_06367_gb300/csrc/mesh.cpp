@@ -96,8 +96,7 @@ std::string build_mesh(const double* V, int64_t nv64, const int32_t* F, int64_t 
         }
     m.D = std::sqrt(D);
 
-    // ---------------- barycentric refinement
-    // longest edge; ordered pairs of triangles that share a vertex
+    // ---------------- for the quadrature: longest edge; ordered pairs of triangles that share a vertex
     for (int e = 0; e < ne; ++e) {
         double l2 = 0.0;
         for (int k = 0; k < 3; ++k) {
@@ -119,6 +118,8 @@ std::string build_mesh(const double* V, int64_t nv64, const int32_t* F, int64_t 
             for (int o : nb) { m.touch.push_back(c); m.touch.push_back(o); }
         }
     }
+
+    // ---------------- barycentric refinement
     const int nfv = nv + ne + nc;
     m.fV.resize(3 * (size_t)nfv);
     for (int i = 0; i < 3 * nv; ++i) m.fV[i] = m.V[i];
