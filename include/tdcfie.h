@@ -230,7 +230,8 @@ tdcfie_status tdcfie_history_stats(tdcfie_t h, int32_t* form, int64_t* nnz, doub
  * tdcfie_replan or tdcfie_set_solver on a member.  Host work plus the work lists' upload.
  * tdcfie_batch_step: every handle must have its excitation set; currents_out is NULL (discard) or a
  * host array of n DEVICE pointers laid out as in tdcfie_step for each handle (entries may be NULL).
- * Synchronous; a member's non-finite current or device timeout is returned with its index.
+ * Synchronous, and ordered after what is queued on the members' streams (opts.stream; the legacy default
+ * stream for handles without one); a member's non-finite current or device timeout is returned with its index.
  * tdcfie_batch_tune (persistent form): times every candidate launch shape (units per turn of a warp
  * 1/2/4, 64/128/256 threads per block, 1/2/4 blocks per SM within the occupancy limit) for
  * steps_per_candidate steps each (rounded up to a multiple of 16) and keeps the fastest; the candidates march the members, which

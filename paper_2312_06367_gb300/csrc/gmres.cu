@@ -10,7 +10,7 @@
 // touches its rows, and what the group sums passes through one partial per block, added by every
 // block in the same order: the Hessenberg column, the rotations and every decision are formed by all
 // blocks alike, and the results do not depend on timing.  Latency bounds it; 100 steps at 768 unknowns,
-// FP32, took 46.3 ms with an iteration as seven kernels in a graph loop, 23.9 ms so.
+// FP32, took 45.6 ms with an iteration as seven kernels in a graph loop, 22.8 ms so.
 #include <cmath>
 
 #include "gmres.h"

@@ -89,9 +89,9 @@ __device__ __forceinline__ void advance(const SimtDev<T>& d, int adv) {
 // Columns lo .. hi - 1 of the current chunk whose tests and pre-sums are formed at this step: all of them
 // where a chunk starts.  In the march's first chunk (the steps 1 .. C), where the lags that reach back before
 // it meet y_i = 0 and only the tests' blocks count, each call forms those of its own steps: a march may
-// end there, and one of a few steps does not pay for C (a march of one step, 1920 edges, K = 42, FP64: 2.33 ms
-// with the chunk formed whole, 0.33 ms so; with eight waves 15.8 and 0.74 ms).  most: the call's steps from this one on, 0: up to
-// ctl->last.
+// end there, and one of a few steps does not pay for C (one step, 1920 edges, K = 42, FP64: 2.33 ms with
+// the chunk formed whole, 0.20 ms so; with eight waves 15.8 and 0.64 ms).  most: the call's steps from this
+// one on, 0: up to ctl->last.
 struct Cols { int lo, hi; bool first; };
 __device__ __forceinline__ Cols new_cols(const Ctl* ctl, int C, int64_t n, int col, int most) {
     if (n - col != 1) return Cols{0, col ? 0 : C, false};

@@ -753,7 +753,7 @@ __global__ void __launch_bounds__(256) k_split_x(const double* __restrict__ x, i
 // The tests of a chunk's TC_C steps are formed when it starts (in the march's first chunk: of the steps that
 // the calls make, new_cols), in two kernels: the envelope increments
 // once per quadrature point, step and wave (a point belongs to three RWG or about twelve BC functions:
-// with one exponential pair per edge and point this took 106 us per step at 1920 edges, now 27 + 82 us per
+// with one exponential pair per edge and point this took 106 us per step at 1920 edges, now 28 + 93 us per
 // four steps), then one block
 // per (64-edge tile, step) gathers them, compensated FP32 sums over the points, and splits the tile into
 // the e and h slices of the step's slots with one scale per (slot, tile, wave).
